@@ -6,9 +6,13 @@
 // followed by F^{-1} = F^*/n3; the imaginary parts of the DC and Nyquist
 // slices are ignored, i.e. the real part of the mirrored inverse).
 //
-// Layout: the plane index e = i*n2 + j runs fastest, so a CTA that owns a tile
-// of consecutive e for every t reads and writes whole cache lines; the
-// transform of one tube runs out of shared memory.
+// Layout: the plane index e = i*n2 + j runs fastest, so neighbouring threads own
+// neighbouring tubes and every load and store is a contiguous run.  Which kernel:
+//   n3 = 2, 4, .., 128      one thread (FP64, 128: two) per tube, in registers;
+//   other n3 <= 160         folded direct products (FP64: where they take fewer
+//                           operations than mixed-radix passes, rdft_better);
+//   the rest                mixed-radix passes out of shared memory, and a direct
+//                           sum for tubes too long for those.
 #include "common.cuh"
 #include "kernels.cuh"
 
@@ -117,8 +121,8 @@ static int tile_e(int n3, size_t elem, size_t celem, bool inverse) {
 }
 
 // ---------------------------------------------------------------------------
-// Mixed-radix FFT of the tubes (Stockham autosort, radices 4, 2, 3, 5 and any
-// remaining prime).  A CTA owns a tile of FFT_TUBES consecutive tubes; two real
+// Mixed-radix FFT of the tubes for the lengths above 160 and the smooth FP64 ones
+// (Stockham autosort, radices 4, 2, 3, 5 and any remaining prime).  A CTA owns a tile of FFT_TUBES consecutive tubes; two real
 // tubes are packed into one complex sequence z = x + i y and each warp
 // transforms whole sequences in shared memory (lane-parallel butterflies,
 // warp barriers between passes).  The half spectra are separated as
@@ -240,49 +244,23 @@ __device__ C* fft_run(C* a, C* b, const C* tw, const FftPlan& P, int lane, int n
   return a;
 }
 
-// The same transform for a length known at compile time (powers of two up to
-// 128): the pass sequence (radix 4 while possible, then 2, as make_plan) is
-// unrolled and every index division and modulus becomes a shift or a mask.
-template <typename C, int N, int NS>
-__device__ __forceinline__ C* fft_run_c(C* a, C* b, const C* tw, int lane, int nseq) {
-  if constexpr (NS >= N) {
-    return a;
-  } else {
-    constexpr int R = ((N / NS) % 4 == 0) ? 4 : 2;
-    fft_pass_fixed<C, R>(a, b, tw, N, NS, lane, nseq);
-    __syncwarp();
-    return fft_run_c<C, N, NS * R>(b, a, tw, lane, nseq);
-  }
-}
-
-template <typename T>
-constexpr size_t fft_smem_c(int n, int tt) {
-  return sizeof(cx_t<T>) * ((size_t)n + (size_t)FFT_WARPS * 2 * fft_seqs(n) * n + (size_t)(n / 2 + 1) * (tt + 1)) +
-         sizeof(T) * (size_t)n * (tt + 1);
-}
-// tubes per CTA (the choice fft_setup makes at run time): the widest tile that leaves room for
-// three CTAs per SM (measured: n = 128 in FP32 went from 64 tubes, two CTAs per SM, to 32),
-// else the widest within 110 KB
+// tubes per CTA of the mixed-radix kernels: the widest tile that leaves room for three CTAs per
+// SM, else the widest within 110 KB
 constexpr size_t FFT_SMEM_3 = 72 * 1024, FFT_SMEM_MAX = 110 * 1024;
 constexpr int fft_pick_tt(size_t s64, size_t s32, size_t s16) {
   return s64 <= FFT_SMEM_3 ? 64 : s32 <= FFT_SMEM_3 ? 32 : s16 <= FFT_SMEM_3 ? 16 :
          s64 <= FFT_SMEM_MAX ? 64 : s32 <= FFT_SMEM_MAX ? 32 : s16 <= FFT_SMEM_MAX ? 16 : 0;
 }
 template <typename T>
-constexpr int fft_tt(int n) {
-  return fft_pick_tt(fft_smem_c<T>(n, 64), fft_smem_c<T>(n, 32), fft_smem_c<T>(n, 16));
-}
-
-template <typename T, int NC>  // NC: compile-time length (0: the plan's)
 __global__ void __launch_bounds__(FFT_WARPS * 32) k_rfft3_fft(const T* __restrict__ X, cx_t<T>* __restrict__ Xh,
                                                               long plane, FftPlan P) {
   using C = cx_t<T>;
   extern __shared__ __align__(16) unsigned char fsm[];
-  const int n = NC ? NC : P.n, h = n / 2 + 1, TT = NC ? fft_tt<T>(NC) : P.tubes;
+  const int n = P.n, h = n / 2 + 1, TT = P.tubes;
   C* tw = (C*)fsm;                                  // [n]
   C* zb = tw + n;                                   // [FFT_WARPS][2][seqs][n]
   const int LD = TT + 1;                            // padded row stride: conflict-free column walks
-  C* otile = zb + (size_t)FFT_WARPS * 2 * (NC ? fft_seqs(NC) : P.seqs) * n;  // [h][LD] complex
+  C* otile = zb + (size_t)FFT_WARPS * 2 * P.seqs * n;  // [h][LD] complex
   T* itile = (T*)(otile + (size_t)h * LD);          // [n][LD] real
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long e0 = (long)blockIdx.x * TT;
@@ -331,7 +309,7 @@ __global__ void __launch_bounds__(FFT_WARPS * 32) k_rfft3_fft(const T* __restric
     }
   }
   __syncthreads();
-  const int B = NC ? fft_seqs(NC) : P.seqs;
+  const int B = P.seqs;
   C* za = zb + (size_t)warp * 2 * B * n;
   C* zc = za + (size_t)B * n;
   const T hf = T(0.5);
@@ -342,9 +320,7 @@ __global__ void __launch_bounds__(FFT_WARPS * 32) k_rfft3_fft(const T* __restric
       za[q] = mkc(itile[t * LD + 2 * s], itile[t * LD + 2 * s + 1]);
     }
     __syncwarp();
-    const C* Z;
-    if constexpr (NC > 0) Z = fft_run_c<C, NC, 1>(za, zc, tw, lane, nseq);
-    else Z = fft_run<C>(za, zc, tw, P, lane, nseq);
+    const C* Z = fft_run<C>(za, zc, tw, P, lane, nseq);
     for (int q = lane; q < nseq * h; q += 32) {
       const int sq = q / h, k = q - sq * h, s = s0 + sq;
       const C zk = Z[sq * n + k], zn = Z[sq * n + (n - k) % n];
@@ -371,16 +347,16 @@ __global__ void __launch_bounds__(FFT_WARPS * 32) k_rfft3_fft(const T* __restric
   }
 }
 
-template <typename T, int NC>  // NC: compile-time length (0: the plan's)
+template <typename T>
 __global__ void __launch_bounds__(FFT_WARPS * 32) k_irfft3_fft(const cx_t<T>* __restrict__ Xh, T* __restrict__ X,
                                                                long plane, FftPlan P) {
   using C = cx_t<T>;
   extern __shared__ __align__(16) unsigned char fsm[];
-  const int n = NC ? NC : P.n, h = n / 2 + 1, TT = NC ? fft_tt<T>(NC) : P.tubes;
+  const int n = P.n, h = n / 2 + 1, TT = P.tubes;
   C* tw = (C*)fsm;                                  // [n]
   C* zb = tw + n;                                   // [FFT_WARPS][2][seqs][n]
   const int LD = TT + 1;                            // padded row stride: conflict-free column walks
-  C* itile = zb + (size_t)FFT_WARPS * 2 * (NC ? fft_seqs(NC) : P.seqs) * n;  // [h][LD] complex
+  C* itile = zb + (size_t)FFT_WARPS * 2 * P.seqs * n;  // [h][LD] complex
   T* otile = (T*)(itile + (size_t)h * LD);          // [n][LD] real
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long e0 = (long)blockIdx.x * TT;
@@ -406,7 +382,7 @@ __global__ void __launch_bounds__(FFT_WARPS * 32) k_irfft3_fft(const cx_t<T>* __
     }
   }
   __syncthreads();
-  const int B = NC ? fft_seqs(NC) : P.seqs;
+  const int B = P.seqs;
   C* za = zb + (size_t)warp * 2 * B * n;
   C* zc = za + (size_t)B * n;
   const T inv = T(1) / T(n);
@@ -425,9 +401,7 @@ __global__ void __launch_bounds__(FFT_WARPS * 32) k_irfft3_fft(const cx_t<T>* __
       za[q] = mkc(x.x - y.y, x.y + y.x);  // Z = X + i Y
     }
     __syncwarp();
-    const C* z;
-    if constexpr (NC > 0) z = fft_run_c<C, NC, 1>(za, zc, tw, lane, nseq);
-    else z = fft_run<C>(za, zc, tw, P, lane, nseq);
+    const C* z = fft_run<C>(za, zc, tw, P, lane, nseq);
     for (int q = lane; q < nseq * n; q += 32) {
       const int sq = q / n, t = q - sq * n, s = s0 + sq;
       otile[t * LD + 2 * s] = z[q].x * inv;
@@ -441,6 +415,656 @@ __global__ void __launch_bounds__(FFT_WARPS * 32) k_irfft3_fft(const cx_t<T>* __
     const long ge = e0 + e;
     if (ge < plane) X[(long)t * plane + ge] = otile[t * LD + e];
   }
+}
+
+// ---------------------------------------------------------------------------
+// Powers of two up to 64 (FP32: 128): one thread transforms one tube in its
+// registers.  The n = 2 M real samples are the complex sequence
+// z_j = x_2j + i x_2j+1; its M-point transform (radix 4, then 2, decimation in
+// frequency, every index and twiddle a compile-time constant) is separated into
+// the half spectrum with one rotation per pair of frequencies.  Neighbouring
+// threads hold neighbouring tubes, so every load and store of a warp is one
+// contiguous run and a thread has its n loads in flight together; nothing goes
+// through shared memory, whose butterfly passes bounded the earlier kernel.
+// Bound: the bytes in FP32 (n = 128, 512 x 512 plane: 110 -> 55 us forward, 147 ->
+// 54 inverse, 40 us at the copy rate; 64: 56 -> 25, 73 -> 23, 20), the FP64 pipe
+// in FP64 (64: 539 -> 341 us).
+// ---------------------------------------------------------------------------
+namespace ct {
+constexpr double kTau = 6.283185307179586476925286766559;
+constexpr double csin(double x) {
+  double t = x, s = x;
+  for (int k = 1; k < 12; ++k) {
+    t *= -x * x / (2.0 * k * (2.0 * k + 1.0));
+    s += t;
+  }
+  return s;
+}
+constexpr double ccos(double x) {
+  double t = 1.0, s = 1.0;
+  for (int k = 1; k < 12; ++k) {
+    t *= -x * x / ((2.0 * k - 1.0) * 2.0 * k);
+    s += t;
+  }
+  return s;
+}
+// cos and sin of 2 pi p / n (Taylor series on the first octant; exact on the axes)
+constexpr double cos2pi(long p, long n) {
+  p %= n;
+  if (2 * p > n) p = n - p;
+  if (4 * p == n) return 0.0;
+  if (4 * p > n) return -cos2pi(n - 2 * p, 2 * n);
+  if (8 * p > n) return csin(kTau * (double)(n - 4 * p) / (4.0 * (double)n));
+  return ccos(kTau * (double)p / (double)n);
+}
+constexpr double sin2pi(long p, long n) {  // cos(theta - pi/2)
+  return cos2pi(((4 * p - n) % (4 * n) + 4 * n) % (4 * n), 4 * n);
+}
+// position of frequency k in the output of dif_fft<., M, .>
+constexpr int pos(int k, int len) { return len <= 2 ? k : (k % 4) * (len / 4) + pos(k / 4, len / 4); }
+}  // namespace ct
+
+template <int V>
+struct IntC {
+  static constexpr int value = V;
+};
+template <int B, int E, typename F>
+__device__ __forceinline__ void static_for(F&& f) {
+  if constexpr (B < E) {
+    f(IntC<B>());
+    static_for<B + 1, E>(static_cast<F&&>(f));
+  }
+}
+
+// v <- v * exp(SGN 2 pi i p / n)
+template <typename T, int SGN, int P, int N>
+__device__ __forceinline__ cx_t<T> rot(cx_t<T> v) {
+  if constexpr (P % N == 0) {
+    return v;
+  } else {
+    constexpr T c = (T)ct::cos2pi(P, N), sn = (T)(SGN * ct::sin2pi(P, N));
+    return mkc(v.x * c - v.y * sn, v.x * sn + v.y * c);
+  }
+}
+
+template <typename T, int SGN, int M, int LEN = M>
+__device__ __forceinline__ void dif_fft(cx_t<T> (&v)[M]) {
+  using C = cx_t<T>;
+  if constexpr (LEN >= 4) {
+    constexpr int Q = LEN / 4;
+    static_for<0, M / LEN>([&](auto b_) {
+      static_for<0, Q>([&](auto j_) {
+        constexpr int j = decltype(j_)::value, i0 = decltype(b_)::value * LEN + j;
+        const C a = cadd(v[i0], v[i0 + 2 * Q]), b = csub(v[i0], v[i0 + 2 * Q]);
+        const C c = cadd(v[i0 + Q], v[i0 + 3 * Q]), d = csub(v[i0 + Q], v[i0 + 3 * Q]);
+        const C di = SGN < 0 ? mkc(d.y, -d.x) : mkc(-d.y, d.x);
+        v[i0] = cadd(a, c);
+        v[i0 + Q] = rot<T, SGN, j, LEN>(cadd(b, di));
+        v[i0 + 2 * Q] = rot<T, SGN, 2 * j, LEN>(csub(a, c));
+        v[i0 + 3 * Q] = rot<T, SGN, 3 * j, LEN>(csub(b, di));
+      });
+    });
+    dif_fft<T, SGN, M, Q>(v);
+  } else if constexpr (LEN == 2) {
+    static_for<0, M / 2>([&](auto b_) {
+      constexpr int i0 = 2 * decltype(b_)::value;
+      const C a = v[i0], b = v[i0 + 1];
+      v[i0] = cadd(a, b);
+      v[i0 + 1] = csub(a, b);
+    });
+  }
+}
+
+template <typename T, int N>
+__global__ void __launch_bounds__(128) k_rfft3_reg(const T* __restrict__ X, cx_t<T>* __restrict__ Xh, long plane) {
+  using C = cx_t<T>;
+  constexpr int M = N / 2;
+  const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= plane) return;
+  X += e;
+  Xh += e;
+  C v[M];
+  static_for<0, M>([&](auto j_) {
+    constexpr int j = decltype(j_)::value;
+    v[j] = mkc(__ldg(X + (2 * j) * plane), __ldg(X + (2 * j + 1) * plane));
+  });
+  dif_fft<T, -1, M>(v);
+  Xh[0] = mkc(v[0].x + v[0].y, T(0));
+  Xh[M * plane] = mkc(v[0].x - v[0].y, T(0));
+  static_for<1, M / 2 + 1>([&](auto k_) {
+    constexpr int k = decltype(k_)::value;
+    const C z = v[ct::pos(k, M)];
+    if constexpr (2 * k == M) {
+      Xh[k * plane] = mkc(z.x, -z.y);
+    } else if constexpr (2 * k < M) {
+      const C y = v[ct::pos(M - k, M)];
+      const T hf = T(0.5);
+      const C ev = mkc(hf * (z.x + y.x), hf * (z.y - y.y));
+      const C od = rot<T, -1, k, N>(mkc(hf * (z.y + y.y), hf * (y.x - z.x)));
+      Xh[k * plane] = cadd(ev, od);
+      Xh[(M - k) * plane] = mkc(ev.x - od.x, od.y - ev.y);
+    }
+  });
+}
+
+template <typename T, int N>
+__global__ void __launch_bounds__(128) k_irfft3_reg(const cx_t<T>* __restrict__ Xh, T* __restrict__ X, long plane) {
+  using C = cx_t<T>;
+  constexpr int M = N / 2;
+  const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= plane) return;
+  X += e;
+  Xh += e;
+  C v[M];
+  {
+    const T a = Xh[0].x, b = Xh[M * plane].x;  // the DC and Nyquist slices are real
+    v[0] = mkc(a + b, a - b);
+  }
+  static_for<1, M / 2 + 1>([&](auto k_) {
+    constexpr int k = decltype(k_)::value;
+    const C x = Xh[k * plane];
+    if constexpr (2 * k == M) {
+      v[k] = mkc(T(2) * x.x, T(-2) * x.y);
+    } else if constexpr (2 * k < M) {
+      const C y = Xh[(M - k) * plane];
+      const C ev = mkc(x.x + y.x, x.y - y.y);
+      const C od = rot<T, +1, k, N>(mkc(x.x - y.x, x.y + y.y));
+      v[k] = mkc(ev.x - od.y, ev.y + od.x);
+      v[M - k] = mkc(ev.x + od.y, od.x - ev.y);
+    }
+  });
+  dif_fft<T, +1, M>(v);
+  constexpr T inv = T(1) / T(N);
+  static_for<0, M>([&](auto j_) {
+    constexpr int j = decltype(j_)::value;
+    const C z = v[ct::pos(j, M)];
+    X[(2 * j) * plane] = z.x * inv;
+    X[(2 * j + 1) * plane] = z.y * inv;
+  });
+}
+
+// FP64, n = 128: two threads per tube (16 lanes apart), each with the 64-point transform of every
+// second sample in its registers (the whole tube would not fit): X_k = E_k + omega^k O_k and
+// X_n/2-k = conj(E_k - omega^k O_k), E of the even and O of the odd samples, exchanged by shuffles.
+template <typename T, int N>
+__global__ void __launch_bounds__(128) k_rfft3_reg2(const T* __restrict__ X, cx_t<T>* __restrict__ Xh, long plane) {
+  using C = cx_t<T>;
+  constexpr int M = N / 4;  // complex points per thread
+  const int odd = (threadIdx.x >> 4) & 1;
+  const long e = ((long)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / 2 + (threadIdx.x & 15);
+  const bool live = e < plane;
+  X += (live ? e : 0) + odd * plane;
+  Xh += live ? e : 0;
+  C v[M];
+  static_for<0, M>([&](auto j_) {
+    constexpr int j = decltype(j_)::value;
+    v[j] = mkc(__ldg(X + (4 * j) * plane), __ldg(X + (4 * j + 2) * plane));
+  });
+  dif_fft<T, -1, M>(v);
+  // this thread's spectrum value f of frequency k: combined with its partner's, stored
+  auto emit = [&](auto k_, C f) {
+    constexpr int k = decltype(k_)::value;
+    const C own = odd ? rot<T, -1, k, N>(f) : f;
+    const C other = mkc(__shfl_xor_sync(0xffffffffu, own.x, 16), __shfl_xor_sync(0xffffffffu, own.y, 16));
+    if (!live) return;
+    if (!odd) Xh[k * plane] = mkc(own.x + other.x, k == 0 ? T(0) : own.y + other.y);
+    else if constexpr (4 * k != N) Xh[(N / 2 - k) * plane] = mkc(other.x - own.x, k == 0 ? T(0) : own.y - other.y);
+  };
+  emit(IntC<0>(), mkc(v[0].x + v[0].y, T(0)));
+  emit(IntC<M>(), mkc(v[0].x - v[0].y, T(0)));
+  static_for<1, M / 2 + 1>([&](auto k_) {
+    constexpr int k = decltype(k_)::value;
+    const C z = v[ct::pos(k, M)];
+    if constexpr (2 * k == M) {
+      emit(k_, mkc(z.x, -z.y));
+    } else if constexpr (2 * k < M) {
+      const C y = v[ct::pos(M - k, M)];
+      const T hf = T(0.5);
+      const C ev = mkc(hf * (z.x + y.x), hf * (z.y - y.y));
+      const C od = rot<T, -1, k, 2 * M>(mkc(hf * (z.y + y.y), hf * (y.x - z.x)));
+      emit(k_, cadd(ev, od));
+      emit(IntC<M - k>(), mkc(ev.x - od.x, od.y - ev.y));
+    }
+  });
+}
+
+template <typename T, int N>
+__global__ void __launch_bounds__(128) k_irfft3_reg2(const cx_t<T>* __restrict__ Xh, T* __restrict__ X, long plane) {
+  using C = cx_t<T>;
+  constexpr int M = N / 4;
+  const int odd = (threadIdx.x >> 4) & 1;
+  const long e = ((long)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / 2 + (threadIdx.x & 15);
+  if (e >= plane) return;
+  Xh += e;
+  X += e + odd * plane;
+  // twice the spectrum of this thread's samples: X_k + conj X_n/2-k, or omega^-k (X_k - conj X_n/2-k)
+  auto part = [&](auto k_) {
+    constexpr int k = decltype(k_)::value;
+    C a = Xh[k * plane], b = Xh[(N / 2 - k) * plane];
+    if constexpr (k == 0) a.y = b.y = T(0);  // the DC and Nyquist slices are real
+    const C od = rot<T, +1, k, N>(mkc(a.x - b.x, a.y + b.y));
+    return odd ? od : mkc(a.x + b.x, a.y - b.y);
+  };
+  C v[M];
+  {
+    const T a = part(IntC<0>()).x, b = part(IntC<M>()).x;
+    v[0] = mkc(a + b, a - b);
+  }
+  static_for<1, M / 2 + 1>([&](auto k_) {
+    constexpr int k = decltype(k_)::value;
+    const C x = part(k_);
+    if constexpr (2 * k == M) {
+      v[k] = mkc(T(2) * x.x, T(-2) * x.y);
+    } else if constexpr (2 * k < M) {
+      const C y = part(IntC<M - k>());
+      const C ev = mkc(x.x + y.x, x.y - y.y);
+      const C od = rot<T, +1, k, 2 * M>(mkc(x.x - y.x, x.y + y.y));
+      v[k] = mkc(ev.x - od.y, ev.y + od.x);
+      v[M - k] = mkc(ev.x + od.y, od.x - ev.y);
+    }
+  });
+  dif_fft<T, +1, M>(v);
+  constexpr T inv = T(1) / T(N);
+  static_for<0, M>([&](auto j_) {
+    constexpr int j = decltype(j_)::value;
+    const C z = v[ct::pos(j, M)];
+    X[(4 * j) * plane] = z.x * inv;
+    X[(4 * j + 2) * plane] = z.y * inv;
+  });
+}
+
+// ---------------------------------------------------------------------------
+// Any other length up to RDFT_MAX: the half spectrum as a small real matrix
+// product.  The samples are folded by symmetry while they are staged: for odd n
+//   Re X_k = x_0 + sum_j P_j cos(j k tau/n),  Im X_k = -sum_j Q_j sin(j k tau/n),
+//   P_j = x_j + x_n-j, Q_j = x_j - x_n-j, j = 1 .. (n-1)/2;
+// for even n = 2m the even and the odd frequencies first separate into the sums
+// s_j = x_j + x_j+m and differences d_j = x_j - x_j+m, each folded again (odd
+// frequencies: P_j = d_j - d_m-j, Q_j = d_j + d_m-j), which halves the products:
+// n/2 (odd n) or n/4 (even n) multiply-adds per sample, inside the time the
+// bytes take in FP32.  The inverse runs the same table the other way: for each
+// t the sums over even and odd k give the samples t, m-t, m+t and n-t.
+// A thread holds KB frequencies of a vector of neighbouring tubes; each operand
+// pair read from shared memory feeds 2 KB V multiply-adds.  Sums are taken in
+// runs of 8 terms (their rounding then stays below a mixed-radix transform's).
+// 512 x 512 plane, against the mixed-radix passes: FP32 n = 33 235 -> 36 us, 100
+// 199 -> 122, 31 1446 -> 32 (prime radices ran serially), FP64 33 2304 -> 378;
+// FP32 is bound by load latency and shared-memory reads (bytes alone: 31 us at
+// n = 100), FP64 by its multiply-adds (1130 of 1480 us at n = 100).
+// ---------------------------------------------------------------------------
+constexpr int RDFT_MAX = 160;
+template <typename T>
+struct RVec;
+template <>
+struct RVec<float> {  // (64 tubes x 8 frequencies per warp and 256 threads measured slower: 121 -> 140 us at n = 100)
+  using type = float4;
+  static constexpr int V = 4, KB = 4, THREADS = 128;
+};
+template <>
+struct RVec<double> {
+  using type = double2;
+  static constexpr int V = 2, KB = 4, THREADS = 128;
+};
+__device__ __forceinline__ void unpack(float4 v, float* o) { o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w; }
+__device__ __forceinline__ void unpack(double2 v, double* o) { o[0] = v.x; o[1] = v.y; }
+
+// KB consecutive twiddles (16-byte aligned) in 16-byte loads
+template <int KB>
+__device__ __forceinline__ void load_row(const float2* p, float2* o) {
+#pragma unroll
+  for (int q = 0; q < KB; q += 2) {
+    const float4 v = *(const float4*)(p + q);
+    o[q] = make_float2(v.x, v.y);
+    o[q + 1] = make_float2(v.z, v.w);
+  }
+}
+template <int KB>
+__device__ __forceinline__ void load_row(const double2* p, double2* o) {
+#pragma unroll
+  for (int q = 0; q < KB; ++q) o[q] = p[q];
+}
+
+// the two halves of the folded problem (one for odd n)
+struct RdftDims {
+  int n, types, m, J, half, hc[2], hp[2], HP;
+};
+__host__ __device__ inline RdftDims rdft_dims(int n, int KB) {
+  RdftDims d;
+  d.n = n;
+  d.types = (n % 2 == 0) ? 2 : 1;
+  d.m = n / d.types;
+  d.J = (d.m - 1) / 2;
+  d.half = (d.m % 2 == 0) ? 1 : 0;  // a middle sample (only for even n)
+  const int h = n / 2 + 1;
+  d.hc[0] = d.types == 2 ? (h + 1) / 2 : h;
+  d.hc[1] = d.types == 2 ? h / 2 : 0;
+  for (int t = 0; t < 2; ++t) d.hp[t] = (d.hc[t] + KB - 1) / KB * KB;
+  d.HP = d.hp[0] + d.hp[1];
+  return d;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(RVec<T>::THREADS, 4) k_rdft3(const T* __restrict__ X, cx_t<T>* __restrict__ Xh, long plane,
+                                                        int n, int lgE) {
+  using C = cx_t<T>;
+  using VT = typename RVec<T>::type;
+  constexpr int V = RVec<T>::V, KB = RVec<T>::KB, THR = RVec<T>::THREADS;
+  extern __shared__ __align__(16) unsigned char fsm[];
+  const RdftDims d = rdft_dims(n, KB);
+  const int J = d.J, m = d.m, rows = 2 * J + 2;  // per half: P_1..P_J, Q_1..Q_J, first, middle
+  T* dat = (T*)fsm;                              // [types][rows][E]
+  C* tab = (C*)(dat + ((size_t)d.types * rows << lgE));  // [J][HP]
+  C* tw = tab + (size_t)J * d.HP;                   // [n]
+  const int tid = threadIdx.x, E = 1 << lgE;
+  for (int p = tid; p < n; p += THR) tw[p] = twiddle<T>(p, n, +1);
+  __syncthreads();
+  for (int i = tid; i < J * d.HP; i += THR) {
+    const int j = i / d.HP + 1, c = i - (j - 1) * d.HP;
+    const int t = c >= d.hp[0], q = c - (t ? d.hp[0] : 0);
+    tab[i] = tw[(j * (d.types == 2 ? 2 * q + t : q)) % n];
+  }
+  // persistent CTAs: the table is made once for all the tiles a CTA takes
+  for (long tile = blockIdx.x; (tile << lgE) < plane; tile += gridDim.x) {
+  const long e0 = tile << lgE;
+  __syncthreads();  // the previous tile's samples have been read
+  auto ld = [&](int j, long ge) { return ge < plane ? __ldg(X + (long)j * plane + ge) : T(0); };
+#pragma unroll 4
+  for (int i = tid; i < J * E; i += THR) {
+    const int j = (i >> lgE) + 1, e = i & (E - 1);
+    const long ge = e0 + e;
+    if (d.types == 1) {
+      const T a = ld(j, ge), b = ld(n - j, ge);
+      dat[(j - 1) * E + e] = a + b;
+      dat[(J + j - 1) * E + e] = a - b;
+    } else {
+      const T a = ld(j, ge), b = ld(m - j, ge), c = ld(m + j, ge), f = ld(n - j, ge);
+      const T s0 = a + c, s1 = b + f, d0 = a - c, d1 = b - f;
+      T* o = dat + (size_t)rows * E;
+      dat[(j - 1) * E + e] = s0 + s1;
+      dat[(J + j - 1) * E + e] = s0 - s1;
+      o[(j - 1) * E + e] = d0 - d1;
+      o[(J + j - 1) * E + e] = d0 + d1;
+    }
+  }
+  for (int e = tid; e < E; e += THR) {
+    const long ge = e0 + e;
+    T* f0 = dat + 2 * J * E + e;
+    if (d.types == 1) {
+      f0[0] = ld(0, ge);
+    } else {
+      const T a = ld(0, ge), b = ld(m, ge);
+      T* f1 = f0 + (size_t)rows * E;
+      f0[0] = a + b;
+      f1[0] = a - b;
+      if (d.half) {
+        const T c = ld(m / 2, ge), f = ld(m / 2 + m, ge);
+        f0[E] = c + f;
+        f1[E] = c - f;
+      }
+    }
+  }
+  __syncthreads();
+  const int L = E / V, items = d.HP / KB * L;
+  for (int it = tid; it < items; it += THR) {
+    const int lane = it % L, c0 = it / L * KB;
+    const int t = c0 >= d.hp[0];
+    const T* P = dat + (size_t)t * rows * E + lane * V;
+    const T* Q = P + J * E;
+    T re[KB][V], im[KB][V];
+    {
+      T f[V], g[V];
+      unpack(*(const VT*)(P + 2 * J * E), f);
+#pragma unroll
+      for (int u = 0; u < V; ++u) g[u] = T(0);
+      if (d.half) unpack(*(const VT*)(P + (2 * J + 1) * E), g);
+#pragma unroll
+      for (int q = 0; q < KB; ++q) {
+        // the middle sample: (-1)^k' on the real part (even frequencies) or on -Im (odd ones)
+        const T sg = ((c0 - (t ? d.hp[0] : 0) + q) & 1) ? T(-1) : T(1);
+#pragma unroll
+        for (int u = 0; u < V; ++u) {
+          re[q][u] = t ? f[u] : f[u] + sg * g[u];
+          im[q][u] = t ? sg * g[u] : T(0);
+        }
+      }
+    }
+    const C* w = tab + c0;
+    for (int j0 = 0; j0 < J; j0 += 8) {
+      T sr[KB][V], si[KB][V];
+#pragma unroll
+      for (int q = 0; q < KB; ++q)
+#pragma unroll
+        for (int u = 0; u < V; ++u) sr[q][u] = si[q][u] = T(0);
+      const int j1 = min(J, j0 + 8);
+#pragma unroll 4
+      for (int j = j0; j < j1; ++j) {
+        T pv[V], qv[V];
+        unpack(*(const VT*)(P + j * E), pv);
+        unpack(*(const VT*)(Q + j * E), qv);
+        C c[KB];
+        load_row<KB>(w + (size_t)j * d.HP, c);
+#pragma unroll
+        for (int q = 0; q < KB; ++q)
+#pragma unroll
+          for (int u = 0; u < V; ++u) {
+            sr[q][u] = fma(pv[u], c[q].x, sr[q][u]);
+            si[q][u] = fma(qv[u], c[q].y, si[q][u]);
+          }
+      }
+#pragma unroll
+      for (int q = 0; q < KB; ++q)
+#pragma unroll
+        for (int u = 0; u < V; ++u) {
+          re[q][u] += sr[q][u];
+          im[q][u] += si[q][u];
+        }
+    }
+    const int q0 = c0 - (t ? d.hp[0] : 0);
+#pragma unroll
+    for (int q = 0; q < KB; ++q) {
+      if (q0 + q >= d.hc[t]) continue;
+      const int k = d.types == 2 ? 2 * (q0 + q) + t : q0 + q;
+      const long ge = e0 + lane * V;
+      C* dst = Xh + (long)k * plane + ge;
+      if (sizeof(T) == 4 && ge + V <= plane && ((uintptr_t)dst & 15) == 0) {
+#pragma unroll
+        for (int u = 0; u < V; u += 2)
+          *(float4*)(dst + u) = make_float4((float)re[q][u], (float)-im[q][u], (float)re[q][u + 1],
+                                            (float)-im[q][u + 1]);
+      } else {
+#pragma unroll
+        for (int u = 0; u < V; ++u)
+          if (ge + u < plane) dst[u] = mkc(re[q][u], -im[q][u]);
+      }
+    }
+  }
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(RVec<T>::THREADS, 3) k_irdft3(const cx_t<T>* __restrict__ Xh, T* __restrict__ X,
+                                                         long plane, int n, int lgE) {
+  using C = cx_t<T>;
+  using VT = typename RVec<T>::type;
+  constexpr int V = RVec<T>::V, KB = RVec<T>::KB, THR = RVec<T>::THREADS;
+  extern __shared__ __align__(16) unsigned char fsm[];
+  const int types = (n % 2 == 0) ? 2 : 1, m = n / types;
+  const int K = (n - 1) / 2;                       // interior frequencies 1 .. K
+  const int K0 = types == 2 ? K / 2 : K;           // even ones (2, 4, ..) first, then the odd ones
+  const int tc = m / 2 + 1, HP = (tc + KB - 1) / KB * KB;  // t = 0 .. m/2
+  const int tid = threadIdx.x, E = 1 << lgE;
+  T* dr = (T*)fsm;                                 // [K + 2][E] 2 Re X_k, then Re X_0, Re X_n/2
+  T* di = dr + (size_t)(K + 2) * E;                // [K][E] 2 Im X_k
+  C* tab = (C*)(di + (size_t)K * E);               // [K][HP]
+  C* tw = tab + (size_t)K * HP;                    // [n]
+  for (int p = tid; p < n; p += THR) tw[p] = twiddle<T>(p, n, +1);
+  auto freq = [&](int r) { return types == 1 ? r + 1 : r < K0 ? 2 * r + 2 : 2 * (r - K0) + 1; };
+  __syncthreads();
+  for (int i = tid; i < K * HP; i += THR) {
+    const int r = i / HP, t = i - r * HP;
+    tab[i] = tw[(freq(r) * t) % n];
+  }
+  for (long tile = blockIdx.x; (tile << lgE) < plane; tile += gridDim.x) {
+  const long e0 = tile << lgE;
+  __syncthreads();  // the previous tile's samples have been read
+#pragma unroll 8
+  for (int i = tid; i < K * E; i += THR) {
+    const int r = i >> lgE, e = i & (E - 1);
+    const long ge = e0 + e;
+    const C x = ge < plane ? Xh[(long)freq(r) * plane + ge] : mkc(T(0), T(0));
+    dr[i] = T(2) * x.x;
+    di[i] = T(2) * x.y;
+  }
+  for (int e = tid; e < E; e += THR) {
+    const long ge = e0 + e;
+    dr[K * E + e] = ge < plane ? Xh[ge].x : T(0);
+    dr[(K + 1) * E + e] = (types == 2 && ge < plane) ? Xh[(long)m * plane + ge].x : T(0);
+  }
+  __syncthreads();
+  const T inv = T(1) / T(n);
+  const int L = E / V, items = HP / KB * L;
+  for (int it = tid; it < items; it += THR) {
+    const int lane = it % L, t0 = it / L * KB;
+    T a[2][KB][V], b[2][KB][V];  // sums over the even and the odd frequencies
+    {
+      T f[V], g[V];
+      unpack(*(const VT*)(dr + (size_t)K * E + lane * V), f);
+      unpack(*(const VT*)(dr + (size_t)(K + 1) * E + lane * V), g);
+#pragma unroll
+      for (int q = 0; q < KB; ++q) {
+        const T sg = ((t0 + q) & 1) ? T(-1) : T(1);  // Nyquist: (-1)^t, with the frequencies of m's parity
+#pragma unroll
+        for (int u = 0; u < V; ++u) {
+          a[0][q][u] = (m & 1) ? f[u] : f[u] + sg * g[u];
+          a[1][q][u] = (m & 1) ? sg * g[u] : T(0);
+          b[0][q][u] = b[1][q][u] = T(0);
+        }
+      }
+    }
+#pragma unroll
+    for (int ty = 0; ty < 2; ++ty) {
+      const int rb = ty ? K0 : 0, re = ty ? K : K0;
+      for (int r0 = rb; r0 < re; r0 += 8) {
+        T sr[KB][V], si[KB][V];
+#pragma unroll
+        for (int q = 0; q < KB; ++q)
+#pragma unroll
+          for (int u = 0; u < V; ++u) sr[q][u] = si[q][u] = T(0);
+        const int r1 = min(re, r0 + 8);
+#pragma unroll 4
+        for (int r = r0; r < r1; ++r) {
+          T pv[V], qv[V];
+          unpack(*(const VT*)(dr + (size_t)r * E + lane * V), pv);
+          unpack(*(const VT*)(di + (size_t)r * E + lane * V), qv);
+          C c[KB];
+          load_row<KB>(tab + (size_t)r * HP + t0, c);
+#pragma unroll
+          for (int q = 0; q < KB; ++q)
+#pragma unroll
+            for (int u = 0; u < V; ++u) {
+              sr[q][u] = fma(pv[u], c[q].x, sr[q][u]);
+              si[q][u] = fma(qv[u], c[q].y, si[q][u]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < KB; ++q)
+#pragma unroll
+          for (int u = 0; u < V; ++u) {
+            a[ty][q][u] += sr[q][u];
+            b[ty][q][u] += si[q][u];
+          }
+      }
+    }
+    const long ge = e0 + lane * V;
+    auto put = [&](int t, const T* v) {
+      T* dst = X + (long)t * plane + ge;
+      if (ge + V <= plane && ((uintptr_t)dst & (sizeof(VT) - 1)) == 0) {
+        if constexpr (V == 4) *(float4*)dst = make_float4(v[0], v[1], v[2], v[3]);
+        else *(double2*)dst = make_double2(v[0], v[1]);
+      } else {
+#pragma unroll
+        for (int u = 0; u < V; ++u)
+          if (ge + u < plane) dst[u] = v[u];
+      }
+    };
+#pragma unroll
+    for (int q = 0; q < KB; ++q) {
+      const int t = t0 + q;
+      if (t >= tc) continue;
+      T v[V];
+      if (types == 1) {
+#pragma unroll
+        for (int u = 0; u < V; ++u) v[u] = (a[0][q][u] - b[0][q][u]) * inv;
+        put(t, v);
+        if (t > 0) {
+#pragma unroll
+          for (int u = 0; u < V; ++u) v[u] = (a[0][q][u] + b[0][q][u]) * inv;
+          put(n - t, v);
+        }
+        continue;
+      }
+#pragma unroll
+      for (int u = 0; u < V; ++u) v[u] = ((a[0][q][u] + a[1][q][u]) - (b[0][q][u] + b[1][q][u])) * inv;
+      put(t, v);
+      if (2 * t < m) {
+#pragma unroll
+        for (int u = 0; u < V; ++u) v[u] = ((a[0][q][u] - a[1][q][u]) + (b[0][q][u] - b[1][q][u])) * inv;
+        put(m - t, v);
+      }
+      if (t > 0) {
+#pragma unroll
+        for (int u = 0; u < V; ++u) v[u] = ((a[0][q][u] + a[1][q][u]) + (b[0][q][u] + b[1][q][u])) * inv;
+        put(n - t, v);
+        if (2 * t < m) {
+#pragma unroll
+          for (int u = 0; u < V; ++u) v[u] = ((a[0][q][u] - a[1][q][u]) - (b[0][q][u] - b[1][q][u])) * inv;
+          put(m + t, v);
+        }
+      }
+    }
+  }
+  }
+}
+
+// log2 of the tubes per tile: about 32 KB of samples, fewer where that would leave SMs idle (down to 32 tubes)
+template <typename T>
+static int rdft_tile(int n, long plane) {
+  int lg = 9;
+  while (lg > 6 && ((size_t)n * sizeof(T) << lg) > 34 * 1024) --lg;
+  while (lg > 5 && cdiv(plane, 1 << lg) < 2 * 152) --lg;
+  return lg;
+}
+// persistent CTAs: as many per SM as registers (the launch bounds) and shared memory allow
+static unsigned rdft_grid(long plane, int lgE, size_t smem, bool inverse) {
+  const unsigned fit = std::max<unsigned>(1, 227 * 1024 / (unsigned)(smem + 1024));
+  return std::min<unsigned>(cdiv(plane, 1L << lgE), 152 * std::min(fit, inverse ? 3u : 4u));
+}
+// FP64 arithmetic runs at 1/64 of FP32's rate, so there the operation count decides: picoseconds per
+// sample of the two forms as measured on a 512 x 512 plane (the mixed-radix passes by radix; the
+// folded product by n, and 100 = 4 5 5: 96 against 58, 128: 36 against 73).  In FP32 the folded
+// product is the faster one at every length that is not a power of two (97: 213 us against 27 ms,
+// 100: 139 against 199, 160: 289 against 346).
+template <typename T>
+static bool rdft_better(int n) {
+  if (n < 3 || n > RDFT_MAX) return false;
+  if (sizeof(T) == 4) return true;
+  double passes = 0;
+  int m = n;
+  while (m % 4 == 0) { passes += 9; m /= 4; }
+  while (m % 2 == 0) { passes += 8; m /= 2; }
+  while (m % 3 == 0) { passes += 18; m /= 3; }
+  while (m % 5 == 0) { passes += 42; m /= 5; }
+  if (m > 1) return true;
+  return n <= 128 && (n % 2 ? 1.13 : 0.57) * n < passes;
+}
+template <typename T>
+static size_t rdft_smem(int n, int E, bool inverse) {
+  constexpr int KB = RVec<T>::KB;
+  const RdftDims d = rdft_dims(n, KB);
+  if (!inverse)
+    return sizeof(T) * (size_t)d.types * (2 * d.J + 2) * E + sizeof(cx_t<T>) * ((size_t)d.J * d.HP + n);
+  const int K = (n - 1) / 2, HP = (d.m / 2 + KB) / KB * KB;
+  return sizeof(T) * (size_t)(2 * K + 2) * E + sizeof(cx_t<T>) * ((size_t)K * HP + n);
 }
 
 // shared bytes of the FFT kernels for tile width tt (0 when the plan does not exist)
@@ -461,27 +1085,47 @@ static bool fft_setup(int n, FftPlan* P, size_t* smem) {
   return true;
 }
 
+// threads per CTA of the register kernels: fewer where the plane would leave SMs idle
+static int reg_fft_threads(long plane) { return cdiv(plane, 128) >= 152 ? 128 : cdiv(plane, 64) >= 152 ? 64 : 32; }
+
 template <typename T>
 int launch_rfft3(const T* X, cx_t<T>* Xh, long plane, int n3, cudaStream_t s) {
   if (plane <= 0) return TSVD_OK;
-  FftPlan P;
-  size_t smem;
-  if (fft_setup<T>(n3, &P, &smem)) {
-    auto go = [&](auto kern) {
-      if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      kern<<<cdiv(plane, P.tubes), FFT_WARPS * 32, smem, s>>>(X, Xh, plane, P);
+  {  // powers of two in registers
+    auto go = [&](auto kern, int per_tube = 1) {
+      const int thr = reg_fft_threads(plane);
+      kern<<<cdiv(per_tube * plane, thr), thr, 0, s>>>(X, Xh, plane);
       TSVD_LAUNCHED();
       return TSVD_OK;
     };
-    switch (n3) {  // compile-time lengths (same tile width as the plan's)
-      case 4: return go(k_rfft3_fft<T, 4>);
-      case 8: return go(k_rfft3_fft<T, 8>);
-      case 16: return go(k_rfft3_fft<T, 16>);
-      case 32: return go(k_rfft3_fft<T, 32>);
-      case 64: return go(k_rfft3_fft<T, 64>);
-      case 128: return go(k_rfft3_fft<T, 128>);
-      default: return go(k_rfft3_fft<T, 0>);
+    switch (n3) {
+      case 2: return go(k_rfft3_reg<T, 2>);
+      case 4: return go(k_rfft3_reg<T, 4>);
+      case 8: return go(k_rfft3_reg<T, 8>);
+      case 16: return go(k_rfft3_reg<T, 16>);
+      case 32: return go(k_rfft3_reg<T, 32>);
+      case 64: return go(k_rfft3_reg<T, 64>);
+      case 128:
+        if constexpr (sizeof(T) == 4) return go(k_rfft3_reg<T, 128>);
+        else return go(k_rfft3_reg2<T, 128>, 2);
+      default: break;
     }
+  }
+  if (rdft_better<T>(n3)) {
+    const int lg = rdft_tile<T>(n3, plane);
+    const size_t sm = rdft_smem<T>(n3, 1 << lg, false);
+    if (sm > 48 * 1024) cudaFuncSetAttribute(k_rdft3<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    k_rdft3<T><<<rdft_grid(plane, lg, sm, false), RVec<T>::THREADS, sm, s>>>(X, Xh, plane, n3, lg);
+    TSVD_LAUNCHED();
+    return TSVD_OK;
+  }
+  FftPlan P;
+  size_t smem;
+  if (fft_setup<T>(n3, &P, &smem)) {
+    if (smem > 48 * 1024) cudaFuncSetAttribute(k_rfft3_fft<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_rfft3_fft<T><<<cdiv(plane, P.tubes), FFT_WARPS * 32, smem, s>>>(X, Xh, plane, P);
+    TSVD_LAUNCHED();
+    return TSVD_OK;
   }
   // very long tubes: direct transform
   const int te = tile_e(n3, sizeof(T), sizeof(cx_t<T>), false);
@@ -496,24 +1140,41 @@ int launch_rfft3(const T* X, cx_t<T>* Xh, long plane, int n3, cudaStream_t s) {
 template <typename T>
 int launch_irfft3(const cx_t<T>* Xh, T* X, long plane, int n3, cudaStream_t s) {
   if (plane <= 0) return TSVD_OK;
-  FftPlan P;
-  size_t smem;
-  if (fft_setup<T>(n3, &P, &smem)) {
-    auto go = [&](auto kern) {
-      if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      kern<<<cdiv(plane, P.tubes), FFT_WARPS * 32, smem, s>>>(Xh, X, plane, P);
+  {
+    auto go = [&](auto kern, int per_tube = 1) {
+      const int thr = reg_fft_threads(plane);
+      kern<<<cdiv(per_tube * plane, thr), thr, 0, s>>>(Xh, X, plane);
       TSVD_LAUNCHED();
       return TSVD_OK;
     };
     switch (n3) {
-      case 4: return go(k_irfft3_fft<T, 4>);
-      case 8: return go(k_irfft3_fft<T, 8>);
-      case 16: return go(k_irfft3_fft<T, 16>);
-      case 32: return go(k_irfft3_fft<T, 32>);
-      case 64: return go(k_irfft3_fft<T, 64>);
-      case 128: return go(k_irfft3_fft<T, 128>);
-      default: return go(k_irfft3_fft<T, 0>);
+      case 2: return go(k_irfft3_reg<T, 2>);
+      case 4: return go(k_irfft3_reg<T, 4>);
+      case 8: return go(k_irfft3_reg<T, 8>);
+      case 16: return go(k_irfft3_reg<T, 16>);
+      case 32: return go(k_irfft3_reg<T, 32>);
+      case 64: return go(k_irfft3_reg<T, 64>);
+      case 128:
+        if constexpr (sizeof(T) == 4) return go(k_irfft3_reg<T, 128>);
+        else return go(k_irfft3_reg2<T, 128>, 2);
+      default: break;
     }
+  }
+  if (rdft_better<T>(n3)) {
+    const int lg = rdft_tile<T>(n3, plane);
+    const size_t sm = rdft_smem<T>(n3, 1 << lg, true);
+    if (sm > 48 * 1024) cudaFuncSetAttribute(k_irdft3<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    k_irdft3<T><<<rdft_grid(plane, lg, sm, true), RVec<T>::THREADS, sm, s>>>(Xh, X, plane, n3, lg);
+    TSVD_LAUNCHED();
+    return TSVD_OK;
+  }
+  FftPlan P;
+  size_t smem;
+  if (fft_setup<T>(n3, &P, &smem)) {
+    if (smem > 48 * 1024) cudaFuncSetAttribute(k_irfft3_fft<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_irfft3_fft<T><<<cdiv(plane, P.tubes), FFT_WARPS * 32, smem, s>>>(Xh, X, plane, P);
+    TSVD_LAUNCHED();
+    return TSVD_OK;
   }
   const int h = n3 / 2 + 1;
   const int te = tile_e(n3, sizeof(T), sizeof(cx_t<T>), true);
