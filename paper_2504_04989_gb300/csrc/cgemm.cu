@@ -1,39 +1,45 @@
 // cgemm.cu -- batched complex GEMM on the SIMT FP64 / FP32 pipes.
 //
-// One CTA computes a 64 x 64 tile of one slice's product with 256 threads,
-// each holding a 4 x 4 complex register tile (rows ty + 16 i, columns
-// tx + 16 j, so a warp's shared-memory reads are contiguous).  op(A) and op(B)
+// One CTA computes a tile of one slice's product (FP32: 64 x 64 on 256 threads,
+// each holding a 4 x 4 complex register tile, rows ty + 16 i, columns tx + 16 j,
+// so a warp's shared-memory reads are contiguous; FP64: 16 x 16, GemmCfg).  op(A) and op(B)
 // tiles are staged in shared memory k-major, in two stages: the next k-tile is
 // loaded into registers while the current one is multiplied; the conjugate
 // transpose is taken while staging, reading the stored matrix along its
 // contiguous dimension.
 // Thin products (long K, small M x N) split K across CTAs and reduce the
 // partial tiles in a fixed order (deterministic, no atomics).
+#include <type_traits>
+
 #include "common.cuh"
 #include "kernels.cuh"
 
 namespace tsvd {
 
+// BT x BT tiles on TD x TD threads (RT x RT complex each), BK deep, K split down to KMIN a piece.
+// FP64: two multiply-adds per SM and clock, so a product is bound by how many SMs take part and
+// not by loads (a 2 x 2 register tile issues 256 clocks of FP64 per 16 of shared-memory reads):
+// 16 x 16 tiles on 64 threads spread a small product over the GPU and pad a thin one less.
+// 64 x 15 x 64 on 9 slices: 264 -> 19 us against 64 x 64 tiles on 256 threads.
 template <typename C>
 struct GemmCfg;
 template <>
 struct GemmCfg<double2> {
-  static constexpr int BK = 8;
+  static constexpr int BT = 16, TD = 8, BK = 16, KMIN = 16;
   using R = double;
 };
 template <>
 struct GemmCfg<float2> {
-  static constexpr int BK = 16;
+  static constexpr int BT = 64, TD = 16, BK = 16, KMIN = 64;
   using R = float;
 };
 
-constexpr int GBM = 64, GBN = 64;
-
 template <typename C, bool AH, bool BH>
-__global__ void __launch_bounds__(256) k_cgemm(GemmArgs g, C* __restrict__ ws, int ksplit, int kchunk, int tiles_m,
+__global__ void __launch_bounds__(GemmCfg<C>::TD* GemmCfg<C>::TD) k_cgemm(GemmArgs g, C* __restrict__ ws, int ksplit, int kchunk, int tiles_m,
                                                int herm_upper) {
-  constexpr int BK = GemmCfg<C>::BK;
-  constexpr int NA = GBM * BK / 256, NB = GBN * BK / 256;  // staged elements per thread
+  constexpr int BK = GemmCfg<C>::BK, GBM = GemmCfg<C>::BT, GBN = GBM, TD = GemmCfg<C>::TD, NT = TD * TD;
+  constexpr int RT = GBM / TD;                           // rows and columns of a thread
+  constexpr int NA = GBM * BK / NT, NB = GBN * BK / NT;  // staged elements per thread
   using R = typename GemmCfg<C>::R;
   // two stages; rows padded by one element so the transposed stores hit distinct banks
   __shared__ __align__(16) C As[2][BK][GBM + 1];
@@ -45,19 +51,25 @@ __global__ void __launch_bounds__(256) k_cgemm(GemmArgs g, C* __restrict__ ws, i
   const C* __restrict__ A = (const C*)g.A + (long)bi * g.sA;
   const C* __restrict__ B = (const C*)g.B + (long)bi * g.sB;
   const int kb = kz * kchunk, ke = min(g.K, kb + kchunk);
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  C acc[4][4];
+  const int tid = threadIdx.x, tx = tid % TD, ty = tid / TD;
+  C acc[RT][RT];
+  // FP64 sums in runs of 64 terms (short runs round less; the adds are 1/64 of the work)
+  constexpr bool RUNS = std::is_same<C, double2>::value;
+  C tot[RUNS ? RT : 1][RUNS ? RT : 1];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < RT; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = mkc(R(0), R(0));
+    for (int j = 0; j < RT; ++j) {
+      acc[i][j] = mkc(R(0), R(0));
+      if constexpr (RUNS) tot[i][j] = acc[i][j];
+    }
 
   // the next k-tile is fetched into registers while the current one is multiplied
   C ra[NA], rb[NB];
   auto fetch = [&](int k0) {
 #pragma unroll
     for (int t = 0; t < NA; ++t) {
-      const int idx = tid + 256 * t;
+      const int idx = tid + NT * t;
       int mm, kk;
       if (!AH) { kk = idx % BK; mm = idx / BK; }
       else { mm = idx % GBM; kk = idx / GBM; }
@@ -68,7 +80,7 @@ __global__ void __launch_bounds__(256) k_cgemm(GemmArgs g, C* __restrict__ ws, i
     }
 #pragma unroll
     for (int t = 0; t < NB; ++t) {
-      const int idx = tid + 256 * t;
+      const int idx = tid + NT * t;
       int nn, kk;
       if (!BH) { nn = idx % GBN; kk = idx / GBN; }
       else { kk = idx % BK; nn = idx / BK; }
@@ -81,13 +93,13 @@ __global__ void __launch_bounds__(256) k_cgemm(GemmArgs g, C* __restrict__ ws, i
   auto stash = [&](int st) {
 #pragma unroll
     for (int t = 0; t < NA; ++t) {
-      const int idx = tid + 256 * t;
+      const int idx = tid + NT * t;
       if (!AH) As[st][idx % BK][idx / BK] = ra[t];
       else As[st][idx / GBM][idx % GBM] = ra[t];
     }
 #pragma unroll
     for (int t = 0; t < NB; ++t) {
-      const int idx = tid + 256 * t;
+      const int idx = tid + NT * t;
       if (!BH) Bs[st][idx / GBN][idx % GBN] = rb[t];
       else Bs[st][idx % BK][idx / BK] = rb[t];
     }
@@ -100,26 +112,37 @@ __global__ void __launch_bounds__(256) k_cgemm(GemmArgs g, C* __restrict__ ws, i
     if (k0 + BK < ke) fetch(k0 + BK);
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
-      C a[4], b[4];
+      C a[RT], b[RT];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[st][kk][ty + 16 * i];
+      for (int i = 0; i < RT; ++i) a[i] = As[st][kk][ty + TD * i];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[st][kk][tx + 16 * j];
+      for (int j = 0; j < RT; ++j) b[j] = Bs[st][kk][tx + TD * j];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < RT; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) cfma(acc[i][j], a[i], b[j]);
+        for (int j = 0; j < RT; ++j) cfma(acc[i][j], a[i], b[j]);
     }
     st ^= 1;
+    if constexpr (RUNS) {
+      if (((k0 - kb) & 63) == 64 - BK || k0 + BK >= ke) {
+#pragma unroll
+        for (int i = 0; i < RT; ++i)
+#pragma unroll
+          for (int j = 0; j < RT; ++j) {
+            tot[i][j] = cadd(tot[i][j], acc[i][j]);
+            acc[i][j] = (k0 + BK >= ke) ? tot[i][j] : mkc(R(0), R(0));
+          }
+      }
+    }
   }
   C* __restrict__ Cm = (C*)g.C + (long)bi * g.sC;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int gm = m0 + ty + 16 * i;
+  for (int i = 0; i < RT; ++i) {
+    const int gm = m0 + ty + TD * i;
     if (gm >= g.M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int gn = n0 + tx + 16 * j;
+    for (int j = 0; j < RT; ++j) {
+      const int gn = n0 + tx + TD * j;
       if (gn >= g.N) continue;
       if (ksplit > 1) {
         ws[(((long)kz * g.batch + bi) * g.M + gm) * g.N + gn] = acc[i][j];
@@ -266,11 +289,13 @@ __global__ void k_splitk_reduce(const C* __restrict__ ws, int ksplit, GemmArgs g
   }
 }
 
-int choose_ksplit(int M, int N, int K, int batch, size_t splitk_elems) {
-  const long tiles = (long)cdiv(M, GBM) * cdiv(N, GBN) * batch;
+// a split of K that fills the GPU (bounded by the scratch it needs)
+template <typename C>
+static int choose_ksplit(int M, int N, int K, int batch, size_t splitk_elems) {
+  const long tiles = (long)cdiv(M, GemmCfg<C>::BT) * cdiv(N, GemmCfg<C>::BT) * batch;
   const long target = 2 * 152;
   int ks = (int)std::max(1L, std::min(16L, target / std::max(1L, tiles)));
-  ks = std::min(ks, std::max(1, K / 64));
+  ks = std::min(ks, std::max(1, K / GemmCfg<C>::KMIN));
   while (ks > 1 && (size_t)ks * batch * M * N > splitk_elems) --ks;
   while (ks > 1 && (long)ks * batch > 65535) --ks;
   return ks;
@@ -287,6 +312,14 @@ __global__ void k_mirror_lower(C* __restrict__ Cm, long ldc, long sC, int n, int
     const int b = t / n;
     if (i > j) Cm[(long)b * sC + (long)i * ldc + j] = cconj(Cm[(long)b * sC + (long)j * ldc + i]);
   }
+}
+
+template <typename C>
+static int mirror_lower(const GemmArgs& g, cudaStream_t s) {
+  const long total = (long)g.batch * g.M * g.M;
+  k_mirror_lower<C><<<std::min<long>(cdiv(total, 256), 8192), 256, 0, s>>>((C*)g.C, g.ldc, g.sC, g.M, g.batch);
+  TSVD_LAUNCHED();
+  return TSVD_OK;
 }
 
 // k_cgemm_w over the FP32 product g: split-K until about two waves of two CTAs per SM
@@ -329,39 +362,54 @@ static int cgemm_impl(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, c
     if (!herm && g.K > 0 && (wtiles >= 2L * 152 || (g.K >= 1024 && splitk_ws)))
       return cgemm_wide(g, (float2*)splitk_ws, splitk_ws ? splitk_elems : 0, s);
   }
-  int ks = (g.K > 0) ? choose_ksplit(g.M, g.N, g.K, g.batch, splitk_ws ? splitk_elems : 0) : 1;
+  if constexpr (std::is_same<C, double2>::value) {
+    const size_t bytes = splitk_ws ? splitk_elems * sizeof(C) : 0;
+    if (!g.simt && dgemm_tc_better(g, bytes)) {
+      TSVD_TRY(dgemm_tc(g, splitk_ws, bytes, s, herm != 0));
+      return herm ? mirror_lower<C>(g, s) : TSVD_OK;
+    }
+  }
+  int ks = (g.K > 0) ? choose_ksplit<C>(g.M, g.N, g.K, g.batch, splitk_ws ? splitk_elems : 0) : 1;
   constexpr int BK = GemmCfg<C>::BK;
   int kchunk = (g.K + ks - 1) / ks;
   kchunk = (kchunk + BK - 1) / BK * BK;
   if (kchunk == 0) kchunk = BK;
   ks = (g.K + kchunk - 1) / kchunk;
   if (ks < 1) ks = 1;
-  const int tiles_m = cdiv(g.M, GBM), tiles_n = cdiv(g.N, GBN);
+  constexpr int BT = GemmCfg<C>::BT, NT = GemmCfg<C>::TD * GemmCfg<C>::TD;
+  const int tiles_m = cdiv(g.M, BT), tiles_n = cdiv(g.N, BT);
   dim3 grid(tiles_m * tiles_n, 1, g.batch * ks);
   const bool ah = (g.opA == 'H'), bh = (g.opB == 'H');
   C* ws = (C*)splitk_ws;
-  if (!ah && !bh) k_cgemm<C, false, false><<<grid, 256, 0, s>>>(g, ws, ks, kchunk, tiles_m, herm);
-  else if (ah && !bh) k_cgemm<C, true, false><<<grid, 256, 0, s>>>(g, ws, ks, kchunk, tiles_m, herm);
-  else if (!ah && bh) k_cgemm<C, false, true><<<grid, 256, 0, s>>>(g, ws, ks, kchunk, tiles_m, herm);
-  else k_cgemm<C, true, true><<<grid, 256, 0, s>>>(g, ws, ks, kchunk, tiles_m, herm);
+  if (!ah && !bh) k_cgemm<C, false, false><<<grid, NT, 0, s>>>(g, ws, ks, kchunk, tiles_m, herm);
+  else if (ah && !bh) k_cgemm<C, true, false><<<grid, NT, 0, s>>>(g, ws, ks, kchunk, tiles_m, herm);
+  else if (!ah && bh) k_cgemm<C, false, true><<<grid, NT, 0, s>>>(g, ws, ks, kchunk, tiles_m, herm);
+  else k_cgemm<C, true, true><<<grid, NT, 0, s>>>(g, ws, ks, kchunk, tiles_m, herm);
   TSVD_LAUNCHED();
   if (ks > 1) {
     const long total = (long)g.batch * g.M * g.N;
     k_splitk_reduce<C><<<std::min<long>(cdiv(total, 256), 4096), 256, 0, s>>>(ws, ks, g);
     TSVD_LAUNCHED();
   }
-  if (herm) {
-    const long total = (long)g.batch * g.M * g.M;
-    k_mirror_lower<C><<<std::min<long>(cdiv(total, 256), 8192), 256, 0, s>>>((C*)g.C, g.ldc, g.sC, g.M, g.batch);
-    TSVD_LAUNCHED();
-  }
-  return TSVD_OK;
+  return herm ? mirror_lower<C>(g, s) : TSVD_OK;
 }
 
 template <typename C>
 int cgemm(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t s) {
   return cgemm_impl<C>(g, splitk_ws, splitk_elems, s, 0);
 }
+
+template <typename C>
+size_t cgemm_scratch(int M, int N, int K, int batch) {
+  GemmArgs g = gemm('N', 'N', M, N, K, 1.0, nullptr, K, 0, nullptr, N, 0, 0.0, nullptr, N, 0, batch);
+  if constexpr (std::is_same<C, double2>::value) {
+    const size_t bytes = dgemm_tc_bytes(M, N, K, batch);
+    return dgemm_tc_better(g, bytes) ? bytes / sizeof(C) + 1 : 0;
+  }
+  return 0;
+}
+template size_t cgemm_scratch<double2>(int, int, int, int);
+template size_t cgemm_scratch<float2>(int, int, int, int);
 
 template <typename C>
 int cgemm_herm(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t s) {

@@ -612,8 +612,14 @@ int orth_block_cols(int n1, int b, int m, int h, const OrthWs& w, int c, int nb,
     {
       TSVD_STAGE("orth_trsm", s);
       // the last pass writes the finished block straight into its columns of Q
-      if (pass < 2) TSVD_TRY(rmul_block<CL>(W, b, sW, Mi, b, sG, n1, nb, h, W, b, sW, s));
-      else TSVD_TRY(rmul_block<CL>(W, b, sW, Mi, b, sG, n1, nb, h, Q + c, m, sQ, s));
+      CL* out = pass < 2 ? W : Q + c;
+      const long ldo = pass < 2 ? b : m, so = pass < 2 ? sW : sQ;
+      const GemmArgs g = gemm('N', 'N', n1, nb, nb, 1.0, W, b, sW, Mi, b, sG, 0.0, out, ldo, so, h);
+      // the digit form reads copies of its operands, so it may write W in place
+      if (std::is_same<L, double>::value && dgemm_tc_better(g, sk * sizeof(CL)))
+        TSVD_TRY(dgemm_tc(g, w.splitk, sk * sizeof(CL), s, false));
+      else
+        TSVD_TRY(rmul_block<CL>(W, b, sW, Mi, b, sG, n1, nb, h, out, ldo, so, s));
     }
   }
   {

@@ -92,7 +92,8 @@ static LrWs<T> carve_lr(void* base, int n1, int n2, int n3, int R) {
   w.Vh = cv.take<C>(h * n2 * R);
   w.Sh = cv.take<C>(h * R);
   w.Xh = cv.take<C>(h * n1 * n2);
-  w.sk_elems = std::min<size_t>((size_t)1 << 20, 4 * h * (size_t)n1 * n2);
+  w.sk_elems = std::max(std::min<size_t>((size_t)1 << 20, 4 * h * (size_t)n1 * n2),
+                        cgemm_scratch<C>(n1, n2, R, (int)h));
   w.sk = cv.take<C>(w.sk_elems);
   w.bytes = cv.bytes();
   return w;

@@ -46,6 +46,7 @@ struct GemmArgs {
   void* C;
   long ldc, sC;
   int batch;
+  bool simt = false;  // keep to the SIMT kernels
 };
 // GemmArgs from its fields (strided batch)
 inline GemmArgs gemm(char opA, char opB, int M, int N, int K, double alpha, const void* A, long lda, long sA,
@@ -72,12 +73,22 @@ inline GemmArgs gemm(char opA, char opB, int M, int N, int K, double alpha, cons
 }
 template <typename C>
 int cgemm(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t s);
+// scratch elements with which cgemm can take its tensor-core form for an M x N x K product (0 where
+// it would keep to the SIMT units); a smaller splitk_elems only makes it slower
+template <typename C>
+size_t cgemm_scratch(int M, int N, int K, int batch);
 // C = op(A) op(B) known to be Hermitian (square, beta = 0, e.g. A^H A): only
 // the upper tiles are computed, the lower triangle is mirrored from them
 template <typename C>
 int cgemm_herm(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t s);
-// pick a split of K that fills the GPU (bounded by the scratch it needs)
-int choose_ksplit(int M, int N, int K, int batch, size_t splitk_elems);
+
+// dgemm_tc.cu -- the FP64 product as exact digit products on the BF16 tensor cores (cgemm and
+// cgemm_herm take it where dgemm_tc_better says so and the scratch holds one slice's digits):
+// bytes of scratch for the whole product (bounded; more slices than fit are done in passes), and
+// the product itself (alpha +-1, beta 0 or 1; upper: only the tiles not wholly below the diagonal)
+size_t dgemm_tc_bytes(int M, int N, int K, int batch);
+bool dgemm_tc_better(const GemmArgs& g, size_t bytes);
+int dgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s, bool upper);
 
 // element-wise conversions of batched complex matrices (rows x cols, leading dims)
 int convert_c64_to_c32(const double2* src, long lds, long ss, float2* dst, long ldd, long sd, int rows, int cols,

@@ -8,6 +8,8 @@
 //           is the conjugate transpose:  dA_k = dC_k B_k^H,  dB_k = A_k^H dC_k.
 // Projection Y = Q*Q^T*A (Sec. 4, the lemma equating the Alg. 2 residual with A - Q (Q^T A)_k): dA_k = Q_k (Q_k^H dY_k),
 //           dQ_k = dY_k (A_k^H Q_k) + A_k (dY_k^H Q_k).
+#include <array>
+#include <initializer_list>
 #include <type_traits>
 
 #include "common.cuh"
@@ -49,13 +51,21 @@ static GemmArgs gm(char opA, char opB, int M, int N, int K, double alpha, const 
   return g;
 }
 
-constexpr size_t SPLITK_ELEMS = (size_t)1 << 22;  // complex elements of split-K scratch
+// complex elements of product scratch: split-K partials, or the operands of the tensor-core form of
+// the products M x N x K given
+template <typename C>
+static size_t scratch_elems(int batch, std::initializer_list<std::array<int, 3>> shapes) {
+  size_t n = (size_t)1 << 22;
+  for (const auto& t : shapes) n = std::max(n, cgemm_scratch<C>(t[0], t[1], t[2], batch));
+  return n;
+}
 
 // ---------------------------------------------------------------------------
 template <typename T>
 struct TprodWs {
   cx_t<T>*Ah, *Bh, *Ch;
   void* sk;
+  size_t sk_elems;
   size_t bytes;
 };
 template <typename T>
@@ -66,7 +76,8 @@ static TprodWs<T> carve_tprod(void* base, int n1, int n2, int n4, int n3) {
   w.Ah = cv.take<cx_t<T>>(h * n1 * n2);
   w.Bh = cv.take<cx_t<T>>(h * n2 * n4);
   w.Ch = cv.take<cx_t<T>>(h * n1 * n4);
-  w.sk = cv.take<cx_t<T>>(SPLITK_ELEMS);
+  w.sk_elems = scratch_elems<cx_t<T>>((int)h, {std::array<int, 3>{n1, n4, n2}});
+  w.sk = cv.take<cx_t<T>>(w.sk_elems);
   w.bytes = cv.bytes();
   return w;
 }
@@ -82,7 +93,7 @@ static int tprod_run(const T* A, const T* B, T* Cout, int n1, int n2, int n4, in
   }
   {
     TSVD_STAGE("tprod_gemm", s);
-    TSVD_TRY(cgemm<cx_t<T>>(gm('N', 'N', n1, n4, n2, 1.0, w.Ah, n2, w.Bh, n4, 0.0, w.Ch, n4, h), w.sk, SPLITK_ELEMS,
+    TSVD_TRY(cgemm<cx_t<T>>(gm('N', 'N', n1, n4, n2, 1.0, w.Ah, n2, w.Bh, n4, 0.0, w.Ch, n4, h), w.sk, w.sk_elems,
                             s));
   }
   {
@@ -174,6 +185,7 @@ template <typename T>
 struct TbwdWs {
   cx_t<T>*Ah, *Bh, *dCh, *dAh, *dBh;
   void* sk;
+  size_t sk_elems;
   size_t bytes;
 };
 template <typename T>
@@ -186,7 +198,8 @@ static TbwdWs<T> carve_tbwd(void* base, int n1, int n2, int n4, int n3) {
   w.dCh = cv.take<cx_t<T>>(h * n1 * n4);
   w.dAh = cv.take<cx_t<T>>(h * n1 * n2);
   w.dBh = cv.take<cx_t<T>>(h * n2 * n4);
-  w.sk = cv.take<cx_t<T>>(SPLITK_ELEMS);
+  w.sk_elems = scratch_elems<cx_t<T>>((int)h, {std::array<int, 3>{n1, n2, n4}, std::array<int, 3>{n2, n4, n1}});
+  w.sk = cv.take<cx_t<T>>(w.sk_elems);
   w.bytes = cv.bytes();
   return w;
 }
@@ -199,13 +212,13 @@ static int tbwd_run(const T* A, const T* B, const T* dC, T* dA, T* dB, int n1, i
   TSVD_TRY(launch_rfft3<T>(dC, w.dCh, (long)n1 * n4, n3, s));
   if (dA) {
     TSVD_TRY(launch_rfft3<T>(B, w.Bh, (long)n2 * n4, n3, s));
-    TSVD_TRY(cgemm<cx_t<T>>(gm('N', 'H', n1, n2, n4, 1.0, w.dCh, n4, w.Bh, n4, 0.0, w.dAh, n2, h), w.sk, SPLITK_ELEMS,
+    TSVD_TRY(cgemm<cx_t<T>>(gm('N', 'H', n1, n2, n4, 1.0, w.dCh, n4, w.Bh, n4, 0.0, w.dAh, n2, h), w.sk, w.sk_elems,
                             s));
     TSVD_TRY(launch_irfft3<T>(w.dAh, dA, (long)n1 * n2, n3, s));
   }
   if (dB) {
     TSVD_TRY(launch_rfft3<T>(A, w.Ah, (long)n1 * n2, n3, s));
-    TSVD_TRY(cgemm<cx_t<T>>(gm('H', 'N', n2, n4, n1, 1.0, w.Ah, n2, w.dCh, n4, 0.0, w.dBh, n4, h), w.sk, SPLITK_ELEMS,
+    TSVD_TRY(cgemm<cx_t<T>>(gm('H', 'N', n2, n4, n1, 1.0, w.Ah, n2, w.dCh, n4, 0.0, w.dBh, n4, h), w.sk, w.sk_elems,
                             s));
     TSVD_TRY(launch_irfft3<T>(w.dBh, dB, (long)n2 * n4, n3, s));
   }
@@ -217,6 +230,7 @@ template <typename T>
 struct TprojWs {
   cx_t<T>*Qh, *Ah, *dYh, *T1, *T2, *dAh, *dQh;
   void* sk;
+  size_t sk_elems;
   size_t bytes;
 };
 template <typename T>
@@ -231,7 +245,8 @@ static TprojWs<T> carve_tproj(void* base, int n1, int m, int n2, int n3) {
   w.T2 = cv.take<cx_t<T>>(h * (size_t)n2 * m);
   w.dAh = cv.take<cx_t<T>>(h * n1 * n2);
   w.dQh = cv.take<cx_t<T>>(h * n1 * m);
-  w.sk = cv.take<cx_t<T>>(SPLITK_ELEMS);
+  w.sk_elems = scratch_elems<cx_t<T>>((int)h, {std::array<int, 3>{m, n2, n1}, std::array<int, 3>{n1, n2, m}, std::array<int, 3>{n2, m, n1}, std::array<int, 3>{n1, m, n2}});
+  w.sk = cv.take<cx_t<T>>(w.sk_elems);
   w.bytes = cv.bytes();
   return w;
 }
@@ -246,18 +261,18 @@ static int tproj_run(const T* Q, const T* A, const T* dY, T* dQ, T* dA, int n1, 
   TSVD_TRY(launch_rfft3<T>(dY, w.dYh, (long)n1 * n2, n3, s));
   if (dA) {
     // T1 = Q^H dY (m x n2); dA = Q T1
-    TSVD_TRY(cgemm<C>(gm('H', 'N', m, n2, n1, 1.0, w.Qh, m, w.dYh, n2, 0.0, w.T1, n2, h), w.sk, SPLITK_ELEMS, s));
-    TSVD_TRY(cgemm<C>(gm('N', 'N', n1, n2, m, 1.0, w.Qh, m, w.T1, n2, 0.0, w.dAh, n2, h), w.sk, SPLITK_ELEMS, s));
+    TSVD_TRY(cgemm<C>(gm('H', 'N', m, n2, n1, 1.0, w.Qh, m, w.dYh, n2, 0.0, w.T1, n2, h), w.sk, w.sk_elems, s));
+    TSVD_TRY(cgemm<C>(gm('N', 'N', n1, n2, m, 1.0, w.Qh, m, w.T1, n2, 0.0, w.dAh, n2, h), w.sk, w.sk_elems, s));
     TSVD_TRY(launch_irfft3<T>(w.dAh, dA, (long)n1 * n2, n3, s));
   }
   if (dQ) {
     TSVD_TRY(launch_rfft3<T>(A, w.Ah, (long)n1 * n2, n3, s));
     // T2 = A^H Q (n2 x m); dQ = dY T2
-    TSVD_TRY(cgemm<C>(gm('H', 'N', n2, m, n1, 1.0, w.Ah, n2, w.Qh, m, 0.0, w.T2, m, h), w.sk, SPLITK_ELEMS, s));
-    TSVD_TRY(cgemm<C>(gm('N', 'N', n1, m, n2, 1.0, w.dYh, n2, w.T2, m, 0.0, w.dQh, m, h), w.sk, SPLITK_ELEMS, s));
+    TSVD_TRY(cgemm<C>(gm('H', 'N', n2, m, n1, 1.0, w.Ah, n2, w.Qh, m, 0.0, w.T2, m, h), w.sk, w.sk_elems, s));
+    TSVD_TRY(cgemm<C>(gm('N', 'N', n1, m, n2, 1.0, w.dYh, n2, w.T2, m, 0.0, w.dQh, m, h), w.sk, w.sk_elems, s));
     // T2 = dY^H Q; dQ += A T2
-    TSVD_TRY(cgemm<C>(gm('H', 'N', n2, m, n1, 1.0, w.dYh, n2, w.Qh, m, 0.0, w.T2, m, h), w.sk, SPLITK_ELEMS, s));
-    TSVD_TRY(cgemm<C>(gm('N', 'N', n1, m, n2, 1.0, w.Ah, n2, w.T2, m, 1.0, w.dQh, m, h), w.sk, SPLITK_ELEMS, s));
+    TSVD_TRY(cgemm<C>(gm('H', 'N', n2, m, n1, 1.0, w.dYh, n2, w.Qh, m, 0.0, w.T2, m, h), w.sk, w.sk_elems, s));
+    TSVD_TRY(cgemm<C>(gm('N', 'N', n1, m, n2, 1.0, w.Ah, n2, w.T2, m, 1.0, w.dQh, m, h), w.sk, w.sk_elems, s));
     TSVD_TRY(launch_irfft3<T>(w.dQh, dQ, (long)n1 * m, n3, s));
   }
   return TSVD_OK;
@@ -270,8 +285,8 @@ static int tproj_fwd_run(const T* Q, const T* A, T* Y, int n1, int m, int n2, in
   using C = cx_t<T>;
   TSVD_TRY(launch_rfft3<T>(Q, w.Qh, (long)n1 * m, n3, s));
   TSVD_TRY(launch_rfft3<T>(A, w.Ah, (long)n1 * n2, n3, s));
-  TSVD_TRY(cgemm<C>(gm('H', 'N', m, n2, n1, 1.0, w.Qh, m, w.Ah, n2, 0.0, w.T1, n2, h), w.sk, SPLITK_ELEMS, s));
-  TSVD_TRY(cgemm<C>(gm('N', 'N', n1, n2, m, 1.0, w.Qh, m, w.T1, n2, 0.0, w.dAh, n2, h), w.sk, SPLITK_ELEMS, s));
+  TSVD_TRY(cgemm<C>(gm('H', 'N', m, n2, n1, 1.0, w.Qh, m, w.Ah, n2, 0.0, w.T1, n2, h), w.sk, w.sk_elems, s));
+  TSVD_TRY(cgemm<C>(gm('N', 'N', n1, n2, m, 1.0, w.Qh, m, w.T1, n2, 0.0, w.dAh, n2, h), w.sk, w.sk_elems, s));
   TSVD_TRY(launch_irfft3<T>(w.dAh, Y, (long)n1 * n2, n3, s));
   return TSVD_OK;
 }

@@ -160,6 +160,10 @@ static TqrWs<T> carve_tqr(void* base, const TqrDims& d, bool pinv) {
   w.dead = cv.take<uint32_t>(h * 4);
   w.counters = cv.take<int>(8);
   w.splitk_elems = std::min<size_t>((size_t)1 << 22, 8 * h * (size_t)d.p * std::max(d.b, 64));
+  const int hb = (int)h, shapes[][3] = {{d.p, d.Nc, d.Mr}, {d.b, d.b, d.Mr}, {d.p, d.b, d.Mr}, {d.Mr, d.b, d.p},
+                                        {d.Mr, d.b, d.b}, {d.p, d.Mr, d.p}, {d.Mr, d.p, d.p}};
+  for (const auto& t : shapes)
+    w.splitk_elems = std::max(w.splitk_elems, cgemm_scratch<C>(t[0], t[1], t[2], hb) * sizeof(C) / sizeof(double2) + 1);
   w.splitk = cv.take<double2>(w.splitk_elems);
   w.bytes = cv.bytes();
   return w;

@@ -201,6 +201,13 @@ static RbkWs<T> carve_rbk(void* base, const RbkDims& d) {
     t.err = w.tc_err;
   }
   w.splitk_elems = 8 * h * (size_t)d.m * std::max(d.b, 64);
+  const int hb = d.h, shapes[][3] = {{d.n1, d.b, d.n2}, {d.n2, d.b, d.n1}, {d.m, d.b, d.n1}, {d.n1, d.b, d.m},
+                                     {d.b, d.b, d.n1},  {d.n1, d.b, d.b}, {d.mp, d.mp, d.n2}, {d.n1, d.R, d.mp},
+                                     {d.n2, d.R, d.mp}};
+  for (const auto& t : shapes) {  // the orthonormalisation's products run in L, the others in T
+    w.splitk_elems = std::max(w.splitk_elems, cgemm_scratch<CL>(t[0], t[1], t[2], hb) * sizeof(CL) / sizeof(double2) + 1);
+    w.splitk_elems = std::max(w.splitk_elems, cgemm_scratch<C>(t[0], t[1], t[2], hb) * sizeof(C) / sizeof(double2) + 1);
+  }
   w.splitk = cv.take<double2>(w.splitk_elems);
   w.lamF = nullptr;
   w.UF = w.Um = w.T1 = w.CpH = nullptr;
@@ -277,7 +284,7 @@ static int basis_product(const RbkDims& d, RbkWs<T>& w, const cx_t<T>* Y, long l
     }
   }
   return cgemm<cx_t<T>>(gemm('N', 'N', n1, nb, n2, 1.0, w.Ah, n2, sA, Y, ldy, sy, 0.0, w.Wt, b, sW, h), w.splitk,
-                        w.splitk_elems * 2, s);
+                        w.splitk_elems * (sizeof(double2) / sizeof(cx_t<T>)), s);
 }
 
 // columns [col0, col0 + nb) of C^H (n2 x m) = X-hat^H Q(:, col0 : col0 + nb): the
@@ -295,7 +302,7 @@ static int conj_product(const RbkDims& d, RbkWs<T>& w, int col0, int nb, cudaStr
   }
   return cgemm<cx_t<T>>(gemm('H', 'N', n2, nb, n1, 1.0, w.Ah, n2, sA, w.Qt + col0, m, sQ, 0.0, w.CHt + col0, m, sCH,
                              h),
-                        w.splitk, w.splitk_elems * 2, s);
+                        w.splitk, w.splitk_elems * (sizeof(double2) / sizeof(cx_t<T>)), s);
 }
 
 // Deflated Rayleigh-Ritz passes of the small SVD (FP64 path, deflate.cu):
@@ -463,7 +470,7 @@ static int rbk_run(const T* A, const RbkDims& d, const tsvd_params& p, const T* 
       } else {
         TSVD_TRY(cgemm<C>(gemm('N', 'N', n2, R, mp, 1.0, w.CHt, m, sCH, w.Uct, R, (long)mp * R, 0.0, w.Vh, R,
                                (long)n2 * R, h),
-                          w.splitk, w.splitk_elems * 2, s));
+                          w.splitk, w.splitk_elems * (sizeof(double2) / sizeof(cx_t<T>)), s));
         done = true;
       }
     }
@@ -471,10 +478,10 @@ static int rbk_run(const T* A, const RbkDims& d, const tsvd_params& p, const T* 
   if (!done) {
     TSVD_TRY(cgemm<C>(gemm('N', 'N', n1, R, mp, 1.0, w.Qt, m, sQ, w.Uct, R, (long)mp * R, 0.0, w.Uh, R,
                            (long)n1 * R, h),
-                      w.splitk, w.splitk_elems * 2, s));
+                      w.splitk, w.splitk_elems * (sizeof(double2) / sizeof(cx_t<T>)), s));
     TSVD_TRY(cgemm<C>(gemm('N', 'N', n2, R, mp, 1.0, w.CHt, m, sCH, w.Uct, R, (long)mp * R, 0.0, w.Vh, R,
                            (long)n2 * R, h),
-                      w.splitk, w.splitk_elems * 2, s));
+                      w.splitk, w.splitk_elems * (sizeof(double2) / sizeof(cx_t<T>)), s));
   }
   TSVD_TRY(scale_columns_inv<T>(w.Vh, R, (long)n2 * R, n2, R, w.lam, h, s));
   }
