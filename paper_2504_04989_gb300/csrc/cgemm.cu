@@ -356,6 +356,8 @@ static int cgemm_impl(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, c
   if (g.batch > 65535) return TSVD_ERR_UNSUPPORTED;
   if (g.beta != 0.0 && g.beta != 1.0) return TSVD_ERR_INVALID_ARG;
   if constexpr (std::is_same<C, float2>::value) {
+    const size_t bytes = splitk_ws ? splitk_elems * sizeof(C) : 0;
+    if (!g.simt && !herm && sgemm_tc_better(g, bytes)) return sgemm_tc(g, splitk_ws, bytes, s);
     // the wide tiles where they fill the GPU (two CTAs per SM), directly or by splitting a long K;
     // smaller products keep the 64 x 64 tiles (measured faster there)
     const long wtiles = (long)cdiv(g.M, WBM) * cdiv(g.N, WBN) * g.batch;
@@ -405,8 +407,10 @@ size_t cgemm_scratch(int M, int N, int K, int batch) {
   if constexpr (std::is_same<C, double2>::value) {
     const size_t bytes = dgemm_tc_bytes(M, N, K, batch);
     return dgemm_tc_better(g, bytes) ? bytes / sizeof(C) + 1 : 0;
+  } else {
+    const size_t bytes = sgemm_tc_bytes(M, N, K, batch);
+    return sgemm_tc_better(g, bytes) ? bytes / sizeof(C) + 1 : 0;
   }
-  return 0;
 }
 template size_t cgemm_scratch<double2>(int, int, int, int);
 template size_t cgemm_scratch<float2>(int, int, int, int);

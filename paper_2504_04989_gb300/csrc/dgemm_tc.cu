@@ -193,6 +193,7 @@ __device__ __forceinline__ double fixed_to_double(long long hi, long long lo, in
 
 __global__ void __launch_bounds__(DG_THREADS, 1) k_dgemm_tc(const __grid_constant__ CUtensorMap tmA,
                                                             const __grid_constant__ CUtensorMap tmB,
+                                                            const __grid_constant__ DotSrc<double2> src,
                                                             const int* __restrict__ EA, const int* __restrict__ EB,
                                                             double2* __restrict__ C, long ldc, long sC, int M, int N,
                                                             int nk, double alpha, int beta, int upper) {
@@ -340,7 +341,9 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dgemm_tc(const __grid_constan
           if (ok && ea < 0x7ff && eb < 0x7ff) {
             const int e = ea + eb + 40 - 2 * 1077;  // the levels carry 256^5 = 2^40
             v = make_double2(fixed_to_double(hi[q], lo[q], e), fixed_to_double(hi[q + 1], lo[q + 1], e));
-          } else {  // a row or column holding an infinity or NaN (or a pipeline that gave up)
+          } else if (ok && src.A) {  // a row or column holding an infinity or NaN
+            v = direct_dot(src, bz, row, col);
+          } else {  // (or its operand overwritten in place, or a pipeline that gave up)
             v = make_double2(__longlong_as_double(0x7ff8000000000000ll), __longlong_as_double(0x7ff8000000000000ll));
           }
           if (alpha != 1.0) v = cscale(v, alpha);
@@ -439,7 +442,8 @@ int dgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s, bool upp
     TSVD_TRY(digit_map(&ma, DA, g.M, 2 * g.K, ldk, n * DG_D, DG_BM));
     TSVD_TRY(digit_map(&mb, DB, N2, 2 * g.K, ldk, n * DG_D, DG_BN));
     const dim3 grid(cdiv(N2, DG_BN), cdiv(g.M, DG_BM), n);
-    k_dgemm_tc<<<grid, DG_THREADS, DG_SMEM, s>>>(ma, mb, EA, EB, (double2*)g.C + (long)b0 * g.sC, g.ldc, g.sC, g.M,
+    const DotSrc<double2> src{g.C == g.A || g.C == g.B ? nullptr : A, B, g.lda, g.sA, g.ldb, g.sB, g.K, ta, !tb};
+    k_dgemm_tc<<<grid, DG_THREADS, DG_SMEM, s>>>(ma, mb, src, EA, EB, (double2*)g.C + (long)b0 * g.sC, g.ldc, g.sC, g.M,
                                                  g.N, cdiv(2L * g.K, DG_KB), g.alpha, g.beta != 0.0, upper ? 1 : 0);
     TSVD_LAUNCHED();
   }

@@ -90,6 +90,12 @@ size_t dgemm_tc_bytes(int M, int N, int K, int batch);
 bool dgemm_tc_better(const GemmArgs& g, size_t bytes);
 int dgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s, bool upper);
 
+// sgemm_tc.cu -- the FP32 product on the TF32 tensor cores at FP32 accuracy (cgemm takes it where
+// sgemm_tc_better says so), as above
+size_t sgemm_tc_bytes(int M, int N, int K, int batch);
+bool sgemm_tc_better(const GemmArgs& g, size_t bytes);
+int sgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s);
+
 // element-wise conversions of batched complex matrices (rows x cols, leading dims)
 int convert_c64_to_c32(const double2* src, long lds, long ss, float2* dst, long ldd, long sd, int rows, int cols,
                        int batch, cudaStream_t s);

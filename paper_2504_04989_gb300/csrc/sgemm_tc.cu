@@ -1,0 +1,333 @@
+// sgemm_tc.cu -- FP32 complex GEMM on the TF32 tensor cores with FP32 accuracy.
+//
+// Each operand is split x = hi + lo, hi the nearest TF32 and lo the nearest TF32 of
+// the rest (2^-23 relative), and hi hi + hi lo + lo hi is accumulated on tcgen05.  The
+// tensor cores truncate when they add to an accumulator (measured: a sum kept in TMEM
+// shrinks by about 2e-8 per instruction, 1.4e-5 after 1024 complex terms), so an
+// accumulator holds 32 terms of K only -- the two small products first, then four
+// instructions of hi hi -- and is then read and added to sums in registers, rounded to
+// nearest, in runs of eight readings; two accumulators alternate so that the reading
+// runs under the next products.  Against exact dot products of normal data the result
+// is closer than FP32 multiply-adds' (the figures stand at sgemm_tc_better).
+//
+// A complex product is the real product of the interleaved rows of op(A) with the
+// expanded real form of op(B) (rows 2n and 2n + 1 per column n, as in tc_gemm.cu),
+// both written as hi / lo rows by one pass over each operand.
+//
+// Bound: the tensor cores at a third of the TF32 rate (355 TFLOP/s), just above what L2
+// delivers of the 64 KB of operands per 128 x 128 x 32 block.
+#include <cmath>
+
+#include "common.cuh"
+#include "kernels.cuh"
+#include "tc_common.cuh"
+
+namespace tsvd {
+
+constexpr int SG_BM = 128, SG_BN = 128;  // complex rows x real columns
+constexpr int SG_KB = 32;                // K per stage: rows of 128 bytes, 128-byte swizzle
+constexpr int SG_STAGES = 3;
+constexpr int SG_TILE = SG_BM * SG_KB * 4;
+constexpr int SG_STAGE_BYTES = 4 * SG_TILE;  // A hi, B hi, A lo, B lo
+constexpr int SG_SMEM = SG_STAGES * SG_STAGE_BYTES + 1024 + 256;
+constexpr int SG_RUN = 8;                // readings summed before they join the total
+constexpr int SG_DRAIN = 256;            // threads reading the accumulators, then one TMA and one MMA warp
+constexpr int SG_THREADS = SG_DRAIN + 64;
+constexpr int SG_OUT = SG_BN / 2;        // columns per reading thread
+static_assert(SG_SMEM <= 227 * 1024, "the stages must fit a CTA's shared memory");
+
+__device__ __forceinline__ float rna_tf32(float x) {
+  uint32_t r;
+  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
+  return __uint_as_float(r);
+}
+
+// One stored complex matrix to hi / lo rows of 2K floats (row length ldk): TRANS, EXPAND and conj
+// as in k_dig_pack.
+template <bool TRANS, bool EXPAND>
+__global__ void __launch_bounds__(256) k_split_pack(const float2* __restrict__ S, long ld, long ss, int rows, int K,
+                                                    bool conj, float* __restrict__ Hi, float* __restrict__ Lo,
+                                                    long ldk) {
+  __shared__ float2 t[TRANS ? 32 : 1][33];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, b = blockIdx.z;
+  const int k0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
+  S += (long)b * ss;
+  if (TRANS) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int k = k0 + ty + 8 * i, r = r0 + tx;
+      t[ty + 8 * i][tx] = (k < K && r < rows) ? S[(long)k * ld + r] : make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+  }
+  const int k = k0 + tx;
+  if (k >= K) return;
+  const long so = (long)b * rows * (EXPAND ? 2 : 1) * ldk;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int r = r0 + ty + 8 * i;
+    if (r >= rows) continue;
+    float2 v = TRANS ? t[tx][ty + 8 * i] : S[(long)r * ld + k];
+    if (conj) v.y = -v.y;
+    const float hx = rna_tf32(v.x), hy = rna_tf32(v.y), lx = rna_tf32(v.x - hx), ly = rna_tf32(v.y - hy);
+    const long o = so + (long)(EXPAND ? 2 * r : r) * ldk + 2 * k;
+    if (EXPAND) {
+      *(float2*)(Hi + o) = make_float2(hx, -hy);
+      *(float2*)(Lo + o) = make_float2(lx, -ly);
+      *(float2*)(Hi + o + ldk) = make_float2(hy, hx);
+      *(float2*)(Lo + o + ldk) = make_float2(ly, lx);
+    } else {
+      *(float2*)(Hi + o) = make_float2(hx, hy);
+      *(float2*)(Lo + o) = make_float2(lx, ly);
+    }
+  }
+}
+
+__device__ __forceinline__ uint64_t smem_desc_sw128_k(uint32_t addr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((addr & 0x3FFFFu) >> 4);
+  d |= (uint64_t)1 << 16;
+  d |= (uint64_t)(1024 >> 4) << 32;  // 8 rows of 128 bytes
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)2 << 61;  // swizzle 128B
+  return d;
+}
+
+__global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constant__ CUtensorMap tmAh,
+                                                            const __grid_constant__ CUtensorMap tmAl,
+                                                            const __grid_constant__ CUtensorMap tmBh,
+                                                            const __grid_constant__ CUtensorMap tmBl,
+                                                            const __grid_constant__ DotSrc<float2> src,
+                                                            float2* __restrict__ C, long ldc, long sC, int M, int N,
+                                                            int nk, float alpha, int beta) {
+  extern __shared__ unsigned char sg_raw[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int n0 = blockIdx.x * SG_BN, m0 = blockIdx.y * SG_BM, bz = blockIdx.z;
+  unsigned char* base = (unsigned char*)(((uintptr_t)sg_raw + 1023) & ~(uintptr_t)1023);
+  uint64_t* bars = (uint64_t*)(base + SG_STAGES * SG_STAGE_BYTES);  // full[S], empty[S], tfull[2], tempty[2]
+  uint32_t* tslot = (uint32_t*)(bars + 2 * SG_STAGES + 4);
+  const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + SG_STAGES);
+  const uint32_t tfull = smem_u32(bars + 2 * SG_STAGES), tempty = tfull + 16;
+  if (tid == 0) {
+    for (int s = 0; s < SG_STAGES; ++s) {
+      mbar_init(full0 + 8 * s, 1);
+      mbar_init(empty0 + 8 * s, 1);
+    }
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(tfull + 8 * s, 1);
+      mbar_init(tempty + 8 * s, SG_DRAIN);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
+                 "r"(2 * SG_BN));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  const uint32_t tmem = *tslot;
+
+  if (tid == SG_DRAIN) {  // TMA producer
+    int issued = 0;
+    bool ok = true;
+    for (int kb = 0; kb < nk; ++kb) {
+      const int s = kb % SG_STAGES, round = kb / SG_STAGES;
+      if (round > 0 && !mbar_wait(empty0 + 8 * s, (round - 1) & 1)) {
+        ok = false;
+        break;
+      }
+      const uint32_t dst = smem_u32(base + s * SG_STAGE_BYTES), bar = full0 + 8 * s;
+      mbar_expect_tx(bar, SG_STAGE_BYTES);
+      tma_load_3d(dst, &tmAh, kb * SG_KB, m0, bz, bar);
+      tma_load_3d(dst + SG_TILE, &tmBh, kb * SG_KB, n0, bz, bar);
+      tma_load_3d(dst + 2 * SG_TILE, &tmAl, kb * SG_KB, m0, bz, bar);
+      tma_load_3d(dst + 3 * SG_TILE, &tmBl, kb * SG_KB, n0, bz, bar);
+      issued = kb + 1;
+    }
+    if (!ok) {  // copies in flight land before the CTA gives its shared memory back
+      for (int kb = (issued > SG_STAGES ? issued - SG_STAGES : 0); kb < issued; ++kb)
+        mbar_wait(full0 + 8 * (kb % SG_STAGES), (kb / SG_STAGES) & 1);
+    }
+  } else if (tid == SG_DRAIN + 32) {  // MMA issuer
+    const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(SG_BN >> 3) << 17) |
+                           ((uint32_t)(SG_BM >> 4) << 24);  // FP32 += TF32 TF32^T
+    for (int kb = 0; kb < nk; ++kb) {
+      const int s = kb % SG_STAGES, a = kb & 1;
+      if (kb >= 2 && !mbar_wait(tempty + 8 * a, ((kb >> 1) - 1) & 1)) break;
+      if (!mbar_wait(full0 + 8 * s, (kb / SG_STAGES) & 1)) break;
+      asm volatile("tcgen05.fence::after_thread_sync;");
+      const uint32_t sm = smem_u32(base + s * SG_STAGE_BYTES);
+      const uint64_t ah = smem_desc_sw128_k(sm), bh = smem_desc_sw128_k(sm + SG_TILE);
+      const uint64_t al = smem_desc_sw128_k(sm + 2 * SG_TILE), bl = smem_desc_sw128_k(sm + 3 * SG_TILE);
+      const uint32_t d = tmem + (uint32_t)(a * SG_BN);
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) {  // 32 bytes of K per instruction
+        mma_issue<false>(d, ah + 2 * kk, bl + 2 * kk, idesc, kk > 0);
+        mma_issue<false>(d, al + 2 * kk, bh + 2 * kk, idesc, 1);
+      }
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) mma_issue<false>(d, ah + 2 * kk, bh + 2 * kk, idesc, 1);
+      mma_commit(empty0 + 8 * s);
+      mma_commit(tfull + 8 * a);
+    }
+  } else if (warp < SG_DRAIN / 32) {
+    const int row = m0 + (warp & 3) * 32 + lane;
+    const int col0 = (warp >> 2) * SG_OUT;
+    const uint32_t tw = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)col0;
+    float run[SG_OUT], tot[SG_OUT];
+#pragma unroll
+    for (int q = 0; q < SG_OUT; ++q) run[q] = tot[q] = 0.f;
+    bool ok = true;
+    for (int kb = 0; kb < nk; ++kb) {
+      const int a = kb & 1;
+      ok = mbar_wait(tfull + 8 * a, (kb >> 1) & 1);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      asm volatile("tcgen05.fence::after_thread_sync;");
+#pragma unroll
+      for (int q0 = 0; q0 < SG_OUT; q0 += 16) {
+        uint32_t r[16];
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+            "%14, %15}, [%16];"
+            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+              "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+            : "r"(tw + (uint32_t)(a * SG_BN + q0)));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int u = 0; u < 16; ++u) run[q0 + u] += __uint_as_float(r[u]);
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;");
+      mbar_arrive(tempty + 8 * a);
+      if ((kb & (SG_RUN - 1)) == SG_RUN - 1 || kb == nk - 1) {
+#pragma unroll
+        for (int q = 0; q < SG_OUT; ++q) {
+          tot[q] += run[q];
+          run[q] = 0.f;
+        }
+      }
+    }
+    if (row < M) {
+      float2* crow = C + (long)bz * sC + (long)row * ldc + ((n0 + col0) >> 1);
+      const int left = N - ((n0 + col0) >> 1);  // complex columns from this thread's first
+#pragma unroll
+      for (int q = 0; q < SG_OUT; q += 4) {
+        float2 v[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          v[u] = make_float2(alpha * tot[q + 2 * u], alpha * tot[q + 2 * u + 1]);
+          const int c = q / 2 + u;
+          if (c >= left) continue;
+          if (!ok) v[u] = make_float2(__int_as_float(0x7fc00000), __int_as_float(0x7fc00000));
+          else if (!(fabsf(v[u].x) <= FLT_MAX && fabsf(v[u].y) <= FLT_MAX))  // operands that are not finite
+            v[u] = cscale(direct_dot(src, bz, row, ((n0 + col0) >> 1) + c), alpha);
+          if (beta) v[u] = cadd(v[u], crow[c]);
+        }
+        const int c = q / 2;
+        if (c + 1 < left && ((uintptr_t)(crow + c) & 15) == 0) {
+          *(float4*)(crow + c) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+        } else {
+          if (c < left) crow[c] = v[0];
+          if (c + 1 < left) crow[c + 1] = v[1];
+        }
+      }
+    }
+  }
+  __syncwarp();
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  if (warp == 0) {
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * SG_BN));
+  }
+}
+
+// ---------------------------------------------------------------------------
+// host side
+// ---------------------------------------------------------------------------
+static int split_map(CUtensorMap* tm, const float* ptr, int rows, int K2, long ldk, int batch) {
+  auto enc = get_encode();
+  if (!enc) return TSVD_ERR_CUDA;
+  cuuint64_t dims[3] = {(cuuint64_t)K2, (cuuint64_t)rows, (cuuint64_t)batch};
+  cuuint64_t strides[2] = {(cuuint64_t)(ldk * 4), (cuuint64_t)(ldk * 4 * rows)};
+  cuuint32_t box[3] = {(cuuint32_t)SG_KB, 128, 1};
+  cuuint32_t estr[3] = {1, 1, 1};
+  const CUresult r = enc(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, (void*)ptr, dims, strides, box, estr,
+                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? TSVD_OK : TSVD_ERR_UNSUPPORTED;
+}
+
+static long sg_ldk(int K) { return (2L * K + 3) / 4 * 4; }
+static size_t sg_slice_bytes(int M, int N, int K) { return 8 * (size_t)sg_ldk(K) * (M + 2 * (size_t)N); }
+size_t sgemm_tc_bytes(int M, int N, int K, int batch) {
+  return std::min<size_t>(sg_slice_bytes(M, N, K) * batch, (size_t)3 << 30) + sg_slice_bytes(M, N, K) + 2048;
+}
+
+// Estimated times in microseconds of the two forms: a SIMT tile takes 0.104 (64 x 64) or 0.25 us (128 x
+// 64) per term of K and SM, K split as cgemm splits it.  Measured, product with its operand passes: 1024 x
+// 1024 x 1024 on 33 slices 5.08 -> 1.56 ms (the product alone 1.23: 230 TFLOP/s), 2048 x 100 x 2048 on
+// 17 1230 -> 561 us, 512 x 60 x 512 on 33 109 -> 70.  Error, 2-norm, normal data, K = 97, 512, 1024,
+// 2048, 4096: 1.4, 1.4, 1.4, 1.6, 1.8e-7, the SIMT kernels 1.8, 4.0, 2.6, 4.2, 4.5e-7.
+bool sgemm_tc_better(const GemmArgs& g, size_t bytes) {
+  if (g.K < 1 || g.M < 1 || g.N < 1 || g.K > (1 << 24)) return false;
+  const size_t slice = sg_slice_bytes(g.M, g.N, g.K) + 2048;
+  if (bytes < slice) return false;
+  const double wtiles = (double)cdiv(g.M, 128) * cdiv(g.N, 64) * g.batch;
+  const bool wide = g.K >= 1024 || wtiles >= 2 * 152;
+  const double stiles = wide ? wtiles : (double)cdiv(g.M, 64) * cdiv(g.N, 64) * g.batch;
+  double ks = std::min(16.0, std::max(1.0, std::floor(wide ? (4 * 152 + stiles - 1) / stiles : 2 * 152 / stiles)));
+  ks = std::min(ks, std::max(1.0, g.K / 64.0));
+  const double simt = 4.0 + (ks > 1.0 ? 3.0 : 0.0) + std::ceil(stiles * ks / 152) * (g.K / ks) * (wide ? 0.25 : 0.104);
+  const double tiles = (double)cdiv(g.M, SG_BM) * cdiv(2L * g.N, SG_BN) * g.batch;
+  const double tile_us = 3.0 + cdiv(2L * g.K, SG_KB) * 0.55;
+  const double pack_us = ((double)slice * 1.4 * g.batch) / 4.0e6;
+  const double calls = std::ceil((double)g.batch * slice / (double)bytes);
+  return simt > 10.0 * calls + pack_us + std::ceil(tiles / 152.0) * tile_us;
+}
+
+int sgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s) {
+  const long ldk = sg_ldk(g.K);
+  const int N2 = 2 * g.N;
+  const uintptr_t p0 = ((uintptr_t)ws + 255) & ~(uintptr_t)255;
+  const size_t avail = bytes - (p0 - (uintptr_t)ws) - 1024;
+  const int nb = (int)std::min<size_t>(g.batch, avail / sg_slice_bytes(g.M, g.N, g.K));
+  if (nb < 1) return TSVD_ERR_WORKSPACE;
+  auto up = [](uintptr_t p) { return (p + 255) & ~(uintptr_t)255; };
+  const size_t an = (size_t)nb * g.M * ldk * 4, bn = (size_t)nb * N2 * ldk * 4;
+  float* Ah = (float*)p0;
+  float* Al = (float*)up(p0 + an);
+  float* Bh = (float*)up((uintptr_t)Al + an);
+  float* Bl = (float*)up((uintptr_t)Bh + bn);
+  if (cudaFuncSetAttribute(k_sgemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, SG_SMEM) != cudaSuccess) {
+    cudaGetLastError();
+    return TSVD_ERR_CUDA;
+  }
+  for (int b0 = 0; b0 < g.batch; b0 += nb) {
+    const int n = std::min(nb, g.batch - b0);
+    const float2* A = (const float2*)g.A + (long)b0 * g.sA;
+    const float2* B = (const float2*)g.B + (long)b0 * g.sB;
+    const dim3 ga(cdiv(g.K, 32), cdiv(g.M, 32), n), gb(cdiv(g.K, 32), cdiv(g.N, 32), n);
+    if (g.opA == 'H') k_split_pack<true, false><<<ga, 256, 0, s>>>(A, g.lda, g.sA, g.M, g.K, true, Ah, Al, ldk);
+    else k_split_pack<false, false><<<ga, 256, 0, s>>>(A, g.lda, g.sA, g.M, g.K, false, Ah, Al, ldk);
+    TSVD_LAUNCHED();
+    if (g.opB == 'N') k_split_pack<true, true><<<gb, 256, 0, s>>>(B, g.ldb, g.sB, g.N, g.K, false, Bh, Bl, ldk);
+    else k_split_pack<false, true><<<gb, 256, 0, s>>>(B, g.ldb, g.sB, g.N, g.K, true, Bh, Bl, ldk);
+    TSVD_LAUNCHED();
+    CUtensorMap mah, mal, mbh, mbl;
+    TSVD_TRY(split_map(&mah, Ah, g.M, 2 * g.K, ldk, n));
+    TSVD_TRY(split_map(&mal, Al, g.M, 2 * g.K, ldk, n));
+    TSVD_TRY(split_map(&mbh, Bh, N2, 2 * g.K, ldk, n));
+    TSVD_TRY(split_map(&mbl, Bl, N2, 2 * g.K, ldk, n));
+    const DotSrc<float2> src{A, B, g.lda, g.sA, g.ldb, g.sB, g.K, g.opA == 'H', g.opB == 'H'};
+    k_sgemm_tc<<<dim3(cdiv(N2, SG_BN), cdiv(g.M, SG_BM), n), SG_THREADS, SG_SMEM, s>>>(
+        mah, mal, mbh, mbl, src, (float2*)g.C + (long)b0 * g.sC, g.ldc, g.sC, g.M, g.N, cdiv(2L * g.K, SG_KB),
+        (float)g.alpha, g.beta != 0.0);
+    TSVD_LAUNCHED();
+  }
+  return TSVD_OK;
+}
+
+}  // namespace tsvd
