@@ -24,177 +24,293 @@ namespace tsvd {
 //   vector (so R-tilde = diag(R_live, I) up to a permutation);
 //   M: R-tilde^{-1} with the dead columns set to zero, so that W M is
 //   W_live R_live^{-1} on the live columns and zero on the dead ones.
-// Warp w keeps the entries [32 EPT w, 32 EPT (w+1)) of the packed upper
-// triangle (row-major; lane-strided) in registers, so each step is one round
-// of independent register updates between two barriers, and a warp whose rows
-// are all finished skips the step:
-//   factorisation, step j: S(i,k) -= conj(S(j,i)) S(j,k) / d_j for
-//   j < i <= k, with row j read from shared memory, where its owners
-//   published it when it became final (end of step j-1); the published rows
-//   are R unscaled (row j is divided by sqrt(d_j) when read);
-//   inverse, step l = nb-1 .. 1 (backward substitution R X = I for all
-//   columns at once, B = I initially): B(i,k) -= R(i,l) X(l,k) for
-//   i < l <= k, where X(l,k) = B(l,k) / R_ll, final after step l+1, is
-//   published in a double-buffered row.
+// Panels of P rows, two barriers each.  Every thread keeps a T x T tile of the
+// upper triangle in registers:
+//   factorisation, panel p: the tiles of its rows are published; each warp
+//   eliminates the P diagonal columns (its first lanes, redundantly) together with
+//   32 - P further columns, one lane per column, the row R(j, .) of the diagonal
+//   columns handed round by shuffles; the finished rows are kept in shared
+//   memory and every later tile subtracts their rank-P product;
+//   inverse, panel from the last to the first (R X = I for all columns at
+//   once): the tiles of its rows are published, solved against the panel's
+//   triangle with one lane per column, written out as rows of M, and
+//   subtracted, times R's columns, from every tile above.
+// Bound: the chain of pivots in a panel, and in FP64 its pipe (64 clocks per
+// instruction of one warp).  P = 8, T = 4 in FP32; FP64 takes P = 4 and the
+// smallest tiles that fit (an instruction costs the same whatever the lanes).
+// Against one step and barrier per row, 33 slices: FP32 nb = 25: 23 -> 16 us, 60:
+// 59 -> 29, 120: 272 -> 61; FP64 15: 35 -> 28, 60: 271 -> 202, 120: 1910 -> 1240.
 // ---------------------------------------------------------------------------
-template <typename GC, int EPT, int NTHR>  // NTHR threads, EPT >= nb (nb+1) / 2 / NTHR entries per thread
-__global__ void __launch_bounds__(NTHR) k_chol_inv(const GC* __restrict__ G, long ldg, long sG,
-                                                       GC* __restrict__ Mo, long ldm, long sM, int nb,
-                                                       double shift_rel, double dead_rel,
-                                                       uint32_t* __restrict__ dead_out) {
+
+__device__ __forceinline__ float2 shfl_c(float2 v, int l) {
+  return make_float2(__shfl_sync(0xffffffffu, v.x, l), __shfl_sync(0xffffffffu, v.y, l));
+}
+__device__ __forceinline__ double2 shfl_c(double2 v, int l) {
+  return make_double2(__shfl_sync(0xffffffffu, v.x, l), __shfl_sync(0xffffffffu, v.y, l));
+}
+// T consecutive complex values of shared memory (16-byte aligned)
+template <int T>
+__device__ __forceinline__ void load_t(const float2* p, float2* o) {
+#pragma unroll
+  for (int q = 0; q < T; q += 2) {
+    const float4 a = *(const float4*)(p + q);
+    o[q] = make_float2(a.x, a.y);
+    o[q + 1] = make_float2(a.z, a.w);
+  }
+}
+template <int T>
+__device__ __forceinline__ void load_t(const double2* p, double2* o) {
+#pragma unroll
+  for (int q = 0; q < T; ++q) o[q] = p[q];
+}
+// acc -= a b and acc -= conj(a) b
+template <typename C>
+__device__ __forceinline__ void cfms(C& acc, C a, C b) {
+  acc.x = fma(-a.x, b.x, acc.x);
+  acc.x = fma(a.y, b.y, acc.x);
+  acc.y = fma(-a.x, b.y, acc.y);
+  acc.y = fma(-a.y, b.x, acc.y);
+}
+template <typename C>
+__device__ __forceinline__ void cfmsc(C& acc, C a, C b) {
+  acc.x = fma(-a.x, b.x, acc.x);
+  acc.x = fma(-a.y, b.y, acc.x);
+  acc.y = fma(-a.x, b.y, acc.y);
+  acc.y = fma(a.y, b.x, acc.y);
+}
+
+// P rows per panel
+template <int P>
+__host__ __device__ inline int ch_pad(int nb) { return (nb + P - 1) / P * P; }
+// panel p's rows in the store of R: P rows of n8 - P p values (columns P p ..)
+template <int P>
+__host__ __device__ inline int ch_off(int p, int n8) { return P * (n8 * p - P * (p * (p - 1) / 2)); }
+
+// 1 / sqrt(d) for d > 0, to a rounding or two of the last place: the hardware's FP32 estimate y and one
+// step of its series in e = 1 - d y^2 (to e in FP32, to e^2 in FP64, whose correctly rounded root and
+// division, and even a second Newton step, weigh on the chain of pivots)
+__device__ __forceinline__ float inv_sqrt(float d) {
+  const float y = rsqrtf(d);
+  return fmaf(y, fmaf(-0.5f * d * y, y, 0.5f), y);
+}
+__device__ __forceinline__ double inv_sqrt(double d) {
+  const int h = (__double2hiint(d) >> 20) - 1023;  // d = m 4^e with m in [1, 4)
+  if (h < -1000 || h > 1000) return 1.0 / sqrt(d);
+  const int e2 = h & ~1;
+  const double m = __hiloint2double(__double2hiint(d) - (e2 << 20), __double2loint(d));
+  double y = (double)rsqrtf((float)m);
+  const double e = fma(-m * y, y, 1.0);  // below 2^-21
+  y = fma(y * e, fma(0.375, e, 0.5), y);
+  return __hiloint2double(__double2hiint(y) - (e2 << 19), __double2loint(y));  // y 2^(-e2/2)
+}
+
+// Tiles to threads.  FP32: the triangle's rows one after another.  FP64, whose pipe takes 16 clocks per
+// instruction and warp whatever the lanes: a warp holds a block of 4 x 8 tiles, so that the tiles of a
+// warp are active in the same steps of the inverse (23 instead of 49 warp-steps at n8 = 64).
+template <typename GC>
+struct ChMap {  // float2
+  static __host__ __device__ int threads(int ntl) { return (ntl * (ntl + 1) / 2 + 31) / 32 * 32; }
+  static __device__ void tile(int tid, int ntl, int* ta, int* tb) {
+    int a = 0, b = tid;
+    while (a < ntl && b >= ntl - a) {
+      b -= ntl - a;
+      ++a;
+    }
+    *ta = a;
+    *tb = a + b;
+  }
+};
+template <>
+struct ChMap<double2> {
+  static __host__ __device__ int first(int a) { return a / 2; }  // first block column of block row a
+  static __host__ __device__ int threads(int ntl) {
+    int n = 0;
+    for (int a = 0; 4 * a < ntl; ++a) n += (ntl + 7) / 8 - first(a);
+    return 32 * n;
+  }
+  static __device__ void tile(int tid, int ntl, int* ta, int* tb) {
+    int a = 0, w = tid >> 5;
+    const int cols = (ntl + 7) / 8, lane = tid & 31;
+    while (4 * a < ntl && w >= cols - first(a)) {
+      w -= cols - first(a);
+      ++a;
+    }
+    *ta = 4 * a + (lane >> 3);
+    *tb = 8 * (first(a) + w) + (lane & 7);
+  }
+};
+
+template <typename GC, int CH_P, int CH_T, int NT>  // CH_P rows per panel, tiles of edge CH_T; NT: most threads
+__global__ void __launch_bounds__(NT, 1) k_chol_inv(const GC* __restrict__ G, long ldg, long sG,
+                                                      GC* __restrict__ Mo, long ldm, long sM, int nb,
+                                                      double shift_rel, double dead_rel,
+                                                      uint32_t* __restrict__ dead_out) {
   using Rt = decltype(GC().x);
+  constexpr int TPP = CH_P / CH_T, CH_COLS = 32 - CH_P;  // tile rows per panel; columns a warp eliminates beside the diagonal ones
   extern __shared__ __align__(16) unsigned char chsm[];
-  GC* S = (GC*)chsm;               // published rows of the packed triangle: S(i, k) = S[rb(i) + k]
-  GC* Xr = S + nb * (nb + 1) / 2;  // [2][nb] published rows of X
-  __shared__ Rt dg[128];           // diagonal of G (pivot test of the plain passes)
-  __shared__ Rt dj[128];           // pivots d_j (0 for a dead column)
-  __shared__ Rt pinv[128];         // 1 / d_j (0 for a dead column)
-  __shared__ Rt ri[128];           // 1 / R-tilde_jj
-  __shared__ double red[NTHR / 32];
-  const int b = blockIdx.x, tid = threadIdx.x;
-  const int np = nb * (nb + 1) / 2;
-  auto rb = [nb](int i) { return i * nb - (i * (i + 1)) / 2; };  // packed offset of row i, minus i
+  const int n8 = ch_pad<CH_P>(nb), NP = n8 / CH_P, NTL = n8 / CH_T;
+  GC* S = (GC*)chsm;           // R by panels
+  GC* Raw = S + ch_off<CH_P>(NP, n8);  // [8][n8] published rows
+  GC* Xb = Raw + CH_P * n8;      // [8][n8] solved rows of the inverse
+  __shared__ Rt thr[128];        // a pivot at or below it is dead
+  __shared__ Rt ri[128];         // 1 / R-tilde_jj
+  __shared__ int live[128];
+  __shared__ double red[NT / 32];
+  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   G += (long)b * sG;
   Mo += (long)b * sM;
-  if (tid < nb) dg[tid] = G[(long)tid * ldg + tid].x;
-  // row of packed index p: largest i with rb(i) + i <= p (closed form in FP32 -- GB300's FP64
-  // unit is narrow -- then corrected exactly)
-  auto row_of = [&](int p) {
-    const float q = 2.0f * nb + 1.0f;
-    int i = (int)((q - sqrtf(fmaxf(q * q - 8.0f * p, 0.0f))) * 0.5f);
-    i = max(0, min(i, nb - 1));
-    while (i > 0 && rb(i) + i > p) --i;
-    while (i + 1 < nb && rb(i + 1) + i + 1 <= p) ++i;
-    return i;
-  };
-  // warp w owns the packed range [32 EPT w, 32 EPT (w+1)), lane-strided; its first and last
-  // rows decide when it has nothing left to do (rows <= j in the factorisation, >= l in the inverse)
-  const int warp = tid >> 5, lane = tid & 31;
-  const int pw0 = 32 * EPT * warp, pw1 = min(pw0 + 32 * EPT, np) - 1;
-  const int wrow0 = (pw0 < np) ? row_of(pw0) : nb, wrow1 = (pw0 < np) ? row_of(pw1) : -1;
-  // owned entries: (row, column) (-1 if none), packed offset and value
-  int ei[EPT], ek[EPT];  // the packed offset of entry e is pw0 + 32 e + lane (a constant per e)
-  GC v[EPT];
+  const GC zero{Rt(0), Rt(0)};
+  int ta, tb;  // this thread's tile; none off the upper triangle
+  ChMap<GC>::tile(tid, NTL, &ta, &tb);
+  const bool own = ta < NTL && tb < NTL && ta <= tb;
+  GC v[CH_T][CH_T];
+  const Rt gd = tid < nb ? G[(long)tid * ldg + tid].x : Rt(0);
+  if (tid < 128) thr[tid] = (shift_rel > 0.0 || tid >= nb) ? Rt(0) : (Rt)dead_rel * gd;
 #pragma unroll
-  for (int e = 0; e < EPT; ++e) {
-    const int p = pw0 + 32 * e + lane;
-    int i = -1, k = -1;
-    if (p < np) {
-      i = row_of(p);
-      k = p - rb(i);
+  for (int x = 0; x < CH_T; ++x)
+#pragma unroll
+    for (int y = 0; y < CH_T; ++y) {
+      const int i = CH_T * ta + x, k = CH_T * tb + y;
+      v[x][y] = (own && i <= k && k < nb) ? G[(long)i * ldg + k] : zero;
+      if (i == k && i >= nb) v[x][y].x = Rt(1);  // padding rows: the unit matrix
     }
-    ei[e] = i;
-    ek[e] = k;
-    v[e] = (p < np) ? G[(long)i * ldg + k] : GC{Rt(0), Rt(0)};
-  }
   __syncthreads();
-  const double trace = block_sum(tid < nb ? (double)dg[tid] : 0.0, red);
+  const double trace = block_sum((double)gd, red);
   const Rt sft = (shift_rel > 0.0) ? (Rt)(shift_rel * trace) : Rt(0);
-  // a final diagonal entry d_i: pivot test, published with its row
-  auto pivot = [&](int i, Rt d) {
-    const bool dead = (shift_rel > 0.0) ? !(d > Rt(0)) : !(d > (Rt)dead_rel * dg[i]);
-    dj[i] = dead ? Rt(0) : d;
-    pinv[i] = dead ? Rt(0) : Rt(1) / d;
+  if (own && ta == tb) {
+#pragma unroll
+    for (int x = 0; x < CH_T; ++x)
+      if (CH_T * ta + x < nb) v[x][x].x += sft;
+  }
+  // publish this thread's tile if it lies in panel p's rows
+  auto publish = [&](int p) {
+    if (own && ta / TPP == p) {
+#pragma unroll
+      for (int x = 0; x < CH_T; ++x)
+#pragma unroll
+        for (int y = 0; y < CH_T; ++y) Raw[(CH_T * (ta % TPP) + x) * n8 + CH_T * tb + y] = v[x][y];
+    }
   };
+
+  for (int p = 0; p < NP; ++p) {
+    publish(p);
+    __syncthreads();
+    const int j0 = CH_P * p;
+    // columns of this warp: the 8 diagonal ones and 24 of the rest
+    const int rest = n8 - j0 - CH_P;
+    if (warp == 0 || warp * CH_COLS < rest) {
+      const int kc = lane < CH_P ? lane : CH_P + warp * CH_COLS + lane - CH_P;  // column j0 + kc
+      const bool in = kc < n8 - j0;
+      GC c[CH_P];
 #pragma unroll
-  for (int e = 0; e < EPT; ++e) {
-    if (ei[e] >= 0 && ei[e] == ek[e]) v[e].x += sft;
-    if (ei[e] == 0) {  // row 0 is final
-      S[pw0 + 32 * e + lane] = v[e];
-      if (ek[e] == 0) pivot(0, v[e].x);
-    }
-  }
-  __syncthreads();
-  // every step is branch-free: the operands of each entry are loaded whether or not it is
-  // active (in-range addresses), and the update is selected
-  for (int j = 0; j < nb; ++j) {
-    const GC* Sj = S + rb(j);
-    const Rt inv = pinv[j];
-    if (wrow1 > j) {
+      for (int r = 0; r < CH_P; ++r) c[r] = in ? Raw[r * n8 + j0 + kc] : zero;
 #pragma unroll
-      for (int e = 0; e < EPT; ++e) {
-        const int i = ei[e], k = ek[e];
-        const GC a = Sj[max(i, 0)];
-        const GC c = Sj[max(k, 0)];
-        const Rt ax = a.x * inv, ay = a.y * inv;  // conj(a) / d times c
-        GC t = v[e];
-        t.x = fma(-ax, c.x, t.x);
-        t.x = fma(-ay, c.y, t.x);
-        t.y = fma(-ax, c.y, t.y);
-        t.y = fma(ay, c.x, t.y);
-        if (i > j) v[e] = t;
-        if (i == j + 1) {  // row j+1 is final
-          S[pw0 + 32 * e + lane] = v[e];
-          if (k == i) pivot(i, v[e].x);
+      for (int r = 0; r < CH_P; ++r) {
+        const Rt d = __shfl_sync(0xffffffffu, c[r].x, r);
+        const int j = j0 + r;
+        const bool alive = d > thr[j];
+        const Rt iv = alive ? inv_sqrt(d) : Rt(0);
+        c[r].x *= iv;
+        c[r].y *= iv;
+        if (lane == r) c[r].y = Rt(0);
+        if (warp == 0 && lane == r) {
+          live[j] = alive;
+          ri[j] = alive ? iv : Rt(1);
         }
+#pragma unroll
+        for (int i = r + 1; i < CH_P; ++i) cfmsc(c[i], shfl_c(c[r], i), c[r]);
+      }
+      if (in && (warp == 0 || lane >= CH_P)) {
+        GC* o = S + ch_off<CH_P>(p, n8) + kc;
+#pragma unroll
+        for (int r = 0; r < CH_P; ++r) o[r * (n8 - j0)] = (kc >= r) ? c[r] : zero;
       }
     }
     __syncthreads();
+    if (own && ta / TPP > p) {
+      const GC* P = S + ch_off<CH_P>(p, n8);
+      const int ra = CH_T * ta - j0, rb = CH_T * tb - j0;
+#pragma unroll
+      for (int r = 0; r < CH_P; ++r) {
+        GC x4[CH_T], y4[CH_T];
+        load_t<CH_T>(P + r * (n8 - j0) + ra, x4);
+        load_t<CH_T>(P + r * (n8 - j0) + rb, y4);
+#pragma unroll
+        for (int x = 0; x < CH_T; ++x)
+#pragma unroll
+          for (int y = 0; y < CH_T; ++y) cfmsc(v[x][y], x4[x], y4[y]);
+      }
+    }
   }
-  if (tid < nb) ri[tid] = (dj[tid] > Rt(0)) ? Rt(1) / sqrt(dj[tid]) : Rt(1);
   __syncthreads();
-  // inverse: B in the registers (0 above the diagonal, 1 on it); R-tilde(i, l) = R(i, l) / sqrt(d_i)
-  // read from the published rows (0 where row i or column l is dead)
-  Rt er[EPT];  // 1 / R-tilde_ii of the entry's row, 0 for a dead row
+  // R-tilde: dead columns zero (dead rows are already)
+  for (int k = warp; k < nb; k += blockDim.x >> 5)
+    if (!live[k])
+      for (int i = lane; i < k; i += 32) {
+        const int q = i / CH_P;
+        S[ch_off<CH_P>(q, n8) + (i - CH_P * q) * (n8 - CH_P * q) + k - CH_P * q] = zero;
+      }
 #pragma unroll
-  for (int e = 0; e < EPT; ++e) {
-    const int i = max(ei[e], 0);
-    er[e] = (dj[i] > Rt(0)) ? ri[i] : Rt(0);
-    v[e] = GC{Rt(0), Rt(0)};
-  }
-  for (int l = nb - 1; l >= 1; --l) {
-    const GC* xl = Xr + (l & 1) * nb;  // X(l, k), k > l
-    const Rt rl = ri[l];
-    const bool live_l = dj[l] > Rt(0);
-    if (wrow0 < l) {
+  for (int x = 0; x < CH_T; ++x)
 #pragma unroll
-      for (int e = 0; e < EPT; ++e) {
-        const int i = ei[e], k = ek[e];
-        const int ic = max(i, 0), kc = max(k, 0);
-        const GC cr = S[rb(ic) + l];
-        const GC xv = xl[kc];
-        const Rt sc = live_l ? er[e] : Rt(0);
-        const Rt cx = cr.x * sc, cy = cr.y * sc;
-        const GC x = (k == l) ? GC{rl, Rt(0)} : xv;
-        GC t = v[e];
-        t.x = fma(-cx, x.x, t.x);
-        t.x = fma(cy, x.y, t.x);
-        t.y = fma(-cx, x.y, t.y);
-        t.y = fma(-cy, x.x, t.y);
-        if (i >= 0 && i < l && k >= l) v[e] = t;
-        if (i == l - 1 && k > i) {  // row l-1 of B is final: publish X(l-1, k)
-          const Rt s2 = ri[i];
-          Xr[((l - 1) & 1) * nb + k] = GC{v[e].x * s2, v[e].y * s2};
-        }
+    for (int y = 0; y < CH_T; ++y) {
+      v[x][y] = zero;
+      if (ta == tb && x == y) v[x][y].x = Rt(1);
+    }
+  for (int p = NP - 1; p >= 0; --p) {
+    publish(p);
+    __syncthreads();
+    const int j0 = CH_P * p, len = n8 - j0;
+    const GC* P = S + ch_off<CH_P>(p, n8);
+    for (int kc = tid; kc < len; kc += blockDim.x) {
+      const int k = j0 + kc;
+      GC x[CH_P];
+#pragma unroll
+      for (int r = 0; r < CH_P; ++r) x[r] = (kc >= r || kc >= CH_P) ? Raw[r * n8 + k] : zero;
+#pragma unroll
+      for (int r = CH_P - 1; r >= 0; --r) {
+#pragma unroll
+        for (int q = r + 1; q < CH_P; ++q) cfms(x[r], P[r * len + q], x[q]);
+        const Rt s = ri[j0 + r];
+        x[r].x *= s;
+        x[r].y *= s;
+      }
+#pragma unroll
+      for (int r = 0; r < CH_P; ++r) {
+        Xb[r * n8 + k] = x[r];
+        if (j0 + r < nb && k < nb && k >= j0 + r) Mo[(long)(j0 + r) * ldm + k] = live[k] ? x[r] : zero;
       }
     }
     __syncthreads();
-  }
-  // M(i, k) = B(i, k) / R_ii (M(i, i) = 1 / R_ii); dead columns and the lower triangle zero
+    if (own && ta / TPP < p && tb / TPP >= p) {
+      const int rp = ta / TPP, rl = n8 - CH_P * rp;  // the panel that holds this tile's rows of R
+      const GC* A = S + ch_off<CH_P>(rp, n8) + CH_T * (ta % TPP) * rl + j0 - CH_P * rp;
 #pragma unroll
-  for (int e = 0; e < EPT; ++e) {
-    const int i = ei[e], k = ek[e];
-    if (i < 0) continue;
-    GC mv = GC{Rt(0), Rt(0)};
-    if (dj[k] > Rt(0)) {
-      if (k == i) {
-        mv.x = ri[i];
-      } else {
-        mv.x = v[e].x * ri[i];
-        mv.y = v[e].y * ri[i];
+      for (int q0 = 0; q0 < CH_P; q0 += CH_T) {
+        GC a4[CH_T][CH_T];
+#pragma unroll
+        for (int x = 0; x < CH_T; ++x) load_t<CH_T>(A + x * rl + q0, a4[x]);
+#pragma unroll
+        for (int q = 0; q < CH_T; ++q) {
+          GC y4[CH_T];
+          load_t<CH_T>(Xb + (q0 + q) * n8 + CH_T * tb, y4);
+#pragma unroll
+          for (int x = 0; x < CH_T; ++x)
+#pragma unroll
+            for (int y = 0; y < CH_T; ++y) cfms(v[x][y], a4[x][q], y4[y]);
+        }
       }
     }
-    Mo[(long)i * ldm + k] = mv;
   }
-  for (int e = tid; e < nb * nb; e += NTHR) {
+  for (int e = tid; e < nb * nb; e += blockDim.x) {
     const int i = e / nb, k = e - i * nb;
-    if (k < i) Mo[(long)i * ldm + k] = GC{Rt(0), Rt(0)};
+    if (k < i) Mo[(long)i * ldm + k] = zero;
   }
   if (tid < 4) {
     uint32_t msk = 0;
     for (int q = 0; q < 32; ++q) {
       const int jj = tid * 32 + q;
-      if (jj < nb && !(dj[jj] > Rt(0))) msk |= 1u << q;
+      if (jj < nb && !live[jj]) msk |= 1u << q;
     }
     dead_out[b * 4 + tid] = msk;
   }
@@ -205,10 +321,8 @@ int chol_inv(const GC* G, long ldg, long sG, GC* M, long ldm, long sM, int nb, i
              double dead_rel, uint32_t* dead, cudaStream_t s) {
   if (nb <= 0 || batch <= 0) return TSVD_OK;
   if (nb > 128) return TSVD_ERR_UNSUPPORTED;
-  const int np = nb * (nb + 1) / 2;
-  const size_t smem = ((size_t)np + 2 * (size_t)nb) * sizeof(GC);  // published rows + X rows
-  auto go = [&](auto kern, int nthr) {
-    // with the kernel's static arrays (about 4 KB) the total passes the 48 KB default earlier
+  auto go = [&](auto kern, int n8, int off, int nthr) {
+    const size_t smem = ((size_t)off + 2 * (size_t)(n8 % 8 ? 4 : 8) * n8) * sizeof(GC);
     if (smem > 40 * 1024 &&
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
       cudaGetLastError();
@@ -218,18 +332,24 @@ int chol_inv(const GC* G, long ldg, long sG, GC* M, long ldm, long sM, int nb, i
     TSVD_LAUNCHED();
     return TSVD_OK;
   };
-  // 512 threads (16 warps: a step's latency is hidden across warps; 128 threads with 16 entries
-  // each measured twice as slow at nb = 60)
-  if (np <= 2 * 512) return go(k_chol_inv<GC, 2, 512>, 512);
-  if (np <= 4 * 512) return go(k_chol_inv<GC, 4, 512>, 512);
-  if (np <= 8 * 512) return go(k_chol_inv<GC, 8, 512>, 512);
-  // larger Grams up to 8192 packed entries (90 < nb <= 127), FP32: 1024 threads with 8 entries
-  // each rather than 17 on 512 (each warp's chain of a step halves and twice the warps hide it;
-  // FP64 spills at 1024 x 8)
-  if constexpr (std::is_same<GC, float2>::value)
-    if (np <= 8 * 1024) return go(k_chol_inv<GC, 8, 1024>, 1024);
-  static_assert(17 * 512 >= 128 * 129 / 2, "the last variant covers every nb <= 128");
-  return go(k_chol_inv<GC, 17, 512>, 512);
+  // at least 128 threads: one per diagonal entry
+  if constexpr (std::is_same<GC, double2>::value) {
+    // FP64: panels of 4 (the panel's own elimination is one warp's work, at 64 clocks per FP64
+    // instruction of one warp) and the smallest tiles that fit 1024 threads
+    const int n4 = ch_pad<4>(nb), t1 = ChMap<GC>::threads(n4), t2 = ChMap<GC>::threads(n4 / 2);
+    if (t1 <= 1024) return go(k_chol_inv<GC, 4, 1, 1024>, n4, ch_off<4>(n4 / 4, n4), std::max(128, t1));
+    if (t2 <= 1024) return go(k_chol_inv<GC, 4, 2, 1024>, n4, ch_off<4>(n4 / 4, n4), t2);
+  }
+  const int n8 = ch_pad<8>(nb), off = ch_off<8>(n8 / 8, n8), nthr = std::max(128, ChMap<GC>::threads(n8 / 4));
+  // registers: 4 x 4 tiles and a panel's operands take 125 in FP32, 167 in FP64
+  if constexpr (std::is_same<GC, float2>::value) {
+    if (nthr <= 256) return go(k_chol_inv<GC, 8, 4, 256>, n8, off, nthr);
+    if (nthr <= 512) return go(k_chol_inv<GC, 8, 4, 512>, n8, off, nthr);  // n8 <= 120
+    return go(k_chol_inv<GC, 8, 4, 544>, n8, off, nthr);                   // 128: 32 * 33 / 2 tiles
+  } else {
+    if (nthr <= 384) return go(k_chol_inv<GC, 8, 4, 384>, n8, off, nthr);  // n8 <= 96
+    return go(k_chol_inv<GC, 8, 4, 640>, n8, off, nthr);                   // 128: 20 blocks
+  }
 }
 template int chol_inv<double2>(const double2*, long, long, double2*, long, long, int, int, double, double, uint32_t*,
                                cudaStream_t);
@@ -615,9 +735,11 @@ int orth_block_cols(int n1, int b, int m, int h, const OrthWs& w, int c, int nb,
       CL* out = pass < 2 ? W : Q + c;
       const long ldo = pass < 2 ? b : m, so = pass < 2 ? sW : sQ;
       const GemmArgs g = gemm('N', 'N', n1, nb, nb, 1.0, W, b, sW, Mi, b, sG, 0.0, out, ldo, so, h);
-      // the digit form reads copies of its operands, so it may write W in place
+      // the tensor-core forms read copies of their operands, so they may write W in place
       if (std::is_same<L, double>::value && dgemm_tc_better(g, sk * sizeof(CL)))
         TSVD_TRY(dgemm_tc(g, w.splitk, sk * sizeof(CL), s, false));
+      else if (std::is_same<L, float>::value && sgemm_tc_better(g, sk * sizeof(CL)))
+        TSVD_TRY(sgemm_tc(g, w.splitk, sk * sizeof(CL), s));
       else
         TSVD_TRY(rmul_block<CL>(W, b, sW, Mi, b, sG, n1, nb, h, out, ldo, so, s));
     }

@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constan
           const int c = q / 2 + u;
           if (c >= left) continue;
           if (!ok) v[u] = make_float2(__int_as_float(0x7fc00000), __int_as_float(0x7fc00000));
-          else if (!(fabsf(v[u].x) <= FLT_MAX && fabsf(v[u].y) <= FLT_MAX))  // operands that are not finite
+          else if (src.A && !(fabsf(v[u].x) <= FLT_MAX && fabsf(v[u].y) <= FLT_MAX))  // operands that are not finite
             v[u] = cscale(direct_dot(src, bz, row, ((n0 + col0) >> 1) + c), alpha);
           if (beta) v[u] = cadd(v[u], crow[c]);
         }
@@ -321,7 +321,7 @@ int sgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s) {
     TSVD_TRY(split_map(&mal, Al, g.M, 2 * g.K, ldk, n));
     TSVD_TRY(split_map(&mbh, Bh, N2, 2 * g.K, ldk, n));
     TSVD_TRY(split_map(&mbl, Bl, N2, 2 * g.K, ldk, n));
-    const DotSrc<float2> src{A, B, g.lda, g.sA, g.ldb, g.sB, g.K, g.opA == 'H', g.opB == 'H'};
+    const DotSrc<float2> src{g.C == g.A || g.C == g.B ? nullptr : A, B, g.lda, g.sA, g.ldb, g.sB, g.K, g.opA == 'H', g.opB == 'H'};
     k_sgemm_tc<<<dim3(cdiv(N2, SG_BN), cdiv(g.M, SG_BM), n), SG_THREADS, SG_SMEM, s>>>(
         mah, mal, mbh, mbl, src, (float2*)g.C + (long)b0 * g.sC, g.ldc, g.sC, g.M, g.N, cdiv(2L * g.K, SG_KB),
         (float)g.alpha, g.beta != 0.0);
