@@ -91,6 +91,24 @@ __device__ __forceinline__ float2 from_c64<float2>(double2 a) {
   return make_float2((float)a.x, (float)a.y);
 }
 
+// 1 / sqrt(d) for d > 0, to a rounding or two of the last place: the hardware's FP32 estimate y and one
+// step of its series in e = 1 - d y^2 (to e in FP32, to e^2 in FP64, whose correctly rounded root and
+// division, and even a second Newton step, weigh on a serial chain)
+__device__ __forceinline__ float inv_sqrt(float d) {
+  const float y = rsqrtf(d);
+  return fmaf(y, fmaf(-0.5f * d * y, y, 0.5f), y);
+}
+__device__ __forceinline__ double inv_sqrt(double d) {
+  const int h = (__double2hiint(d) >> 20) - 1023;  // d = m 4^e with m in [1, 4)
+  if (h < -1000 || h > 1000) return 1.0 / sqrt(d);
+  const int e2 = h & ~1;
+  const double m = __hiloint2double(__double2hiint(d) - (e2 << 20), __double2loint(d));
+  double y = (double)rsqrtf((float)m);
+  const double e = fma(-m * y, y, 1.0);  // below 2^-21
+  y = fma(y * e, fma(0.375, e, 0.5), y);
+  return __hiloint2double(__double2hiint(y) - (e2 << 19), __double2loint(y));  // y 2^(-e2/2)
+}
+
 // warp reductions
 __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

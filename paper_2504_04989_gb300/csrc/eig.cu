@@ -15,6 +15,9 @@
 #include <cooperative_groups.h>
 #include <float.h>
 
+#include <mutex>
+#include <type_traits>
+
 #include "common.cuh"
 #include "kernels.cuh"
 
@@ -22,555 +25,43 @@ namespace cg = cooperative_groups;
 
 namespace tsvd {
 
-constexpr int HETRD_CLUSTER = 4;
-
 struct EigScratch {
   double* d;       // [batch][m] diagonal of T
   double* f;       // [batch][m] off-diagonal |alpha_j|
   double2* alpha;  // [batch][m] complex off-diagonals of T'
   double2* delta;  // [batch][m] phases making T real
   double2* Hv;     // [batch][m][m] Householder vectors (row j, columns j+1..m-1)
-  double2* pbuf;   // [batch][HETRD_CLUSTER][m] partial matrix-vector products of a cluster
   double* Z;       // [batch][R][m] real eigenvectors of T (vector-contiguous)
   double* lu;      // [batch][5][m][R] inverse-iteration LU factors
   double* tnorm;   // [batch]
   double2* Sg;     // packed own rows of the cluster reduction when they do not fit in shared memory
+  double2* Cp;     // the warps' partials of p where they do not
 };
 
-static bool hetrd_needs_global_rows(int m, int batch);
-
-static EigScratch carve_eig(void* base, int m, int R, int batch, size_t* bytes) {
-  Carver cv(base);
-  EigScratch e;
-  e.d = cv.take<double>((size_t)batch * m);
-  e.f = cv.take<double>((size_t)batch * m);
-  e.alpha = cv.take<double2>((size_t)batch * m);
-  e.delta = cv.take<double2>((size_t)batch * m);
-  e.Hv = cv.take<double2>((size_t)batch * m * m);
-  e.pbuf = cv.take<double2>((size_t)batch * HETRD_CLUSTER * m);
-  e.Z = cv.take<double>((size_t)batch * m * R);
-  e.lu = cv.take<double>((size_t)batch * 5 * m * R);
-  e.tnorm = cv.take<double>((size_t)batch);
-  // CL CTAs of a slice own at most m(m+1)/2 + CL m packed elements together (CL <= 8)
-  e.Sg = hetrd_needs_global_rows(m, batch) ? cv.take<double2>((size_t)batch * ((size_t)m * (m + 1) / 2 + 8 * (size_t)m))
-                                           : nullptr;
-  if (bytes) *bytes = cv.bytes();
-  return e;
-}
-
-size_t eig_scratch_bytes(int m, int R, int batch) {
-  size_t b = 0;
-  carve_eig(nullptr, m, R, batch, &b);
-  return b;
-}
-
-__device__ __forceinline__ double2 ldcg2(const double2* p) { return __ldcg(p); }
-
 // ---------------------------------------------------------------------------
-// Householder tridiagonalisation, one cluster of CL CTAs per slice; only the
-// lower triangle of G is read and updated.  Rows of the trailing block are
-// owned round-robin (global row g by CTA g mod CL).  Step j:
-//   x = G(j+1:, j), alpha = -e^{i arg x_0} ||x||, v = (x - alpha e_1)/||.||
-//   (every CTA forms the same v);
-//   p = 2 A v from the lower triangle: each CTA adds, for its rows r, the row
-//   part sum_{k<=r} A(r,k) v_k to p_r and the transposed part conj(A(r,k)) v_r
-//   to p_k (k < r) into a shared partial, then the CL partials are summed
-//   after a cluster barrier;
-//   w = p - (v^H p) v;  A(r,k) -= v_r conj(w_k) + w_r conj(v_k) for k <= r.
-// Data another CTA wrote is read with L2-coherent loads after the barrier
-// (release / acquire at cluster scope).
+// Householder tridiagonalisation: a cluster of CL CTAs (one per SM) holds the
+// lower triangle of one slice, row g in CTA g mod CL.
 // ---------------------------------------------------------------------------
-template <int CL>
-__global__ void __launch_bounds__(512) k_hetrd(double2* __restrict__ G, long ldg, long sG, int m, EigScratch e) {
-  extern __shared__ __align__(16) double2 sh[];
-  double2* v = sh;            // [m]
-  double2* p = sh + m;        // [m] full product / w
-  double2* pw = sh + 2 * m;   // [nwarp][m] per-warp partial products (fixed-order sum: deterministic)
-  __shared__ double red[64];
-  cg::cluster_group cluster = cg::this_cluster();
-  const int rank = (CL > 1) ? (int)cluster.block_rank() : 0;
-  const int b = blockIdx.x / CL;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
-  G += (long)b * sG;
-  double2* Hv = e.Hv + (long)b * m * m;
-  double2* pb = e.pbuf + (long)b * CL * m;  // [CL][m] partial products of the cluster's CTAs
-  double2* mine = pw + (long)warp * m;
-  for (int j = 0; j < m - 1; ++j) {
-    const int n = m - j - 1;
-    double part = 0;
-    for (int i = tid; i < n; i += blockDim.x) {
-      const double2 x = ldcg2(G + (long)(j + 1 + i) * ldg + j);
-      v[i] = x;
-      part += cabs2(x);
-    }
-    for (int i = lane; i < n; i += 32) mine[i] = make_double2(0, 0);
-    const double nrm2 = block_sum(part, red);  // synchronises: v visible
-    const double2 x0 = v[0];
-    const double djj = ldcg2(G + (long)j * ldg + j).x;
-    __syncthreads();
-    if (rank == 0 && tid == 0) e.d[(long)b * m + j] = djj;
-    const bool skip = !(nrm2 > 0.0);  // identical in every CTA of the cluster
-    const int r0 = ((rank - (j + 1)) % CL + CL) % CL;
-    if (!skip) {
-      const double nrm = sqrt(nrm2), ax0 = sqrt(cabs2(x0));
-      const double2 ph = (ax0 > 0) ? cscale(x0, 1.0 / ax0) : make_double2(1, 0);
-      const double2 alpha = cscale(ph, -nrm);
-      const double vinv = 1.0 / sqrt(2.0 * nrm * (nrm + ax0));
-      for (int i = tid; i < n; i += blockDim.x) {
-        double2 vi = v[i];
-        if (i == 0) vi = csub(vi, alpha);
-        vi = cscale(vi, vinv);
-        v[i] = vi;
-        if (rank == 0) Hv[(long)j * m + j + 1 + i] = vi;
-      }
-      if (rank == 0 && tid == 0) e.alpha[(long)b * m + j] = alpha;
-      __syncthreads();
-      // this warp's rows: row part into mine[r], transposed part conj(A(r,k)) v_r into mine[k]
-      for (int r = r0 + warp * CL; r < n; r += nwarp * CL) {
-        const double2* row = G + (long)(j + 1 + r) * ldg + j + 1;
-        const double2 vr = v[r];
-        double2 acc = make_double2(0, 0);
-        for (int k = lane; k <= r; k += 32) {
-          const double2 a = row[k];
-          cfma(acc, a, v[k]);
-          if (k < r) {  // t += conj(a) v_r
-            double2 t = mine[k];
-            t.x = fma(a.x, vr.x, t.x);
-            t.x = fma(a.y, vr.y, t.x);
-            t.y = fma(a.x, vr.y, t.y);
-            t.y = fma(-a.y, vr.x, t.y);
-            mine[k] = t;
-          }
-        }
-        acc = warp_sum(acc);
-        __syncwarp();
-        if (lane == 0) mine[r] = cadd(mine[r], acc);
-        __syncwarp();
-      }
-      __syncthreads();
-      for (int i = tid; i < n; i += blockDim.x) {
-        double2 s = make_double2(0, 0);
-        for (int w = 0; w < nwarp; ++w) s = cadd(s, pw[(long)w * m + i]);
-        __stcg(pb + (long)rank * m + i, s);
-      }
-    } else {
-      for (int i = tid; i < n; i += blockDim.x)
-        if (rank == 0) Hv[(long)j * m + j + 1 + i] = make_double2(0, 0);
-      if (rank == 0 && tid == 0) e.alpha[(long)b * m + j] = make_double2(0, 0);
-    }
-    if (CL > 1) cluster.sync();
-    else __syncthreads();
-    if (!skip) {
-      double2 kp = make_double2(0, 0);
-      for (int i = tid; i < n; i += blockDim.x) {
-        double2 pi = make_double2(0, 0);
-#pragma unroll
-        for (int c = 0; c < CL; ++c) pi = cadd(pi, ldcg2(pb + (long)c * m + i));
-        pi = cscale(pi, 2.0);
-        p[i] = pi;
-        cfmac(kp, v[i], pi);
-      }
-      const double K = block_sum2(kp, red).x;
-      for (int i = tid; i < n; i += blockDim.x) p[i] = csub(p[i], cscale(v[i], K));  // p <- w
-      __syncthreads();
-      // lower-triangle update of this CTA's rows, one warp per row
-      for (int r = r0 + warp * CL; r < n; r += nwarp * CL) {
-        double2* row = G + (long)(j + 1 + r) * ldg + j + 1;
-        const double2 vr = v[r], wr = p[r];
-        for (int k = lane; k <= r; k += 32) {
-          const double2 vk = v[k], wk = p[k];
-          double2 t = row[k];
-          // t -= v_r conj(w_k) + w_r conj(v_k), as four fused multiply-adds per component
-          t.x = fma(-vr.x, wk.x, t.x);
-          t.x = fma(-vr.y, wk.y, t.x);
-          t.x = fma(-wr.x, vk.x, t.x);
-          t.x = fma(-wr.y, vk.y, t.x);
-          t.y = fma(-vr.y, wk.x, t.y);
-          t.y = fma(vr.x, wk.y, t.y);
-          t.y = fma(-wr.y, vk.x, t.y);
-          t.y = fma(wr.x, vk.y, t.y);
-          row[k] = t;
-        }
-      }
-    }
-    if (CL > 1) cluster.sync();
-    else __syncthreads();
-  }
-  if (rank == 0 && tid == 0) {
-    e.d[(long)b * m + m - 1] = ldcg2(G + (long)(m - 1) * ldg + m - 1).x;
-    // phases: T = D^H T' D real with T(j+1, j) = |alpha_j|
-    double2 dl = make_double2(1, 0);
-    e.delta[(long)b * m] = dl;
-    double tn = 0;
-    for (int j = 0; j < m - 1; ++j) {
-      const double2 a = e.alpha[(long)b * m + j];
-      const double aa = sqrt(cabs2(a));
-      e.f[(long)b * m + j] = aa;
-      if (aa > 0) dl = cmul(dl, cscale(a, 1.0 / aa));
-      e.delta[(long)b * m + j + 1] = dl;
-    }
-    for (int j = 0; j < m; ++j) {
-      const double fl = (j > 0) ? e.f[(long)b * m + j - 1] : 0.0, fr = (j < m - 1) ? e.f[(long)b * m + j] : 0.0;
-      tn = fmax(tn, fabs(e.d[(long)b * m + j]) + fl + fr);
-    }
-    e.tnorm[b] = tn;
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Householder tridiagonalisation with the lower triangle resident in shared
-// memory.  One cluster of CL CTAs per slice; CTA c owns global rows
-// g = c + CL q, stored packed (row g holds columns 0..g).  GB300 issues FP64
-// at 2 DFMA per clock per SM, so the kernel is organised to spend its FP64
-// instructions on the 16 DFMA per trailing element and step that the method
-// needs, on full warps:
-//   * the rank-2 update of step j-1 is applied lazily inside step j's pass
-//     over the trailing triangle (one visit per element and step);
-//   * the work of a pass is cut into equal contiguous segments, one per
-//     thread, of a row-major enumeration (row part sum_k A(g,k) v_k) and of
-//     a column-major enumeration (transposed part sum_g conj(A(g,k)) v_g), so
-//     every accumulation is private to a thread; rows or columns split
-//     between threads are summed from per-thread slots in thread order
-//     (deterministic);
-//   * the column x_j and the partial products are exchanged through
-//     distributed shared memory with two cluster barriers per step.
-// Step j (A^{(j)} = the matrix after j reflectors; the stored S lags one
-// update behind: S = A^{(j-1)} on the trailing block):
-//   x_g = S(g,j) - v'_g conj(w'_j) - w'_g conj(v'_j)      (v', w' of step j-1)
-//   alpha = -e^{i arg x_0} ||x||,  v = (x - alpha e_1) / ||x - alpha e_1||
-//   S(g,k) <- S(g,k) - v'_g conj(w'_k) - w'_g conj(v'_k)   (k <= g, both > j)
-//   p = 2 A^{(j)} v,  w = p - (v^H p) v
-// ---------------------------------------------------------------------------
-constexpr int HS_THREADS = 256;
-constexpr int HS_U_GLOBAL = 4;  // row-store elements a thread loads before using them, rows in L2
-
 __host__ __device__ __forceinline__ int hs_own_rows(int m, int c, int CL) { return (c < m) ? (m - 1 - c) / CL + 1 : 0; }
 __host__ __device__ __forceinline__ int hs_rowbase(int q, int c, int CL) { return q * (c + 1) + CL * q * (q - 1) / 2; }
 // first own row index q with c + CL q > j
 __host__ __device__ __forceinline__ int hs_qfirst(int j, int c, int CL) { return (j < c) ? 0 : (j - c) / CL + 1; }
 
-static size_t hetrd_smem_elems(int m, int CL) {
+static size_t hetrd_row_elems(int m, int CL) {  // packed own rows of the CTA that has most
   int mx = 0;
   for (int c = 0; c < CL; ++c) mx = std::max(mx, hs_rowbase(hs_own_rows(m, c, CL), c, CL));
   return (size_t)mx;
 }
-static size_t hetrd_smem_bytes(int m, int CL, int nt = HS_THREADS, bool global_rows = false) {
-  const size_t vown = (size_t)(m + CL - 1) / CL;  // v at the own rows, compacted
-  const size_t rows = global_rows ? 0 : hetrd_smem_elems(m, CL);
-  const size_t el = (rows + 5 * (size_t)m + 2 * (size_t)nt + vown) * sizeof(double2);
-  return el + (size_t)(m + 1) * sizeof(int);
-}
-
-// A pass of E elements is cut into contiguous segments of L elements (the
-// last one shorter), one per thread: L is odd and at least 5, so the
-// addresses of neighbouring lanes inside a row differ by an odd multiple of
-// 16 bytes and fall in different shared-memory bank groups.
-template <int NT>
-__device__ __forceinline__ int hs_seglen(int E) {
-  int L = max(5, E / NT) | 1;
-  while ((E + L - 1) / L > NT) L += 2;
-  return L;
-}
-__device__ __forceinline__ int hs_seg(int t, int E, int L) { return min(t * L, E); }
-// the segment holding element e
-__device__ __forceinline__ int hs_owner(int e, int L) { return e / L; }
-
-template <int CL, bool GS>
-__global__ void __launch_bounds__(HS_THREADS, 1) k_hetrd_smem(const double2* __restrict__ G, long ldg, long sG, int m,
-                                                           int s_elems, EigScratch e, int b0) {
-  extern __shared__ __align__(16) double2 hsm[];
-  // own rows, packed: in shared memory, or (GS) in this CTA's private part of a
-  // global array, which stays L2-resident (only this CTA reads or writes it)
-  double2* S = GS ? e.Sg + (long)blockIdx.x * s_elems : hsm;
-  double2* bufV = GS ? hsm : S + s_elems;      // [2][m] v of this and of the previous step
-  double2* bufW = bufV + 2 * m;                // [2][m] w
-  double2* pv = bufW + 2 * m;                  // [m] this CTA's part of p
-  double2* slotF = pv + m;                     // [T] partial of a thread's first (split) row / column
-  double2* slotL = slotF + HS_THREADS;         // [T] partial of a thread's last (split) row / column
-  double2* vown = slotL + HS_THREADS;          // [ceil(m/CL)] v at the own rows (odd lane stride in the column pass)
-  int* CP = (int*)(vown + (m + CL - 1) / CL);  // [m+1] prefix of the per-column own-row counts
-  __shared__ double red[2 * (HS_THREADS / 32)];
-  cg::cluster_group cluster = cg::this_cluster();
-  const int c = (CL > 1) ? (int)cluster.block_rank() : 0;
-  const int b = b0 + (int)blockIdx.x / CL;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int NW = HS_THREADS / 32;
-  G += (long)b * sG;
-  double2* Hv = e.Hv + (long)b * m * m;
-  const int nq = hs_own_rows(m, c, CL);
-
-  // load the own rows of the lower triangle; column prefix counts
-  for (int q = warp; q < nq; q += NW) {
-    const int g = c + CL * q;
-    const double2* src = G + (long)g * ldg;
-    double2* dst = S + hs_rowbase(q, c, CL);
-    for (int k = lane; k <= g; k += 32) dst[k] = __ldcg(src + k);
-  }
-  if (tid == 0) {
-    int acc = 0;
-    for (int k = 0; k < m; ++k) {
-      CP[k] = acc;
-      acc += max(0, nq - hs_qfirst(k, c, CL));
-    }
-    CP[m] = acc;
-  }
-  for (int i = tid; i < 4 * m; i += HS_THREADS) bufV[i] = make_double2(0, 0);  // v', w' of "step -1"
-  if (CL > 1) cluster.sync();
-  else __syncthreads();
-
-  for (int j = 0; j < m - 1; ++j) {
-    const int cur = j & 1;
-    double2* v = bufV + cur * m;
-    double2* w = bufW + cur * m;
-    const double2* vp = bufV + (cur ^ 1) * m;
-    const double2* wp = bufW + (cur ^ 1) * m;
-    const bool lag = j > 0;
-    // (0) column j of A^{(j)} from the own rows, pushed to every CTA's v
-    {
-      const double2 vpj = vp[j], wpj = wp[j];
-      for (int q = hs_qfirst(j, c, CL) + tid; q < nq; q += HS_THREADS) {
-        const int g = c + CL * q;
-        double2 a = S[hs_rowbase(q, c, CL) + j];
-        if (lag) {
-          const double2 vg = vp[g], wg = wp[g];
-          a.x -= vg.x * wpj.x + vg.y * wpj.y + wg.x * vpj.x + wg.y * vpj.y;
-          a.y -= vg.y * wpj.x - vg.x * wpj.y + wg.y * vpj.x - wg.x * vpj.y;
-        }
-#pragma unroll
-        for (int rr = 0; rr < CL; ++rr) {
-          double2* dst = (CL > 1) ? cluster.map_shared_rank(v, rr) : v;
-          dst[g] = a;
-        }
-      }
-      if (tid == 0 && (j % CL) == c) {
-        const double2 s = S[hs_rowbase((j - c) / CL, c, CL) + j];
-        e.d[(long)b * m + j] = s.x - 2.0 * (vpj.x * wpj.x + vpj.y * wpj.y);
-      }
-    }
-    if (CL > 1) cluster.sync();
-    else __syncthreads();
-    // (1) the reflector (every CTA forms the same v)
-    const int n = m - j - 1;
-    const double2 x0 = v[j + 1];
-    double part = 0;
-    for (int i = tid; i < n; i += HS_THREADS) part += cabs2(v[j + 1 + i]);
-    for (int i = tid; i < n; i += HS_THREADS) pv[j + 1 + i] = make_double2(0, 0);
-    const double nrm2 = block_sum(part, red);
-    const bool skip = !(nrm2 > 0.0);
-    double2 alpha = make_double2(0, 0);
-    double vinv = 0.0;
-    if (!skip) {
-      const double nrm = sqrt(nrm2), ax0 = sqrt(cabs2(x0));
-      const double2 ph = (ax0 > 0) ? cscale(x0, 1.0 / ax0) : make_double2(1, 0);
-      alpha = cscale(ph, -nrm);
-      vinv = 1.0 / sqrt(2.0 * nrm * (nrm + ax0));
-    }
-    for (int i = tid; i < n; i += HS_THREADS) {
-      double2 vi = v[j + 1 + i];
-      if (i == 0) vi = csub(vi, alpha);
-      vi = cscale(vi, vinv);
-      v[j + 1 + i] = vi;
-      if (c == 0) Hv[(long)j * m + j + 1 + i] = vi;
-    }
-    if (c == 0 && tid == 0) e.alpha[(long)b * m + j] = alpha;
-    __syncthreads();
-
-    // (2) row pass: lazy update of S and the row part of A v over own rows g > j, columns j+1..g
-    const int q0 = hs_qfirst(j, c, CL);
-    for (int q = q0 + tid; q < nq; q += HS_THREADS) vown[q] = v[c + CL * q];
-    const int nr = max(0, nq - q0);
-    const int g0 = c + CL * q0;
-    const int E1 = nr * (g0 - j) + CL * nr * (nr - 1) / 2;  // sum of the row lengths g - j
-    if (E1 > 0) {
-      const int L1 = hs_seglen<HS_THREADS>(E1);
-      const int e0 = hs_seg(tid, E1, L1), e1 = hs_seg(tid + 1, E1, L1);
-      if (e0 < e1) {
-        // row i holds elements [P(i), P(i+1)), P(i) = i (g0 - j) + CL i (i - 1) / 2
-        int lo = 0, hi = nr - 1;
-        while (lo < hi) {
-          const int mid = (lo + hi + 1) >> 1;
-          if (mid * (g0 - j) + CL * mid * (mid - 1) / 2 <= e0) lo = mid;
-          else hi = mid - 1;
-        }
-        int i = lo;
-        int Pi = i * (g0 - j) + CL * i * (i - 1) / 2;
-        int g = g0 + CL * i;
-        int k = j + 1 + (e0 - Pi);
-        double2* row = S + hs_rowbase(q0 + i, c, CL);
-        bool whole = (e0 == Pi), first = true;
-        double2 vg = vp[g], wg = wp[g];
-        double2 acc = make_double2(0, 0);
-        for (int el = e0; el < e1; ++el) {
-          double2 a = row[k];
-          if (lag) {
-            const double2 wk = wp[k], vk = vp[k];
-            a.x = fma(-vg.x, wk.x, a.x);
-            a.x = fma(-vg.y, wk.y, a.x);
-            a.x = fma(-wg.x, vk.x, a.x);
-            a.x = fma(-wg.y, vk.y, a.x);
-            a.y = fma(-vg.y, wk.x, a.y);
-            a.y = fma(vg.x, wk.y, a.y);
-            a.y = fma(-wg.y, vk.x, a.y);
-            a.y = fma(wg.x, vk.y, a.y);
-            if (k == g) a.y = 0.0;  // the diagonal stays real
-            row[k] = a;
-          }
-          cfma(acc, a, v[k]);
-          if (++k > g) {  // row g done
-            if (whole) pv[g] = acc;
-            else slotF[tid] = acc;  // a row ending here but started earlier is this thread's first row
-            first = false;
-            whole = true;
-            acc = make_double2(0, 0);
-            row += g + 1;
-            g += CL;
-            k = j + 1;
-            if (el + 1 < e1) {
-              vg = vp[g];
-              wg = wp[g];
-            }
-          }
-        }
-        if (k != j + 1) {  // the segment ends inside row g
-          if (first) slotF[tid] = acc;
-          else slotL[tid] = acc;
-        }
-      }
-      __syncthreads();
-      // rows split between threads: fixed-order sum of the slots
-      for (int i = tid; i < nr; i += HS_THREADS) {
-        const int Pi = i * (g0 - j) + CL * i * (i - 1) / 2;
-        const int len = g0 + CL * i - j;
-        const int ta = hs_owner(Pi, L1), tb = hs_owner(Pi + len - 1, L1);
-        if (ta == tb) continue;
-        double2 s = (hs_seg(ta, E1, L1) == Pi) ? slotF[ta] : slotL[ta];
-        for (int t = ta + 1; t <= tb; ++t)
-          if (hs_seg(t, E1, L1) < hs_seg(t + 1, E1, L1)) s = cadd(s, slotF[t]);
-        pv[g0 + CL * i] = s;
-      }
-    }
-    __syncthreads();
-
-    // (3) column pass: transposed part sum_{g > k} conj(S(g,k)) v_g, columns k > j
-    const int cb = CP[j + 1];
-    const int E2 = CP[m] - cb;
-    if (E2 > 0) {
-      const int L2 = hs_seglen<HS_THREADS>(E2);
-      const int e0 = hs_seg(tid, E2, L2), e1 = hs_seg(tid + 1, E2, L2);
-      if (e0 < e1) {
-        int lo = j + 1, hi = m - 1;  // last column k with CP[k] <= cb + e0
-        while (lo < hi) {
-          const int mid = (lo + hi + 1) >> 1;
-          if (CP[mid] <= cb + e0) lo = mid;
-          else hi = mid - 1;
-        }
-        int k = lo;
-        int o = cb + e0 - CP[k];
-        int cnt = CP[k + 1] - CP[k];
-        int q = hs_qfirst(k, c, CL) + o;
-        int g = c + CL * q, base = hs_rowbase(q, c, CL);
-        bool whole = (o == 0), first = true;
-        double2 acc = make_double2(0, 0);
-        for (int el = e0; el < e1; ++el) {
-          cfmac(acc, S[base + k], vown[q]);
-          base += g + 1;  // next own row
-          g += CL;
-          ++q;
-          if (++o == cnt) {  // column k done
-            if (whole) pv[k] = cadd(pv[k], acc);
-            else slotF[tid] = acc;
-            first = false;
-            whole = true;
-            acc = make_double2(0, 0);
-            if (el + 1 < e1) {
-              do {
-                ++k;
-              } while (CP[k + 1] == CP[k]);
-              cnt = CP[k + 1] - CP[k];
-              q = hs_qfirst(k, c, CL);
-              g = c + CL * q;
-              base = hs_rowbase(q, c, CL);
-              o = 0;
-            }
-          }
-        }
-        if (o != cnt && o != 0) {  // the segment ends inside column k
-          if (first) slotF[tid] = acc;
-          else slotL[tid] = acc;
-        }
-      }
-      __syncthreads();
-      for (int k = j + 1 + tid; k < m; k += HS_THREADS) {
-        const int cnt = CP[k + 1] - CP[k];
-        if (cnt == 0) continue;
-        const int s0 = CP[k] - cb;
-        const int ta = hs_owner(s0, L2), tb = hs_owner(s0 + cnt - 1, L2);
-        if (ta == tb) continue;
-        double2 s = (hs_seg(ta, E2, L2) == s0) ? slotF[ta] : slotL[ta];
-        for (int t = ta + 1; t <= tb; ++t)
-          if (hs_seg(t, E2, L2) < hs_seg(t + 1, E2, L2)) s = cadd(s, slotF[t]);
-        pv[k] = cadd(pv[k], s);
-      }
-    }
-    if (CL > 1) cluster.sync();
-    else __syncthreads();
-
-    // (4) p = 2 sum over the cluster's parts (fixed order), w = p - (v^H p) v
-    double2 kp = make_double2(0, 0);
-    for (int i = j + 1 + tid; i < m; i += HS_THREADS) {
-      double2 pi = make_double2(0, 0);
-#pragma unroll
-      for (int rr = 0; rr < CL; ++rr) {
-        const double2* src = (CL > 1) ? cluster.map_shared_rank(pv, rr) : pv;
-        pi = cadd(pi, src[i]);
-      }
-      pi = cscale(pi, 2.0);
-      w[i] = pi;
-      cfmac(kp, v[i], pi);
-    }
-    const double K = block_sum2(kp, red).x;
-    for (int i = j + 1 + tid; i < m; i += HS_THREADS) w[i] = csub(w[i], cscale(v[i], K));
-    __syncthreads();
-  }
-  // last diagonal entry: apply the pending update of step m-2
-  if (tid == 0 && ((m - 1) % CL) == c) {
-    const double2 s = S[hs_rowbase((m - 1 - c) / CL, c, CL) + m - 1];
-    const double2 vq = bufV[((m - 2) & 1) * m + m - 1], wq = bufW[((m - 2) & 1) * m + m - 1];
-    e.d[(long)b * m + m - 1] = (m > 1) ? s.x - 2.0 * (vq.x * wq.x + vq.y * wq.y) : s.x;
-  }
-  __threadfence();
-  if (CL > 1) cluster.sync();
-  else __syncthreads();
-  if (c == 0 && tid == 0) {
-    double2 dl = make_double2(1, 0);
-    e.delta[(long)b * m] = dl;
-    double tn = 0;
-    for (int jj = 0; jj < m - 1; ++jj) {
-      const double2 a = __ldcg(e.alpha + (long)b * m + jj);
-      const double aa = sqrt(cabs2(a));
-      e.f[(long)b * m + jj] = aa;
-      if (aa > 0) dl = cmul(dl, cscale(a, 1.0 / aa));
-      e.delta[(long)b * m + jj + 1] = dl;
-    }
-    for (int jj = 0; jj < m; ++jj) {
-      const double fl = (jj > 0) ? e.f[(long)b * m + jj - 1] : 0.0, fr = (jj < m - 1) ? e.f[(long)b * m + jj] : 0.0;
-      tn = fmax(tn, fabs(__ldcg(e.d + (long)b * m + jj)) + fl + fr);
-    }
-    e.tnorm[b] = tn;
-  }
-}
 
 // ---------------------------------------------------------------------------
-// Double-float variant of k_hetrd_smem for the FP32 path.  GB300 issues FP32
-// at 64x its FP64 rate, so the same reduction is carried in unevaluated pairs
+// Double-float arithmetic of the FP32 path's eigen-solver: unevaluated pairs
 // (hi, lo) of floats (about 48 significant bits) built from the error-free
-// transformations TwoSum (Knuth) and TwoProduct via FMA (Dekker): a
-// multiply-add costs about 15 FP32 instructions instead of one DFMA at 1/64
-// of the rate.  G is first scaled by a power of two so its entries stay far
-// inside the FP32 exponent range; the per-step scalars (norm, alpha, the
-// scale of v, v^H p) are formed in FP64 by one thread.  The rounding level
-// (about 2^-47 ||G|| per operation) is far below what the FP32 path's
-// accuracy needs; the FP64 path keeps k_hetrd_smem.
+// transformations TwoSum (Knuth) and TwoProduct via FMA (Dekker).  GB300
+// issues FP32 at 64x its FP64 rate, so a multiply-add of about 15 FP32
+// instructions replaces one DFMA at 1/64 of the rate.  G is first scaled by a
+// power of two so its entries stay far inside the FP32 exponent range; the
+// rounding level (about 2^-47 ||G|| per operation) is far below what the FP32
+// path's accuracy needs.
 // ---------------------------------------------------------------------------
 struct __align__(8) dfl {
   float hi, lo;
@@ -615,13 +106,6 @@ __device__ __forceinline__ dfl df_sqrt(dfl a) {
   const float r = ((a.hi - p) - pe) + a.lo;
   return df_fast_two_sum(x, r / (2.f * x));
 }
-// quotient: FP32 quotient, then one correction with the residual a - q b
-__device__ __forceinline__ dfl df_div(dfl a, dfl b) {
-  const float q = a.hi / b.hi;
-  const float p = q * b.hi, pe = fmaf(q, b.hi, -p);
-  const float r = (((a.hi - p) - pe) + a.lo) - q * b.lo;
-  return df_fast_two_sum(q, r / b.hi);
-}
 // Reciprocal square root and square root without a division: the correctly
 // rounded FP32 reciprocal square root y, then one Newton correction with the
 // residual formed in double-float (y (1 + e/2), e = 1 - a y^2; for the root,
@@ -650,7 +134,6 @@ __device__ __forceinline__ dfl cre(cdf a) { return dfl{a.rh, a.rl}; }
 __device__ __forceinline__ dfl cim(cdf a) { return dfl{a.ih, a.il}; }
 __device__ __forceinline__ cdf cdf_make(dfl r, dfl i) { return cdf{r.hi, r.lo, i.hi, i.lo}; }
 __device__ __forceinline__ cdf cdf_from(double2 x) { return cdf_make(df_from(x.x), df_from(x.y)); }
-__device__ __forceinline__ double2 cdf_to(cdf a) { return make_double2(df_to(cre(a)), df_to(cim(a))); }
 __device__ __forceinline__ cdf cdf_zero() { return cdf{0.f, 0.f, 0.f, 0.f}; }
 __device__ __forceinline__ cdf cdf_add(cdf a, cdf b) { return cdf_make(df_add(cre(a), cre(b)), df_add(cim(a), cim(b))); }
 // acc += a b
@@ -671,18 +154,6 @@ __device__ __forceinline__ dfl df_dot(dfl a, const dfl (&x)[N], const dfl (&y)[N
     s = t;
   }
   return df_fast_two_sum(s, e);
-}
-// acc += a b
-__device__ __forceinline__ void cdf_fma(cdf& acc, cdf a, cdf b) {
-  const dfl xr[2] = {cre(a), df_neg(cim(a))}, yr[2] = {cre(b), cim(b)};
-  const dfl xi[2] = {cre(a), cim(a)}, yi[2] = {cim(b), cre(b)};
-  acc = cdf_make(df_dot<2>(cre(acc), xr, yr), df_dot<2>(cim(acc), xi, yi));
-}
-// acc += conj(a) b
-__device__ __forceinline__ void cdf_fmac(cdf& acc, cdf a, cdf b) {
-  const dfl xr[2] = {cre(a), cim(a)}, yr[2] = {cre(b), cim(b)};
-  const dfl xi[2] = {cre(a), df_neg(cim(a))}, yi[2] = {cim(b), cre(b)};
-  acc = cdf_make(df_dot<2>(cre(acc), xr, yr), df_dot<2>(cim(acc), xi, yi));
 }
 // acc += a b and acc += conj(a) b with acc kept unnormalised: the high words
 // carry the running sums, the low words every rounding error (the loop of
@@ -727,894 +198,488 @@ __device__ __forceinline__ cdf cdf_shfl_xor(cdf a, int o) {
   return cdf{__shfl_xor_sync(0xffffffffu, a.rh, o), __shfl_xor_sync(0xffffffffu, a.rl, o),
              __shfl_xor_sync(0xffffffffu, a.ih, o), __shfl_xor_sync(0xffffffffu, a.il, o)};
 }
-// block-wide sum in a fixed order, result on every thread (two barriers)
-__device__ __forceinline__ dfl df_block_sum(dfl v, dfl* red) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+// ---------------------------------------------------------------------------
+// The reduction, for cdf (double-float, FP32 path) and double2 (FP64 path).
+// Step j (A^(j) = the matrix after j reflectors; the stored rows S lag one
+// update behind, S = A^(j-1) on the trailing block; v', w' of step j-1):
+//   w' = p' - K v',  K = Re(v'^H p')
+//   x = S(:,j) - v' conj(w'_j) - w' conj(v'_j)
+//   alpha = -e^{i arg x_0} ||x||,  v = (x - alpha e_1) / ||x - alpha e_1||
+//   S(g,k) <- S(g,k) - v'_g conj(w'_k) - w'_g conj(v'_k)   (k <= g, both > j)
+//   p = 2 A^(j) v from the lower triangle: row part sum_k S(g,k) v_k and
+//       column part sum_g conj(S(g,k)) v_g
+// One sweep per step does the update, the store and both parts, and sends the
+// updated column j+1 to every CTA of the cluster, so that after the one
+// cluster barrier of the step each CTA has the parts of p and the next column
+// and goes on alone (the same sums in the same order in every CTA).
+//
+// Warp w takes every NW-th own row from the last but w on, in strips of HF_SR
+// and 32 columns at a time with lane l on column k0 + l: every load is one
+// contiguous 512-byte run, the row sums stay in the lane until the strip's
+// end, the column sums go to a partial of p private to the warp.  Every sum
+// has one order, so reruns agree bitwise.  Rows sit in shared memory where
+// they fit, else in a private part of a global array (L2), read 32 columns
+// ahead; the warps' partials likewise (`cp_global`).
+//
+// Bound: in double-float its instructions (about 200 of FP32 per element and
+// step) and, per step, a chain of two block sums, the reflector's scalars and a
+// cluster barrier (7 to 9 of 14 us at m = 300 in the three-sweep form this
+// replaces, about 4 of 11 here); in FP64 its pipe (16 multiply-adds per element
+// and step).  Two rows' chains interleave without branches on the lane (all
+// eight in turn: 3692 us at m = 300, two at a time 3405, four 3400).  Against
+// the former kernels, us: double-float m = 45 on 9 slices 350 -> 215, 135 on 33
+// 1420 -> 816, 300 on 33 4363 -> 3405, 480 on 65 (rows in L2) 17330 -> 16500;
+// FP64 45 on 9 623 -> 346, 300 on 33 9318 -> 8090, 480 on 9 34880 -> 15650.
+// ---------------------------------------------------------------------------
+
+constexpr int HETRD_NT = 256;  // threads (m = 300 on 33 slices in double-float: 512 threads 3764 us, 256 3405)
+
+// operations the kernel takes from its arithmetic
+__device__ __forceinline__ dfl r_zero(dfl) { return dfl{0.f, 0.f}; }
+__device__ __forceinline__ double r_zero(double) { return 0.0; }
+__device__ __forceinline__ cdf c_zero(cdf) { return cdf_zero(); }
+__device__ __forceinline__ double2 c_zero(double2) { return make_double2(0.0, 0.0); }
+__device__ __forceinline__ cdf c_one(cdf) { return cdf{1.f, 0.f, 0.f, 0.f}; }
+__device__ __forceinline__ double2 c_one(double2) { return make_double2(1.0, 0.0); }
+__device__ __forceinline__ dfl r_add(dfl a, dfl b) { return df_add(a, b); }
+__device__ __forceinline__ double r_add(double a, double b) { return a + b; }
+__device__ __forceinline__ dfl r_neg(dfl a) { return df_neg(a); }
+__device__ __forceinline__ double r_neg(double a) { return -a; }
+__device__ __forceinline__ dfl r_fma(dfl a, dfl x, dfl y) { return df_fma(a, x, y); }
+__device__ __forceinline__ double r_fma(double a, double x, double y) { return fma(x, y, a); }
+__device__ __forceinline__ dfl r_mul(dfl a, dfl b) { return df_mul(a, b); }
+__device__ __forceinline__ double r_mul(double a, double b) { return a * b; }
+__device__ __forceinline__ bool r_pos(dfl a) { return a.hi > 0.f; }
+__device__ __forceinline__ bool r_pos(double a) { return a > 0.0; }
+__device__ __forceinline__ dfl r_rsqrt(dfl a) { return df_rsqrt(a); }
+__device__ __forceinline__ double r_rsqrt(double a) { return inv_sqrt(a); }
+__device__ __forceinline__ dfl r_sqrt(dfl a) { return df_sqrt_nodiv(a); }
+__device__ __forceinline__ double r_sqrt(double a) { return a * inv_sqrt(a); }
+__device__ __forceinline__ dfl r_shfl(dfl a, int o) { return df_shfl_xor(a, o); }
+__device__ __forceinline__ double r_shfl(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+__device__ __forceinline__ double r_double(dfl a) { return df_to(a); }
+__device__ __forceinline__ double r_double(double a) { return a; }
+__device__ __forceinline__ double cre(double2 a) { return a.x; }
+__device__ __forceinline__ double cim(double2 a) { return a.y; }
+__device__ __forceinline__ cdf c_make(dfl r, dfl i) { return cdf_make(r, i); }
+__device__ __forceinline__ double2 c_make(double r, double i) { return make_double2(r, i); }
+__device__ __forceinline__ cdf c_add(cdf a, cdf b) { return cdf_add(a, b); }
+__device__ __forceinline__ double2 c_add(double2 a, double2 b) { return cadd(a, b); }
+__device__ __forceinline__ cdf c_twice(cdf a) { return cdf{2.f * a.rh, 2.f * a.rl, 2.f * a.ih, 2.f * a.il}; }
+__device__ __forceinline__ double2 c_twice(double2 a) { return make_double2(2.0 * a.x, 2.0 * a.y); }
+__device__ __forceinline__ void c_real(cdf& a) { a.ih = a.il = 0.f; }
+__device__ __forceinline__ void c_real(double2& a) { a.y = 0.0; }
+__device__ __forceinline__ cdf c_shfl(cdf a, int o) { return cdf_shfl_xor(a, o); }
+__device__ __forceinline__ double2 c_shfl(double2 a, int o) {
+  return make_double2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
+}
+__device__ __forceinline__ cdf c_scale_r(cdf a, dfl s) { return cdf_scale(a, s); }
+__device__ __forceinline__ double2 c_scale_r(double2 a, double s) { return cscale(a, s); }
+__device__ __forceinline__ cdf c_lag(cdf a, cdf vg, cdf wg, cdf vk, cdf wk) { return cdf_lag(a, vg, wg, vk, wk); }
+__device__ __forceinline__ double2 c_lag(double2 a, double2 vg, double2 wg, double2 vk, double2 wk) {
+  a.x = fma(-vg.x, wk.x, a.x);
+  a.x = fma(-vg.y, wk.y, a.x);
+  a.x = fma(-wg.x, vk.x, a.x);
+  a.x = fma(-wg.y, vk.y, a.x);
+  a.y = fma(-vg.y, wk.x, a.y);
+  a.y = fma(vg.x, wk.y, a.y);
+  a.y = fma(-wg.y, vk.x, a.y);
+  a.y = fma(wg.x, vk.y, a.y);
+  return a;
+}
+__device__ __forceinline__ void c_fma_acc(cdf& s, cdf a, cdf b) { cdf_fma_acc(s, a, b); }
+__device__ __forceinline__ void c_fma_acc(double2& s, double2 a, double2 b) { cfma(s, a, b); }
+__device__ __forceinline__ void c_fmac_acc(cdf& s, cdf a, cdf b) { cdf_fmac_acc(s, a, b); }
+__device__ __forceinline__ void c_fmac_acc(double2& s, double2 a, double2 b) { cfmac(s, a, b); }
+__device__ __forceinline__ cdf c_from(cdf, double2 x, int ex) {
+  return cdf_from(make_double2(ldexp(x.x, -ex), ldexp(x.y, -ex)));
+}
+__device__ __forceinline__ double2 c_from(double2, double2 x, int) { return x; }
+// the Householder vector as the back-transformation reads it (FP32 path: evict-first, so the row
+// store keeps the L2)
+__device__ __forceinline__ void put_hv(void* Hv, long i, cdf v) { __stcs((float2*)Hv + i, make_float2(v.rh, v.ih)); }
+__device__ __forceinline__ void put_hv(void* Hv, long i, double2 v) { ((double2*)Hv)[i] = v; }
+
+// Sum over the block in a fixed order, the result on every thread.  Double-float: every warp adds the
+// warps' sums (one barrier).  FP64: one warp adds them (two barriers), since an FP64 instruction of
+// every warp costs 64 clocks times the warps of a scheduler.
+template <int NW>
+__device__ __forceinline__ dfl hf_block_sum(dfl v, dfl* red, int lane, int warp) {
+#pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = df_add(v, df_shfl_xor(v, o));
+  if (lane == 0) red[warp] = v;
   __syncthreads();
-  if (lane == 0) red[wid] = v;
+  v = red[lane & (NW - 1)];
+#pragma unroll
+  for (int o = NW / 2; o > 0; o >>= 1) v = df_add(v, df_shfl_xor(v, o));
+  return v;
+}
+template <int NW>
+__device__ __forceinline__ double hf_block_sum(double v, double* red, int lane, int warp) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lane == 0) red[warp] = v;
   __syncthreads();
-  dfl t = (lane < nw) ? red[lane] : dfl{0.f, 0.f};
-  for (int o = 16; o > 0; o >>= 1) t = df_add(t, df_shfl_xor(t, o));
-  return t;
+  if (warp == 0) {
+    v = lane < NW ? red[lane] : 0.0;
+#pragma unroll
+    for (int o = NW / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) red[NW] = v;
+  }
+  __syncthreads();
+  return red[NW];
 }
 
-template <int CL, int NT, bool GS>
-__global__ void __launch_bounds__(NT, 1) k_hetrd_df(const double2* __restrict__ G, long ldg, long sG, int m,
-                                                            int s_elems, EigScratch e, int b0) {
-  extern __shared__ __align__(16) cdf dsm[];
-  // own rows, packed: in shared memory, or (GS) in this CTA's private part of a
-  // global array, which stays L2-resident (only this CTA reads or writes it)
-  cdf* S = GS ? (cdf*)e.Sg + (long)blockIdx.x * s_elems : dsm;
-  cdf* bufV = GS ? dsm : S + s_elems;
-  constexpr int HS_U = HS_U_GLOBAL;
-  cdf* bufW = bufV + 2 * m;
-  cdf* pv = bufW + 2 * m;
-  cdf* slotF = pv + m;
-  cdf* slotL = slotF + NT;
-  cdf* vown = slotL + NT;
-  int* CP = (int*)(vown + (m + CL - 1) / CL);
-  __shared__ dfl red[NT / 32];
-  __shared__ int s_exp;
-  __shared__ cdf s_am;   // -alpha of the current reflector
-  __shared__ dfl s_vinv; // its normalisation
-  cg::cluster_group cluster = cg::this_cluster();
-  const int c = (CL > 1) ? (int)cluster.block_rank() : 0;
-  const int b = b0 + (int)blockIdx.x / CL;  // slice (launches may cover a range of slices from b0)
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int NW = NT / 32;
-  G += (long)b * sG;
-  float2* Hv32 = (float2*)e.Hv + (long)b * m * m;
-  const int nq = hs_own_rows(m, c, CL);
-
-  // power-of-two scale from the largest diagonal entry (identical in every CTA)
-  {
-    double mx = 0;
-    for (int i = tid; i < m; i += NT) mx = fmax(mx, fabs(__ldcg(G + (long)i * ldg + i).x));
-    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    __shared__ double wmx[NW];
-    if (lane == 0) wmx[warp] = mx;
-    __syncthreads();
-    if (tid == 0) {
-      double t = 0;
-      for (int w = 0; w < NW; ++w) t = fmax(t, wmx[w]);
-      int ex = 0;
-      if (t > 0 && isfinite(t)) frexp(t, &ex);
-      s_exp = ex;
-    }
-    __syncthreads();
-  }
-  const int ex = s_exp;
-  for (int q = warp; q < nq; q += NW) {
-    const int g = c + CL * q;
-    const double2* src = G + (long)g * ldg;
-    cdf* dst = S + hs_rowbase(q, c, CL);
-    for (int k = lane; k <= g; k += 32) {
-      const double2 x = __ldcg(src + k);
-      dst[k] = cdf_from(make_double2(ldexp(x.x, -ex), ldexp(x.y, -ex)));
-    }
-  }
-  if (tid == 0) {
-    int acc = 0;
-    for (int k = 0; k < m; ++k) {
-      CP[k] = acc;
-      acc += max(0, nq - hs_qfirst(k, c, CL));
-    }
-    CP[m] = acc;
-  }
-  for (int i = tid; i < 4 * m; i += NT) bufV[i] = cdf_zero();
-  if (CL > 1) cluster.sync();
-  else __syncthreads();
-
-  for (int j = 0; j < m - 1; ++j) {
-    const int cur = j & 1;
-    cdf* v = bufV + cur * m;
-    cdf* w = bufW + cur * m;
-    const cdf* vp = bufV + (cur ^ 1) * m;
-    const cdf* wp = bufW + (cur ^ 1) * m;
-    const bool lag = j > 0;
-    {
-      const cdf vpj = vp[j], wpj = wp[j];
-      for (int q = hs_qfirst(j, c, CL) + tid; q < nq; q += NT) {
-        const int g = c + CL * q;
-        cdf a = S[hs_rowbase(q, c, CL) + j];
-        if (lag) a = cdf_lag(a, vp[g], wp[g], vpj, wpj);
-#pragma unroll
-        for (int rr = 0; rr < CL; ++rr) {
-          cdf* dst = (CL > 1) ? cluster.map_shared_rank(v, rr) : v;
-          dst[g] = a;
-        }
-      }
-      if (tid == 0 && (j % CL) == c) {
-        const cdf sj = S[hs_rowbase((j - c) / CL, c, CL) + j];
-        dfl t = cre(sj);
-        t = df_fma(t, df_neg(cre(vpj)), cre(wpj));
-        t = df_fma(t, df_neg(cim(vpj)), cim(wpj));
-        t = df_fma(t, df_neg(cre(vpj)), cre(wpj));
-        t = df_fma(t, df_neg(cim(vpj)), cim(wpj));
-        e.d[(long)b * m + j] = ldexp(df_to(t), ex);
-      }
-    }
-    if (CL > 1) cluster.sync();
-    else __syncthreads();
-    const int n = m - j - 1;
-    {
-      // |x|^2 and the reflector scalars by warp 0 alone (the other warps clear the partial
-      // products meanwhile), handed over through shared memory: lanes take entries
-      // lane + 32 u + 128 k in four independent chains, then a butterfly of double-float sums;
-      // -alpha = e^{i arg x0} |x|, v = (x - alpha e1) / sqrt(2 |x| (|x| + |x0|))
-      for (int i = tid; i < n; i += NT) pv[j + 1 + i] = cdf_zero();
-      if (warp > 0 && lag) {
-        // meanwhile the other warps apply the pending rank-2 update of step j-1 to the own rows'
-        // entries k in [j+1, g] (contiguous segments over NT - 32 threads), so that the
-        // matrix-vector passes below read updated values and need only v_j
-        const int q0 = hs_qfirst(j, c, CL);
-        const int nr = max(0, nq - q0);
-        const int g0 = c + CL * q0;
-        const int E1 = nr * (g0 - j) + CL * nr * (nr - 1) / 2;
-        if (E1 > 0) {
-          const int lt = tid - 32;
-          const int L = hs_seglen<NT - 32>(E1);
-          const int e0 = hs_seg(lt, E1, L), e1 = hs_seg(lt + 1, E1, L);
-          if (e0 < e1) {
-            int lo = 0, hi = nr - 1;
-            while (lo < hi) {
-              const int mid = (lo + hi + 1) >> 1;
-              if (mid * (g0 - j) + CL * mid * (mid - 1) / 2 <= e0) lo = mid;
-              else hi = mid - 1;
-            }
-            const int i = lo;
-            const int Pi = i * (g0 - j) + CL * i * (i - 1) / 2;
-            int g = g0 + CL * i;
-            int k = j + 1 + (e0 - Pi);
-            cdf* row = S + hs_rowbase(q0 + i, c, CL);
-            if constexpr (GS) {
-              // HS_U elements at a time: their addresses first, then independent loads
-              // (several row-store accesses in flight per thread), then the updates
-              for (int el = e0; el < e1; el += HS_U) {
-                cdf* p[HS_U];
-                int kk[HS_U], gg[HS_U];
-  #pragma unroll
-                for (int u = 0; u < HS_U; ++u) {
-                  p[u] = row + k;
-                  kk[u] = k;
-                  gg[u] = g;
-                  if (++k > g) {
-                    row += g + 1;
-                    g += CL;
-                    k = j + 1;
-                  }
-                }
-                cdf a[HS_U];
-  #pragma unroll
-                for (int u = 0; u < HS_U; ++u)
-                  if (el + u < e1) a[u] = *p[u];
-  #pragma unroll
-                for (int u = 0; u < HS_U; ++u)
-                  if (el + u < e1) {
-                    cdf x = cdf_lag(a[u], vp[gg[u]], wp[gg[u]], vp[kk[u]], wp[kk[u]]);
-                    if (kk[u] == gg[u]) {
-                      x.ih = 0.f;
-                      x.il = 0.f;
-                    }
-                    *p[u] = x;
-                  }
-              }
-            } else {
-              cdf vg = vp[g], wg = wp[g];
-              for (int el = e0; el < e1; ++el) {
-                cdf a = cdf_lag(row[k], vg, wg, vp[k], wp[k]);
-                if (k == g) {
-                  a.ih = 0.f;
-                  a.il = 0.f;
-                }
-                row[k] = a;
-                if (++k > g) {
-                  row += g + 1;
-                  g += CL;
-                  k = j + 1;
-                  if (el + 1 < e1) {
-                    vg = vp[g];
-                    wg = wp[g];
-                  }
-                }
-              }
-            }
-          }
-        }
-      }
-      if (warp == 0) {
-        dfl pa[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-        for (int i0 = 0; i0 < n; i0 += 128) {
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int i = i0 + 32 * u + lane;
-            if (i < n) {
-              const cdf x = v[j + 1 + i];
-              pa[u] = df_fma(pa[u], cre(x), cre(x));
-              pa[u] = df_fma(pa[u], cim(x), cim(x));
-            }
-          }
-        }
-        dfl nrm2d = df_add(df_add(pa[0], pa[1]), df_add(pa[2], pa[3]));
-        for (int o = 16; o > 0; o >>= 1) nrm2d = df_add(nrm2d, df_shfl_xor(nrm2d, o));
-        cdf am = cdf_zero();  // -alpha
-        dfl vinv{0.f, 0.f};
-        if (nrm2d.hi > 0.f) {
-          const cdf x0 = v[j + 1];
-          const dfl nrm = df_sqrt_nodiv(nrm2d);
-          const dfl ax2 = df_fma(df_fma(dfl{0.f, 0.f}, cre(x0), cre(x0)), cim(x0), cim(x0));
-          dfl phr{1.f, 0.f}, phi{0.f, 0.f}, ax0{0.f, 0.f};
-          if (ax2.hi > 0.f) {
-            const dfl iax = df_rsqrt(ax2);  // 1 / |x0|
-            ax0 = df_mul(ax2, iax);
-            phr = df_mul(cre(x0), iax);
-            phi = df_mul(cim(x0), iax);
-          }
-          am = cdf_make(df_mul(phr, nrm), df_mul(phi, nrm));
-          vinv = df_rsqrt(df_mul(df_add(nrm, nrm), df_add(nrm, ax0)));
-        }
-        if (lane == 0) {
-          s_am = am;
-          s_vinv = vinv;
-          if (c == 0) {
-            const double2 al = cdf_to(am);
-            e.alpha[(long)b * m + j] = make_double2(-ldexp(al.x, ex), -ldexp(al.y, ex));
-          }
-        }
-      }
-      __syncthreads();
-      const cdf am = s_am;
-      const dfl vinv = s_vinv;
-      for (int i = tid; i < n; i += NT) {
-        cdf vi = v[j + 1 + i];
-        if (i == 0) vi = cdf_add(vi, am);
-        vi = cdf_scale(vi, vinv);
-        v[j + 1 + i] = vi;
-        // read by the FP32 back-transform after this kernel: evict-first, so the
-        // row store keeps the L2
-        if (c == 0) __stcs(Hv32 + (long)j * m + j + 1 + i, make_float2(vi.rh, vi.ih));
-      }
-    }
-    __syncthreads();
-
-    // row pass (as in k_hetrd_smem, the pending update already applied)
-    const int q0 = hs_qfirst(j, c, CL);
-    for (int q = q0 + tid; q < nq; q += NT) vown[q] = v[c + CL * q];
-    const int nr = max(0, nq - q0);
-    const int g0 = c + CL * q0;
-    const int E1 = nr * (g0 - j) + CL * nr * (nr - 1) / 2;
-    if (E1 > 0) {
-      const int L1 = hs_seglen<NT>(E1);
-      const int e0 = hs_seg(tid, E1, L1), e1 = hs_seg(tid + 1, E1, L1);
-      if (e0 < e1) {
-        int lo = 0, hi = nr - 1;
-        while (lo < hi) {
-          const int mid = (lo + hi + 1) >> 1;
-          if (mid * (g0 - j) + CL * mid * (mid - 1) / 2 <= e0) lo = mid;
-          else hi = mid - 1;
-        }
-        int i = lo;
-        const int Pi = i * (g0 - j) + CL * i * (i - 1) / 2;
-        int g = g0 + CL * i;
-        int k = j + 1 + (e0 - Pi);
-        const cdf* row = S + hs_rowbase(q0 + i, c, CL);
-        if constexpr (GS) {
-          bool whole = (e0 == Pi), first = true, pending = false;
-          cdf acc = cdf_zero();
-          for (int el = e0; el < e1; el += HS_U) {
-            const cdf* p[HS_U];
-            int kk[HS_U], gend[HS_U];  // gend: the row an element ends, else -1
-  #pragma unroll
-            for (int u = 0; u < HS_U; ++u) {
-              p[u] = row + k;
-              kk[u] = k;
-              gend[u] = -1;
-              if (++k > g) {
-                gend[u] = g;
-                row += g + 1;
-                g += CL;
-                k = j + 1;
-              }
-            }
-            cdf a[HS_U];
-  #pragma unroll
-            for (int u = 0; u < HS_U; ++u)
-              if (el + u < e1) a[u] = *p[u];
-  #pragma unroll
-            for (int u = 0; u < HS_U; ++u)
-              if (el + u < e1) {
-                cdf_fma(acc, a[u], v[kk[u]]);
-                pending = gend[u] < 0;
-                if (!pending) {
-                  if (whole) pv[gend[u]] = acc;
-                  else slotF[tid] = acc;
-                  first = false;
-                  whole = true;
-                  acc = cdf_zero();
-                }
-              }
-          }
-          if (pending) {
-            if (first) slotF[tid] = acc;
-            else slotL[tid] = acc;
-          }
-        } else {
-          bool whole = (e0 == Pi), first = true;
-          cdf acc = cdf_zero();
-          for (int el = e0; el < e1; ++el) {
-            cdf_fma(acc, row[k], v[k]);
-            if (++k > g) {
-              if (whole) pv[g] = acc;
-              else slotF[tid] = acc;
-              first = false;
-              whole = true;
-              acc = cdf_zero();
-              row += g + 1;
-              g += CL;
-              k = j + 1;
-            }
-          }
-          if (k != j + 1) {
-            if (first) slotF[tid] = acc;
-            else slotL[tid] = acc;
-          }
-        }
-      }
-      __syncthreads();
-      // rows split between threads: 8 lanes per row sum every 8th slot, then a 3-level butterfly
-      for (int base = 0; base < nr; base += NT / 8) {
-        const int i = base + (tid >> 3), q = tid & 7;
-        cdf sacc = cdf_zero();
-        bool split = false;
-        if (i < nr) {
-          const int Pi = i * (g0 - j) + CL * i * (i - 1) / 2;
-          const int len = g0 + CL * i - j;
-          const int ta = hs_owner(Pi, L1), tb = hs_owner(Pi + len - 1, L1);
-          split = ta != tb;
-          if (split) {
-            if (q == 0) sacc = (hs_seg(ta, E1, L1) == Pi) ? slotF[ta] : slotL[ta];
-            for (int t = ta + 1 + q; t <= tb; t += 8)
-              if (hs_seg(t, E1, L1) < hs_seg(t + 1, E1, L1)) sacc = cdf_add(sacc, slotF[t]);
-          }
-        }
-        for (int o = 1; o < 8; o <<= 1) sacc = cdf_add(sacc, cdf_shfl_xor(sacc, o));
-        if (split && q == 0) pv[g0 + CL * i] = sacc;
-      }
-    }
-    __syncthreads();
-
-    // column pass
-    const int cb = CP[j + 1];
-    const int E2 = CP[m] - cb;
-    if (E2 > 0) {
-      const int L2 = hs_seglen<NT>(E2);
-      const int e0 = hs_seg(tid, E2, L2), e1 = hs_seg(tid + 1, E2, L2);
-      if (e0 < e1) {
-        int lo = j + 1, hi = m - 1;
-        while (lo < hi) {
-          const int mid = (lo + hi + 1) >> 1;
-          if (CP[mid] <= cb + e0) lo = mid;
-          else hi = mid - 1;
-        }
-        int k = lo;
-        int o = cb + e0 - CP[k];
-        int cnt = CP[k + 1] - CP[k];
-        int q = hs_qfirst(k, c, CL) + o;
-        int g = c + CL * q, base = hs_rowbase(q, c, CL);
-        if constexpr (GS) {
-          bool whole = (o == 0), first = true, pending = false;
-          cdf acc = cdf_zero();
-          for (int el = e0; el < e1; el += HS_U) {
-            int addr[HS_U], qq[HS_U], kend[HS_U];  // kend: the column an element ends, else -1
-  #pragma unroll
-            for (int u = 0; u < HS_U; ++u) {
-              addr[u] = base + k;
-              qq[u] = q;
-              kend[u] = -1;
-              base += g + 1;
-              g += CL;
-              ++q;
-              if (++o == cnt) {
-                kend[u] = k;
-                if (el + u + 1 < e1) {
-                  do {
-                    ++k;
-                  } while (CP[k + 1] == CP[k]);
-                  cnt = CP[k + 1] - CP[k];
-                  q = hs_qfirst(k, c, CL);
-                  g = c + CL * q;
-                  base = hs_rowbase(q, c, CL);
-                  o = 0;
-                }
-              }
-            }
-            cdf a[HS_U];
-  #pragma unroll
-            for (int u = 0; u < HS_U; ++u)
-              if (el + u < e1) a[u] = S[addr[u]];
-  #pragma unroll
-            for (int u = 0; u < HS_U; ++u)
-              if (el + u < e1) {
-                cdf_fmac(acc, a[u], vown[qq[u]]);
-                pending = kend[u] < 0;
-                if (!pending) {
-                  if (whole) pv[kend[u]] = cdf_add(pv[kend[u]], acc);
-                  else slotF[tid] = acc;
-                  first = false;
-                  whole = true;
-                  acc = cdf_zero();
-                }
-              }
-          }
-          if (pending) {
-            if (first) slotF[tid] = acc;
-            else slotL[tid] = acc;
-          }
-        } else {
-          bool whole = (o == 0), first = true;
-          cdf acc = cdf_zero();
-          for (int el = e0; el < e1; ++el) {
-            cdf_fmac(acc, S[base + k], vown[q]);
-            base += g + 1;
-            g += CL;
-            ++q;
-            if (++o == cnt) {
-              if (whole) pv[k] = cdf_add(pv[k], acc);
-              else slotF[tid] = acc;
-              first = false;
-              whole = true;
-              acc = cdf_zero();
-              if (el + 1 < e1) {
-                do {
-                  ++k;
-                } while (CP[k + 1] == CP[k]);
-                cnt = CP[k + 1] - CP[k];
-                q = hs_qfirst(k, c, CL);
-                g = c + CL * q;
-                base = hs_rowbase(q, c, CL);
-                o = 0;
-              }
-            }
-          }
-          if (o != cnt && o != 0) {
-            if (first) slotF[tid] = acc;
-            else slotL[tid] = acc;
-          }
-        }
-      }
-      __syncthreads();
-      for (int k = j + 1 + tid; k < m; k += NT) {
-        const int cnt = CP[k + 1] - CP[k];
-        if (cnt == 0) continue;
-        const int s0 = CP[k] - cb;
-        const int ta = hs_owner(s0, L2), tb = hs_owner(s0 + cnt - 1, L2);
-        if (ta == tb) continue;
-        cdf sacc = (hs_seg(ta, E2, L2) == s0) ? slotF[ta] : slotL[ta];
-        for (int t = ta + 1; t <= tb; ++t)
-          if (hs_seg(t, E2, L2) < hs_seg(t + 1, E2, L2)) sacc = cdf_add(sacc, slotF[t]);
-        pv[k] = cdf_add(pv[k], sacc);
-      }
-    }
-    if (CL > 1) cluster.sync();
-    else __syncthreads();
-
-    // p = 2 sum of the parts; K = Re(v^H p); w = p - K v
-    dfl kp{0.f, 0.f};
-    for (int i = j + 1 + tid; i < m; i += NT) {
-      cdf pi = cdf_zero();
-#pragma unroll
-      for (int rr = 0; rr < CL; ++rr) {
-        const cdf* src = (CL > 1) ? cluster.map_shared_rank(pv, rr) : pv;
-        pi = cdf_add(pi, src[i]);
-      }
-      pi = cdf_make(dfl{2.f * pi.rh, 2.f * pi.rl}, dfl{2.f * pi.ih, 2.f * pi.il});
-      w[i] = pi;
-      const cdf vi = v[i];
-      kp = df_fma(kp, cre(vi), cre(pi));
-      kp = df_fma(kp, cim(vi), cim(pi));
-    }
-    const dfl K = df_block_sum(kp, red);
-    const dfl nK = df_neg(K);
-    for (int i = j + 1 + tid; i < m; i += NT) {
-      const cdf vi = v[i];
-      cdf wi = w[i];
-      wi = cdf_make(df_fma(cre(wi), cre(vi), nK), df_fma(cim(wi), cim(vi), nK));
-      w[i] = wi;
-    }
-    __syncthreads();
-  }
-  if (tid == 0 && ((m - 1) % CL) == c) {
-    const cdf sl = S[hs_rowbase((m - 1 - c) / CL, c, CL) + m - 1];
-    dfl t = cre(sl);
-    if (m > 1) {
-      const cdf vq = bufV[((m - 2) & 1) * m + m - 1], wq = bufW[((m - 2) & 1) * m + m - 1];
-      t = df_fma(t, df_neg(cre(vq)), cre(wq));
-      t = df_fma(t, df_neg(cim(vq)), cim(wq));
-      t = df_fma(t, df_neg(cre(vq)), cre(wq));
-      t = df_fma(t, df_neg(cim(vq)), cim(wq));
-    }
-    e.d[(long)b * m + m - 1] = ldexp(df_to(t), ex);
-  }
-  __threadfence();
-  if (CL > 1) cluster.sync();
-  else __syncthreads();
-  if (c == 0 && tid == 0) {
-    double2 dl = make_double2(1, 0);
-    e.delta[(long)b * m] = dl;
-    double tn = 0;
-    for (int jj = 0; jj < m - 1; ++jj) {
-      const double2 a = __ldcg(e.alpha + (long)b * m + jj);
-      const double aa = sqrt(cabs2(a));
-      e.f[(long)b * m + jj] = aa;
-      if (aa > 0) dl = cmul(dl, cscale(a, 1.0 / aa));
-      e.delta[(long)b * m + jj + 1] = dl;
-    }
-    for (int jj = 0; jj < m; ++jj) {
-      const double fl = (jj > 0) ? e.f[(long)b * m + jj - 1] : 0.0, fr = (jj < m - 1) ? e.f[(long)b * m + jj] : 0.0;
-      tn = fmax(tn, fabs(__ldcg(e.d + (long)b * m + jj)) + fl + fr);
-    }
-    e.tnorm[b] = tn;
-  }
-}
-
-// ---------------------------------------------------------------------------
-// One-pass double-float reduction with the rows in global memory (L2): the
-// same steps as k_hetrd_df (the update of step j-1 applied lazily in step j),
-// but its three sweeps of the trailing triangle (the pending rank-2 update,
-// the row and the column matrix-vector passes) become one.  Warps take strips
-// of HF_SR consecutive own rows and walk them 32 columns at a time, lane l on
-// column k0 + l (512-byte coalesced loads); each element is updated, stored
-// once and used twice:
-//   row part     p_g += a_gk v_k              (k <= g; lane-local over the
-//                                              strip, reduced across lanes once
-//                                              per strip)
-//   column part  p_k += conj(a_gk) v_g        (k < g; the lane's column, summed
-//                                              over the strip's rows, added to a
-//                                              warp-private partial of p)
-// The warp partials are summed per column after the sweep.  The strips go to
-// the warps by a schedule fixed for every step in the prologue: longest first
-// to the least loaded warp, which balances the sweep to about one short strip
-// and keeps every sum in a fixed order.
-// ---------------------------------------------------------------------------
-constexpr int HF_SR = 4;  // own rows per strip
-
-// strips of the sweep of one CTA (the most of any CTA of a cluster of CL)
-static int hetrd_df1_strips(int m, int CL) { return (hs_own_rows(m, 0, CL) + HF_SR - 1) / HF_SR; }
-// v[2], w[2], p, the warp partials [NW]; with `sched`, the strip schedule [m-1][strips] after them
-static size_t hetrd_df1_smem_bytes(int m, int nt, int CL = 1, bool sched = false) {
-  const size_t base = (size_t)(5 + nt / 32) * (size_t)m * sizeof(double2);
-  return sched ? base + (((size_t)(m - 1) * hetrd_df1_strips(m, CL) + 15) & ~(size_t)15) : base;
-}
-
-template <int CL, int NT>
-__global__ void __launch_bounds__(NT, 1) k_hetrd_df1(const double2* __restrict__ G, long ldg, long sG, int m,
-                                                     int s_elems, EigScratch e, int use_sched) {
-  extern __shared__ __align__(16) cdf dsm[];
-  constexpr int NW = NT / 32;
-  static_assert(HF_SR == 4, "the row-sum reduction below is written for strips of four rows");
-  cdf* S = (cdf*)e.Sg + (long)blockIdx.x * s_elems;  // own rows, packed, private to this CTA
-  cdf* bufV = dsm;                                   // [2][m] v of this and of the previous step
-  cdf* bufW = bufV + 2 * m;                          // [2][m] w
-  cdf* pv = bufW + 2 * m;                            // [m] this CTA's part of p
-  cdf* cpart = pv + m;                               // [NW][m] column parts of p, one per warp
-  uint8_t* sched = (uint8_t*)(cpart + NW * m);       // [m-1][NSM] the warp of every strip of every step
-  __shared__ dfl red[NW];
-  __shared__ int s_exp;
+template <typename C, int CL, bool GS>
+__global__ void __launch_bounds__(HETRD_NT, 1) k_hetrd(const double2* __restrict__ G, long ldg, long sG, int m, int s_elems,
+                                                 EigScratch e, int cp_global) {
+  using R = decltype(cre(C()));
+  constexpr bool DF = std::is_same<C, cdf>::value;
+  constexpr int NT = HETRD_NT, NW = NT / 32, IPT = 512 / NT;  // indices of a vector per thread (m <= 512)
+  constexpr int HF_SR = DF && !GS ? 8 : 4;       // rows per strip
+  constexpr int RP = DF ? 2 : 1;                 // of which interleaved
+  extern __shared__ __align__(16) unsigned char hfsm[];
+  C* S = GS ? (C*)e.Sg + (long)blockIdx.x * s_elems : (C*)hfsm;  // own rows, packed, private to this CTA
+  C* bufV = GS ? (C*)hfsm : S + s_elems;  // [2][m] v of this and of the previous step
+  C* w = bufV + 2 * m;                    // [m] w of the previous step
+  C* bufP = w + m;                        // [2][m] this CTA's part of p, by step parity (read by the partners)
+  C* bufX = bufP + 2 * m;                 // [2][m] the next column before its update, by step parity
+  C* cpart = cp_global ? (C*)e.Cp + (long)blockIdx.x * NW * m : bufX + 2 * m;  // [NW][m] column parts of p
+  __shared__ R redK[NW + 1], redN[NW + 1];
+  __shared__ C s_p2[2], s_ph, s_am;  // p of the entries j and j + 1; the phase of x_0; -alpha
+  __shared__ R s_ax0, s_vinv;
+  __shared__ int s_exp, s_glast[NW];
   cg::cluster_group cluster = cg::this_cluster();
   const int c = (CL > 1) ? (int)cluster.block_rank() : 0;
   const int b = (int)blockIdx.x / CL;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   G += (long)b * sG;
-  float2* Hv32 = (float2*)e.Hv + (long)b * m * m;
+  void* Hv = DF ? (void*)((float2*)e.Hv + (long)b * m * m) : (void*)(e.Hv + (long)b * m * m);
   const int nq = hs_own_rows(m, c, CL);
-  const int NSM = (hs_own_rows(m, 0, CL) + HF_SR - 1) / HF_SR;
+  const int qlast = nq - 1 - warp;  // this warp's last own row: qlast, qlast - NW, ..
+  const C z = c_zero(C());
 
-  // The strip schedule of every step, fixed before the first (so the column parts are
-  // summed in the same order on every run): longest strip first to the least loaded
-  // warp (lowest index on ties), a strip costing its 32-column chunks x 4 rows plus one
-  // for its row-sum reduction.  Without room for it, the warps take the strips in snake
-  // order (w, 2 NW - 1 - w, 2 NW + w, ...).
-  if (use_sched) {
-    for (int jj = tid; jj < m - 1; jj += NT) {
-      const int q0j = hs_qfirst(jj, c, CL);
-      const int nsj = (max(0, nq - q0j) + HF_SR - 1) / HF_SR;
-      int load[NW];
-#pragma unroll
-      for (int w2 = 0; w2 < NW; ++w2) load[w2] = 0;
-      for (int t = 0; t < nsj; ++t) {
-        const int sj = nsj - 1 - t;
-        const int glast = c + CL * min(q0j + sj * HF_SR + HF_SR - 1, nq - 1);
-        const int cost = ((glast - jj) + 31) / 32 * HF_SR + 1;
-        int wb = 0, lb = load[0];
-#pragma unroll
-        for (int w2 = 1; w2 < NW; ++w2)
-          if (load[w2] < lb) {
-            lb = load[w2];
-            wb = w2;
-          }
-#pragma unroll
-        for (int w2 = 0; w2 < NW; ++w2)
-          if (w2 == wb) load[w2] += cost;
-        sched[jj * NSM + sj] = (uint8_t)wb;
-      }
-    }
-  }
-
-  // power-of-two scale from the largest diagonal entry (identical in every CTA)
-  {
+  // double-float: power-of-two scale from the largest diagonal entry (identical in every CTA)
+  if (tid == 0) s_exp = 0;
+  if (lane == 0) s_glast[warp] = qlast >= 0 ? c + CL * qlast : -1;
+  if constexpr (DF) {
+    __shared__ double wmx[NW];
     double mx = 0;
     for (int i = tid; i < m; i += NT) mx = fmax(mx, fabs(__ldcg(G + (long)i * ldg + i).x));
     for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    __shared__ double wmx[NW];
     if (lane == 0) wmx[warp] = mx;
     __syncthreads();
     if (tid == 0) {
       double t = 0;
-      for (int w = 0; w < NW; ++w) t = fmax(t, wmx[w]);
+      for (int q = 0; q < NW; ++q) t = fmax(t, wmx[q]);
       int ex = 0;
       if (t > 0 && isfinite(t)) frexp(t, &ex);
       s_exp = ex;
     }
-    __syncthreads();
   }
+  __syncthreads();
   const int ex = s_exp;
   for (int q = warp; q < nq; q += NW) {
     const int g = c + CL * q;
     const double2* src = G + (long)g * ldg;
-    cdf* dst = S + hs_rowbase(q, c, CL);
-    for (int k = lane; k <= g; k += 32) {
-      const double2 x = __ldcg(src + k);
-      dst[k] = cdf_from(make_double2(ldexp(x.x, -ex), ldexp(x.y, -ex)));
-    }
+    C* dst = S + hs_rowbase(q, c, CL);
+    for (int k = lane; k <= g; k += 32) dst[k] = c_from(C(), __ldcg(src + k), ex);
   }
-  for (int i = tid; i < (5 + NW) * m; i += NT) bufV[i] = cdf_zero();
+  for (int i = tid; i < m; i += NT) {
+    bufX[i] = c_from(C(), __ldcg(G + (long)i * ldg), ex);
+    // no update is pending in the first step; entries a vector never gets multiply zeros: finite
+    bufV[i] = bufV[m + i] = w[i] = z;
+  }
   if (CL > 1) cluster.sync();
   else __syncthreads();
 
-  for (int j = 0; j < m - 1; ++j) {
+  for (int j = 0; j < m; ++j) {
     const int cur = j & 1;
-    cdf* v = bufV + cur * m;
-    cdf* w = bufW + cur * m;
-    const cdf* vp = bufV + (cur ^ 1) * m;
-    const cdf* wp = bufW + (cur ^ 1) * m;
+    C* v = bufV + cur * m;
+    const C* vp = bufV + (cur ^ 1) * m;
+    const C* xr = bufX + cur * m;
     const bool lag = j > 0;
-    // column j of A^(j) (the pending update applied) to every CTA's v; the diagonal d_j
-    {
-      const cdf vpj = vp[j], wpj = wp[j];
-      for (int q = hs_qfirst(j, c, CL) + tid; q < nq; q += NT) {
-        const int g = c + CL * q;
-        cdf a = S[hs_rowbase(q, c, CL) + j];
-        if (lag) a = cdf_lag(a, vp[g], wp[g], vpj, wpj);
+    // w of step j-1 and the column j of A^(j); indices i = tid + NT u
+    C x[IPT], x0 = (j + 1 < m) ? xr[j + 1] : z;
+    if (lag) {
+      C pi[IPT], vi[IPT];
+      R kp = r_zero(R());
 #pragma unroll
-        for (int rr = 0; rr < CL; ++rr) {
-          cdf* dst = (CL > 1) ? cluster.map_shared_rank(v, rr) : v;
-          dst[g] = a;
+      for (int u = 0; u < IPT; ++u) {
+        const int i = tid + NT * u;
+        pi[u] = vi[u] = z;
+        if (i >= j && i < m) {
+          const C* part = bufP + (cur ^ 1) * m + i;
+#pragma unroll
+          for (int rr = 0; rr < CL; ++rr) {
+            const C* src = (CL > 1) ? cluster.map_shared_rank(part, rr) : part;
+            pi[u] = rr == 0 ? *src : c_add(pi[u], *src);
+          }
+          pi[u] = c_twice(pi[u]);
+          vi[u] = vp[i];
+          kp = r_fma(kp, cre(vi[u]), cre(pi[u]));
+          kp = r_fma(kp, cim(vi[u]), cim(pi[u]));
+          if (i - j < 2) s_p2[i - j] = pi[u];
         }
       }
-      if (tid == 0 && (j % CL) == c) {
-        const cdf sj = S[hs_rowbase((j - c) / CL, c, CL) + j];
-        dfl t = cre(sj);
-        t = df_fma(t, df_neg(cre(vpj)), cre(wpj));
-        t = df_fma(t, df_neg(cim(vpj)), cim(wpj));
-        t = df_fma(t, df_neg(cre(vpj)), cre(wpj));
-        t = df_fma(t, df_neg(cim(vpj)), cim(wpj));
-        e.d[(long)b * m + j] = ldexp(df_to(t), ex);
+      const R nK = r_neg(hf_block_sum<NW>(kp, redK, lane, warp));
+      const C vj = vp[j], pj = s_p2[0];
+      const C wj = c_make(r_fma(cre(pj), cre(vj), nK), r_fma(cim(pj), cim(vj), nK));
+      if (warp == NW - 1 && j + 1 < m) {  // x_0 once more, for its phase
+        const C v1 = vp[j + 1], p1 = s_p2[1];
+        const C w1 = c_make(r_fma(cre(p1), cre(v1), nK), r_fma(cim(p1), cim(v1), nK));
+        x0 = c_lag(x0, v1, w1, vj, wj);
       }
+#pragma unroll
+      for (int u = 0; u < IPT; ++u) {
+        const int i = tid + NT * u;
+        x[u] = z;
+        if (i >= j && i < m) {
+          const C wi = c_make(r_fma(cre(pi[u]), cre(vi[u]), nK), r_fma(cim(pi[u]), cim(vi[u]), nK));
+          w[i] = wi;
+          x[u] = c_lag(xr[i], vi[u], wi, vj, wj);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < IPT; ++u) x[u] = (tid + NT * u < m) ? xr[tid + NT * u] : z;
     }
-    if (CL > 1) cluster.sync();
-    else __syncthreads();
-    const int n = m - j - 1;
-    // the reflector: |x|^2 by the whole block (fixed order, so both CTAs agree), then every
-    // thread forms -alpha = e^{i arg x0} |x| and 1 / sqrt(2 |x| (|x| + |x0|)) itself
+    if (c == 0) {
+#pragma unroll
+      for (int u = 0; u < IPT; ++u)
+        if (tid + NT * u == j) e.d[(long)b * m + j] = DF ? ldexp(r_double(cre(x[u])), ex) : r_double(cre(x[u]));
+    }
+    if (j == m - 1) break;
+    // the reflector
     {
-      const cdf x0 = v[j + 1];
-      dfl t{0.f, 0.f};
-      for (int i = tid; i < n; i += NT) {
-        const cdf x = v[j + 1 + i];
-        t = df_fma(t, cre(x), cre(x));
-        t = df_fma(t, cim(x), cim(x));
-      }
-      const dfl nrm2d = df_block_sum(t, red);
-      cdf am = cdf_zero();  // -alpha
-      dfl vinv{0.f, 0.f};
-      if (nrm2d.hi > 0.f) {
-        const dfl nrm = df_sqrt_nodiv(nrm2d);
-        const dfl ax2 = df_fma(df_fma(dfl{0.f, 0.f}, cre(x0), cre(x0)), cim(x0), cim(x0));
-        dfl phr{1.f, 0.f}, phi{0.f, 0.f}, ax0{0.f, 0.f};
-        if (ax2.hi > 0.f) {
-          const dfl iax = df_rsqrt(ax2);  // 1 / |x0|
-          ax0 = df_mul(ax2, iax);
-          phr = df_mul(cre(x0), iax);
-          phi = df_mul(cim(x0), iax);
+      R t = r_zero(R());
+#pragma unroll
+      for (int u = 0; u < IPT; ++u) {
+        const int i = tid + NT * u;
+        if (i > j && i < m) {
+          t = r_fma(t, cre(x[u]), cre(x[u]));
+          t = r_fma(t, cim(x[u]), cim(x[u]));
         }
-        am = cdf_make(df_mul(phr, nrm), df_mul(phi, nrm));
-        vinv = df_rsqrt(df_mul(df_add(nrm, nrm), df_add(nrm, ax0)));
       }
-      if (tid == 0 && c == 0) {
-        const double2 al = cdf_to(am);
-        e.alpha[(long)b * m + j] = make_double2(-ldexp(al.x, ex), -ldexp(al.y, ex));
+      if (warp == NW - 1) {  // |x_0| and e^{i arg x_0}, beside the norm
+        const R ax2 = r_fma(r_fma(r_zero(R()), cre(x0), cre(x0)), cim(x0), cim(x0));
+        R ax0 = r_zero(R());
+        C phase = c_one(C());
+        if (r_pos(ax2)) {
+          const R iax = r_rsqrt(ax2);
+          ax0 = r_mul(ax2, iax);
+          phase = c_make(r_mul(cre(x0), iax), r_mul(cim(x0), iax));
+        }
+        if (lane == 0) {
+          s_ax0 = ax0;
+          s_ph = phase;
+        }
       }
-      for (int i = tid; i < n; i += NT) {
-        cdf vi = v[j + 1 + i];
-        if (i == 0) vi = cdf_add(vi, am);
-        vi = cdf_scale(vi, vinv);
-        v[j + 1 + i] = vi;
-        // read by the FP32 back-transform after this kernel: evict-first, so the
-        // row store keeps the L2
-        if (c == 0) __stcs(Hv32 + (long)j * m + j + 1 + i, make_float2(vi.rh, vi.ih));
+      const R nrm2 = hf_block_sum<NW>(t, redN, lane, warp);
+      C am = z;  // -alpha = e^{i arg x0} |x|
+      R vinv = r_zero(R());
+      if (DF || warp == 0) {  // FP64: by one warp (one more barrier)
+        if (r_pos(nrm2)) {
+          const R nrm = r_sqrt(nrm2);
+          vinv = r_rsqrt(r_mul(r_add(nrm, nrm), r_add(nrm, s_ax0)));
+          am = c_make(r_mul(cre(s_ph), nrm), r_mul(cim(s_ph), nrm));
+        }
+        if (!DF && lane == 0) {
+          s_am = am;
+          s_vinv = vinv;
+        }
+        if (tid == 0 && c == 0) {
+          double2 al = make_double2(-r_double(cre(am)), -r_double(cim(am)));
+          if (DF) al = make_double2(ldexp(al.x, ex), ldexp(al.y, ex));
+          e.alpha[(long)b * m + j] = al;
+        }
+      }
+      if constexpr (!DF) {
+        __syncthreads();
+        am = s_am;
+        vinv = s_vinv;
+      }
+#pragma unroll
+      for (int u = 0; u < IPT; ++u) {
+        const int i = tid + NT * u;
+        if (i > j && i < m) {
+          C vi = x[u];
+          if (i == j + 1) vi = c_add(vi, am);
+          vi = c_scale_r(vi, vinv);
+          v[i] = vi;
+          if (c == 0) put_hv(Hv, (long)j * m + i, vi);
+        }
       }
     }
     __syncthreads();
 
-    // the sweep: pending update, store, row and column parts of p = A^(j) v
-    const int q0 = hs_qfirst(j, c, CL);
-    const int nstrip = (max(0, nq - q0) + HF_SR - 1) / HF_SR;
-    cdf* cp = cpart + warp * m;
-    const uint8_t* own = sched + j * NSM;
-    unsigned mine = 0;  // this warp's strips among s0 .. s0 + 31 (with the schedule)
-    for (int s0 = 0, it = 0; s0 < nstrip;) {
-      int s;
-      if (use_sched) {
-        if (it == 0) {
-          const int sl = s0 + lane;
-          mine = __ballot_sync(0xffffffffu, sl < nstrip && own[sl] == warp);
+    // the sweep
+    {
+      const int q0 = hs_qfirst(j, c, CL);
+      const int nr = qlast >= q0 ? (qlast - q0) / NW + 1 : 0;  // own rows of this warp
+      const int nst = (nr + HF_SR - 1) / HF_SR;
+      const int per = nst > 0 ? (nr + nst - 1) / nst : 0;      // rows per strip, evenly
+      C* cp = cpart + warp * m;
+      C* xn = bufX + (cur ^ 1) * m;
+      C* pv = bufP + cur * m;
+      for (int st = 0; st < nst; ++st) {
+        const int r0 = st * per, rn = min(per, nr - r0);
+        int gr[HF_SR], off[HF_SR];
+#pragma unroll
+        for (int r = 0; r < HF_SR; ++r) {
+          const int q = max(qlast - NW * (r0 + r), 0);
+          gr[r] = r < rn ? c + CL * q : -1;  // -1: no row
+          off[r] = hs_rowbase(q, c, CL);
         }
-        if (mine == 0) {  // the next group of 32 strips
-          s0 += 32;
-          it = 0;
-          continue;
+        const int glast = gr[0];
+        C racc[HF_SR];
+#pragma unroll
+        for (int r = 0; r < HF_SR; ++r) racc[r] = z;
+        C next[GS ? HF_SR : 1];  // rows in L2: the next 32 columns, on their way during this one's arithmetic
+        if constexpr (GS) {
+#pragma unroll
+          for (int r = 0; r < HF_SR; ++r) next[r] = (j + 1 + lane <= gr[r]) ? S[off[r] + j + 1 + lane] : z;
         }
-        const int bit = 31 - __clz(mine);
-        mine &= ~(1u << bit);
-        s = s0 + bit;
-        it = 1;
-      } else {
-        s = s0 + (((s0 / NW) & 1) ? NW - 1 - warp : warp);  // snake order
-        s0 += NW;
-        if (s >= nstrip) continue;
-      }
-      const int qs = q0 + s * HF_SR;
-      int gr[HF_SR];
-      cdf* rowp[HF_SR];
+        for (int k0 = j + 1; k0 <= glast; k0 += 32) {
+          const int k = k0 + lane, kc = min(k, glast);
+          C a[GS ? HF_SR : 1];
+          if constexpr (GS) {
 #pragma unroll
-      for (int r = 0; r < HF_SR; ++r) {
-        const int q = min(qs + r, nq - 1);
-        gr[r] = (qs + r < nq) ? c + CL * q : -1;  // -1: no row (past the last own row)
-        rowp[r] = S + hs_rowbase(q, c, CL);
-      }
-      const int glast = c + CL * min(qs + HF_SR - 1, nq - 1);
-      cdf racc[HF_SR];
-#pragma unroll
-      for (int r = 0; r < HF_SR; ++r) racc[r] = cdf_zero();
-      for (int k0 = j + 1; k0 <= glast; k0 += 32) {
-        const int k = k0 + lane;
-        cdf a[HF_SR];
-#pragma unroll
-        for (int r = 0; r < HF_SR; ++r)
-          if (k <= gr[r]) a[r] = rowp[r][k];
-        if (k <= glast) {
-          const cdf vk = v[k];
-          cdf vpk = cdf_zero(), wpk = cdf_zero();
-          if (lag) {
-            vpk = vp[k];
-            wpk = wp[k];
-          }
-          cdf cacc = cdf_zero();
-#pragma unroll
-          for (int r = 0; r < HF_SR; ++r) {
-            if (k <= gr[r]) {
-              const int g = gr[r];
-              cdf x = a[r];
-              if (lag) {
-                x = cdf_lag(x, vp[g], wp[g], vpk, wpk);
-                if (k == g) {
-                  x.ih = 0.f;
-                  x.il = 0.f;
-                }
-                rowp[r][k] = x;
-              }
-              cdf_fma_acc(racc[r], x, vk);
-              if (k < g) cdf_fmac_acc(cacc, x, v[g]);
+            for (int r = 0; r < HF_SR; ++r) {
+              a[r] = next[r];
+              next[r] = (k + 32 <= gr[r]) ? S[off[r] + k + 32] : z;
             }
           }
-          if (k < glast) cp[k] = cdf_add(cp[k], cacc);
-        }
-      }
-      // row sums across the lanes: halve the rows twice (lanes 16-31 keep rows 2, 3; then
-      // lanes with bit 3 set keep the odd row), then a 3-level butterfly; lane l ends with
-      // row l / 8
-      {
-        const bool u16 = (lane & 16) != 0, u8 = (lane & 8) != 0;
-        cdf k0v = u16 ? racc[2] : racc[0], k1v = u16 ? racc[3] : racc[1];
-        const cdf s0v = u16 ? racc[0] : racc[2], s1v = u16 ? racc[1] : racc[3];
-        k0v = cdf_add(k0v, cdf_shfl_xor(s0v, 16));
-        k1v = cdf_add(k1v, cdf_shfl_xor(s1v, 16));
-        cdf kk = u8 ? k1v : k0v;
-        const cdf ss = u8 ? k0v : k1v;
-        kk = cdf_add(kk, cdf_shfl_xor(ss, 8));
-        for (int o = 4; o > 0; o >>= 1) kk = cdf_add(kk, cdf_shfl_xor(kk, o));
-        const int r = lane >> 3;
-        int gsel = gr[0];
+          const C vk = v[kc], vpk = vp[kc], wpk = w[kc];
+          C cacc[RP];
 #pragma unroll
-        for (int rr = 1; rr < HF_SR; ++rr)
-          if (r == rr) gsel = gr[rr];
-        if ((lane & 7) == 0 && gsel >= 0) pv[gsel] = kk;
+          for (int u = 0; u < RP; ++u) cacc[u] = z;
+          // RP rows at a time, without branches on the lane: the chains of the two interleave; lanes
+          // past a row's end carry zeros
+#pragma unroll
+          for (int r = 0; r < HF_SR; r += RP) {
+            if (k0 > gr[r]) break;  // rows get shorter
+            C y[RP];
+#pragma unroll
+            for (int u = 0; u < RP; ++u) {
+              if constexpr (GS) y[u] = a[r + u];
+              else y[u] = (k <= gr[r + u]) ? S[off[r + u] + k] : z;
+            }
+#pragma unroll
+            for (int u = 0; u < RP; ++u) {
+              const int g = max(gr[r + u], 0);
+              y[u] = c_lag(y[u], vp[g], w[g], vpk, wpk);
+              if (k > gr[r + u]) y[u] = z;
+              if (k == gr[r + u]) c_real(y[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < RP; ++u)
+              if (k <= gr[r + u]) S[off[r + u] + k] = y[u];
+            if (k == j + 1) {  // the next column, to every CTA
+#pragma unroll
+              for (int u = 0; u < RP; ++u)
+                if (gr[r + u] >= 0) {
+#pragma unroll
+                  for (int rr = 0; rr < CL; ++rr) {
+                    C* dst = (CL > 1) ? cluster.map_shared_rank(xn, rr) : xn;
+                    dst[gr[r + u]] = y[u];
+                  }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < RP; ++u) {
+              c_fma_acc(racc[r + u], y[u], vk);
+              c_fmac_acc(cacc[u], (k < gr[r + u]) ? y[u] : z, v[max(gr[r + u], 0)]);
+            }
+          }
+          // the first strip has the warp's last row, hence all its columns
+          if (k < glast) {
+            const C cs = RP == 2 ? c_add(cacc[0], cacc[RP - 1]) : cacc[0];
+            cp[k] = st == 0 ? cs : c_add(cp[k], cs);
+          }
+        }
+        // row sums across the lanes: halve the rows (the lanes with the bit set keep the upper half)
+        // until one is left, then a butterfly; lane l ends with row l SR / 32
+        int o = 16;
+#pragma unroll
+        for (int h = HF_SR / 2; h > 0; h >>= 1, o >>= 1) {
+          const bool up = (lane & o) != 0;
+#pragma unroll
+          for (int i = 0; i < h; ++i) {
+            const C keep = up ? racc[h + i] : racc[i], send = up ? racc[i] : racc[h + i];
+            racc[i] = c_add(keep, c_shfl(send, o));
+          }
+        }
+#pragma unroll
+        for (; o > 0; o >>= 1) racc[0] = c_add(racc[0], c_shfl(racc[0], o));
+        constexpr int LR = 32 / HF_SR;  // lanes per row
+        if (lane % LR == 0 && lane / LR < rn) pv[c + CL * (qlast - NW * (r0 + lane / LR))] = racc[0];
       }
     }
     __syncthreads();
-    // p of this CTA: its rows' row parts plus every warp's column parts; the partials are
-    // cleared for the next step as they are read
-    for (int k = j + 1 + tid; k < m; k += NT) {
-      cdf part[NW];  // all loads first, then a pairwise sum (fixed order), then the clearing
+    // this CTA's part of p: its rows' row parts plus the warps' column parts (a warp has them for the
+    // columns before its last row), all loads first, then a pairwise sum
+    {
+      C* pv = bufP + cur * m;
 #pragma unroll
-      for (int w2 = 0; w2 < NW; ++w2) part[w2] = cpart[w2 * m + k];
+      for (int u = 0; u < IPT; ++u) {
+        const int k = tid + NT * u;
+        if (k > j && k < m) {
+          C part[NW];
 #pragma unroll
-      for (int h = NW / 2; h > 0; h >>= 1)
+          for (int q = 0; q < NW; ++q) part[q] = k < s_glast[q] ? cpart[q * m + k] : z;
 #pragma unroll
-        for (int w2 = 0; w2 < h; ++w2) part[w2] = cdf_add(part[w2], part[w2 + h]);
+          for (int h = NW / 2; h > 0; h >>= 1)
 #pragma unroll
-      for (int w2 = 0; w2 < NW; ++w2) cpart[w2 * m + k] = cdf_zero();
-      pv[k] = (k % CL == c) ? cdf_add(pv[k], part[0]) : part[0];
+            for (int q = 0; q < h; ++q) part[q] = c_add(part[q], part[q + h]);
+          pv[k] = (k % CL == c) ? c_add(pv[k], part[0]) : part[0];
+        }
+      }
     }
     if (CL > 1) cluster.sync();
     else __syncthreads();
-    // p = 2 sum of the parts; K = Re(v^H p); w = p - K v
-    dfl kp{0.f, 0.f};
-    for (int i = j + 1 + tid; i < m; i += NT) {
-      cdf pi = cdf_zero();
-#pragma unroll
-      for (int rr = 0; rr < CL; ++rr) {
-        const cdf* src = (CL > 1) ? cluster.map_shared_rank(pv, rr) : pv;
-        pi = cdf_add(pi, src[i]);
-      }
-      pi = cdf_make(dfl{2.f * pi.rh, 2.f * pi.rl}, dfl{2.f * pi.ih, 2.f * pi.il});
-      w[i] = pi;
-      const cdf vi = v[i];
-      kp = df_fma(kp, cre(vi), cre(pi));
-      kp = df_fma(kp, cim(vi), cim(pi));
-    }
-    const dfl K = df_block_sum(kp, red);
-    const dfl nK = df_neg(K);
-    for (int i = j + 1 + tid; i < m; i += NT) {
-      const cdf vi = v[i];
-      cdf wi = w[i];
-      wi = cdf_make(df_fma(cre(wi), cre(vi), nK), df_fma(cim(wi), cim(vi), nK));
-      w[i] = wi;
-    }
-    __syncthreads();
   }
-  if (tid == 0 && ((m - 1) % CL) == c) {
-    const cdf sl = S[hs_rowbase((m - 1 - c) / CL, c, CL) + m - 1];
-    dfl t = cre(sl);
-    if (m > 1) {
-      const cdf vq = bufV[((m - 2) & 1) * m + m - 1], wq = bufW[((m - 2) & 1) * m + m - 1];
-      t = df_fma(t, df_neg(cre(vq)), cre(wq));
-      t = df_fma(t, df_neg(cim(vq)), cim(wq));
-      t = df_fma(t, df_neg(cre(vq)), cre(wq));
-      t = df_fma(t, df_neg(cim(vq)), cim(wq));
-    }
-    e.d[(long)b * m + m - 1] = ldexp(df_to(t), ex);
-  }
-  __threadfence();
-  if (CL > 1) cluster.sync();
+  if (CL > 1) cluster.sync();  // the partners' last reads of this CTA's part of p
   else __syncthreads();
-  if (c == 0 && tid == 0) {
-    double2 dl = make_double2(1, 0);
-    e.delta[(long)b * m] = dl;
+  if (c != 0) return;
+  // |alpha_j|, the phases that make T real (running products of alpha_j / |alpha_j|) and a bound of
+  // its norm
+  double2* ph = (double2*)bufV;
+  __syncthreads();
+  for (int i = tid; i < m - 1; i += NT) {
+    const double2 a = __ldcg(e.alpha + (long)b * m + i);
+    const double aa = sqrt(cabs2(a));
+    e.f[(long)b * m + i] = aa;
+    ph[i] = aa > 0 ? cscale(a, 1.0 / aa) : make_double2(1.0, 0.0);
+  }
+  __syncthreads();
+  if (warp == 0) {
+    const int per = (m - 1 + 31) / 32, i0 = min(lane * per, m - 1), i1 = min(i0 + per, m - 1);
+    double2 t = make_double2(1.0, 0.0);
+    for (int i = i0; i < i1; ++i) t = cmul(t, ph[i]);
+    double2 run = t;  // inclusive products of the lanes' own
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double2 up = make_double2(__shfl_up_sync(0xffffffffu, run.x, o), __shfl_up_sync(0xffffffffu, run.y, o));
+      if (lane >= o) run = cmul(up, run);
+    }
+    double2 dl = make_double2(__shfl_up_sync(0xffffffffu, run.x, 1), __shfl_up_sync(0xffffffffu, run.y, 1));
+    if (lane == 0) {
+      dl = make_double2(1.0, 0.0);
+      e.delta[(long)b * m] = dl;
+    }
+    for (int i = i0; i < i1; ++i) {
+      dl = cmul(dl, ph[i]);
+      e.delta[(long)b * m + i + 1] = dl;
+    }
+  } else if (warp == 1) {
     double tn = 0;
-    for (int jj = 0; jj < m - 1; ++jj) {
-      const double2 a = __ldcg(e.alpha + (long)b * m + jj);
-      const double aa = sqrt(cabs2(a));
-      e.f[(long)b * m + jj] = aa;
-      if (aa > 0) dl = cmul(dl, cscale(a, 1.0 / aa));
-      e.delta[(long)b * m + jj + 1] = dl;
+    for (int i = lane; i < m; i += 32) {
+      const double fl = (i > 0) ? e.f[(long)b * m + i - 1] : 0.0, fr = (i < m - 1) ? e.f[(long)b * m + i] : 0.0;
+      tn = fmax(tn, fabs(e.d[(long)b * m + i]) + fl + fr);
     }
-    for (int jj = 0; jj < m; ++jj) {
-      const double fl = (jj > 0) ? e.f[(long)b * m + jj - 1] : 0.0, fr = (jj < m - 1) ? e.f[(long)b * m + jj] : 0.0;
-      tn = fmax(tn, fabs(__ldcg(e.d + (long)b * m + jj)) + fl + fr);
-    }
-    e.tnorm[b] = tn;
+    for (int o = 16; o > 0; o >>= 1) tn = fmax(tn, __shfl_xor_sync(0xffffffffu, tn, o));
+    if (lane == 0) e.tnorm[b] = tn;
   }
 }
 
@@ -2392,42 +1457,106 @@ static int device_attr(cudaDeviceAttr a, int fallback) {
   return v;
 }
 
-// Cluster size of the shared-memory tridiagonalisation, or 0 when the slice's
-// rows do not fit: the largest CL in {8,4,2,1} with batch * CL CTAs resident
-// at once (one per SM), at least 48 rows per CTA (else the per-step barriers
-// dominate) and the packed rows within the opt-in shared memory.
-static int hetrd_smem_cluster(int m, int batch, int nt, bool global_rows = false) {
-  if (m < 2) return 0;
-  const int sms = device_attr(cudaDevAttrMultiProcessorCount, 148);
-  // the kernels' static arrays (up to about 1.3 KB) share the per-block limit with the dynamic part
+// Clusters of CL CTAs of k_hetrd that the device holds at once, one CTA per SM (clusters stay inside a
+// group of SMs, so 8 x 15 and 4 x 36 of the 152 SMs here); a cluster more would wait for a whole
+// reduction to end.  A property of the device, looked up once per size.
+static int hetrd_clusters(int CL) {
+  static std::mutex mu;
+  static int known[64][9];
+  int dev = 0;
+  const bool have = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64;
+  const int guess = std::max(1, device_attr(cudaDevAttrMultiProcessorCount, 148) - 4 * (CL - 1)) / CL;
+  if (!have || CL == 1) {
+    cudaGetLastError();
+    return guess;
+  }
+  std::lock_guard<std::mutex> lk(mu);
+  int& n = known[dev][CL];
+  if (n == 0) {
+    auto kern = CL == 8 ? k_hetrd<cdf, 8, false> : CL == 4 ? k_hetrd<cdf, 4, false>
+                                                                     : k_hetrd<cdf, 2, false>;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(64 * CL);
+    cfg.blockDim = dim3(HETRD_NT);
+    cfg.dynamicSmemBytes = 200 * 1024;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = CL;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
+      cudaGetLastError();
+      n = guess;
+    }
+  }
+  return n;
+}
+
+// How a batch of m x m reductions is laid out (k_hetrd): the largest cluster in {8, 4, 2, 1} whose CTAs are
+// all resident at once, with at least 20 rows each (m = 90 on 9 slices: 604 us on clusters of 1, 508 on 2,
+// 455 on 4), and whose packed rows fit in shared memory beside the vectors, with the warps' partials there
+// too or, where only those do not fit, in L2; else rows in L2.
+struct HetrdPlan {
+  int CL;
+  bool global_rows, cp_global;
+  size_t smem;
+};
+static HetrdPlan hetrd_plan(int m, int batch) {
+  // the kernel's static arrays (about 1 KB) share the per-block limit with the dynamic part
   const size_t smax = (size_t)device_attr(cudaDevAttrMaxSharedMemoryPerBlockOptin, 232448) - 2048;
+  const size_t el = sizeof(double2), vec = 7 * (size_t)m * el, part = (size_t)(HETRD_NT / 32) * m * el;
+  int most = 1;
   for (int CL = 8; CL >= 1; CL >>= 1) {
-    if (CL > 1 && ((long)batch * CL > sms || m / CL < 48)) continue;
-    if (hetrd_smem_bytes(m, CL, nt, global_rows) <= smax) return CL;
+    if (CL > 1 && (m / CL < 20 || batch > hetrd_clusters(CL))) continue;
+    most = std::max(most, CL);
+    const size_t rows = hetrd_row_elems(m, CL) * el;
+    if (rows + vec + part <= smax) return HetrdPlan{CL, false, false, rows + vec + part};
+    if (rows + vec <= smax) return HetrdPlan{CL, false, true, rows + vec};
   }
-  return 0;
+  return HetrdPlan{most, true, false, vec + part};
 }
 
-// the packed rows do not fit in shared memory for the double-float reduction
-// (the larger of the two): they go to a global array (EigScratch::Sg)
-static bool hetrd_needs_global_rows(int m, int batch) {
-  return m >= 2 && hetrd_smem_cluster(m, batch, 2 * HS_THREADS) == 0;
+static EigScratch carve_eig(void* base, int m, int R, int batch, size_t* bytes) {
+  Carver cv(base);
+  EigScratch e;
+  e.d = cv.take<double>((size_t)batch * m);
+  e.f = cv.take<double>((size_t)batch * m);
+  e.alpha = cv.take<double2>((size_t)batch * m);
+  e.delta = cv.take<double2>((size_t)batch * m);
+  e.Hv = cv.take<double2>((size_t)batch * m * m);
+  e.Z = cv.take<double>((size_t)batch * m * R);
+  e.lu = cv.take<double>((size_t)batch * 5 * m * R);
+  e.tnorm = cv.take<double>((size_t)batch);
+  e.Sg = e.Cp = nullptr;
+  const HetrdPlan pl = hetrd_plan(m, batch);
+  // CL CTAs of a slice own at most m(m+1)/2 + CL m packed elements together (CL <= 8)
+  if (pl.global_rows) e.Sg = cv.take<double2>((size_t)batch * ((size_t)m * (m + 1) / 2 + 8 * (size_t)m));
+  if (pl.cp_global) e.Cp = cv.take<double2>((size_t)batch * pl.CL * (HETRD_NT / 32) * m);
+  if (bytes) *bytes = cv.bytes();
+  return e;
 }
 
-template <int CL, bool DF, bool GS>
-static int launch_hetrd_smem_t(const double2* G, long ldg, long sG, int m, int batch, const EigScratch& e,
-                               cudaStream_t s, int b0 = 0) {
-  constexpr int NT = DF ? 2 * HS_THREADS : HS_THREADS;
-  const size_t smem = hetrd_smem_bytes(m, CL, NT, GS);
-  auto kern = DF ? k_hetrd_df<CL, NT, GS> : k_hetrd_smem<CL, GS>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+size_t eig_scratch_bytes(int m, int R, int batch) {
+  size_t b = 0;
+  carve_eig(nullptr, m, R, batch, &b);
+  return b;
+}
+
+template <typename C, int CL, bool GS>
+static int launch_hetrd_t(const double2* G, long ldg, long sG, int m, int batch, const EigScratch& e,
+                          const HetrdPlan& pl, cudaStream_t s) {
+  auto kern = k_hetrd<C, CL, GS>;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem) != cudaSuccess) {
     cudaGetLastError();
     return TSVD_ERR_CUDA;
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(batch * CL);
-  cfg.blockDim = dim3(NT);
-  cfg.dynamicSmemBytes = smem;
+  cfg.blockDim = dim3(HETRD_NT);
+  cfg.dynamicSmemBytes = pl.smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -2436,7 +1565,8 @@ static int launch_hetrd_smem_t(const double2* G, long ldg, long sG, int m, int b
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, kern, G, ldg, sG, m, (int)hetrd_smem_elems(m, CL), e, b0) != cudaSuccess) {
+  if (cudaLaunchKernelEx(&cfg, kern, G, ldg, sG, m, (int)hetrd_row_elems(m, CL), e, pl.cp_global ? 1 : 0) !=
+      cudaSuccess) {
     cudaGetLastError();
     return TSVD_ERR_CUDA;
   }
@@ -2444,68 +1574,14 @@ static int launch_hetrd_smem_t(const double2* G, long ldg, long sG, int m, int b
   return TSVD_OK;
 }
 
-template <bool DF, bool GS>
-static int launch_hetrd_smem(int CL, const double2* G, long ldg, long sG, int m, int batch, const EigScratch& e,
-                             cudaStream_t s, int b0 = 0) {
-  switch (CL) {
-    case 8: return launch_hetrd_smem_t<8, DF, GS>(G, ldg, sG, m, batch, e, s, b0);
-    case 4: return launch_hetrd_smem_t<4, DF, GS>(G, ldg, sG, m, batch, e, s, b0);
-    case 2: return launch_hetrd_smem_t<2, DF, GS>(G, ldg, sG, m, batch, e, s, b0);
-    default: return launch_hetrd_smem_t<1, DF, GS>(G, ldg, sG, m, batch, e, s, b0);
-  }
-}
-
-// the one-pass reduction with rows in L2 (k_hetrd_df1): same cluster sizes as the
-// sweep kernels; 0 when its per-warp partials of p do not fit in shared memory
-constexpr int HF_THREADS = 2 * HS_THREADS;
-static int hetrd_df1_cluster(int m, int batch) {
-  if (m < 2) return 0;
-  const size_t smax = (size_t)device_attr(cudaDevAttrMaxSharedMemoryPerBlockOptin, 232448) - 2048;
-  if (hetrd_df1_smem_bytes(m, HF_THREADS) > smax) return 0;
-  const int sms = device_attr(cudaDevAttrMultiProcessorCount, 148);
-  for (int CL = 8; CL >= 2; CL >>= 1)
-    if ((long)batch * CL <= sms && m / CL >= 48) return CL;
-  return 1;
-}
-
-template <int CL>
-static int launch_hetrd_df1_t(const double2* G, long ldg, long sG, int m, int batch, const EigScratch& e,
-                              cudaStream_t s) {
-  const size_t smax = (size_t)device_attr(cudaDevAttrMaxSharedMemoryPerBlockOptin, 232448) - 2048;
-  const int use_sched = hetrd_df1_smem_bytes(m, HF_THREADS, CL, true) <= smax ? 1 : 0;
-  const size_t smem = hetrd_df1_smem_bytes(m, HF_THREADS, CL, use_sched != 0);
-  auto kern = k_hetrd_df1<CL, HF_THREADS>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-    cudaGetLastError();
-    return TSVD_ERR_CUDA;
-  }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(batch * CL);
-  cfg.blockDim = dim3(HF_THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = CL;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, kern, G, ldg, sG, m, (int)hetrd_smem_elems(m, CL), e, use_sched) != cudaSuccess) {
-    cudaGetLastError();
-    return TSVD_ERR_CUDA;
-  }
-  TSVD_LAUNCHED();
-  return TSVD_OK;
-}
-
-static int launch_hetrd_df1(int CL, const double2* G, long ldg, long sG, int m, int batch, const EigScratch& e,
-                            cudaStream_t s) {
-  switch (CL) {
-    case 8: return launch_hetrd_df1_t<8>(G, ldg, sG, m, batch, e, s);
-    case 4: return launch_hetrd_df1_t<4>(G, ldg, sG, m, batch, e, s);
-    case 2: return launch_hetrd_df1_t<2>(G, ldg, sG, m, batch, e, s);
-    default: return launch_hetrd_df1_t<1>(G, ldg, sG, m, batch, e, s);
+template <typename C, bool GS>
+static int launch_hetrd(const double2* G, long ldg, long sG, int m, int batch, const EigScratch& e,
+                        const HetrdPlan& pl, cudaStream_t s) {
+  switch (pl.CL) {
+    case 8: return launch_hetrd_t<C, 8, GS>(G, ldg, sG, m, batch, e, pl, s);
+    case 4: return launch_hetrd_t<C, 4, GS>(G, ldg, sG, m, batch, e, pl, s);
+    case 2: return launch_hetrd_t<C, 2, GS>(G, ldg, sG, m, batch, e, pl, s);
+    default: return launch_hetrd_t<C, 1, GS>(G, ldg, sG, m, batch, e, pl, s);
   }
 }
 
@@ -2514,49 +1590,16 @@ int herm_eig_topR(double2* G, long ldg, long sG, int m, int R, int batch, double
                   void* scratch, int* status, cudaStream_t s) {
   (void)status;
   if (m <= 0 || R <= 0 || batch <= 0) return TSVD_OK;
-  if (R > m || R > 128 || m > 768) return TSVD_ERR_UNSUPPORTED;  // shared memory of k_hetrd
+  if (R > m || R > 128 || m > 512) return TSVD_ERR_UNSUPPORTED;  // one or two vector entries per thread of k_hetrd
   EigScratch e = carve_eig(scratch, m, R, batch, nullptr);
-  // FP32 path (C = float2): double-float reduction (twice the threads); FP64 path: FP64
+  // FP32 path (C = float2): double-float reduction; FP64 path: FP64
   constexpr bool kDoubleFloat = std::is_same<C, float2>::value;
-  const int NTh = kDoubleFloat ? 2 * HS_THREADS : HS_THREADS;
-  const int CLs = hetrd_smem_cluster(m, batch, NTh);
-  // rows too large for shared memory: the same double-float cluster reduction on
-  // rows kept in L2 (the FP64 path keeps its FP64 L2 kernel below)
-  const int CLg = (kDoubleFloat && CLs == 0 && e.Sg) ? hetrd_smem_cluster(m, batch, NTh, true) : 0;
-  const int hv32 = (kDoubleFloat && (CLs > 0 || CLg > 0)) ? 1 : 0;  // Householder vectors stored as float2
-  if (CLs > 0) {
+  {
     TSVD_STAGE("eig_hetrd", s);
-    TSVD_TRY((launch_hetrd_smem<kDoubleFloat, false>(CLs, G, ldg, sG, m, batch, e, s)));
-  } else if (CLg > 0) {
-    // one launch over all slices: measured faster than waves sized to keep each
-    // wave's rows in L2 (the pass is bound by its instructions, not by L2 misses)
-    TSVD_STAGE("eig_hetrd", s);
-    const int CL1 = hetrd_df1_cluster(m, batch);
-    if (CL1 > 0) TSVD_TRY(launch_hetrd_df1(CL1, G, ldg, sG, m, batch, e, s));
-    else TSVD_TRY((launch_hetrd_smem<kDoubleFloat, true>(CLg, G, ldg, sG, m, batch, e, s)));
-  } else {
-    TSVD_STAGE("eig_hetrd", s);
-    const size_t smem = (2 + 16) * (size_t)m * sizeof(double2);  // v, p and 16 warps' partials
-    if (smem > 40 * 1024) {  // with the static reduction arrays
-      cudaFuncSetAttribute(k_hetrd<HETRD_CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(batch * HETRD_CLUSTER);
-    cfg.blockDim = dim3(512);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = HETRD_CLUSTER;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, k_hetrd<HETRD_CLUSTER>, G, ldg, sG, m, e) != cudaSuccess) {
-      cudaGetLastError();
-      return TSVD_ERR_CUDA;
-    }
-    TSVD_LAUNCHED();
+    const HetrdPlan pl = hetrd_plan(m, batch);
+    using T = typename std::conditional<kDoubleFloat, cdf, double2>::type;
+    if (pl.global_rows) TSVD_TRY((launch_hetrd<T, true>(G, ldg, sG, m, batch, e, pl, s)));
+    else TSVD_TRY((launch_hetrd<T, false>(G, ldg, sG, m, batch, e, pl, s)));
   }
   {
     TSVD_STAGE("eig_bisect", s);
@@ -2614,10 +1657,8 @@ int herm_eig_topR(double2* G, long ldg, long sG, int m, int R, int batch, double
     TSVD_LAUNCHED();
   }
   TSVD_STAGE("eig_backtransform", s);
-  if constexpr (kDoubleFloat) {
-    if (hv32) return launch_backtransform<C, float2>(m, R, batch, e, U, ldu, sU, s);
-  }
-  return launch_backtransform<C, double2>(m, R, batch, e, U, ldu, sU, s);
+  using VT = typename std::conditional<kDoubleFloat, float2, double2>::type;  // the Householder vectors as stored
+  return launch_backtransform<C, VT>(m, R, batch, e, U, ldu, sU, s);
 }
 template int herm_eig_topR<double2>(double2*, long, long, int, int, int, double*, double2*, long, long, void*, int*,
                                     cudaStream_t);
