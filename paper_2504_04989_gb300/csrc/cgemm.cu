@@ -16,31 +16,40 @@
 
 namespace tsvd {
 
-// BT x BT tiles on TD x TD threads (RT x RT complex each), BK deep, K split down to KMIN a piece.
+// BT x BT tiles on TD x TD threads (RT x RT complex each), BK deep, K split down to KMIN a piece until
+// TARGET tiles are in flight.
 // FP64: two multiply-adds per SM and clock, so a product is bound by how many SMs take part and
 // not by loads (a 2 x 2 register tile issues 256 clocks of FP64 per 16 of shared-memory reads):
 // 16 x 16 tiles on 64 threads spread a small product over the GPU and pad a thin one less.
 // 64 x 15 x 64 on 9 slices: 264 -> 19 us against 64 x 64 tiles on 256 threads.
-template <typename C>
+// FP32: 64 x 64, or 32 x 32 (SMALL) for products that the larger tiles would leave on few SMs or mostly
+// pad (128 x 64 x 128 on 5 slices: 19 -> 13 us, 100 x 100 x 100 on 3: 22 -> 14).
+template <typename C, bool SMALL>
 struct GemmCfg;
-template <>
-struct GemmCfg<double2> {
-  static constexpr int BT = 16, TD = 8, BK = 16, KMIN = 16;
+template <bool SMALL>
+struct GemmCfg<double2, SMALL> {
+  static constexpr int BT = 16, TD = 8, BK = 16, KMIN = 16, TARGET = 2 * 152;
   using R = double;
 };
 template <>
-struct GemmCfg<float2> {
-  static constexpr int BT = 64, TD = 16, BK = 16, KMIN = 64;
+struct GemmCfg<float2, false> {
+  static constexpr int BT = 64, TD = 16, BK = 16, KMIN = 64, TARGET = 2 * 152;
+  using R = float;
+};
+template <>
+struct GemmCfg<float2, true> {
+  static constexpr int BT = 32, TD = 8, BK = 16, KMIN = 32, TARGET = 4 * 152;
   using R = float;
 };
 
-template <typename C, bool AH, bool BH>
-__global__ void __launch_bounds__(GemmCfg<C>::TD* GemmCfg<C>::TD) k_cgemm(GemmArgs g, C* __restrict__ ws, int ksplit, int kchunk, int tiles_m,
+template <typename C, bool AH, bool BH, bool SMALL>
+__global__ void __launch_bounds__(GemmCfg<C, SMALL>::TD* GemmCfg<C, SMALL>::TD) k_cgemm(GemmArgs g, C* __restrict__ ws, int ksplit, int kchunk, int tiles_m,
                                                int herm_upper) {
-  constexpr int BK = GemmCfg<C>::BK, GBM = GemmCfg<C>::BT, GBN = GBM, TD = GemmCfg<C>::TD, NT = TD * TD;
+  using Cfg = GemmCfg<C, SMALL>;
+  constexpr int BK = Cfg::BK, GBM = Cfg::BT, GBN = GBM, TD = Cfg::TD, NT = TD * TD;
   constexpr int RT = GBM / TD;                           // rows and columns of a thread
   constexpr int NA = GBM * BK / NT, NB = GBN * BK / NT;  // staged elements per thread
-  using R = typename GemmCfg<C>::R;
+  using R = typename Cfg::R;
   // two stages; rows padded by one element so the transposed stores hit distinct banks
   __shared__ __align__(16) C As[2][BK][GBM + 1];
   __shared__ __align__(16) C Bs[2][BK][GBN + 1];
@@ -273,7 +282,7 @@ __global__ void __launch_bounds__(256, 2) k_cgemm_w(GemmArgs g, float2* __restri
 
 template <typename C>
 __global__ void k_splitk_reduce(const C* __restrict__ ws, int ksplit, GemmArgs g) {
-  using R = typename GemmCfg<C>::R;
+  using R = decltype(C().x);
   const long total = (long)g.batch * g.M * g.N;
   for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
     const int n = idx % g.N;
@@ -290,12 +299,11 @@ __global__ void k_splitk_reduce(const C* __restrict__ ws, int ksplit, GemmArgs g
 }
 
 // a split of K that fills the GPU (bounded by the scratch it needs)
-template <typename C>
+template <typename Cfg>
 static int choose_ksplit(int M, int N, int K, int batch, size_t splitk_elems) {
-  const long tiles = (long)cdiv(M, GemmCfg<C>::BT) * cdiv(N, GemmCfg<C>::BT) * batch;
-  const long target = 2 * 152;
-  int ks = (int)std::max(1L, std::min(16L, target / std::max(1L, tiles)));
-  ks = std::min(ks, std::max(1, K / GemmCfg<C>::KMIN));
+  const long tiles = (long)cdiv(M, Cfg::BT) * cdiv(N, Cfg::BT) * batch;
+  int ks = (int)std::max(1L, std::min(16L, Cfg::TARGET / std::max(1L, tiles)));
+  ks = std::min(ks, std::max(1, K / Cfg::KMIN));
   while (ks > 1 && (size_t)ks * batch * M * N > splitk_elems) --ks;
   while (ks > 1 && (long)ks * batch > 65535) --ks;
   return ks;
@@ -350,6 +358,32 @@ static int cgemm_wide(const GemmArgs& g, float2* ws, size_t splitk_elems, cudaSt
   return TSVD_OK;
 }
 
+template <typename C, bool SMALL>
+static int cgemm_tiles(const GemmArgs& g, C* ws, size_t splitk_elems, cudaStream_t s, int herm) {
+  using Cfg = GemmCfg<C, SMALL>;
+  int ks = (g.K > 0) ? choose_ksplit<Cfg>(g.M, g.N, g.K, g.batch, splitk_elems) : 1;
+  constexpr int BK = Cfg::BK, BT = Cfg::BT, NT = Cfg::TD * Cfg::TD;
+  int kchunk = (g.K + ks - 1) / ks;
+  kchunk = (kchunk + BK - 1) / BK * BK;
+  if (kchunk == 0) kchunk = BK;
+  ks = (g.K + kchunk - 1) / kchunk;
+  if (ks < 1) ks = 1;
+  const int tiles_m = cdiv(g.M, BT), tiles_n = cdiv(g.N, BT);
+  dim3 grid(tiles_m * tiles_n, 1, g.batch * ks);
+  const bool ah = (g.opA == 'H'), bh = (g.opB == 'H');
+  if (!ah && !bh) k_cgemm<C, false, false, SMALL><<<grid, NT, 0, s>>>(g, ws, ks, kchunk, tiles_m, herm);
+  else if (ah && !bh) k_cgemm<C, true, false, SMALL><<<grid, NT, 0, s>>>(g, ws, ks, kchunk, tiles_m, herm);
+  else if (!ah && bh) k_cgemm<C, false, true, SMALL><<<grid, NT, 0, s>>>(g, ws, ks, kchunk, tiles_m, herm);
+  else k_cgemm<C, true, true, SMALL><<<grid, NT, 0, s>>>(g, ws, ks, kchunk, tiles_m, herm);
+  TSVD_LAUNCHED();
+  if (ks > 1) {
+    const long total = (long)g.batch * g.M * g.N;
+    k_splitk_reduce<C><<<std::min<long>(cdiv(total, 256), 4096), 256, 0, s>>>(ws, ks, g);
+    TSVD_LAUNCHED();
+  }
+  return herm ? mirror_lower<C>(g, s) : TSVD_OK;
+}
+
 template <typename C>
 static int cgemm_impl(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t s, int herm) {
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return TSVD_OK;
@@ -371,29 +405,13 @@ static int cgemm_impl(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, c
       return herm ? mirror_lower<C>(g, s) : TSVD_OK;
     }
   }
-  int ks = (g.K > 0) ? choose_ksplit<C>(g.M, g.N, g.K, g.batch, splitk_ws ? splitk_elems : 0) : 1;
-  constexpr int BK = GemmCfg<C>::BK;
-  int kchunk = (g.K + ks - 1) / ks;
-  kchunk = (kchunk + BK - 1) / BK * BK;
-  if (kchunk == 0) kchunk = BK;
-  ks = (g.K + kchunk - 1) / kchunk;
-  if (ks < 1) ks = 1;
-  constexpr int BT = GemmCfg<C>::BT, NT = GemmCfg<C>::TD * GemmCfg<C>::TD;
-  const int tiles_m = cdiv(g.M, BT), tiles_n = cdiv(g.N, BT);
-  dim3 grid(tiles_m * tiles_n, 1, g.batch * ks);
-  const bool ah = (g.opA == 'H'), bh = (g.opB == 'H');
-  C* ws = (C*)splitk_ws;
-  if (!ah && !bh) k_cgemm<C, false, false><<<grid, NT, 0, s>>>(g, ws, ks, kchunk, tiles_m, herm);
-  else if (ah && !bh) k_cgemm<C, true, false><<<grid, NT, 0, s>>>(g, ws, ks, kchunk, tiles_m, herm);
-  else if (!ah && bh) k_cgemm<C, false, true><<<grid, NT, 0, s>>>(g, ws, ks, kchunk, tiles_m, herm);
-  else k_cgemm<C, true, true><<<grid, NT, 0, s>>>(g, ws, ks, kchunk, tiles_m, herm);
-  TSVD_LAUNCHED();
-  if (ks > 1) {
-    const long total = (long)g.batch * g.M * g.N;
-    k_splitk_reduce<C><<<std::min<long>(cdiv(total, 256), 4096), 256, 0, s>>>(ws, ks, g);
-    TSVD_LAUNCHED();
-  }
-  return herm ? mirror_lower<C>(g, s) : TSVD_OK;
+  const size_t sk = splitk_ws ? splitk_elems : 0;
+  // small tiles where the 64 x 64 ones would be mostly padding or, even with K split, leave SMs idle
+  const long tiles64 = (long)cdiv(g.M, 64) * cdiv(g.N, 64) * g.batch;
+  if (std::is_same<C, float2>::value &&
+      (g.N <= 32 || g.M <= 32 || tiles64 * std::max(1, std::min(16, g.K / 64)) < 152))
+    return cgemm_tiles<C, true>(g, (C*)splitk_ws, sk, s, herm);
+  return cgemm_tiles<C, false>(g, (C*)splitk_ws, sk, s, herm);
 }
 
 template <typename C>
