@@ -633,10 +633,14 @@ static int lane_pool(LanePool** out) {
   return TSVD_OK;
 }
 
-// work estimate of one T-SVD: Krylov products, orthonormalisation, eigen-solve
+// time estimate of one T-SVD on a lane, in microseconds: its launches (a block's three orthonormalisation
+// passes are chains of small kernels), the steps of its tridiagonalisation, and its arithmetic (Krylov
+// products, orthonormalisation, eigen-solve).  Most tensors of a batch are latency: by arithmetic alone
+// the lanes of a 24-tensor batch ended between 6.2 and 13.0 ms.
 static double rbk_cost(const RbkDims& d) {
-  const double n1 = d.n1, n2 = d.n2, m = d.m;
-  return d.h * (8.0 * n1 * n2 * 2.0 * m + 16.0 * n1 * m * m + (16.0 / 3.0) * m * m * m) + 2e6;
+  const double n1 = d.n1, n2 = d.n2, m = d.m, blocks = d.alg1 ? 1 : d.q + 1;
+  const double flops = d.h * (8.0 * n1 * n2 * 2.0 * m + 16.0 * n1 * m * m + (16.0 / 3.0) * m * m * m);
+  return 25.0 * (13.0 * blocks + 20.0) + 5.0 * m + flops / 5.0e6;
 }
 
 struct BatchPlan {
