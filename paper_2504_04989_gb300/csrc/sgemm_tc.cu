@@ -83,16 +83,6 @@ __global__ void __launch_bounds__(256) k_split_pack(const float2* __restrict__ S
   }
 }
 
-__device__ __forceinline__ uint64_t smem_desc_sw128_k(uint32_t addr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((addr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)1 << 16;
-  d |= (uint64_t)(1024 >> 4) << 32;  // 8 rows of 128 bytes
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;  // swizzle 128B
-  return d;
-}
-
 __global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constant__ CUtensorMap tmAh,
                                                             const __grid_constant__ CUtensorMap tmAl,
                                                             const __grid_constant__ CUtensorMap tmBh,
@@ -159,8 +149,8 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constan
       if (!mbar_wait(full0 + 8 * s, (kb / SG_STAGES) & 1)) break;
       asm volatile("tcgen05.fence::after_thread_sync;");
       const uint32_t sm = smem_u32(base + s * SG_STAGE_BYTES);
-      const uint64_t ah = smem_desc_sw128_k(sm), bh = smem_desc_sw128_k(sm + SG_TILE);
-      const uint64_t al = smem_desc_sw128_k(sm + 2 * SG_TILE), bl = smem_desc_sw128_k(sm + 3 * SG_TILE);
+      const uint64_t ah = smem_desc_sw128(sm), bh = smem_desc_sw128(sm + SG_TILE);
+      const uint64_t al = smem_desc_sw128(sm + 2 * SG_TILE), bl = smem_desc_sw128(sm + 3 * SG_TILE);
       const uint32_t d = tmem + (uint32_t)(a * SG_BN);
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk) {  // 32 bytes of K per instruction

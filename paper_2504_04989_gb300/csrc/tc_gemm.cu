@@ -13,9 +13,8 @@
 // tcgen05.ld and store it (thread = row, 16 columns at a time as four 16-byte
 // accesses where aligned; C = alpha A B^T + beta C, the old values loaded
 // before any store).  Every wait is bounded: on a timeout the kernel records
-// an error flag instead of hanging.  Options: `upper` skips the tiles wholly
-// below the diagonal of a symmetric product (B = A); the split-TF32 epilogue
-// can also write hi / lo copies of C and of C^T for a following product.
+// an error flag instead of hanging.  The split-TF32 epilogue can also write
+// hi / lo copies of C and of C^T for a following product.
 //
 // A third mode keeps FP32 accuracy on the TF32 units ("split TF32"): each
 // operand is split as x = hi + lo with hi = x rounded to TF32 and lo = x - hi
@@ -56,18 +55,6 @@ __device__ __forceinline__ float tf32_hi(float x) {
   return __uint_as_float(r);
 }
 
-// shared-memory matrix descriptor: K-major operand tile, 128-byte swizzle,
-// 8-row groups 1024 bytes apart (SBO), descriptor version 1
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((addr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)1 << 16;            // leading byte offset (unused for this layout)
-  d |= (uint64_t)(1024 >> 4) << 32;  // stride byte offset
-  d |= (uint64_t)1 << 46;            // version
-  d |= (uint64_t)2 << 61;            // swizzle 128B
-  return d;
-}
-
 // instruction descriptor: D FP32, A/B TF32 (kind::tf32) or BF16 (kind::f16),
 // both K-major, M = 128, N = BN
 template <bool BF16, int BN>
@@ -83,7 +70,7 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUte
                                                     const __grid_constant__ CUtensorMap tmA2,
                                                     const __grid_constant__ CUtensorMap tmB2, float* __restrict__ C,
                                                     long ldc, long sC, int M, int N, int nk, int* __restrict__ err,
-                                                    float alpha, float beta, int upper, TcSplitOut o2) {
+                                                    float alpha, float beta, TcSplitOut o2) {
   constexpr bool BF16 = MODE == 1, SPLIT = MODE == 2;
   constexpr int STAGES = tc_stages<MODE, BN>(), SB = tc_stage_bytes<MODE, BN>();
   static_assert(tc_smem<MODE, BN>() <= 227 * 1024, "the stages must fit the opt-in shared memory of a CTA");
@@ -99,8 +86,6 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUte
   __shared__ int s_fail;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n0 = blockIdx.x * BN, m0 = blockIdx.y * TC_BM, bz = blockIdx.z;
-  // upper: a symmetric product (B = A) needs only the tiles not wholly below the diagonal
-  if (upper && n0 + BN <= m0) return;
   const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STAGES), done = smem_u32(bars + 2 * STAGES);
   constexpr int KE = BF16 ? 64 : 32;  // elements per 128 bytes of K
 
@@ -309,7 +294,7 @@ bool tc_gemm_supported(const void* A, long lda, long sA, const void* B, long ldb
 template <int MODE, int BN>
 static int tc_launch(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& ta2, const CUtensorMap& tb2,
                      float* C, long ldc, long sC, int M, int N, int nk, int batch, int* err, cudaStream_t s,
-                     float alpha = 1.0f, float beta = 0.0f, int upper = 0, const TcSplitOut& o2 = TcSplitOut()) {
+                     float alpha = 1.0f, float beta = 0.0f, const TcSplitOut& o2 = TcSplitOut()) {
   dim3 grid(cdiv(N, BN), cdiv(M, TC_BM), batch);
   if (cudaFuncSetAttribute(k_tc_gemm<MODE, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem<MODE, BN>()) !=
       cudaSuccess) {
@@ -317,16 +302,15 @@ static int tc_launch(const CUtensorMap& ta, const CUtensorMap& tb, const CUtenso
     return TSVD_ERR_CUDA;
   }
   k_tc_gemm<MODE, BN><<<grid, 128, tc_smem<MODE, BN>(), s>>>(ta, tb, ta2, tb2, C, ldc, sC, M, N, nk, err, alpha,
-                                                               beta, upper, o2);
+                                                               beta, o2);
   TSVD_LAUNCHED();
   return TSVD_OK;
 }
 // tile width: 256 columns when N > 128 (one tile row covers the whole of N <= 256)
 static int tc_bn(int N) { return N > 128 ? 256 : 128; }
-int tc_gemm_tile_n(int N, bool bf16) { (void)bf16; return tc_bn(N); }
 
 int tc_gemm(const void* A, long lda, long sA, int M, const void* B, long ldb, long sB, int N, int K, float* C, long ldc,
-            long sC, int batch, bool bf16, int* err, cudaStream_t s, bool upper) {
+            long sC, int batch, bool bf16, int* err, cudaStream_t s) {
   if (M <= 0 || N <= 0 || batch <= 0) return TSVD_OK;
   if (!tc_gemm_supported(A, lda, sA, B, ldb, sB, batch, bf16)) return TSVD_ERR_UNSUPPORTED;
   CUtensorMap ta, tb;
@@ -335,12 +319,11 @@ int tc_gemm(const void* A, long lda, long sA, int M, const void* B, long ldb, lo
   TSVD_TRY(make_map(&tb, B, N, K, ldb, sB, batch, bf16, bn));
   const int kelem = bf16 ? 64 : 32;
   const int nk = (K + kelem - 1) / kelem;
-  const int up = upper ? 1 : 0;
   if (bf16)
-    return bn == 256 ? tc_launch<1, 256>(ta, tb, ta, tb, C, ldc, sC, M, N, nk, batch, err, s, 1.f, 0.f, up)
-                     : tc_launch<1, 128>(ta, tb, ta, tb, C, ldc, sC, M, N, nk, batch, err, s, 1.f, 0.f, up);
-  return bn == 256 ? tc_launch<0, 256>(ta, tb, ta, tb, C, ldc, sC, M, N, nk, batch, err, s, 1.f, 0.f, up)
-                   : tc_launch<0, 128>(ta, tb, ta, tb, C, ldc, sC, M, N, nk, batch, err, s, 1.f, 0.f, up);
+    return bn == 256 ? tc_launch<1, 256>(ta, tb, ta, tb, C, ldc, sC, M, N, nk, batch, err, s)
+                     : tc_launch<1, 128>(ta, tb, ta, tb, C, ldc, sC, M, N, nk, batch, err, s);
+  return bn == 256 ? tc_launch<0, 256>(ta, tb, ta, tb, C, ldc, sC, M, N, nk, batch, err, s)
+                   : tc_launch<0, 128>(ta, tb, ta, tb, C, ldc, sC, M, N, nk, batch, err, s);
 }
 
 int tc_gemm_split(const float* Ahi, const float* Alo, long lda, long sA, int M, const float* Bhi, const float* Blo,
@@ -357,7 +340,7 @@ int tc_gemm_split(const float* Ahi, const float* Alo, long lda, long sA, int M, 
   TSVD_TRY(make_map(&tb, Bhi, N, K, ldb, sB, batch, false));
   TSVD_TRY(make_map(&ta2, Alo, M, K, lda, sA, batch, false));
   TSVD_TRY(make_map(&tb2, Blo, N, K, ldb, sB, batch, false));
-  return tc_launch<2, 128>(ta, tb, ta2, tb2, C, ldc, sC, M, N, (K + 31) / 32, batch, err, s, alpha, beta, 0,
+  return tc_launch<2, 128>(ta, tb, ta2, tb2, C, ldc, sC, M, N, (K + 31) / 32, batch, err, s, alpha, beta,
                            out2 ? *out2 : TcSplitOut());
 }
 
