@@ -160,16 +160,6 @@ __global__ void __launch_bounds__(256) k_dig_pack(const double2* __restrict__ S,
 // ---------------------------------------------------------------------------
 // the product
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t addr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((addr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)1 << 16;
-  d |= (uint64_t)(512 >> 4) << 32;  // 8 rows of 64 bytes
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)4 << 61;  // swizzle 64B
-  return d;
-}
-
 // (hi 2^32 + lo) 2^e rounded to nearest, in integer arithmetic (FP64 conversions run on the FP64 pipe)
 __device__ __forceinline__ double fixed_to_double(long long hi, long long lo, int e) {
   __int128 v = ((__int128)hi << 32) + lo;

@@ -58,6 +58,17 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
   return d;
 }
 
+// the same of 64-byte rows, 64-byte swizzle, 8-row groups of 512 bytes
+__device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t addr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((addr & 0x3FFFFu) >> 4);
+  d |= (uint64_t)1 << 16;
+  d |= (uint64_t)(512 >> 4) << 32;  // 8 rows of 64 bytes
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)4 << 61;  // swizzle 64B
+  return d;
+}
+
 template <bool BF16>
 __device__ __forceinline__ void mma_issue(uint32_t tmem, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t acc) {
   if (BF16) {

@@ -3,7 +3,7 @@
 // A and B K-major (K contiguous), TF32 (FP32 storage) or BF16 operands, FP32
 // accumulation in tensor memory.
 //
-// One CTA computes a 128 x BN tile, BN = 128, or (TF32 and BF16) 256 when
+// One CTA computes a 128 x BN tile, BN = 128, or 256 when
 // N > 128 (a product with N in (128, 256], as the Krylov products' 2b real
 // columns, then reads each row panel of A once).  Operand tiles of 128 (A) and BN (B) rows x 128
 // bytes of K are staged by TMA (128-byte swizzle) through a ring of shared
@@ -20,7 +20,8 @@
 // operand is split as x = hi + lo with hi = x rounded to TF32 and lo = x - hi
 // (exact in FP32), and the tile product is hi*hi + hi*lo + lo*hi accumulated
 // in the same TMEM tile (about 22 significant bits per product; lo*lo, below
-// FP32 rounding, is dropped).  Four operand tiles per stage, three stages.
+// FP32 rounding, is dropped).  Four operand tiles per stage: three stages of 128
+// bytes of K at 128 columns, four of 64 bytes at 256 columns.
 //
 // Complex products use it without moving the big operand: an interleaved
 // complex matrix X (rows x cols) is the real matrix [Re Im Re Im ...] of
@@ -37,14 +38,19 @@
 namespace tsvd {
 
 constexpr int TC_BM = 128;
-constexpr int TC_A_BYTES = TC_BM * 128;  // 128 rows x 128 bytes of K
 // MODE 0: TF32, 1: BF16, 2: split TF32; BN: 128 or 256 columns per tile
-template <int BN>
-constexpr int tc_b_bytes() { return BN * 128; }
 template <int MODE, int BN>
-constexpr int tc_stage_bytes() { return (MODE == 2 ? 2 : 1) * (TC_A_BYTES + tc_b_bytes<BN>()); }  // A, B[, A lo, B lo]
+constexpr int tc_row() { return MODE == 2 && BN == 256 ? 64 : 128; }  // bytes of K per stage
 template <int MODE, int BN>
-constexpr int tc_stages() { return MODE == 2 ? 3 : 4; }
+constexpr int tc_a_bytes() { return TC_BM * tc_row<MODE, BN>(); }
+template <int MODE, int BN>
+constexpr int tc_b_bytes() { return BN * tc_row<MODE, BN>(); }
+template <int MODE, int BN>
+constexpr int tc_stage_bytes() {  // A, B[, A lo, B lo]
+  return (MODE == 2 ? 2 : 1) * (tc_a_bytes<MODE, BN>() + tc_b_bytes<MODE, BN>());
+}
+template <int MODE, int BN>
+constexpr int tc_stages() { return MODE == 2 && BN == 128 ? 3 : 4; }
 template <int MODE, int BN>
 constexpr int tc_smem() { return tc_stages<MODE, BN>() * tc_stage_bytes<MODE, BN>() + 1024 + 256; }
 
@@ -74,12 +80,13 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUte
   constexpr bool BF16 = MODE == 1, SPLIT = MODE == 2;
   constexpr int STAGES = tc_stages<MODE, BN>(), SB = tc_stage_bytes<MODE, BN>();
   static_assert(tc_smem<MODE, BN>() <= 227 * 1024, "the stages must fit the opt-in shared memory of a CTA");
-  constexpr int BB = tc_b_bytes<BN>();
+  constexpr int AB = tc_a_bytes<MODE, BN>(), BB = tc_b_bytes<MODE, BN>(), ROW = tc_row<MODE, BN>();
+  auto desc = [](uint32_t addr) { return ROW == 64 ? smem_desc_sw64(addr) : smem_desc_sw128(addr); };
   extern __shared__ unsigned char tc_raw[];
   unsigned char* base = (unsigned char*)(((uintptr_t)tc_raw + 1023) & ~(uintptr_t)1023);
   // o: A, B, A lo, B lo (every offset a multiple of 1024 bytes)
   auto tile = [&](int s, int o) {
-    return base + s * SB + (o & 1) * TC_A_BYTES + (o >> 1) * (TC_A_BYTES + BB);
+    return base + s * SB + (o & 1) * AB + (o >> 1) * (AB + BB);
   };
   uint64_t* bars = (uint64_t*)(base + STAGES * SB);  // full[S], empty[S], done
   uint32_t* tslot = (uint32_t*)(bars + 2 * STAGES + 1);
@@ -87,7 +94,7 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUte
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n0 = blockIdx.x * BN, m0 = blockIdx.y * TC_BM, bz = blockIdx.z;
   const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STAGES), done = smem_u32(bars + 2 * STAGES);
-  constexpr int KE = BF16 ? 64 : 32;  // elements per 128 bytes of K
+  constexpr int KE = ROW / (BF16 ? 2 : 4);  // elements of K per stage
 
   if (tid == 0) {
     s_fail = 0;
@@ -134,14 +141,14 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUte
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;");
-      const uint64_t ad = smem_desc_sw128(smem_u32(tile(s, 0)));
-      const uint64_t bd = smem_desc_sw128(smem_u32(tile(s, 1)));
+      const uint64_t ad = desc(smem_u32(tile(s, 0)));
+      const uint64_t bd = desc(smem_u32(tile(s, 1)));
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {  // 32 bytes of K per instruction: advance the start address by 2 x 16 B
+      for (int kk = 0; kk < ROW / 32; ++kk) {  // 32 bytes of K per instruction: advance the start address by 2 x 16 B
         mma_issue<BF16>(tmem, ad + 2 * kk, bd + 2 * kk, idesc, (kb | kk) != 0);
         if (SPLIT) {
-          const uint64_t ad2 = smem_desc_sw128(smem_u32(tile(s, 2)));
-          const uint64_t bd2 = smem_desc_sw128(smem_u32(tile(s, 3)));
+          const uint64_t ad2 = desc(smem_u32(tile(s, 2)));
+          const uint64_t bd2 = desc(smem_u32(tile(s, 3)));
           mma_issue<BF16>(tmem, ad + 2 * kk, bd2 + 2 * kk, idesc, 1);
           mma_issue<BF16>(tmem, ad2 + 2 * kk, bd + 2 * kk, idesc, 1);
         }
@@ -266,18 +273,19 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUte
 // host side
 // ---------------------------------------------------------------------------
 // rows x K (elements) per batch, row stride ld, batch stride sb (elements); boxes of
-// box_rows rows x 128 bytes of K
+// box_rows rows x row bytes of K
 static int make_map(CUtensorMap* tm, const void* ptr, int rows, int K, long ld, long sb, int batch, bool bf16,
-                    int box_rows = TC_BM) {
+                    int box_rows = TC_BM, int row = 128) {
   auto enc = get_encode();
   if (!enc) return TSVD_ERR_CUDA;
   const size_t es = bf16 ? 2 : 4;
   cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)rows, (cuuint64_t)batch};
   cuuint64_t strides[2] = {(cuuint64_t)(ld * es), (cuuint64_t)(sb * es)};
-  cuuint32_t box[3] = {(cuuint32_t)(128 / es), (cuuint32_t)box_rows, 1};
+  cuuint32_t box[3] = {(cuuint32_t)(row / es), (cuuint32_t)box_rows, 1};
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = enc(tm, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, (void*)ptr, dims,
-                   strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                   strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                   row == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? TSVD_OK : TSVD_ERR_UNSUPPORTED;
 }
@@ -333,15 +341,21 @@ int tc_gemm_split(const float* Ahi, const float* Alo, long lda, long sA, int M, 
   if (!tc_gemm_supported(Ahi, lda, sA, Bhi, ldb, sB, batch, false) ||
       !tc_gemm_supported(Alo, lda, sA, Blo, ldb, sB, batch, false))
     return TSVD_ERR_UNSUPPORTED;
-  // split TF32 keeps 128-column tiles: with four operand tiles per stage a 256-column tile
-  // leaves room for two stages only, which measured slower
+  // columns per tile: shared memory feeds the products (every instruction reads its 128 rows of A and
+  // BN of B, 160 KB per 32 terms at 128 columns with the filling, 240 KB at 256, against 128 bytes per
+  // clock), so a term of K costs a tile of 256 about 1.5 times one of 128.  The 48 products of a T-SVD
+  // of 2048 x 2048 x 128 took 12.2 ms with 128 columns throughout, 11.1 so.
+  const long rows = (long)cdiv(M, TC_BM) * batch;
+  const bool wide = 3 * cdiv(rows * cdiv(N, 256), 152) <= 2 * cdiv(rows * cdiv(N, 128), 152);
+  const int bn = wide ? 256 : 128, row = wide ? 64 : 128;
   CUtensorMap ta, tb, ta2, tb2;
-  TSVD_TRY(make_map(&ta, Ahi, M, K, lda, sA, batch, false));
-  TSVD_TRY(make_map(&tb, Bhi, N, K, ldb, sB, batch, false));
-  TSVD_TRY(make_map(&ta2, Alo, M, K, lda, sA, batch, false));
-  TSVD_TRY(make_map(&tb2, Blo, N, K, ldb, sB, batch, false));
-  return tc_launch<2, 128>(ta, tb, ta2, tb2, C, ldc, sC, M, N, (K + 31) / 32, batch, err, s, alpha, beta,
-                           out2 ? *out2 : TcSplitOut());
+  TSVD_TRY(make_map(&ta, Ahi, M, K, lda, sA, batch, false, TC_BM, row));
+  TSVD_TRY(make_map(&tb, Bhi, N, K, ldb, sB, batch, false, bn, row));
+  TSVD_TRY(make_map(&ta2, Alo, M, K, lda, sA, batch, false, TC_BM, row));
+  TSVD_TRY(make_map(&tb2, Blo, N, K, ldb, sB, batch, false, bn, row));
+  const TcSplitOut o2 = out2 ? *out2 : TcSplitOut();
+  return wide ? tc_launch<2, 256>(ta, tb, ta2, tb2, C, ldc, sC, M, N, (K + 15) / 16, batch, err, s, alpha, beta, o2)
+              : tc_launch<2, 128>(ta, tb, ta2, tb2, C, ldc, sC, M, N, (K + 31) / 32, batch, err, s, alpha, beta, o2);
 }
 
 // ---------------------------------------------------------------------------
