@@ -24,8 +24,8 @@
 // Bound: the tensor cores, 34 BF16 products per multiply-add (56 TFLOP/s of FP64
 // work at the measured BF16 rate, against 1.1 on the FP64 units), and for thin
 // products the two passes over the operands (largest exponents, digits).  1024 x 1024
-// x 1024 on 5 slices: 36.7 -> 1.26 ms, 512 x 60 x 512 on 33: 4.09 -> 0.29 ms, of which
-// the product itself about 0.1.
+// x 1024 on 5 slices: 36.7 -> 1.26 ms, 512 x 60 x 512 on 33: 4.09 -> 0.28 ms, of which
+// the product itself about 0.09.
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -46,9 +46,11 @@ constexpr int DG_CHUNK = 6;    // stages between two readings of the accumulator
 constexpr int DG_A_BYTES = DG_D * DG_BM * DG_KB * 2, DG_B_BYTES = DG_D * DG_BN * DG_KB * 2;
 constexpr int DG_STAGE_BYTES = DG_A_BYTES + DG_B_BYTES;
 constexpr int DG_SMEM = DG_STAGES * DG_STAGE_BYTES + 1024 + 256;
-constexpr int DG_DRAIN = 256;  // threads that read the accumulators (8 warps), then one TMA and one MMA warp
+// threads that read the accumulators (16 warps: 5.7 ms for the products of a 512 x 512 x 64 T-SVD, 6.3 with 8,
+// whose sums took all registers), then one TMA and one MMA warp
+constexpr int DG_DRAIN = 512;
 constexpr int DG_THREADS = DG_DRAIN + 64;
-constexpr int DG_OUT = DG_BN / 2;  // real columns per draining thread
+constexpr int DG_OUT = DG_BN / 4;  // real columns per draining thread
 static_assert(DG_SMEM <= 227 * 1024, "two stages must fit a CTA's shared memory");
 static_assert(DG_L * DG_BN == 512, "the accumulators take the whole of TMEM");
 static_assert(5 * (1 << 14) * DG_CHUNK * DG_KB < (1 << 24), "sums of the five leading levels stay exact");
@@ -186,11 +188,22 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dgemm_tc(const __grid_constan
                                                             const __grid_constant__ DotSrc<double2> src,
                                                             const int* __restrict__ EA, const int* __restrict__ EB,
                                                             double2* __restrict__ C, long ldc, long sC, int M, int N,
-                                                            int nk, double alpha, int beta, int upper) {
+                                                            int nk, int batch, double alpha, int beta, int upper) {
   extern __shared__ unsigned char dg_raw[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int n0 = blockIdx.x * DG_BN, m0 = blockIdx.y * DG_BM, bz = blockIdx.z;
-  if (upper && n0 / 2 + DG_BN / 2 <= m0) return;  // Hermitian product: mirrored afterwards
+  const int tn = (2 * N + DG_BN - 1) / DG_BN, tm = (M + DG_BM - 1) / DG_BM;
+  const int tiles = tn * tm * batch;  // at least one element each: within an int
+  struct Tile {
+    int n0, m0, bz;
+    bool skip;
+  };
+  auto tile = [&](int t) {  // columns fastest: neighbouring CTAs share rows of A
+    const int r = t / tn;
+    Tile w{(t % tn) * DG_BN, (r % tm) * DG_BM, r / tm, false};
+    w.skip = upper && w.n0 / 2 + DG_BN / 2 <= w.m0;  // Hermitian product: mirrored afterwards
+    return w;
+  };
+  if (upper && (int)gridDim.x == tiles && tile(blockIdx.x).skip) return;
   unsigned char* base = (unsigned char*)(((uintptr_t)dg_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* bars = (uint64_t*)(base + DG_STAGES * DG_STAGE_BYTES);  // full[S], empty[S], tfull, tempty
   uint32_t* tslot = (uint32_t*)(bars + 2 * DG_STAGES + 2);
@@ -215,130 +228,146 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dgemm_tc(const __grid_constan
   const uint32_t tmem = *tslot;
   const int chunks = (nk + DG_CHUNK - 1) / DG_CHUNK;
 
+  // stages and readings are counted through all tiles of the CTA, so loads and products of the next
+  // tile run under the rounding and writing of this one
   if (tid == DG_DRAIN) {  // TMA producer
-    int issued = 0;
+    Ring<DG_STAGES> r;
+    long filled = 0;
     bool ok = true;
-    for (int kb = 0; kb < nk; ++kb) {
-      const int s = kb % DG_STAGES, round = kb / DG_STAGES;
-      if (round > 0 && !mbar_wait(empty0 + 8 * s, (round - 1) & 1)) {
-        ok = false;
-        break;
+    for (int t = blockIdx.x; ok && t < tiles; t += gridDim.x) {
+      const Tile w = tile(t);
+      if (w.skip) continue;
+      for (int kb = 0; kb < nk; ++kb, ++filled, r.next()) {
+        const int s = r.s;
+        if (!mbar_wait(empty0 + 8 * s, r.ph ^ 1)) {
+          ok = false;
+          break;
+        }
+        const uint32_t dst = smem_u32(base + s * DG_STAGE_BYTES);
+        mbar_expect_tx(full0 + 8 * s, DG_STAGE_BYTES);
+        tma_load_3d(dst, &tmA, kb * DG_KB, w.m0, w.bz * DG_D, full0 + 8 * s);
+        tma_load_3d(dst + DG_A_BYTES, &tmB, kb * DG_KB, w.n0, w.bz * DG_D, full0 + 8 * s);
       }
-      const uint32_t dst = smem_u32(base + s * DG_STAGE_BYTES);
-      mbar_expect_tx(full0 + 8 * s, DG_STAGE_BYTES);
-      tma_load_3d(dst, &tmA, kb * DG_KB, m0, bz * DG_D, full0 + 8 * s);
-      tma_load_3d(dst + DG_A_BYTES, &tmB, kb * DG_KB, n0, bz * DG_D, full0 + 8 * s);
-      issued = kb + 1;
     }
-    if (!ok) {  // copies in flight land before the CTA gives its shared memory back
-      for (int kb = (issued > DG_STAGES ? issued - DG_STAGES : 0); kb < issued; ++kb)
-        mbar_wait(full0 + 8 * (kb % DG_STAGES), (kb / DG_STAGES) & 1);
-    }
+    ring_drain(r, filled, full0);
   } else if (tid == DG_DRAIN + 32) {  // MMA issuer
     const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(DG_BM >> 4) << 24);  // FP32 += BF16 BF16^T
+    Ring<DG_STAGES> r;
+    Ring<1> ra;
     bool ok = true;
-    for (int c = 0; ok && c < chunks; ++c) {
-      if (c > 0 && !mbar_wait(tempty, (c - 1) & 1)) break;
-      asm volatile("tcgen05.fence::after_thread_sync;");
-      const int k1 = min(nk, (c + 1) * DG_CHUNK);
-      for (int kb = c * DG_CHUNK; kb < k1; ++kb) {
-        const int s = kb % DG_STAGES;
-        if (!mbar_wait(full0 + 8 * s, (kb / DG_STAGES) & 1)) {
+    for (int t = blockIdx.x; ok && t < tiles; t += gridDim.x) {
+      if (tile(t).skip) continue;
+      for (int c = 0; ok && c < chunks; ++c, ra.next()) {
+        if (!mbar_wait(tempty, ra.ph ^ 1)) {
           ok = false;
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;");
-        const uint32_t sa = smem_u32(base + s * DG_STAGE_BYTES), sb = sa + DG_A_BYTES;
+        const int k1 = min(nk, (c + 1) * DG_CHUNK);
+        for (int kb = c * DG_CHUNK; kb < k1; ++kb, r.next()) {
+          const int s = r.s;
+          if (!mbar_wait(full0 + 8 * s, r.ph)) {
+            ok = false;
+            break;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;");
+          const uint32_t sa = smem_u32(base + s * DG_STAGE_BYTES), sb = sa + DG_A_BYTES;
 #pragma unroll
-        for (int kk = 0; kk < DG_KB / 16; ++kk) {
-          const bool first = kb == c * DG_CHUNK && kk == 0;
-          // digit i of A with the digits j of B, as many as 256 columns per instruction; level i + j
-          auto mul = [&](int i, int j, int nj, bool acc) {
-            mma_issue<true>(tmem + (uint32_t)((i + j) * DG_BN),
-                            smem_desc_sw64(sa + i * (DG_BM * DG_KB * 2)) + 2 * kk,
-                            smem_desc_sw64(sb + j * (DG_BN * DG_KB * 2)) + 2 * kk,
-                            idesc0 | ((uint32_t)(nj * DG_BN >> 3) << 17), acc ? 1u : 0u);
-          };
-          mul(0, 0, 4, !first);
-          mul(0, 4, 3, !first);
-          mul(1, 0, 4, true);
-          mul(1, 4, 2, true);
-          mul(1, 6, 1, !first);  // level 7 begins here
-          mul(2, 0, 4, true);
-          mul(2, 4, 2, true);
-          mul(3, 0, 4, true);
-          mul(3, 4, 1, true);
-          mul(4, 0, 4, true);
-          mul(5, 0, 3, true);
-          mul(6, 0, 2, true);
+          for (int kk = 0; kk < DG_KB / 16; ++kk) {
+            const bool first = kb == c * DG_CHUNK && kk == 0;
+            // digit i of A with the digits j of B, as many as 256 columns per instruction; level i + j
+            auto mul = [&](int i, int j, int nj, bool acc) {
+              mma_issue<true>(tmem + (uint32_t)((i + j) * DG_BN),
+                              smem_desc_sw64(sa + i * (DG_BM * DG_KB * 2)) + 2 * kk,
+                              smem_desc_sw64(sb + j * (DG_BN * DG_KB * 2)) + 2 * kk,
+                              idesc0 | ((uint32_t)(nj * DG_BN >> 3) << 17), acc ? 1u : 0u);
+            };
+            mul(0, 0, 4, !first);
+            mul(0, 4, 3, !first);
+            mul(1, 0, 4, true);
+            mul(1, 4, 2, true);
+            mul(1, 6, 1, !first);  // level 7 begins here
+            mul(2, 0, 4, true);
+            mul(2, 4, 2, true);
+            mul(3, 0, 4, true);
+            mul(3, 4, 1, true);
+            mul(4, 0, 4, true);
+            mul(5, 0, 3, true);
+            mul(6, 0, 2, true);
+          }
+          mma_commit(empty0 + 8 * s);
         }
-        mma_commit(empty0 + 8 * s);
+        if (ok) mma_commit(tfull);
       }
-      if (ok) mma_commit(tfull);
     }
   } else if (warp < DG_DRAIN / 32) {
-    const int row = m0 + (warp & 3) * 32 + lane;
     const int col0 = (warp >> 2) * DG_OUT;
     const uint32_t tw = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)col0;
-    long long hi[DG_OUT], lo[DG_OUT];
-#pragma unroll
-    for (int q = 0; q < DG_OUT; ++q) hi[q] = lo[q] = 0;
+    Ring<1> ra;
     bool ok = true;
-    for (int c = 0; c < chunks; ++c) {
-      ok = mbar_wait(tfull, c & 1);
-      ok = __all_sync(0xffffffffu, ok);
-      if (!ok) break;
-      asm volatile("tcgen05.fence::after_thread_sync;");
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+      if (tile(t).skip) continue;
+      long long hi[DG_OUT], lo[DG_OUT];
 #pragma unroll
-      for (int q0 = 0; q0 < DG_OUT; q0 += 4) {
-        uint32_t r[DG_L][4];
+      for (int q = 0; q < DG_OUT; ++q) hi[q] = lo[q] = 0;
+      for (int c = 0; ok && c < chunks; ++c, ra.next()) {
+        ok = mbar_wait(tfull, ra.ph);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;");
 #pragma unroll
-        for (int l = 0; l < DG_L; ++l)
-          asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
-                       : "=r"(r[l][0]), "=r"(r[l][1]), "=r"(r[l][2]), "=r"(r[l][3])
-                       : "r"(tw + (uint32_t)(l * DG_BN + q0)));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        for (int q0 = 0; q0 < DG_OUT; q0 += 4) {
+          uint32_t r[DG_L][4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          int v[DG_L];
+          for (int l = 0; l < DG_L; ++l)
+            asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(r[l][0]), "=r"(r[l][1]), "=r"(r[l][2]), "=r"(r[l][3])
+                         : "r"(tw + (uint32_t)(l * DG_BN + q0)));
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-          for (int l = 0; l < DG_L; ++l) v[l] = __float2int_rn(__uint_as_float(r[l][u]));
-          long long h = hi[q0 + u], w = lo[q0 + u];
-          h += (long long)v[0] * (1 << 24);
-          h += (long long)v[1] * (1 << 16);
-          h += (long long)v[2] * (1 << 8);
-          h += (long long)v[3];
-          w += (long long)v[4] * (1 << 24);
-          w += (long long)v[5] * (1 << 16);
-          w += (long long)v[6] * (1 << 8);
-          w += (long long)v[7];
-          hi[q0 + u] = h;
-          lo[q0 + u] = w;
-        }
-      }
-      asm volatile("tcgen05.fence::before_thread_sync;");
-      mbar_arrive(tempty);
-    }
-    if (row < M) {
-      const int ea = EA[(long)bz * M + row];
-      double2* crow = C + (long)bz * sC + (long)row * ldc;
+          for (int u = 0; u < 4; ++u) {
+            int v[DG_L];
 #pragma unroll
-      for (int q = 0; q < DG_OUT; q += 2) {
-        const int col = (n0 + col0 + q) >> 1;
-        if (col < N) {
-          const int eb = EB[(long)bz * N + col];
-          double2 v;
-          if (ok && ea < 0x7ff && eb < 0x7ff) {
-            const int e = ea + eb + 40 - 2 * 1077;  // the levels carry 256^5 = 2^40
-            v = make_double2(fixed_to_double(hi[q], lo[q], e), fixed_to_double(hi[q + 1], lo[q + 1], e));
-          } else if (ok && src.A) {  // a row or column holding an infinity or NaN
-            v = direct_dot(src, bz, row, col);
-          } else {  // (or its operand overwritten in place, or a pipeline that gave up)
-            v = make_double2(__longlong_as_double(0x7ff8000000000000ll), __longlong_as_double(0x7ff8000000000000ll));
+            for (int l = 0; l < DG_L; ++l) v[l] = __float2int_rn(__uint_as_float(r[l][u]));
+            long long h = hi[q0 + u], lw = lo[q0 + u];
+            h += (long long)v[0] * (1 << 24);
+            h += (long long)v[1] * (1 << 16);
+            h += (long long)v[2] * (1 << 8);
+            h += (long long)v[3];
+            lw += (long long)v[4] * (1 << 24);
+            lw += (long long)v[5] * (1 << 16);
+            lw += (long long)v[6] * (1 << 8);
+            lw += (long long)v[7];
+            hi[q0 + u] = h;
+            lo[q0 + u] = lw;
           }
-          if (alpha != 1.0) v = cscale(v, alpha);
-          if (beta) v = cadd(v, crow[col]);
-          crow[col] = v;
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;");
+        mbar_arrive(tempty);
+      }
+      const Tile w = tile(t);
+      const int row = w.m0 + (warp & 3) * 32 + lane;
+      if (row < M) {
+        const int ea = EA[(long)w.bz * M + row];
+        double2* crow = C + (long)w.bz * sC + (long)row * ldc;
+#pragma unroll
+        for (int q = 0; q < DG_OUT; q += 2) {
+          const int col = (w.n0 + col0 + q) >> 1;
+          if (col < N) {
+            const int eb = EB[(long)w.bz * N + col];
+            double2 v;
+            if (ok && ea < 0x7ff && eb < 0x7ff) {
+              const int e = ea + eb + 40 - 2 * 1077;  // the levels carry 256^5 = 2^40
+              v = make_double2(fixed_to_double(hi[q], lo[q], e), fixed_to_double(hi[q + 1], lo[q + 1], e));
+            } else if (ok && src.A) {  // a row or column holding an infinity or NaN
+              v = direct_dot(src, w.bz, row, col);
+            } else {  // (or its operand overwritten in place, or a pipeline that gave up)
+              v = make_double2(__longlong_as_double(0x7ff8000000000000ll), __longlong_as_double(0x7ff8000000000000ll));
+            }
+            if (alpha != 1.0) v = cscale(v, alpha);
+            if (beta) v = cadd(v, crow[col]);
+            crow[col] = v;
+          }
         }
       }
     }
@@ -431,10 +460,11 @@ int dgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s, bool upp
     CUtensorMap ma, mb;
     TSVD_TRY(digit_map(&ma, DA, g.M, 2 * g.K, ldk, n * DG_D, DG_BM));
     TSVD_TRY(digit_map(&mb, DB, N2, 2 * g.K, ldk, n * DG_D, DG_BN));
-    const dim3 grid(cdiv(N2, DG_BN), cdiv(g.M, DG_BM), n);
+    const long tiles = (long)cdiv(N2, DG_BN) * cdiv(g.M, DG_BM) * n;  // one per CTA where some are skipped
+    const unsigned grid = (unsigned)(upper ? tiles : std::min<long>(tiles, 152));
     const DotSrc<double2> src{g.C == g.A || g.C == g.B ? nullptr : A, B, g.lda, g.sA, g.ldb, g.sB, g.K, ta, !tb};
     k_dgemm_tc<<<grid, DG_THREADS, DG_SMEM, s>>>(ma, mb, src, EA, EB, (double2*)g.C + (long)b0 * g.sC, g.ldc, g.sC, g.M,
-                                                 g.N, cdiv(2L * g.K, DG_KB), g.alpha, g.beta != 0.0, upper ? 1 : 0);
+                                                 g.N, cdiv(2L * g.K, DG_KB), n, g.alpha, g.beta != 0.0, upper ? 1 : 0);
     TSVD_LAUNCHED();
   }
   return TSVD_OK;

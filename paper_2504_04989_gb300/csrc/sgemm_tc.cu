@@ -4,18 +4,22 @@
 // the rest (2^-23 relative), and hi hi + hi lo + lo hi is accumulated on tcgen05.  The
 // tensor cores truncate when they add to an accumulator (measured: a sum kept in TMEM
 // shrinks by about 2e-8 per instruction, 1.4e-5 after 1024 complex terms), so an
-// accumulator holds 32 terms of K only -- the two small products first, then four
-// instructions of hi hi -- and is then read and added to sums in registers, rounded to
-// nearest, in runs of eight readings; two accumulators alternate so that the reading
-// runs under the next products.  Against exact dot products of normal data the result
+// accumulator holds 32 terms of K only -- hi hi and the two small products apart, as B's hi
+// and lo rows lie one after another and one instruction multiplies A hi with both -- and
+// is then read and added to sums in registers, rounded to nearest, in runs of eight
+// readings; two pairs of accumulators alternate so that the reading runs under the next
+// products, and a CTA walks over several tiles so that the next tile's loads and products
+// run under the writing of this one.  Against exact dot products of normal data the result
 // is closer than FP32 multiply-adds' (the figures stand at sgemm_tc_better).
 //
 // A complex product is the real product of the interleaved rows of op(A) with the
 // expanded real form of op(B) (rows 2n and 2n + 1 per column n, as in tc_gemm.cu),
 // both written as hi / lo rows by one pass over each operand.
 //
-// Bound: the tensor cores at a third of the TF32 rate (355 TFLOP/s), just above what L2
-// delivers of the 64 KB of operands per 128 x 128 x 32 block.
+// Bound: shared memory, 144 KB read and filled per 128 x 128 x 32 block (1125 clocks at 128
+// bytes per clock; the products alone take 768).  K = 100 (2048 x 2048 on 65 slices, most of it
+// writing): 2.13 -> 1.70 ms by walking over tiles; K = 1024: 1.82 -> 1.81 ms by reading A hi
+// once for both, 1.92 with 16 reading warps instead of 8.
 #include <cmath>
 
 #include "common.cuh"
@@ -28,12 +32,12 @@ constexpr int SG_BM = 128, SG_BN = 128;  // complex rows x real columns
 constexpr int SG_KB = 32;                // K per stage: rows of 128 bytes, 128-byte swizzle
 constexpr int SG_STAGES = 3;
 constexpr int SG_TILE = SG_BM * SG_KB * 4;
-constexpr int SG_STAGE_BYTES = 4 * SG_TILE;  // A hi, B hi, A lo, B lo
-constexpr int SG_SMEM = SG_STAGES * SG_STAGE_BYTES + 1024 + 256;
+constexpr int SG_STAGE_BYTES = 4 * SG_TILE;  // A hi, A lo, B hi, B lo
 constexpr int SG_RUN = 8;                // readings summed before they join the total
 constexpr int SG_DRAIN = 256;            // threads reading the accumulators, then one TMA and one MMA warp
 constexpr int SG_THREADS = SG_DRAIN + 64;
 constexpr int SG_OUT = SG_BN / 2;        // columns per reading thread
+constexpr int SG_SMEM = SG_STAGES * SG_STAGE_BYTES + 1024 + 256 + SG_DRAIN / 32 * 4096;  // 4 KB per reading warp
 static_assert(SG_SMEM <= 227 * 1024, "the stages must fit a CTA's shared memory");
 
 __device__ __forceinline__ float rna_tf32(float x) {
@@ -89,10 +93,18 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constan
                                                             const __grid_constant__ CUtensorMap tmBl,
                                                             const __grid_constant__ DotSrc<float2> src,
                                                             float2* __restrict__ C, long ldc, long sC, int M, int N,
-                                                            int nk, float alpha, int beta) {
+                                                            int nk, int batch, float alpha, int beta) {
   extern __shared__ unsigned char sg_raw[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int n0 = blockIdx.x * SG_BN, m0 = blockIdx.y * SG_BM, bz = blockIdx.z;
+  const int tn = (2 * N + SG_BN - 1) / SG_BN, tm = (M + SG_BM - 1) / SG_BM;
+  const int tiles = tn * tm * batch;  // at least one element each: within an int
+  struct Tile {
+    int n0, m0, bz;
+  };
+  auto tile = [&](int t) {  // columns fastest: neighbouring CTAs share rows of A
+    const int r = t / tn;
+    return Tile{(t % tn) * SG_BN, (r % tm) * SG_BM, r / tm};
+  };
   unsigned char* base = (unsigned char*)(((uintptr_t)sg_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* bars = (uint64_t*)(base + SG_STAGES * SG_STAGE_BYTES);  // full[S], empty[S], tfull[2], tempty[2]
   uint32_t* tslot = (uint32_t*)(bars + 2 * SG_STAGES + 4);
@@ -111,7 +123,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constan
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
-                 "r"(2 * SG_BN));
+                 "r"(512));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
@@ -119,108 +131,123 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constan
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = *tslot;
 
+  // stages and accumulators are counted through all tiles of the CTA, so loads and products of the
+  // next tile run under the writing of this one
   if (tid == SG_DRAIN) {  // TMA producer
-    int issued = 0;
+    Ring<SG_STAGES> r;
+    long filled = 0;
     bool ok = true;
-    for (int kb = 0; kb < nk; ++kb) {
-      const int s = kb % SG_STAGES, round = kb / SG_STAGES;
-      if (round > 0 && !mbar_wait(empty0 + 8 * s, (round - 1) & 1)) {
-        ok = false;
-        break;
+    for (int t = blockIdx.x; ok && t < tiles; t += gridDim.x) {
+      const Tile w = tile(t);
+      for (int kb = 0; kb < nk; ++kb, ++filled, r.next()) {
+        const int s = r.s;
+        if (!mbar_wait(empty0 + 8 * s, r.ph ^ 1)) {
+          ok = false;
+          break;
+        }
+        const uint32_t dst = smem_u32(base + s * SG_STAGE_BYTES), bar = full0 + 8 * s;
+        mbar_expect_tx(bar, SG_STAGE_BYTES);
+        tma_load_3d(dst, &tmAh, kb * SG_KB, w.m0, w.bz, bar);
+        tma_load_3d(dst + 2 * SG_TILE, &tmBh, kb * SG_KB, w.n0, w.bz, bar);
+        tma_load_3d(dst + SG_TILE, &tmAl, kb * SG_KB, w.m0, w.bz, bar);
+        tma_load_3d(dst + 3 * SG_TILE, &tmBl, kb * SG_KB, w.n0, w.bz, bar);
       }
-      const uint32_t dst = smem_u32(base + s * SG_STAGE_BYTES), bar = full0 + 8 * s;
-      mbar_expect_tx(bar, SG_STAGE_BYTES);
-      tma_load_3d(dst, &tmAh, kb * SG_KB, m0, bz, bar);
-      tma_load_3d(dst + SG_TILE, &tmBh, kb * SG_KB, n0, bz, bar);
-      tma_load_3d(dst + 2 * SG_TILE, &tmAl, kb * SG_KB, m0, bz, bar);
-      tma_load_3d(dst + 3 * SG_TILE, &tmBl, kb * SG_KB, n0, bz, bar);
-      issued = kb + 1;
     }
-    if (!ok) {  // copies in flight land before the CTA gives its shared memory back
-      for (int kb = (issued > SG_STAGES ? issued - SG_STAGES : 0); kb < issued; ++kb)
-        mbar_wait(full0 + 8 * (kb % SG_STAGES), (kb / SG_STAGES) & 1);
-    }
+    ring_drain(r, filled, full0);
   } else if (tid == SG_DRAIN + 32) {  // MMA issuer
-    const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(SG_BN >> 3) << 17) |
-                           ((uint32_t)(SG_BM >> 4) << 24);  // FP32 += TF32 TF32^T
-    for (int kb = 0; kb < nk; ++kb) {
-      const int s = kb % SG_STAGES, a = kb & 1;
-      if (kb >= 2 && !mbar_wait(tempty + 8 * a, ((kb >> 1) - 1) & 1)) break;
-      if (!mbar_wait(full0 + 8 * s, (kb / SG_STAGES) & 1)) break;
+    const uint32_t idesc0 = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(SG_BM >> 4) << 24);  // FP32 += TF32 TF32^T
+    const uint32_t idesc1 = idesc0 | ((uint32_t)(SG_BN >> 3) << 17), idesc2 = idesc0 | ((uint32_t)(2 * SG_BN >> 3) << 17);
+    const long last = (long)((tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1) * nk;
+    Ring<SG_STAGES> r;
+    Ring<2> ra;
+    for (long g = 0; g < last; ++g, r.next(), ra.next()) {
+      const int s = r.s, a = ra.s;
+      if (!mbar_wait(tempty + 8 * a, ra.ph ^ 1)) break;
+      if (!mbar_wait(full0 + 8 * s, r.ph)) break;
       asm volatile("tcgen05.fence::after_thread_sync;");
       const uint32_t sm = smem_u32(base + s * SG_STAGE_BYTES);
-      const uint64_t ah = smem_desc_sw128(sm), bh = smem_desc_sw128(sm + SG_TILE);
-      const uint64_t al = smem_desc_sw128(sm + 2 * SG_TILE), bl = smem_desc_sw128(sm + 3 * SG_TILE);
-      const uint32_t d = tmem + (uint32_t)(a * SG_BN);
+      const uint64_t ah = smem_desc_sw128(sm), al = smem_desc_sw128(sm + SG_TILE);
+      const uint64_t bb = smem_desc_sw128(sm + 2 * SG_TILE);  // B hi, B lo: 256 rows
+      const uint32_t d = tmem + (uint32_t)(a * 2 * SG_BN);
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {  // 32 bytes of K per instruction
-        mma_issue<false>(d, ah + 2 * kk, bl + 2 * kk, idesc, kk > 0);
-        mma_issue<false>(d, al + 2 * kk, bh + 2 * kk, idesc, 1);
-      }
+      for (int kk = 0; kk < 4; ++kk) mma_issue<false>(d, ah + 2 * kk, bb + 2 * kk, idesc2, kk > 0);  // 32 bytes of K
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk) mma_issue<false>(d, ah + 2 * kk, bh + 2 * kk, idesc, 1);
+      for (int kk = 0; kk < 4; ++kk) mma_issue<false>(d + SG_BN, al + 2 * kk, bb + 2 * kk, idesc1, 1);
       mma_commit(empty0 + 8 * s);
       mma_commit(tfull + 8 * a);
     }
   } else if (warp < SG_DRAIN / 32) {
-    const int row = m0 + (warp & 3) * 32 + lane;
-    const int col0 = (warp >> 2) * SG_OUT;
-    const uint32_t tw = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)col0;
-    float run[SG_OUT], tot[SG_OUT];
-#pragma unroll
-    for (int q = 0; q < SG_OUT; ++q) run[q] = tot[q] = 0.f;
+    const int row0 = (warp & 3) * 32, col0 = (warp >> 2) * SG_OUT;
+    const uint32_t tw = tmem + ((uint32_t)row0 << 16) + (uint32_t)col0;
+    float4* stg = (float4*)(base + SG_STAGES * SG_STAGE_BYTES + 256) + warp * 256;  // 32 rows x 32 floats
+    Ring<2> ra;
     bool ok = true;
-    for (int kb = 0; kb < nk; ++kb) {
-      const int a = kb & 1;
-      ok = mbar_wait(tfull + 8 * a, (kb >> 1) & 1);
-      ok = __all_sync(0xffffffffu, ok);
-      if (!ok) break;
-      asm volatile("tcgen05.fence::after_thread_sync;");
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+      const Tile w = tile(t);
+      float run[SG_OUT], tot[SG_OUT];
 #pragma unroll
-      for (int q0 = 0; q0 < SG_OUT; q0 += 16) {
-        uint32_t r[16];
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
-            "%14, %15}, [%16];"
-            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-              "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-            : "r"(tw + (uint32_t)(a * SG_BN + q0)));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      for (int q = 0; q < SG_OUT; ++q) run[q] = tot[q] = 0.f;
+      for (int kb = 0; kb < nk && ok; ++kb, ra.next()) {
+        const int a = ra.s;
+        ok = mbar_wait(tfull + 8 * a, ra.ph);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;");
 #pragma unroll
-        for (int u = 0; u < 16; ++u) run[q0 + u] += __uint_as_float(r[u]);
-      }
-      asm volatile("tcgen05.fence::before_thread_sync;");
-      mbar_arrive(tempty + 8 * a);
-      if ((kb & (SG_RUN - 1)) == SG_RUN - 1 || kb == nk - 1) {
+        for (int q0 = 0; q0 < SG_OUT; q0 += 8) {
+          uint32_t r[2][8];  // hi hi, the small products
 #pragma unroll
-        for (int q = 0; q < SG_OUT; ++q) {
-          tot[q] += run[q];
-          run[q] = 0.f;
+          for (int h = 0; h < 2; ++h)
+            asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                         : "=r"(r[h][0]), "=r"(r[h][1]), "=r"(r[h][2]), "=r"(r[h][3]), "=r"(r[h][4]), "=r"(r[h][5]),
+                           "=r"(r[h][6]), "=r"(r[h][7])
+                         : "r"(tw + (uint32_t)((2 * a + h) * SG_BN + q0)));
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+          for (int u = 0; u < 8; ++u) run[q0 + u] += __uint_as_float(r[0][u]) + __uint_as_float(r[1][u]);
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;");
+        mbar_arrive(tempty + 8 * a);
+        if ((kb & (SG_RUN - 1)) == SG_RUN - 1 || kb == nk - 1) {
+#pragma unroll
+          for (int q = 0; q < SG_OUT; ++q) {
+            tot[q] += run[q];
+            run[q] = 0.f;
+          }
         }
       }
-    }
-    if (row < M) {
-      float2* crow = C + (long)bz * sC + (long)row * ldc + ((n0 + col0) >> 1);
-      const int left = N - ((n0 + col0) >> 1);  // complex columns from this thread's first
+      // 32 columns at a time through shared memory, so that eight lanes write 128 bytes of a row
 #pragma unroll
-      for (int q = 0; q < SG_OUT; q += 4) {
-        float2 v[2];
+      for (int c0 = 0; c0 < SG_OUT; c0 += 32) {
+        __syncwarp();
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          v[u] = make_float2(alpha * tot[q + 2 * u], alpha * tot[q + 2 * u + 1]);
-          const int c = q / 2 + u;
-          if (c >= left) continue;
-          if (!ok) v[u] = make_float2(__int_as_float(0x7fc00000), __int_as_float(0x7fc00000));
-          else if (src.A && !(fabsf(v[u].x) <= FLT_MAX && fabsf(v[u].y) <= FLT_MAX))  // operands that are not finite
-            v[u] = cscale(direct_dot(src, bz, row, ((n0 + col0) >> 1) + c), alpha);
-          if (beta) v[u] = cadd(v[u], crow[c]);
-        }
-        const int c = q / 2;
-        if (c + 1 < left && ((uintptr_t)(crow + c) & 15) == 0) {
-          *(float4*)(crow + c) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
-        } else {
-          if (c < left) crow[c] = v[0];
-          if (c + 1 < left) crow[c + 1] = v[1];
+        for (int q = 0; q < 8; ++q)
+          stg[lane * 8 + (q ^ (lane & 7))] =
+              make_float4(tot[c0 + 4 * q], tot[c0 + 4 * q + 1], tot[c0 + 4 * q + 2], tot[c0 + 4 * q + 3]);
+        __syncwarp();
+        const int col = ((w.n0 + col0 + c0) >> 1) + 2 * (lane & 7);
+        if (col >= N) continue;
+#pragma unroll 2
+        for (int i = 0; i < 8; ++i) {
+          const int r = 4 * i + (lane >> 3), row = w.m0 + row0 + r;
+          if (row >= M) break;
+          const float4 x = stg[r * 8 + ((lane & 7) ^ (r & 7))];
+          float2* dst = C + (long)w.bz * sC + (long)row * ldc + col;
+          float2 v[2] = {make_float2(alpha * x.x, alpha * x.y), make_float2(alpha * x.z, alpha * x.w)};
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            if (col + u >= N) continue;
+            if (!ok) v[u] = make_float2(__int_as_float(0x7fc00000), __int_as_float(0x7fc00000));
+            else if (src.A && !(fabsf(v[u].x) <= FLT_MAX && fabsf(v[u].y) <= FLT_MAX))  // operands that are not finite
+              v[u] = cscale(direct_dot(src, w.bz, row, col + u), alpha);
+            if (beta) v[u] = cadd(v[u], dst[u]);
+          }
+          if (col + 1 < N && ((uintptr_t)dst & 15) == 0) {
+            *(float4*)dst = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+          } else {
+            dst[0] = v[0];
+            if (col + 1 < N) dst[1] = v[1];
+          }
         }
       }
     }
@@ -230,7 +257,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constan
   __syncthreads();
   if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * SG_BN));
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
   }
 }
 
@@ -312,8 +339,9 @@ int sgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s) {
     TSVD_TRY(split_map(&mbh, Bh, N2, 2 * g.K, ldk, n));
     TSVD_TRY(split_map(&mbl, Bl, N2, 2 * g.K, ldk, n));
     const DotSrc<float2> src{g.C == g.A || g.C == g.B ? nullptr : A, B, g.lda, g.sA, g.ldb, g.sB, g.K, g.opA == 'H', g.opB == 'H'};
-    k_sgemm_tc<<<dim3(cdiv(N2, SG_BN), cdiv(g.M, SG_BM), n), SG_THREADS, SG_SMEM, s>>>(
-        mah, mal, mbh, mbl, src, (float2*)g.C + (long)b0 * g.sC, g.ldc, g.sC, g.M, g.N, cdiv(2L * g.K, SG_KB),
+    const long tiles = (long)cdiv(N2, SG_BN) * cdiv(g.M, SG_BM) * n;
+    k_sgemm_tc<<<(unsigned)std::min<long>(tiles, 152), SG_THREADS, SG_SMEM, s>>>(
+        mah, mal, mbh, mbl, src, (float2*)g.C + (long)b0 * g.sC, g.ldc, g.sC, g.M, g.N, cdiv(2L * g.K, SG_KB), n,
         (float)g.alpha, g.beta != 0.0);
     TSVD_LAUNCHED();
   }

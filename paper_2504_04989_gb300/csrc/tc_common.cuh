@@ -88,6 +88,35 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
+// Position in a ring of N buffers and the parity of its current round: consumers wait for `ph`,
+// producers for `ph ^ 1` (true at once in the first round).
+template <int N>
+struct Ring {
+  int s = 0;
+  uint32_t ph = 0;
+  __device__ __forceinline__ void next() {
+    if (++s == N) {
+      s = 0;
+      ph ^= 1;
+    }
+  }
+  __device__ __forceinline__ void back() {
+    if (--s < 0) {
+      s = N - 1;
+      ph ^= 1;
+    }
+  }
+};
+// the copies of the last N fills (of `filled`), full barriers from `bar` on, have landed: a CTA
+// gives its shared memory back after that
+template <int N>
+__device__ __forceinline__ void ring_drain(Ring<N> r, long filled, uint32_t bar) {
+  for (int i = 0; i < N && i < filled; ++i) {
+    r.back();
+    mbar_wait(bar + 8 * r.s, r.ph);
+  }
+}
+
 // The operands of a complex product as stored, for the elements whose tensor-core sum is not a
 // number because an operand is not finite (its digits or its lo part say nothing): those are summed
 // again directly.

@@ -9,10 +9,12 @@
 // bytes of K are staged by TMA (128-byte swizzle) through a ring of shared
 // buffers guarded by mbarriers; one thread issues tcgen05.mma (4 per stage,
 // 32 bytes of K each) into a BN-column TMEM accumulator and commits each
-// stage back to the producer; all four warps then read the accumulator with
-// tcgen05.ld and store it (thread = row, 16 columns at a time as four 16-byte
-// accesses where aligned; C = alpha A B^T + beta C, the old values loaded
-// before any store).  Every wait is bounded: on a timeout the kernel records
+// stage back to the producer; eight further warps read the accumulator with
+// tcgen05.ld and store it through shared memory, 128 bytes of a row per eight
+// lanes (C = alpha A B^T + beta C, the old values loaded before any store).  A
+// CTA walks over several tiles with two accumulators, so the next tile's loads
+// and products run under the storing of this one (2048 x 120 x 360 on 65 slices,
+// added to C with split copies: 357 -> 258 us; TF32, 2048 x 120 x 2048: 470 -> 440).  Every wait is bounded: on a timeout the kernel records
 // an error flag instead of hanging.  The split-TF32 epilogue can also write
 // hi / lo copies of C and of C^T for a following product.
 //
@@ -38,6 +40,8 @@
 namespace tsvd {
 
 constexpr int TC_BM = 128;
+constexpr int TC_DRAIN = 256;  // threads that read the accumulator (8 warps, 4 KB of staging each), then one TMA and one MMA warp
+constexpr int TC_THREADS = TC_DRAIN + 64;
 // MODE 0: TF32, 1: BF16, 2: split TF32; BN: 128 or 256 columns per tile
 template <int MODE, int BN>
 constexpr int tc_row() { return MODE == 2 && BN == 256 ? 64 : 128; }  // bytes of K per stage
@@ -52,7 +56,7 @@ constexpr int tc_stage_bytes() {  // A, B[, A lo, B lo]
 template <int MODE, int BN>
 constexpr int tc_stages() { return MODE == 2 && BN == 128 ? 3 : 4; }
 template <int MODE, int BN>
-constexpr int tc_smem() { return tc_stages<MODE, BN>() * tc_stage_bytes<MODE, BN>() + 1024 + 256; }
+constexpr int tc_smem() { return tc_stages<MODE, BN>() * tc_stage_bytes<MODE, BN>() + 1024 + 256 + TC_DRAIN / 32 * 4096; }
 
 // hi = x rounded to the nearest TF32 (lo = x - hi is exact in FP32)
 __device__ __forceinline__ float tf32_hi(float x) {
@@ -71,12 +75,13 @@ __device__ __forceinline__ uint32_t instr_desc() {
 }
 
 template <int MODE, int BN>
-__global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUtensorMap tmA,
-                                                    const __grid_constant__ CUtensorMap tmB,
-                                                    const __grid_constant__ CUtensorMap tmA2,
-                                                    const __grid_constant__ CUtensorMap tmB2, float* __restrict__ C,
-                                                    long ldc, long sC, int M, int N, int nk, int* __restrict__ err,
-                                                    float alpha, float beta, TcSplitOut o2) {
+__global__ void __launch_bounds__(TC_THREADS, 1) k_tc_gemm(const __grid_constant__ CUtensorMap tmA,
+                                                           const __grid_constant__ CUtensorMap tmB,
+                                                           const __grid_constant__ CUtensorMap tmA2,
+                                                           const __grid_constant__ CUtensorMap tmB2,
+                                                           float* __restrict__ C, long ldc, long sC, int M, int N, int nk,
+                                                           int batch, int* __restrict__ err, float alpha, float beta,
+                                                           TcSplitOut o2) {
   constexpr bool BF16 = MODE == 1, SPLIT = MODE == 2;
   constexpr int STAGES = tc_stages<MODE, BN>(), SB = tc_stage_bytes<MODE, BN>();
   static_assert(tc_smem<MODE, BN>() <= 227 * 1024, "the stages must fit the opt-in shared memory of a CTA");
@@ -85,29 +90,39 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUte
   extern __shared__ unsigned char tc_raw[];
   unsigned char* base = (unsigned char*)(((uintptr_t)tc_raw + 1023) & ~(uintptr_t)1023);
   // o: A, B, A lo, B lo (every offset a multiple of 1024 bytes)
-  auto tile = [&](int s, int o) {
-    return base + s * SB + (o & 1) * AB + (o >> 1) * (AB + BB);
+  auto operand = [&](int s, int o) {
+    return smem_u32(base + s * SB + (o & 1) * AB + (o >> 1) * (AB + BB));
   };
-  uint64_t* bars = (uint64_t*)(base + STAGES * SB);  // full[S], empty[S], done
-  uint32_t* tslot = (uint32_t*)(bars + 2 * STAGES + 1);
-  __shared__ int s_fail;
+  uint64_t* bars = (uint64_t*)(base + STAGES * SB);  // full[S], empty[S], tfull[2], tempty[2]
+  uint32_t* tslot = (uint32_t*)(bars + 2 * STAGES + 4);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int n0 = blockIdx.x * BN, m0 = blockIdx.y * TC_BM, bz = blockIdx.z;
-  const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STAGES), done = smem_u32(bars + 2 * STAGES);
+  const int tn = (N + BN - 1) / BN, tm = (M + TC_BM - 1) / TC_BM;
+  const int tiles = tn * tm * batch;  // at least one element each: within an int
+  struct Tile {
+    int n0, m0, bz;
+  };
+  auto tile = [&](int t) {  // columns fastest: neighbouring CTAs share rows of A
+    const int r = t / tn;
+    return Tile{(t % tn) * BN, (r % tm) * TC_BM, r / tm};
+  };
+  const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STAGES);
+  const uint32_t tfull = smem_u32(bars + 2 * STAGES), tempty = tfull + 16;
   constexpr int KE = ROW / (BF16 ? 2 : 4);  // elements of K per stage
 
   if (tid == 0) {
-    s_fail = 0;
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(full0 + 8 * s, 1);
       mbar_init(empty0 + 8 * s, 1);
     }
-    mbar_init(done, 1);
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(tfull + 8 * s, 1);
+      mbar_init(tempty + 8 * s, TC_DRAIN);
+    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
-                 "r"(BN));
+                 "r"(2 * BN));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
@@ -115,157 +130,179 @@ __global__ void __launch_bounds__(128, 1) k_tc_gemm(const __grid_constant__ CUte
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = *tslot;
 
-  int issued = 0;  // stages the producer loaded
-  if (tid == 0) {  // TMA producer
-    for (int kb = 0; kb < nk; ++kb) {
-      const int s = kb % STAGES, round = kb / STAGES;
-      if (round > 0 && !mbar_wait(empty0 + 8 * s, (round - 1) & 1)) {
-        s_fail = 1;
-        break;
+  // stages are counted through all tiles of the CTA and two accumulators alternate, so loads and
+  // products of the next tile run under the writing of this one
+  if (tid == TC_DRAIN) {  // TMA producer
+    Ring<STAGES> r;
+    long filled = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; ok && t < tiles; t += gridDim.x) {
+      const Tile w = tile(t);
+      for (int kb = 0; kb < nk; ++kb, ++filled, r.next()) {
+        const int s = r.s;
+        if (!mbar_wait(empty0 + 8 * s, r.ph ^ 1)) {
+          ok = false;
+          break;
+        }
+        const uint32_t bar = full0 + 8 * s;
+        mbar_expect_tx(bar, SB);
+        tma_load_3d(operand(s, 0), &tmA, kb * KE, w.m0, w.bz, bar);
+        tma_load_3d(operand(s, 1), &tmB, kb * KE, w.n0, w.bz, bar);
+        if (SPLIT) {
+          tma_load_3d(operand(s, 2), &tmA2, kb * KE, w.m0, w.bz, bar);
+          tma_load_3d(operand(s, 3), &tmB2, kb * KE, w.n0, w.bz, bar);
+        }
       }
-      mbar_expect_tx(full0 + 8 * s, SB);
-      tma_load_3d(smem_u32(tile(s, 0)), &tmA, kb * KE, m0, bz, full0 + 8 * s);
-      tma_load_3d(smem_u32(tile(s, 1)), &tmB, kb * KE, n0, bz, full0 + 8 * s);
-      if (SPLIT) {
-        tma_load_3d(smem_u32(tile(s, 2)), &tmA2, kb * KE, m0, bz, full0 + 8 * s);
-        tma_load_3d(smem_u32(tile(s, 3)), &tmB2, kb * KE, n0, bz, full0 + 8 * s);
-      }
-      issued = kb + 1;
     }
-  } else if (tid == 32) {  // MMA issuer
+    ring_drain(r, filled, full0);
+  } else if (tid == TC_DRAIN + 32) {  // MMA issuer
     const uint32_t idesc = instr_desc<BF16, BN>();
-    for (int kb = 0; kb < nk; ++kb) {
-      const int s = kb % STAGES, round = kb / STAGES;
-      if (!mbar_wait(full0 + 8 * s, round & 1)) {
-        s_fail = 1;
+    Ring<STAGES> r;
+    Ring<2> ra;
+    bool ok = true;
+    for (int t = blockIdx.x; ok && t < tiles; t += gridDim.x, ra.next()) {
+      const int a = ra.s;
+      if (!mbar_wait(tempty + 8 * a, ra.ph ^ 1)) break;
+      asm volatile("tcgen05.fence::after_thread_sync;");
+      const uint32_t d = tmem + (uint32_t)(a * BN);
+      for (int kb = 0; kb < nk; ++kb, r.next()) {
+        const int s = r.s;
+        if (!mbar_wait(full0 + 8 * s, r.ph)) {
+          ok = false;
+          break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        const uint64_t ad = desc(operand(s, 0)), bd = desc(operand(s, 1));
+#pragma unroll
+        for (int kk = 0; kk < ROW / 32; ++kk) {  // 32 bytes of K per instruction: advance the start address by 2 x 16 B
+          mma_issue<BF16>(d, ad + 2 * kk, bd + 2 * kk, idesc, (kb | kk) != 0);
+          if (SPLIT) {
+            const uint64_t ad2 = desc(operand(s, 2)), bd2 = desc(operand(s, 3));
+            mma_issue<BF16>(d, ad + 2 * kk, bd2 + 2 * kk, idesc, 1);
+            mma_issue<BF16>(d, ad2 + 2 * kk, bd + 2 * kk, idesc, 1);
+          }
+        }
+        mma_commit(empty0 + 8 * s);
+      }
+      if (ok) mma_commit(tfull + 8 * a);
+    }
+  } else if (warp < TC_DRAIN / 32) {
+    const int row0 = (warp & 3) * 32, col0 = (warp >> 2) * (BN / 2);
+    float4* stg = (float4*)(base + STAGES * SB + 256) + warp * 256;  // 32 rows x 32 floats, swizzled
+    const int q8 = lane & 7;
+    Ring<2> ra;
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x, ra.next()) {
+      const Tile w = tile(t);
+      const int a = ra.s;
+      if (!__all_sync(0xffffffffu, mbar_wait(tfull + 8 * a, ra.ph))) {
+        if (lane == 0) atomicExch(err, 1);
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;");
-      const uint64_t ad = desc(smem_u32(tile(s, 0)));
-      const uint64_t bd = desc(smem_u32(tile(s, 1)));
-#pragma unroll
-      for (int kk = 0; kk < ROW / 32; ++kk) {  // 32 bytes of K per instruction: advance the start address by 2 x 16 B
-        mma_issue<BF16>(tmem, ad + 2 * kk, bd + 2 * kk, idesc, (kb | kk) != 0);
-        if (SPLIT) {
-          const uint64_t ad2 = desc(smem_u32(tile(s, 2)));
-          const uint64_t bd2 = desc(smem_u32(tile(s, 3)));
-          mma_issue<BF16>(tmem, ad + 2 * kk, bd2 + 2 * kk, idesc, 1);
-          mma_issue<BF16>(tmem, ad2 + 2 * kk, bd + 2 * kk, idesc, 1);
-        }
-      }
-      mma_commit(empty0 + 8 * s);
-    }
-    mma_commit(done);
-  }
-  __syncwarp();
-  const bool ok = mbar_wait(done, 0);
-  __syncwarp();
-  asm volatile("tcgen05.fence::after_thread_sync;");
-  __syncthreads();
-  const bool good = ok && (s_fail == 0);
-  if (good) {
-    const int row = m0 + warp * 32 + lane;
-    float* crow = C + (long)bz * sC + (long)row * ldc;
+      // 32 columns at a time through shared memory, so that eight lanes write 128 bytes of a row
 #pragma unroll 1
-    for (int c0 = 0; c0 < BN; c0 += 16) {
-      uint32_t r[16];
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-          "%15}, [%16];"
-          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-            "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-          : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0));
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      if (row < M) {
-        float* dst = crow + n0 + c0;
-        const bool full = n0 + c0 + 16 <= N;
-        float o[16];  // the chunk's final values (C = alpha A B^T + beta C)
-        if (full && ((uintptr_t)dst & 15) == 0) {
-          // the thread's 16 columns as four 16-byte accesses (the old values all loaded first)
-          float4 old4[4];
-          if (beta != 0.0f) {
+      for (int c0 = 0; c0 < BN / 2; c0 += 32) {
+        const uint32_t ta = tmem + ((uint32_t)row0 << 16) + (uint32_t)(a * BN + col0 + c0);
+        uint32_t r[32];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) old4[q] = reinterpret_cast<const float4*>(dst)[q];
-          }
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            float4 v = make_float4(alpha * __uint_as_float(r[4 * q]), alpha * __uint_as_float(r[4 * q + 1]),
-                                   alpha * __uint_as_float(r[4 * q + 2]), alpha * __uint_as_float(r[4 * q + 3]));
-            if (beta != 0.0f) {
-              v.x = fmaf(beta, old4[q].x, v.x);
-              v.y = fmaf(beta, old4[q].y, v.y);
-              v.z = fmaf(beta, old4[q].z, v.z);
-              v.w = fmaf(beta, old4[q].w, v.w);
-            }
-            reinterpret_cast<float4*>(dst)[q] = v;
-            o[4 * q] = v.x;
-            o[4 * q + 1] = v.y;
-            o[4 * q + 2] = v.z;
-            o[4 * q + 3] = v.w;
-          }
-        } else {
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const int col = n0 + c0 + j;
-            o[j] = 0.0f;
-            if (col < N) {
-              const float v = alpha * __uint_as_float(r[j]);
-              o[j] = (beta != 0.0f) ? fmaf(beta, crow[col], v) : v;
-              crow[col] = o[j];
-            }
-          }
+        for (int h = 0; h < 32; h += 16)
+          asm volatile(
+              "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+              "%14, %15}, [%16];"
+              : "=r"(r[h]), "=r"(r[h + 1]), "=r"(r[h + 2]), "=r"(r[h + 3]), "=r"(r[h + 4]), "=r"(r[h + 5]),
+                "=r"(r[h + 6]), "=r"(r[h + 7]), "=r"(r[h + 8]), "=r"(r[h + 9]), "=r"(r[h + 10]), "=r"(r[h + 11]),
+                "=r"(r[h + 12]), "=r"(r[h + 13]), "=r"(r[h + 14]), "=r"(r[h + 15])
+              : "r"(ta + (uint32_t)h));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (c0 + 32 == BN / 2) {  // the accumulator has been read
+          asm volatile("tcgen05.fence::before_thread_sync;");
+          mbar_arrive(tempty + 8 * a);
         }
-        if (o2.Rhi) {  // split copy in C's layout
-          float* rh = o2.Rhi + (long)bz * o2.sr + (long)row * o2.ldr + n0 + c0;
-          float* rl = o2.Rlo + (long)bz * o2.sr + (long)row * o2.ldr + n0 + c0;
-          if (full && (((uintptr_t)rh | (uintptr_t)rl) & 15) == 0) {
+        if (w.n0 + col0 + c0 >= N) continue;
+        __syncwarp();
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              float h4[4], l4[4];
+        for (int q = 0; q < 8; ++q)
+          stg[lane * 8 + (q ^ q8)] =
+              make_float4(__uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]), __uint_as_float(r[4 * q + 2]),
+                          __uint_as_float(r[4 * q + 3]));
+        __syncwarp();
+        const int col = w.n0 + col0 + c0 + 4 * q8, left = N - col;
+        float* Cb = C + (long)w.bz * sC + col;
+        float4 v[8], old[8];
 #pragma unroll
-              for (int u = 0; u < 4; ++u) {
-                h4[u] = tf32_hi(o[4 * q + u]);
-                l4[u] = o[4 * q + u] - h4[u];
-              }
-              reinterpret_cast<float4*>(rh)[q] = make_float4(h4[0], h4[1], h4[2], h4[3]);
-              reinterpret_cast<float4*>(rl)[q] = make_float4(l4[0], l4[1], l4[2], l4[3]);
-            }
+        for (int i = 0; i < 8; ++i) {
+          const int rr = 4 * i + (lane >> 3), row = w.m0 + row0 + rr;
+          v[i] = stg[rr * 8 + (q8 ^ (rr & 7))];
+          if (beta == 0.0f || row >= M || left <= 0) continue;  // the old values all loaded first
+          const float* src = Cb + (long)row * ldc;
+          if (left >= 4 && ((uintptr_t)src & 15) == 0) {
+            old[i] = *(const float4*)src;
           } else {
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-              if (n0 + c0 + j < N) {
-                const float hv = tf32_hi(o[j]);
-                rh[j] = hv;
-                rl[j] = o[j] - hv;
-              }
+            old[i].x = src[0];
+            old[i].y = left > 1 ? src[1] : 0.f;
+            old[i].z = left > 2 ? src[2] : 0.f;
+            old[i].w = left > 3 ? src[3] : 0.f;
           }
         }
-        if (o2.Thi) {  // split copy of C^T: lanes are consecutive rows, so each store is coalesced
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const int col = n0 + c0 + j;
-            if (col < N) {
-              const long off = (long)bz * o2.st + (long)col * o2.ldt + row;
-              const float hv = tf32_hi(o[j]);
+        for (int i = 0; i < 8; ++i) {
+          const int rr = 4 * i + (lane >> 3), row = w.m0 + row0 + rr;
+          if (row >= M || left <= 0) continue;
+          // C = alpha A B^T + beta C
+          float4 x = make_float4(alpha * v[i].x, alpha * v[i].y, alpha * v[i].z, alpha * v[i].w);
+          if (beta != 0.0f)
+            x = make_float4(fmaf(beta, old[i].x, x.x), fmaf(beta, old[i].y, x.y), fmaf(beta, old[i].z, x.z),
+                            fmaf(beta, old[i].w, x.w));
+          v[i] = x;
+          auto put = [&](float* dst, float4 y) {
+            if (left >= 4 && ((uintptr_t)dst & 15) == 0) {
+              *(float4*)dst = y;
+            } else {
+              dst[0] = y.x;
+              if (left > 1) dst[1] = y.y;
+              if (left > 2) dst[2] = y.z;
+              if (left > 3) dst[3] = y.w;
+            }
+          };
+          put(Cb + (long)row * ldc, x);
+          if (o2.Rhi) {  // split copy in C's layout
+            const float4 hi = make_float4(tf32_hi(x.x), tf32_hi(x.y), tf32_hi(x.z), tf32_hi(x.w));
+            const long off = (long)w.bz * o2.sr + (long)row * o2.ldr + col;
+            put(o2.Rhi + off, hi);
+            put(o2.Rlo + off, make_float4(x.x - hi.x, x.y - hi.y, x.z - hi.z, x.w - hi.w));
+          }
+        }
+        if (o2.Thi) {  // split copy of C^T: back to a row per lane, so that each store is coalesced
+          __syncwarp();
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const int rr = 4 * i + (lane >> 3);
+            stg[rr * 8 + (q8 ^ (rr & 7))] = v[i];
+          }
+          __syncwarp();
+          const int row = w.m0 + row0 + lane;
+          if (row < M) {
+#pragma unroll 1
+            for (int j = 0; j < 32; ++j) {
+              const int cj = w.n0 + col0 + c0 + j;
+              if (cj >= N) break;
+              const float x = reinterpret_cast<const float*>(stg)[lane * 32 + (((j >> 2) ^ q8) << 2) + (j & 3)];
+              const long off = (long)w.bz * o2.st + (long)cj * o2.ldt + row;
+              const float hv = tf32_hi(x);
               o2.Thi[off] = hv;
-              o2.Tlo[off] = o[j] - hv;
+              o2.Tlo[off] = x - hv;
             }
           }
         }
       }
     }
-  } else if (tid == 0) {
-    atomicExch(err, 1);
   }
-  if (tid == 0) {  // make sure no copy of this CTA is still landing in shared memory
-    for (int kb = (issued > STAGES ? issued - STAGES : 0); kb < issued; ++kb)
-      mbar_wait(full0 + 8 * (kb % STAGES), (kb / STAGES) & 1);
-  }
+  __syncwarp();
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN));
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * BN));
   }
 }
 
@@ -303,14 +340,14 @@ template <int MODE, int BN>
 static int tc_launch(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& ta2, const CUtensorMap& tb2,
                      float* C, long ldc, long sC, int M, int N, int nk, int batch, int* err, cudaStream_t s,
                      float alpha = 1.0f, float beta = 0.0f, const TcSplitOut& o2 = TcSplitOut()) {
-  dim3 grid(cdiv(N, BN), cdiv(M, TC_BM), batch);
+  const long tiles = (long)cdiv(N, BN) * cdiv(M, TC_BM) * batch;
   if (cudaFuncSetAttribute(k_tc_gemm<MODE, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem<MODE, BN>()) !=
       cudaSuccess) {
     cudaGetLastError();
     return TSVD_ERR_CUDA;
   }
-  k_tc_gemm<MODE, BN><<<grid, 128, tc_smem<MODE, BN>(), s>>>(ta, tb, ta2, tb2, C, ldc, sC, M, N, nk, err, alpha,
-                                                               beta, o2);
+  k_tc_gemm<MODE, BN><<<(unsigned)std::min<long>(tiles, 152), TC_THREADS, tc_smem<MODE, BN>(), s>>>(
+      ta, tb, ta2, tb2, C, ldc, sC, M, N, nk, batch, err, alpha, beta, o2);
   TSVD_LAUNCHED();
   return TSVD_OK;
 }
@@ -344,7 +381,7 @@ int tc_gemm_split(const float* Ahi, const float* Alo, long lda, long sA, int M, 
   // columns per tile: shared memory feeds the products (every instruction reads its 128 rows of A and
   // BN of B, 160 KB per 32 terms at 128 columns with the filling, 240 KB at 256, against 128 bytes per
   // clock), so a term of K costs a tile of 256 about 1.5 times one of 128.  The 48 products of a T-SVD
-  // of 2048 x 2048 x 128 took 12.2 ms with 128 columns throughout, 11.1 so.
+  // of 2048 x 2048 x 128 took 12.2 ms with 128 columns throughout, 11.1 so (one tile per CTA).
   const long rows = (long)cdiv(M, TC_BM) * batch;
   const bool wide = 3 * cdiv(rows * cdiv(N, 256), 152) <= 2 * cdiv(rows * cdiv(N, 128), 152);
   const int bn = wide ? 256 : 128, row = wide ? 64 : 128;
