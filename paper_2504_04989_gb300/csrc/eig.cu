@@ -799,16 +799,21 @@ __device__ __forceinline__ int sturm_count_df(const float4* __restrict__ v, int 
 // slice's scaled T); per step the 32 lanes count at 32 interior points of the
 // bracket, so the bracket shrinks 33-fold per step.
 //
-// abs_tol = 0 (FP64 path): FP64 counts until the bracket is within two units
-// in the last place of the eigenvalue.  abs_tol > 0 (FP32 path): BIS_F32_ROUNDS
-// rounds of FP32 counts, the bracket widened by BIS_F32_MARGIN on both sides
-// (about seven times the FP32 count's backward error bound), then
-// double-float counts until the bracket is at most abs_tol wide.  Each round
-// moves an end only to a point whose count was taken, at that point's value
-// in the precision of the count.
+// BIS_F32_ROUNDS rounds of FP32 counts, the bracket widened by BIS_F32_MARGIN
+// on both sides (about seven times the FP32 count's backward error bound), then
+// double-float counts until the bracket is at most abs_tol wide (FP32 path).
+// abs_tol = 0 (FP64 path): until it is 2^-40 ||T|| wide, widened again by
+// BIS_DF_MARGIN (eleven times the double-float count's bound), and from there on
+// FP64 counts until it is within two units in the last place of the eigenvalue:
+// an FP64 count is bound by the FP64 pipe and takes some twenty times a
+// double-float one, and 3 rounds of it remain of 11 (m = 300, 50 eigenvalues on 33
+// slices: 3.15 -> 1.49 ms).  Each round moves an
+// end only to a point whose count was taken, at that point's value in the
+// precision of the count.
 constexpr int BIS_WARPS = 4;
 constexpr int BIS_F32_ROUNDS = 4;
 constexpr double BIS_F32_MARGIN = 0x1p-18;
+constexpr double BIS_DF_MARGIN = 0x1p-43;
 __global__ void __launch_bounds__(BIS_WARPS * 32) k_bisect(int m, int R, EigScratch e, double* __restrict__ lam_out,
                                                           double abs_tol) {
   extern __shared__ __align__(16) double bsm[];
@@ -865,7 +870,8 @@ __global__ void __launch_bounds__(BIS_WARPS * 32) k_bisect(int m, int R, EigScra
   double lo = g_lo - (4.0 * DBL_EPSILON * tn + pivmin);
   double hi = g_hi + (4.0 * DBL_EPSILON * tn + pivmin);
   const int idx = m - 1 - r;  // ascending index of the wanted eigenvalue
-  if (abs_tol > 0.0) {
+  const double wide_lo = lo, wide_hi = hi;
+  {
     for (int it = 0; it < BIS_F32_ROUNDS; ++it) {
       const double w = hi - lo;
       const float x = (float)(lo + w * ((double)(lane + 1) / 33.0));
@@ -876,11 +882,12 @@ __global__ void __launch_bounds__(BIS_WARPS * 32) k_bisect(int m, int R, EigScra
       lo = nlo;
       hi = nhi;
     }
-    lo = fmax(lo - BIS_F32_MARGIN * tn, g_lo - (4.0 * DBL_EPSILON * tn + pivmin));
-    hi = fmin(hi + BIS_F32_MARGIN * tn, g_hi + (4.0 * DBL_EPSILON * tn + pivmin));
+    lo = fmax(lo - BIS_F32_MARGIN * tn, wide_lo);
+    hi = fmin(hi + BIS_F32_MARGIN * tn, wide_hi);
+    const double df_tol = abs_tol > 0.0 ? abs_tol : 0x1p-40 * tn;
     for (int it = 0; it < 16; ++it) {
       const double w = hi - lo;
-      if (w <= abs_tol) break;
+      if (w <= df_tol) break;
       const dfl x = df_from(lo + w * ((double)(lane + 1) / 33.0));
       const unsigned above = __ballot_sync(0xffffffffu, sturm_count_df(v4, m, x) > idx);
       const int first = above ? __ffs(above) - 1 : 32;
@@ -890,7 +897,10 @@ __global__ void __launch_bounds__(BIS_WARPS * 32) k_bisect(int m, int R, EigScra
       lo = nlo;
       hi = nhi;
     }
-  } else {
+  }
+  if (abs_tol == 0.0) {
+    lo = fmax(lo - BIS_DF_MARGIN * tn, wide_lo);
+    hi = fmin(hi + BIS_DF_MARGIN * tn, wide_hi);
     for (int it = 0; it < 64; ++it) {
       const double w = hi - lo;
       // relative to the eigenvalue
@@ -1337,12 +1347,19 @@ __global__ void __launch_bounds__(CO_THREADS) k_cluster_orth(int m, int R, EigSc
 }
 
 // u_r = H_0 H_1 .. H_{m-2} D z_r in the precision of the output (the FP32
-// path rounds U_c to FP32 for its GEMMs anyway): BT_VPC eigenvectors per CTA,
-// one warp each, the vector in the warp's registers (entry i in lane i % 32,
-// slot i / 32).  The reflectors (VT: float2 copies from the double-float
-// reduction, else double2) are staged in shared memory by asynchronous copies
-// one reflector ahead, three buffers deep (one barrier per reflector), and
-// read by all the CTA's warps; slots wholly at or above row j are skipped.
+// path rounds U_c to FP32 for its GEMMs anyway): one warp per eigenvector, the
+// vector in the warp's registers (entry i in lane i % 32, slot i / 32).  The
+// reflectors (VT: float2 copies from the double-float reduction, else double2)
+// are taken in pairs, v1 = v_{2k+1} first, then v0 = v_{2k}: with c = v0^H v1,
+//   a1 = 2 v1^H u,  a0 = 2 (v0^H u - c a1),  u -= v1 a1 + v0 a0,
+// so both products with u come from the same u and their four sums across the
+// warp are halved together (six exchanges a pair instead of twenty).  The pairs
+// are staged in shared memory by asynchronous copies one pair ahead, three
+// buffers deep (one barrier a pair), and read by all the CTA's warps; slots wholly
+// at or above row 2k are skipped.  Bound: FP64 by its pipe (8 multiply-adds per
+// entry and reflector), FP32 by the exchanges and the barrier.  m = 300, 50
+// vectors on 33 slices: FP64 5.53 -> 1.54 ms (one reflector at a time, 16 vectors in every CTA
+// before).
 constexpr int BT_VPC = 16;
 __device__ __forceinline__ void bt_copy(float2* dst, const float2* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src));
@@ -1350,14 +1367,42 @@ __device__ __forceinline__ void bt_copy(float2* dst, const float2* src) {
 __device__ __forceinline__ void bt_copy(double2* dst, const double2* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src));
 }
-template <typename C, typename VT, int NPL>  // NPL >= ceil(m / 32)
+
+// c = v_{2k}^H v_{2k+1} of every pair, one warp each, to the unused place (2k+1, 2k) of the
+// reflectors' array, and zero to (2k+1, 2k+1), where v_{2k+1} has no entry but v_{2k} has (reflector j
+// lies in row j, columns j + 1 on; row m - 1, of an even m, has none)
+template <typename VT>
+__global__ void __launch_bounds__(256) k_reflector_pairs(int m, EigScratch e) {
+  using Rt = decltype(VT().x);
+  const int k = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int j0 = 2 * k, j1 = j0 + 1;
+  if (j1 >= m) return;
+  VT* Hs = (VT*)e.Hv + (long)blockIdx.y * m * m;
+  const VT *v0 = Hs + (long)j0 * m, *v1 = Hs + (long)j1 * m;
+  Rt cx = Rt(0), cy = Rt(0);
+  for (int i = j1 + 1 + lane; i < m; i += 32) {
+    const VT a = v0[i], b = v1[i];
+    cx = fma(a.x, b.x, cx);
+    cx = fma(a.y, b.y, cx);
+    cy = fma(a.x, b.y, cy);
+    cy = fma(-a.y, b.x, cy);
+  }
+  cx = warp_sum(cx);
+  cy = warp_sum(cy);
+  if (lane == 0) {
+    Hs[(long)j1 * m + j0] = VT{cx, cy};
+    Hs[(long)j1 * m + j1] = VT{Rt(0), Rt(0)};
+  }
+}
+
+template <typename C, typename VT, int NPL>  // NPL >= ceil(m / 32); C and VT of one precision
 __global__ void __launch_bounds__(BT_VPC * 32) k_backtransform(int m, int R, EigScratch e, C* __restrict__ U,
                                                                long ldu, long sU) {
   using Rt = decltype(C().x);
   extern __shared__ __align__(16) unsigned char bts[];
-  VT* vb = (VT*)bts;  // [3][m]
+  VT* vb = (VT*)bts;  // [3][2][m]: v1 (from its c on), v0
   const int b = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int r = blockIdx.x * BT_VPC + warp;
+  const int r = blockIdx.x * (blockDim.x >> 5) + warp;
   const bool active = r < R;
   const VT* Hs = (const VT*)e.Hv + (long)b * m * m;  // reflector j at Hs + j m + j + 1
   C u[NPL];
@@ -1367,53 +1412,83 @@ __global__ void __launch_bounds__(BT_VPC * 32) k_backtransform(int m, int R, Eig
     u[t] = C{Rt(0), Rt(0)};
     if (active && i < m) u[t] = from_c64<C>(cscale(e.delta[(long)b * m + i], e.Z[((long)b * R + r) * m + i]));
   }
-  auto stage = [&](int j) {
-    const VT* src = Hs + (long)j * m + j + 1;
-    VT* dst = vb + (j % 3) * m + j + 1;
-    for (int i = tid; i < m - j - 1; i += blockDim.x) bt_copy(dst + i, src + i);
+  auto stage = [&](int k, int buf) {
+    const int j0 = 2 * k;
+    const VT* src = Hs + (long)(j0 + 1) * m;
+    VT* dst = vb + buf * 2 * m;
+    for (int i = j0 + tid; i < m; i += blockDim.x) bt_copy(dst + i, src + i);
+    for (int i = j0 + 1 + tid; i < m; i += blockDim.x) bt_copy(dst + m + i, src - m + i);
     asm volatile("cp.async.commit_group;\n" ::: "memory");
   };
-  if (m >= 2) stage(m - 2);
-  for (int j = m - 2; j >= 0; --j) {
-    if (j > 0) {
-      stage(j - 1);
+  const int pairs = m / 2;  // of an even m the first has a reflector without entries
+  int buf = 0;
+  if (pairs > 0) stage(pairs - 1, 0);
+  for (int k = pairs - 1; k >= 0; --k) {
+    const int nbuf = buf == 2 ? 0 : buf + 1;
+    if (k > 0) {
+      stage(k - 1, nbuf);
       asm volatile("cp.async.wait_group 1;\n" ::: "memory");
     } else {
       asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     }
-    __syncthreads();  // reflector j visible; the buffer staged next was last read two reflectors ago
+    __syncthreads();  // pair k visible; the buffer staged next was last read two pairs ago
     if (active) {
-      const VT* v = vb + (j % 3) * m;
-      Rt ax = Rt(0), ay = Rt(0);
+      const int j0 = 2 * k;
+      const VT *v1 = vb + buf * 2 * m, *v0 = v1 + m;
+      Rt s1x = Rt(0), s1y = Rt(0), s0x = Rt(0), s0y = Rt(0);
 #pragma unroll
       for (int t = 0; t < NPL; ++t) {
-        if (32 * t + 31 > j) {
+        if (32 * t + 31 > j0) {
           const int i = lane + 32 * t;
-          if (i > j && i < m) {
-            const VT vv = v[i];
-            const Rt vx = (Rt)vv.x, vy = (Rt)vv.y;
-            ax = fma(vx, u[t].x, ax);  // conj(v_i) u_i
-            ax = fma(vy, u[t].y, ax);
-            ay = fma(vx, u[t].y, ay);
-            ay = fma(-vy, u[t].x, ay);
+          if (i > j0 && i < m) {
+            const VT a = v1[i], d = v0[i];
+            s1x = fma(a.x, u[t].x, s1x);  // conj(v_i) u_i
+            s1y = fma(a.x, u[t].y, s1y);
+            s0x = fma(d.x, u[t].x, s0x);
+            s0y = fma(d.x, u[t].y, s0y);
+            s1x = fma(a.y, u[t].y, s1x);
+            s1y = fma(-a.y, u[t].x, s1y);
+            s0x = fma(d.y, u[t].y, s0x);
+            s0y = fma(-d.y, u[t].x, s0y);
           }
         }
       }
-      ax = Rt(2) * warp_sum(ax);
-      ay = Rt(2) * warp_sum(ay);
+      // lanes with bit 4 keep v0's sums, those with bit 3 the imaginary parts
+      const bool h4 = lane & 16, h3 = lane & 8;
+      Rt px = (h4 ? s0x : s1x) + __shfl_xor_sync(0xffffffffu, h4 ? s1x : s0x, 16);
+      Rt py = (h4 ? s0y : s1y) + __shfl_xor_sync(0xffffffffu, h4 ? s1y : s0y, 16);
+      Rt p = (h3 ? py : px) + __shfl_xor_sync(0xffffffffu, h3 ? px : py, 8);
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
+      p *= Rt(2);
+      const Rt a1x = __shfl_sync(0xffffffffu, p, 0), a1y = __shfl_sync(0xffffffffu, p, 8);
+      Rt a0x = __shfl_sync(0xffffffffu, p, 16), a0y = __shfl_sync(0xffffffffu, p, 24);
+      const VT c = v1[j0];
+      const Rt cx = Rt(-2) * c.x, cy = Rt(-2) * c.y;
+      a0x = fma(cx, a1x, a0x);
+      a0x = fma(-cy, a1y, a0x);
+      a0y = fma(cx, a1y, a0y);
+      a0y = fma(cy, a1x, a0y);
 #pragma unroll
       for (int t = 0; t < NPL; ++t) {
-        if (32 * t + 31 > j) {
+        if (32 * t + 31 > j0) {
           const int i = lane + 32 * t;
-          if (i > j && i < m) {
-            const VT vv = v[i];
-            const Rt vx = (Rt)vv.x, vy = (Rt)vv.y;
-            u[t].x -= vx * ax - vy * ay;
-            u[t].y -= vx * ay + vy * ax;
+          if (i > j0 && i < m) {
+            const VT a = v1[i], d = v0[i];
+            Rt x = u[t].x, y = u[t].y;
+            x = fma(-a.x, a1x, x);
+            y = fma(-a.x, a1y, y);
+            x = fma(a.y, a1y, x);
+            y = fma(-a.y, a1x, y);
+            x = fma(-d.x, a0x, x);
+            y = fma(-d.x, a0y, y);
+            u[t].x = fma(d.y, a0y, x);
+            u[t].y = fma(-d.y, a0x, y);
           }
         }
       }
     }
+    buf = nbuf;
   }
   if (!active) return;
   C* Ub = U + (long)b * sU;
@@ -1427,15 +1502,31 @@ __global__ void __launch_bounds__(BT_VPC * 32) k_backtransform(int m, int R, Eig
 template <typename C, typename VT>
 static int launch_backtransform(int m, int R, int batch, const EigScratch& e, C* U, long ldu, long sU,
                                 cudaStream_t s) {
-  const size_t smem = 3 * (size_t)m * sizeof(VT);
-  const dim3 grid(cdiv(R, BT_VPC), batch);
+  if (m >= 2) {
+    k_reflector_pairs<VT><<<dim3(cdiv(m / 2, 8), batch), 256, 0, s>>>(m, e);
+    TSVD_LAUNCHED();
+  }
+  const size_t smem = 6 * (size_t)m * sizeof(VT);
+  // eigenvectors per CTA: the parts of R that leave the fewest on the busiest SM (each CTA stages all
+  // reflectors for itself, so no fewer than 4, and of equal choices the largest)
+  int parts = cdiv(R, BT_VPC);
+  long best = -1;
+  for (int p = parts; p <= std::max<int>(parts, cdiv(R, 4)); ++p) {
+    const long load = (long)cdiv((long)p * batch, 152) * cdiv(R, p);
+    if (best < 0 || load < best) {
+      best = load;
+      parts = p;
+    }
+  }
+  const int vpc = cdiv(R, parts);
+  const dim3 grid(cdiv(R, vpc), batch);
   auto go = [&](auto kern) {
     if (smem > 48 * 1024 &&
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
       cudaGetLastError();
       return TSVD_ERR_CUDA;
     }
-    kern<<<grid, BT_VPC * 32, smem, s>>>(m, R, e, U, ldu, sU);
+    kern<<<grid, vpc * 32, smem, s>>>(m, R, e, U, ldu, sU);
     TSVD_LAUNCHED();
     return TSVD_OK;
   };
