@@ -687,16 +687,19 @@ __global__ void __launch_bounds__(128) k_irfft3_reg2(const cx_t<T>* __restrict__
 // A thread holds KB frequencies of a vector of neighbouring tubes; each operand
 // pair read from shared memory feeds 2 KB V multiply-adds.  Sums are taken in
 // runs of 8 terms (their rounding then stays below a mixed-radix transform's).
-// 512 x 512 plane, against the mixed-radix passes: FP32 n = 33 235 -> 36 us, 100
-// 199 -> 122, 31 1446 -> 32 (prime radices ran serially), FP64 33 2304 -> 378;
-// FP32 is bound by load latency and shared-memory reads (bytes alone: 31 us at
-// n = 100), FP64 by its multiply-adds (1130 of 1480 us at n = 100).
+// 512 x 512 plane, against the mixed-radix passes: FP32 n = 33 235 -> 23 us, 100
+// 199 -> 81, 31 1446 -> 20 (prime radices ran serially), FP64 33 2304 -> 371;
+// FP32 is bound by shared-memory reads (bytes alone: 31 us at n = 100), FP64 by its
+// multiply-adds (1130 of 1480 us at n = 100).  The staging keeps eight 16-byte (or
+// sixteen 4-byte) loads of a thread in flight: with eight of 4 bytes it took a
+// third of the time (n = 33: 36 us, 100: 122).  Tubes 32 apart instead of
+// neighbours, for planes whose rows are not aligned, gave no more (33: 44 -> 49).
 // ---------------------------------------------------------------------------
 constexpr int RDFT_MAX = 160;
 template <typename T>
 struct RVec;
 template <>
-struct RVec<float> {  // (64 tubes x 8 frequencies per warp and 256 threads measured slower: 121 -> 140 us at n = 100)
+struct RVec<float> {  // (64 tubes x 8 frequencies per warp and 256 threads measured slower: 121 -> 140 us at n = 100 with the former loads)
   using type = float4;
   static constexpr int V = 4, KB = 4, THREADS = 128;
 };
@@ -768,24 +771,88 @@ __global__ void __launch_bounds__(RVec<T>::THREADS, 4) k_rdft3(const T* __restri
   const long e0 = tile << lgE;
   __syncthreads();  // the previous tile's samples have been read
   auto ld = [&](int j, long ge) { return ge < plane ? __ldg(X + (long)j * plane + ge) : T(0); };
-#pragma unroll 4
-  for (int i = tid; i < J * E; i += THR) {
-    const int j = (i >> lgE) + 1, e = i & (E - 1);
-    const long ge = e0 + e;
+  // 16 bytes per load where the planes are aligned (W tubes), else one sample; 8 or 16 loads in flight
+  auto fold = [&](auto w_) {
+    constexpr int W = decltype(w_)::value;
+    using VW = typename std::conditional<W == 1, T, VT>::type;
+    constexpr int UB = W == 1 ? 8 : 4;  // items of two loads at a time
+    const int lgW = lgE - (W == 4 ? 2 : W == 2 ? 1 : 0), items = J << lgW;
+    auto get = [&](int j, long ge, T* o) {
+      if (ge < plane) {
+        const VW x = __ldg((const VW*)(X + (long)j * plane + ge));
+        if constexpr (W == 1) o[0] = x;
+        else unpack(x, o);
+      } else {
+#pragma unroll
+        for (int q = 0; q < W; ++q) o[q] = T(0);
+      }
+    };
+    auto put = [&](T* dst, const T* v) {
+      if constexpr (W == 4) *(float4*)dst = make_float4(v[0], v[1], v[2], v[3]);
+      else if constexpr (W == 2) *(double2*)dst = make_double2(v[0], v[1]);
+      else dst[0] = v[0];
+    };
     if (d.types == 1) {
-      const T a = ld(j, ge), b = ld(n - j, ge);
-      dat[(j - 1) * E + e] = a + b;
-      dat[(J + j - 1) * E + e] = a - b;
+      for (int i0 = tid; i0 < items; i0 += UB * THR) {
+        T x[UB][2][W];
+#pragma unroll
+        for (int u = 0; u < UB; ++u) {
+          const int i = min(i0 + u * THR, items - 1), j = (i >> lgW) + 1;
+          const long ge = e0 + (i & ((1 << lgW) - 1)) * W;
+          get(j, ge, x[u][0]);
+          get(n - j, ge, x[u][1]);
+        }
+#pragma unroll
+        for (int u = 0; u < UB; ++u) {
+          const int i = i0 + u * THR;
+          if (i >= items) break;
+          T p[W], q[W];
+#pragma unroll
+          for (int k = 0; k < W; ++k) {
+            p[k] = x[u][0][k] + x[u][1][k];
+            q[k] = x[u][0][k] - x[u][1][k];
+          }
+          put(dat + (long)i * W, p);
+          put(dat + J * E + (long)i * W, q);
+        }
+      }
     } else {
-      const T a = ld(j, ge), b = ld(m - j, ge), c = ld(m + j, ge), f = ld(n - j, ge);
-      const T s0 = a + c, s1 = b + f, d0 = a - c, d1 = b - f;
       T* o = dat + (size_t)rows * E;
-      dat[(j - 1) * E + e] = s0 + s1;
-      dat[(J + j - 1) * E + e] = s0 - s1;
-      o[(j - 1) * E + e] = d0 - d1;
-      o[(J + j - 1) * E + e] = d0 + d1;
+      for (int i0 = tid; i0 < items; i0 += UB / 2 * THR) {
+        T x[UB / 2][4][W];
+#pragma unroll
+        for (int u = 0; u < UB / 2; ++u) {
+          const int i = min(i0 + u * THR, items - 1), j = (i >> lgW) + 1;
+          const long ge = e0 + (i & ((1 << lgW) - 1)) * W;
+          get(j, ge, x[u][0]);
+          get(m - j, ge, x[u][1]);
+          get(m + j, ge, x[u][2]);
+          get(n - j, ge, x[u][3]);
+        }
+#pragma unroll
+        for (int u = 0; u < UB / 2; ++u) {
+          const int i = i0 + u * THR;
+          if (i >= items) break;
+          T p0[W], q0[W], p1[W], q1[W];
+#pragma unroll
+          for (int k = 0; k < W; ++k) {
+            const T s0 = x[u][0][k] + x[u][2][k], s1 = x[u][1][k] + x[u][3][k];
+            const T d0 = x[u][0][k] - x[u][2][k], d1 = x[u][1][k] - x[u][3][k];
+            p0[k] = s0 + s1;
+            q0[k] = s0 - s1;
+            p1[k] = d0 - d1;
+            q1[k] = d0 + d1;
+          }
+          put(dat + (long)i * W, p0);
+          put(dat + J * E + (long)i * W, q0);
+          put(o + (long)i * W, p1);
+          put(o + J * E + (long)i * W, q1);
+        }
+      }
     }
-  }
+  };
+  if (plane % V == 0 && ((uintptr_t)X & 15) == 0) fold(IntC<V>());
+  else fold(IntC<1>());
   for (int e = tid; e < E; e += THR) {
     const long ge = e0 + e;
     T* f0 = dat + 2 * J * E + e;
@@ -907,14 +974,39 @@ __global__ void __launch_bounds__(RVec<T>::THREADS, 3) k_irdft3(const cx_t<T>* _
   for (long tile = blockIdx.x; (tile << lgE) < plane; tile += gridDim.x) {
   const long e0 = tile << lgE;
   __syncthreads();  // the previous tile's samples have been read
-#pragma unroll 8
-  for (int i = tid; i < K * E; i += THR) {
-    const int r = i >> lgE, e = i & (E - 1);
-    const long ge = e0 + e;
-    const C x = ge < plane ? Xh[(long)freq(r) * plane + ge] : mkc(T(0), T(0));
-    dr[i] = T(2) * x.x;
-    di[i] = T(2) * x.y;
-  }
+  // FP32: two tubes per load where the planes are aligned; 8 loads in flight
+  auto stage = [&](auto w_) {
+    constexpr int W = decltype(w_)::value, UB = 8;
+    const int lgW = lgE - (W == 2 ? 1 : 0), cnt = K << lgW;
+    for (int i0 = tid; i0 < cnt; i0 += UB * THR) {
+      C x[UB][W];
+#pragma unroll
+      for (int u = 0; u < UB; ++u) {
+        const int i = min(i0 + u * THR, cnt - 1);
+        const long ge = e0 + (i & ((1 << lgW) - 1)) * W;
+        const C* src = Xh + (long)freq(i >> lgW) * plane + ge;
+        if constexpr (W == 2) {
+          const float4 y = ge < plane ? *(const float4*)src : make_float4(0.f, 0.f, 0.f, 0.f);
+          x[u][0] = mkc(T(y.x), T(y.y));
+          x[u][1] = mkc(T(y.z), T(y.w));
+        } else {
+          x[u][0] = ge < plane ? *src : mkc(T(0), T(0));
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < UB; ++u) {
+        const int i = i0 + u * THR;
+        if (i >= cnt) break;
+#pragma unroll
+        for (int k = 0; k < W; ++k) {
+          dr[i * W + k] = T(2) * x[u][k].x;
+          di[i * W + k] = T(2) * x[u][k].y;
+        }
+      }
+    }
+  };
+  if (sizeof(T) == 4 && plane % 2 == 0 && ((uintptr_t)Xh & 15) == 0) stage(IntC<sizeof(T) == 4 ? 2 : 1>());
+  else stage(IntC<1>());
   for (int e = tid; e < E; e += THR) {
     const long ge = e0 + e;
     dr[K * E + e] = ge < plane ? Xh[ge].x : T(0);
@@ -1042,8 +1134,8 @@ static unsigned rdft_grid(long plane, int lgE, size_t smem, bool inverse) {
 // FP64 arithmetic runs at 1/64 of FP32's rate, so there the operation count decides: picoseconds per
 // sample of the two forms as measured on a 512 x 512 plane (the mixed-radix passes by radix; the
 // folded product by n, and 100 = 4 5 5: 96 against 58, 128: 36 against 73).  In FP32 the folded
-// product is the faster one at every length that is not a power of two (97: 213 us against 27 ms,
-// 100: 139 against 199, 160: 289 against 346).
+// product is the faster one at every length that is not a power of two (97: 106 us against 27 ms,
+// 100: 81 against 199, 160: 163 against 346).
 template <typename T>
 static bool rdft_better(int n) {
   if (n < 3 || n > RDFT_MAX) return false;
