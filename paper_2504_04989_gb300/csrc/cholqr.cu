@@ -607,35 +607,29 @@ static int orth_block_tc(int n1, int b, int m, int h, const OrthWs& w, int c, in
   const long sQ = (long)n1 * m, sW = (long)n1 * b, sP = (long)m * b, sG = (long)b * b;
   const long sWT = (long)b * t.ldq2, sWr = (long)n1 * t.ldw2, sE = 2L * b * t.ldq2;
   const long ldd = t.ldq2 / 2;  // de-interleaved rows: >= n1, a multiple of 4 (16-byte rows)
-  // which split copies of the current W exist: wd its de-interleaved rows (WThi / WTlo), wr its
-  // rows (Whi / Wlo), written by the epilogue of the GEMM that produced W
-  bool wd = false, wr = false;
-  TcSplitOut both;
-  both.Rhi = t.Whi;
-  both.Rlo = t.Wlo;
-  both.ldr = t.ldw2;
-  both.sr = sWr;
-  both.Thi = t.WThi;
-  both.Tlo = t.WTlo;
-  both.ldt = ldd;
-  both.st = sWT;
-  TcSplitOut rows_only = both;  // measured: the transposed copy costs the epilogue more than a
-  rows_only.Thi = rows_only.Tlo = nullptr;  // separate de-interleaving pass
+  // wr: the split rows of the current W (Whi / Wlo) exist, written by the epilogue of the GEMM that
+  // produced W (its de-interleaved rows too, transposed there, gave 10.58 + 0.48 ms of products and
+  // passes at 2048 x 120, m = 480 on 65 slices, the separate pass 9.70 + 1.49)
+  bool wr = false;
+  TcSplitOut rows;
+  rows.Rhi = t.Whi;
+  rows.Rlo = t.Wlo;
+  rows.ldr = t.ldw2;
+  rows.sr = sWr;
   for (int pass = 0; pass < 3; ++pass) {
     if (c > 0) {
       // the projection on tcgen05 against the cached split operands of Q's finished columns:
       // Q^H W from the real product Q_d W_d^T (K = n1), then W -= Q (Q^H W) with Q's
       // interleaved rows (K = 2c) against the expanded coefficients
       TSVD_STAGE("orth_cgs", s);
-      if (!wd) TSVD_TRY(split_deinterleave(W, n1, nb, b, sW, h, t.WThi, t.WTlo, ldd, sWT, s));
+      TSVD_TRY(split_deinterleave(W, n1, nb, b, sW, h, t.WThi, t.WTlo, ldd, sWT, s));
       TSVD_TRY(tc_gemm_split(t.Qdhi, t.Qdlo, ldd, 2L * m * ldd, 2 * c, t.WThi, t.WTlo, ldd, sWT, 2 * nb, n1, t.Elo,
                              2L * b, 4L * m * b, h, t.err, s));
       TSVD_TRY(complex_from_real(t.Elo, 2L * b, 4L * m * b, c, nb, P, nb, sP, h, s));
       const long sEq = 2L * b * t.ldqi;
       TSVD_TRY(expand_thin_split(P, nb, sP, c, nb, t.Ehi, t.Elo, t.ldqi, sEq, h, 0, s));
       TSVD_TRY(tc_gemm_split(t.Qhi, t.Qlo, t.ldqi, (long)n1 * t.ldqi, n1, t.Ehi, t.Elo, t.ldqi, sEq, 2 * nb, 2 * c,
-                             (float*)W, 2L * b, 2L * sW, h, t.err, s, -1.0f, 1.0f, &rows_only));
-      wd = false;
+                             (float*)W, 2L * b, 2L * sW, h, t.err, s, -1.0f, 1.0f, &rows));
       wr = true;
     }
     {
@@ -643,7 +637,7 @@ static int orth_block_tc(int n1, int b, int m, int h, const OrthWs& w, int c, in
       // kept in Elo until the Cholesky has read G)
       TSVD_STAGE("orth_gram", s);
       float* Pr = t.Elo;
-      if (!wd) TSVD_TRY(split_deinterleave(W, n1, nb, b, sW, h, t.WThi, t.WTlo, ldd, sWT, s));
+      TSVD_TRY(split_deinterleave(W, n1, nb, b, sW, h, t.WThi, t.WTlo, ldd, sWT, s));
       TSVD_TRY(tc_gemm_split(t.WThi, t.WTlo, ldd, sWT, 2 * nb, t.WThi, t.WTlo, ldd, sWT, 2 * nb, n1, Pr, 2L * b,
                              4L * b * b, h, t.err, s));
       TSVD_TRY(complex_from_real(Pr, 2L * b, 4L * b * b, nb, nb, Gs, b, sG, h, s));
@@ -659,7 +653,7 @@ static int orth_block_tc(int n1, int b, int m, int h, const OrthWs& w, int c, in
       float* out = (pass < 2) ? (float*)W : (float*)(Q + c);
       TSVD_TRY(tc_gemm_split(t.Whi, t.Wlo, t.ldw2, sWr, n1, t.Ehi, t.Elo, t.ldw2, sE, 2 * nb, 2 * nb, out,
                              pass < 2 ? 2L * b : 2L * m, pass < 2 ? 2L * sW : 2L * sQ, h, t.err, s));
-      wd = wr = false;
+      wr = false;
     }
   }
   {

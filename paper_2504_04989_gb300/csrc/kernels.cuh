@@ -180,14 +180,11 @@ int expand_thin(const float2* Y, long ldy, long sy, int K, int N, void* E, long 
 int copy_rows(const float* x, long ldx, void* y, long ldy, int cols, long rows, bool bf16, cudaStream_t s);
 // split TF32: C = alpha A B^T + beta C with A = Ahi + Alo, B = Bhi + Blo (hi*hi + hi*lo + lo*hi),
 // FP32-level accuracy
-// Optional split copies of the result written by the epilogue (null pointers: none):
-//   rows (Rhi / Rlo): hi / lo of C in C's own layout (leading dim ldr, batch stride sr);
-//   cols (Thi / Tlo): hi / lo of C^T (row f of T is column f of C; leading dim ldt, batch stride st).
+// Optional split copy of the result written by the epilogue (null pointers: none): hi / lo of C in C's
+// own layout (leading dim ldr, batch stride sr)
 struct TcSplitOut {
   float *Rhi = nullptr, *Rlo = nullptr;
   long ldr = 0, sr = 0;
-  float *Thi = nullptr, *Tlo = nullptr;
-  long ldt = 0, st = 0;
 };
 int tc_gemm_split(const float* Ahi, const float* Alo, long lda, long sA, int M, const float* Bhi, const float* Blo,
                   long ldb, long sB, int N, int K, float* C, long ldc, long sC, int batch, int* err, cudaStream_t s,

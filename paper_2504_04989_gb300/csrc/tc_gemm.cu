@@ -16,7 +16,7 @@
 // and products run under the storing of this one (2048 x 120 x 360 on 65 slices,
 // added to C with split copies: 357 -> 258 us; TF32, 2048 x 120 x 2048: 470 -> 440).  Every wait is bounded: on a timeout the kernel records
 // an error flag instead of hanging.  The split-TF32 epilogue can also write
-// hi / lo copies of C and of C^T for a following product.
+// hi / lo copies of C for a following product.
 //
 // A third mode keeps FP32 accuracy on the TF32 units ("split TF32"): each
 // operand is split as x = hi + lo with hi = x rounded to TF32 and lo = x - hi
@@ -253,7 +253,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_gemm(const __grid_constant
           if (beta != 0.0f)
             x = make_float4(fmaf(beta, old[i].x, x.x), fmaf(beta, old[i].y, x.y), fmaf(beta, old[i].z, x.z),
                             fmaf(beta, old[i].w, x.w));
-          v[i] = x;
           auto put = [&](float* dst, float4 y) {
             if (left >= 4 && ((uintptr_t)dst & 15) == 0) {
               *(float4*)dst = y;
@@ -270,28 +269,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_gemm(const __grid_constant
             const long off = (long)w.bz * o2.sr + (long)row * o2.ldr + col;
             put(o2.Rhi + off, hi);
             put(o2.Rlo + off, make_float4(x.x - hi.x, x.y - hi.y, x.z - hi.z, x.w - hi.w));
-          }
-        }
-        if (o2.Thi) {  // split copy of C^T: back to a row per lane, so that each store is coalesced
-          __syncwarp();
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const int rr = 4 * i + (lane >> 3);
-            stg[rr * 8 + (q8 ^ (rr & 7))] = v[i];
-          }
-          __syncwarp();
-          const int row = w.m0 + row0 + lane;
-          if (row < M) {
-#pragma unroll 1
-            for (int j = 0; j < 32; ++j) {
-              const int cj = w.n0 + col0 + c0 + j;
-              if (cj >= N) break;
-              const float x = reinterpret_cast<const float*>(stg)[lane * 32 + (((j >> 2) ^ q8) << 2) + (j & 3)];
-              const long off = (long)w.bz * o2.st + (long)cj * o2.ldt + row;
-              const float hv = tf32_hi(x);
-              o2.Thi[off] = hv;
-              o2.Tlo[off] = x - hv;
-            }
           }
         }
       }
