@@ -465,54 +465,60 @@ int copy_rows(const float* x, long ldx, void* y, long ldy, int cols, long rows, 
 // (cvt.rna.tf32.f32), lo = x - hi (exact in FP32).
 // ---------------------------------------------------------------------------
 
-// rows x cols FP32 (leading dim ldx) to hi / lo rows of leading dim ldy (padding zeroed)
-__global__ void k_split_rows(const float* __restrict__ x, long ldx, float* __restrict__ hi, float* __restrict__ lo,
-                             long ldy, int cols, long rows) {
-  const long total = rows * ldy;
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
-    const long r = i / ldy;
-    const long c = i % ldy;
-    const float v = c < cols ? x[r * ldx + c] : 0.0f;
-    const float h = tf32_hi(v);
-    hi[i] = h;
-    lo[i] = v - h;
+// Columns [0, fill) of hi / lo rows (leading dim ldy) from rows x cols FP32 (leading dim ldx, zeros from
+// cols on): 2^lg lanes per row, W floats per lane.  Bound: its bytes (the eight passes of a T-SVD of 2048 x 2048 x
+// 128, 4 GB: 1.01 ms with an element and two 64-bit divisions per thread, 0.65 so).
+template <int W>
+__global__ void __launch_bounds__(256) k_split_rows(const float* __restrict__ x, long ldx, float* __restrict__ hi,
+                                                    float* __restrict__ lo, long ldy, int cols, int fill, long rows,
+                                                    int lg) {
+  const int lane = threadIdx.x & 31, sub = lane & ((1 << lg) - 1);
+  const long warps = (long)gridDim.x * 8 << (5 - lg);
+  for (long r = ((long)blockIdx.x * 8 + (threadIdx.x >> 5) << (5 - lg)) + (lane >> lg); r < rows; r += warps) {
+    const float* src = x + r * ldx;
+    float *h = hi + r * ldy, *l = lo + r * ldy;
+#pragma unroll 4
+    for (int c = sub * W; c < fill; c += W << lg) {
+      if constexpr (W == 4) {
+        const float4 v = c < cols ? *(const float4*)(src + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 y = make_float4(tf32_hi(v.x), tf32_hi(v.y), tf32_hi(v.z), tf32_hi(v.w));
+        *(float4*)(h + c) = y;
+        *(float4*)(l + c) = make_float4(v.x - y.x, v.y - y.y, v.z - y.z, v.w - y.w);
+      } else {
+        const float v = c < cols ? src[c] : 0.f, y = tf32_hi(v);
+        h[c] = y;
+        l[c] = v - y;
+      }
+    }
   }
 }
 
-int split_rows(const float* x, long ldx, float* hi, float* lo, long ldy, int cols, long rows, cudaStream_t s) {
-  const long total = rows * ldy;
-  if (total <= 0) return TSVD_OK;
-  k_split_rows<<<(unsigned)std::min<long>(cdiv(total, 256), 8192), 256, 0, s>>>(x, ldx, hi, lo, ldy, cols, rows);
+static int split_fill(const float* x, long ldx, float* hi, float* lo, long ldy, int cols, int fill, long rows,
+                      cudaStream_t s) {
+  if (rows <= 0 || fill <= 0) return TSVD_OK;
+  const bool vec = (((uintptr_t)x | (uintptr_t)hi | (uintptr_t)lo) & 15) == 0 && ldx % 4 == 0 && ldy % 4 == 0 &&
+                   cols % 4 == 0 && fill % 4 == 0;
+  int lg = 0;
+  while (lg < 5 && (vec ? 4 : 1) << lg < fill) ++lg;
+  const unsigned grid = (unsigned)std::min<long>(cdiv(rows, 8L << (5 - lg)), 152 * 16);
+  if (vec) k_split_rows<4><<<grid, 256, 0, s>>>(x, ldx, hi, lo, ldy, cols, fill, rows, lg);
+  else k_split_rows<1><<<grid, 256, 0, s>>>(x, ldx, hi, lo, ldy, cols, fill, rows, lg);
   TSVD_LAUNCHED();
   return TSVD_OK;
+}
+// rows x cols FP32 (leading dim ldx) to hi / lo rows of leading dim ldy (padding zeroed)
+int split_rows(const float* x, long ldx, float* hi, float* lo, long ldy, int cols, long rows, cudaStream_t s) {
+  return split_fill(x, ldx, hi, lo, ldy, cols, (int)ldy, rows, s);
+}
+// columns [0, cols) of FP32 rows (leading dim ldx) -> hi (nearest TF32) / lo rows of leading dim ldy;
+// the other columns of the destination rows are left as they are
+int split_block(const float* x, long ldx, float* hi, float* lo, long ldy, int cols, long rows, cudaStream_t s) {
+  return split_fill(x, ldx, hi, lo, ldy, cols, cols, rows, s);
 }
 
 // per slice: complex X (rows x cols, interleaved, leading dim cols) transposed
 // to XT (cols x rows complex = real rows of 2 rows floats, leading dim ldt),
 // split into hi / lo; 32 x 32 complex tiles through shared memory
-// columns [0, cols) of FP32 rows (leading dim ldx) -> hi (nearest TF32) / lo rows of leading dim ldy;
-// the other columns of the destination rows are left as they are
-__global__ void k_split_block(const float* __restrict__ x, long ldx, float* __restrict__ hi, float* __restrict__ lo,
-                              long ldy, int cols, long rows) {
-  const long total = rows * cols;
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
-    const long r = i / cols;
-    const long c = i % cols;
-    const float v = x[r * ldx + c];
-    const float h = tf32_hi(v);
-    hi[r * ldy + c] = h;
-    lo[r * ldy + c] = v - h;
-  }
-}
-
-int split_block(const float* x, long ldx, float* hi, float* lo, long ldy, int cols, long rows, cudaStream_t s) {
-  const long total = rows * cols;
-  if (total <= 0) return TSVD_OK;
-  k_split_block<<<(unsigned)std::min<long>(cdiv(total, 256), 8192), 256, 0, s>>>(x, ldx, hi, lo, ldy, cols, rows);
-  TSVD_LAUNCHED();
-  return TSVD_OK;
-}
-
 __global__ void k_split_transpose(const float2* __restrict__ X, int rows, int cols, long ldx, long sx,
                                   float* __restrict__ hi, float* __restrict__ lo, long ldt, long st) {
   __shared__ float2 t[32][33];
