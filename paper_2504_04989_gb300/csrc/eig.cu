@@ -1254,7 +1254,8 @@ template <typename CT, bool STAGED>  // !STAGED (vectors too large for shared me
 __global__ void __launch_bounds__(CO_THREADS) k_cluster_orth(int m, int R, EigScratch e, const double* __restrict__ lam) {
   extern __shared__ __align__(16) unsigned char cosm[];
   __shared__ double red[32];
-  __shared__ CT dots[128];
+  __shared__ CT dots[128], s_inv;
+  __shared__ bool starts[128];  // vector r begins a cluster (R <= 128)
   constexpr bool kBlock = std::is_same<CT, float>::value;
   __shared__ float Gs[kBlock ? CO_BLOCK * CO_BLOCK : 1];  // Gram, then R (upper, row-major)
   __shared__ float Rd[kBlock ? CO_BLOCK : 1];             // 1 / R_jj
@@ -1263,9 +1264,12 @@ __global__ void __launch_bounds__(CO_THREADS) k_cluster_orth(int m, int R, EigSc
   const double* l = lam + (long)b * R;
   const double tol = 1e-3 * e.tnorm[b];
   // only vectors inside a cluster change; find whether there is any
-  bool any = false;
-  for (int r = 1; r < R; ++r) any |= !(l[r - 1] - l[r] > tol);
-  if (!any) return;
+  bool joins = false;
+  for (int r = tid; r < R; r += blockDim.x) {
+    starts[r] = r == 0 || l[r - 1] - l[r] > tol;
+    joins |= !starts[r];
+  }
+  if (!__syncthreads_or(joins)) return;
   CT* zsm = STAGED ? (CT*)cosm : (CT*)Z;  // [R][m]
   if (STAGED) {
     for (int q = tid; q < R * m; q += blockDim.x) zsm[q] = (CT)Z[q];
@@ -1328,14 +1332,24 @@ __global__ void __launch_bounds__(CO_THREADS) k_cluster_orth(int m, int R, EigSc
       }
       double part = 0;
       for (int i = tid; i < m; i += blockDim.x) part += (double)zr[i] * (double)zr[i];
-      const CT inv = (CT)(1.0 / sqrt(block_sum(part, red)));
+      // the root and the quotient by one warp: all 32 of them on the FP64 pipe took 10 us a vector (100
+      // vectors of 480 on 65 slices, clusters up to 69: 903 -> 443 us; FP64 50 of 300 on 33: 764 -> 520)
+      if (32 * warp < m) part = warp_sum(part);
+      if (lane == 0) red[warp] = part;
+      __syncthreads();
+      if (warp == 0) {
+        const double t = warp_sum(lane < nwarp ? red[lane] : 0.0);
+        if (lane == 0) s_inv = (CT)(1.0 / sqrt(t));
+      }
+      __syncthreads();
+      const CT inv = s_inv;
       for (int i = tid; i < m; i += blockDim.x) zr[i] *= inv;
       __syncthreads();
     }
   };
   int c0 = 0;
   for (int r = 1; r <= R; ++r) {
-    if (r < R && !(l[r - 1] - l[r] > tol)) continue;  // r extends the cluster starting at c0
+    if (r < R && !starts[r]) continue;  // r extends the cluster starting at c0
     const int nc = r - c0;
     bool done = nc < 2;
     if constexpr (kBlock) done = done || (nc <= CO_BLOCK && block_qr(c0, nc));
