@@ -81,9 +81,9 @@ __global__ void __launch_bounds__(256) k_gram_quantize(const float2* __restrict_
 //
 // Bound: the operand tiles from L2, 72 KB of digits per 128 x 64 x 64 step (62 bytes per
 // clock and SM at the full tensor rate), and the reading of the accumulators, which
-// is not overlapped.  480 x 480 from 2048 rows on 65 slices: 1.61 ms with its two passes
+// is not overlapped.  480 x 480 from 2048 rows on 65 slices: 1.43 ms with its two passes
 // over C^H (four digits, 16 products of a real GEMM written to memory and added up from
-// there: 4.2 ms); 300 x 300 from 512 rows on 33 slices 0.69 -> 0.18 ms.
+// there: 4.2 ms); 300 x 300 from 512 rows on 33 slices 0.69 -> 0.15 ms.
 // ---------------------------------------------------------------------------
 constexpr int GS_D = 3, GS_L = 5;  // digits, levels
 constexpr int GS_BM = 128, GS_BN = 64, GS_KB = 64;  // rows of 128 bytes per stage, 128-byte swizzle
@@ -144,6 +144,25 @@ __global__ void __launch_bounds__(256) k_gram_digits(const float2* __restrict__ 
       for (int s = 0; s < GS_D; ++s) dst[s * plane + part * w] = gram_digit(y0, s) | (gram_digit(y1, s) << 16);
     }
   }
+}
+
+// v 2^e rounded to nearest, ldexp((double)v, e) in integer arithmetic: those run on the FP64 pipe, which
+// took some 7 us of every tile (480 x 480 on 65 slices: 1303 -> 1127 us)
+__device__ __forceinline__ double int_to_double(long long v, int e) {
+  if (v == 0) return 0.0;
+  const bool neg = v < 0;
+  unsigned long long a = neg ? 0ull - (unsigned long long)v : (unsigned long long)v;
+  const int lz = __clzll((long long)a);
+  a <<= lz;
+  const unsigned rem = (unsigned)a & 0x7ffu;
+  unsigned long long m = a >> 11;
+  m += (rem > 0x400u || (rem == 0x400u && (m & 1))) ? 1 : 0;
+  const int be = 63 - lz + e + 1023;  // biased exponent of the leading bit
+  if (be >= 1 && be < 2046) {
+    const unsigned long long bits = ((unsigned long long)be << 52) + (m - (1ull << 52));
+    return __longlong_as_double((long long)(bits | (neg ? 1ull << 63 : 0)));
+  }
+  return ldexp((double)v, e);
 }
 
 __global__ void __launch_bounds__(GS_THREADS, 1) k_gram_tc(const __grid_constant__ CUtensorMap tmA,
@@ -290,7 +309,7 @@ __global__ void __launch_bounds__(GS_THREADS, 1) k_gram_tc(const __grid_constant
         if (i >= m || j >= m || i > j || (odd && i == j)) continue;
         const long long re = odd ? acc[q + 1] + o0 : acc[q] + o1, im = odd ? o1 - acc[q] : acc[q + 1] - o0;
         const int sc = ei + colexp[(long)bz * m + j] - 2 * B;
-        const double2 g = make_double2(ldexp((double)re, sc), ldexp((double)im, sc));
+        const double2 g = make_double2(int_to_double(re, sc), int_to_double(im, sc));
         if (odd) Gb[(long)j * ldg + i] = make_double2(g.x, -g.y);
         else Gb[(long)i * ldg + j] = g;
       }
