@@ -402,7 +402,11 @@ def main():
         work = algorithmic(stage, d, args.precision)
         t = stages[stage] * 1e-3
         if "flops" in work:
-            if args.precision == "fp64":
+            if args.precision == "fp64" and stage != "eig_hetrd":
+                # exact digit products on the BF16 tensor cores, 34 digit pairs
+                peak = pk.get("bf16_tflops")
+                peak, src = peak and peak / 34, "MEASURED_PEAKS.json bf16_tflops / 34 (digit-pair products)"
+            elif args.precision == "fp64":
                 peak, src = alu["fp64"], "measured here: cuBLAS FP64 GEMM"
             elif stage == "eig_hetrd":
                 peak, src = alu["double_float"], "measured FP32 GEMM rate / 15 instructions per double-float FMA x 2"
@@ -411,11 +415,10 @@ def main():
             elif stage in ("orth_gram", "orth_trsm", "orth_cgs") and d["n1"] >= 1024:
                 # tcgen05 in split TF32 from n1 = 1024 on: three TF32 products per FP32-accurate one
                 peak, src = alu["tf32"] and alu["tf32"] / 3, "measured here: cuBLAS TF32 GEMM / 3 (split TF32)"
-            elif stage == "gram_c" and d["n2"] <= 4096:
-                # the exact Gram in base-64 digits on the BF16 tensor cores: of the 16 digit-pair
-                # products about 8 are computed (the symmetric half skipped)
+            elif stage == "gram_c":
+                # the exact Gram in base-256 digits on the BF16 tensor cores: nine digit-pair products
                 peak = pk.get("bf16_tflops")
-                peak, src = peak and peak / 8, "MEASURED_PEAKS.json bf16_tflops / 8 (digit-pair products)"
+                peak, src = peak and peak / 9, "MEASURED_PEAKS.json bf16_tflops / 9 (digit-pair products)"
             else:
                 peak, src = alu["fp32"], "measured here: cuBLAS FP32 GEMM (no TF32)"
             a = work["flops"] / t / 1e12

@@ -410,8 +410,8 @@ int gram_int_fp32(const float2* CH, long ldc, long sC, int n2, int m, int batch,
   return TSVD_OK;
 }
 
-// the digit form
-bool gram_sliced_ok(int n2, int m) { return n2 >= 1 && m >= 1 && 2L * m <= 65535; }
+// the digit form (n2: 64 rows per block of the grid's second dimension)
+bool gram_sliced_ok(int n2, int m) { return n2 >= 1 && n2 <= (1 << 20) && m >= 1 && 2L * m <= 65535; }
 static long gram_sliced_ldd(int n2) { return (n2 + 7L) / 8 * 8; }
 size_t gram_sliced_bytes(int n2, int m, int batch) {
   return (size_t)batch * GS_D * 2 * m * gram_sliced_ldd(n2) * sizeof(__nv_bfloat16) + 512;
