@@ -122,13 +122,14 @@ __device__ __forceinline__ uint32_t digit_bf16(unsigned long long y, int s) {
 //   TRANS: stored K x rows (read through 32 x 32 tiles), else rows x K;
 //   EXPAND: op(B), two rows 2r and 2r + 1 per column r: (yr, -yi) and (yi, yr); else op(A): (ar, ai);
 //   conj: the stored matrix enters conjugated.
+// Blocks of 32 rows x 32 of K, all along blockIdx.x: rows / 32 passes the 65535 of the other two.
 template <bool TRANS, bool EXPAND>
 __global__ void __launch_bounds__(256) k_dig_pack(const double2* __restrict__ S, long ld, long ss, int rows, int K,
                                                   bool conj, const int* __restrict__ E, uint32_t* __restrict__ D,
                                                   long ldk) {
   __shared__ double2 t[TRANS ? 32 : 1][33];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, b = blockIdx.z;
-  const int k0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
+  const int kblocks = (K + 31) / 32, k0 = blockIdx.x % kblocks * 32, r0 = blockIdx.x / kblocks * 32;
   S += (long)b * ss;
   if (TRANS) {
 #pragma unroll
@@ -450,7 +451,7 @@ int dgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s, bool upp
     if (tb) k_dig_expo_cols<<<dim3(cdiv(g.N, 32), cdiv(g.K, 64), n), 256, 0, s>>>(B, g.ldb, g.sB, g.K, g.N, EB);
     else k_dig_expo_rows<<<dim3(cdiv(g.N, 8), n), 256, 0, s>>>(B, g.ldb, g.sB, g.N, g.K, EB);
     TSVD_LAUNCHED();
-    const dim3 ga(cdiv(g.K, 32), cdiv(g.M, 32), n), gb(cdiv(g.K, 32), cdiv(g.N, 32), n);
+    const dim3 ga(cdiv(g.K, 32) * cdiv(g.M, 32), 1, n), gb(cdiv(g.K, 32) * cdiv(g.N, 32), 1, n);
     if (ta) k_dig_pack<true, false><<<ga, 256, 0, s>>>(A, g.lda, g.sA, g.M, g.K, true, EA, DA, ldk);
     else k_dig_pack<false, false><<<ga, 256, 0, s>>>(A, g.lda, g.sA, g.M, g.K, false, EA, DA, ldk);
     TSVD_LAUNCHED();

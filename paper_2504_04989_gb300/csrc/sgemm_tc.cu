@@ -47,14 +47,14 @@ __device__ __forceinline__ float rna_tf32(float x) {
 }
 
 // One stored complex matrix to hi / lo rows of 2K floats (row length ldk): TRANS, EXPAND and conj
-// as in k_dig_pack.
+// and the blocks as in k_dig_pack.
 template <bool TRANS, bool EXPAND>
 __global__ void __launch_bounds__(256) k_split_pack(const float2* __restrict__ S, long ld, long ss, int rows, int K,
                                                     bool conj, float* __restrict__ Hi, float* __restrict__ Lo,
                                                     long ldk) {
   __shared__ float2 t[TRANS ? 32 : 1][33];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, b = blockIdx.z;
-  const int k0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
+  const int kblocks = (K + 31) / 32, k0 = blockIdx.x % kblocks * 32, r0 = blockIdx.x / kblocks * 32;
   S += (long)b * ss;
   if (TRANS) {
 #pragma unroll
@@ -326,7 +326,7 @@ int sgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s) {
     const int n = std::min(nb, g.batch - b0);
     const float2* A = (const float2*)g.A + (long)b0 * g.sA;
     const float2* B = (const float2*)g.B + (long)b0 * g.sB;
-    const dim3 ga(cdiv(g.K, 32), cdiv(g.M, 32), n), gb(cdiv(g.K, 32), cdiv(g.N, 32), n);
+    const dim3 ga(cdiv(g.K, 32) * cdiv(g.M, 32), 1, n), gb(cdiv(g.K, 32) * cdiv(g.N, 32), 1, n);
     if (g.opA == 'H') k_split_pack<true, false><<<ga, 256, 0, s>>>(A, g.lda, g.sA, g.M, g.K, true, Ah, Al, ldk);
     else k_split_pack<false, false><<<ga, 256, 0, s>>>(A, g.lda, g.sA, g.M, g.K, false, Ah, Al, ldk);
     TSVD_LAUNCHED();
