@@ -687,18 +687,22 @@ int orth_block_cols(int n1, int b, int m, int h, const OrthWs& w, int c, int nb,
                            ? 11.0 * ((double)n1 * nb + (double)nb * (nb + 1)) * 1.1102230246251565e-16
                            : 1e-5;
   const double dead_rel = std::is_same<L, double>::value ? 1e-12 : 1e-7;
+  // the block goes from W to its columns of Q, back, and again: no product writes over its operand
+  CL* Qc = Q + c;
   for (int pass = 0; pass < 3; ++pass) {
+    CL *X = pass == 1 ? Qc : W, *Y = pass == 1 ? W : Qc;
+    const long ldx = pass == 1 ? m : b, sX = pass == 1 ? sQ : sW, ldy = pass == 1 ? b : m, sY = pass == 1 ? sW : sQ;
     // a Gram-Schmidt projection before every pass: without the third, blocks
     // whose new directions are tiny next to the old ones (exact low rank in
     // FP32, the fast-decaying spectra of Sec. 5 Ex. 1 in FP64) lose accuracy
     if (c > 0) {
       TSVD_STAGE("orth_cgs", s);
-      TSVD_TRY(cgemm<CL>(gemm('H', 'N', c, nb, n1, 1.0, Q, m, sQ, W, b, sW, 0.0, P, nb, sP, h), w.splitk, sk, s));
-      TSVD_TRY(cgemm<CL>(gemm('N', 'N', n1, nb, c, -1.0, Q, m, sQ, P, nb, sP, 1.0, W, b, sW, h), w.splitk, sk, s));
+      TSVD_TRY(cgemm<CL>(gemm('H', 'N', c, nb, n1, 1.0, Q, m, sQ, X, ldx, sX, 0.0, P, nb, sP, h), w.splitk, sk, s));
+      TSVD_TRY(cgemm<CL>(gemm('N', 'N', n1, nb, c, -1.0, Q, m, sQ, P, nb, sP, 1.0, X, ldx, sX, h), w.splitk, sk, s));
     }
     {
       TSVD_STAGE("orth_gram", s);
-      TSVD_TRY(cgemm<CL>(gemm('H', 'N', nb, nb, n1, 1.0, W, b, sW, W, b, sW, 0.0, Gs, b, sG, h), w.splitk, sk, s));
+      TSVD_TRY(cgemm<CL>(gemm('H', 'N', nb, nb, n1, 1.0, X, ldx, sX, X, ldx, sX, 0.0, Gs, b, sG, h), w.splitk, sk, s));
     }
     CL* Mi = (CL*)w.Minv;  // R-tilde^{-1}, nb x nb per slice (leading dimension b)
     {
@@ -707,17 +711,13 @@ int orth_block_cols(int n1, int b, int m, int h, const OrthWs& w, int c, int nb,
     }
     {
       TSVD_STAGE("orth_trsm", s);
-      // the last pass writes the finished block straight into its columns of Q
-      CL* out = pass < 2 ? W : Q + c;
-      const long ldo = pass < 2 ? b : m, so = pass < 2 ? sW : sQ;
-      const GemmArgs g = gemm('N', 'N', n1, nb, nb, 1.0, W, b, sW, Mi, b, sG, 0.0, out, ldo, so, h);
-      // the tensor-core forms read copies of their operands, so they may write W in place
+      const GemmArgs g = gemm('N', 'N', n1, nb, nb, 1.0, X, ldx, sX, Mi, b, sG, 0.0, Y, ldy, sY, h);
       if (std::is_same<L, double>::value && dgemm_tc_better(g, sk * sizeof(CL)))
         TSVD_TRY(dgemm_tc(g, w.splitk, sk * sizeof(CL), s, false));
       else if (std::is_same<L, float>::value && sgemm_tc_better(g, sk * sizeof(CL)))
         TSVD_TRY(sgemm_tc(g, w.splitk, sk * sizeof(CL), s));
       else
-        TSVD_TRY(rmul_block<CL>(W, b, sW, Mi, b, sG, n1, nb, h, out, ldo, so, s));
+        TSVD_TRY(rmul_block<CL>(X, ldx, sX, Mi, b, sG, n1, nb, h, Y, ldy, sY, s));
     }
   }
   {

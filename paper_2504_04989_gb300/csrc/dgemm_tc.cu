@@ -33,6 +33,7 @@
 #include "common.cuh"
 #include "kernels.cuh"
 #include "tc_common.cuh"
+#include "tc_redo.cuh"
 
 namespace tsvd {
 
@@ -63,39 +64,56 @@ __device__ __forceinline__ int expo(double2 v) {
   return max(max(a, b), 1);  // subnormals scale as 2^-1022
 }
 
-// largest biased exponent of every row of a stored rows x cols matrix (one warp per row)
-__global__ void __launch_bounds__(256) k_dig_expo_rows(const double2* __restrict__ S, long ld, long ss, int rows,
-                                                       int cols, int* __restrict__ E) {
-  const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31, b = blockIdx.y;
-  if (r >= rows) return;
-  const double2* p = S + (long)b * ss + (long)r * ld;
-  int e = 1;
-#pragma unroll 4
-  for (int c = lane; c < cols; c += 32) e = max(e, expo(p[c]));
-  e = __reduce_max_sync(0xffffffffu, e);
-  if (lane == 0) E[(long)b * rows + r] = e;
-}
+// one operand as its passes see it: rows (columns of op(B)) of K elements
+struct DigOp {
+  const double2* S;
+  long ld, ss;
+  int rows;
+  bool trans;  // stored K x rows, else rows x K
+  bool conj;   // enters conjugated
+  int* E;      // largest biased exponent of each row (zeroed before where trans), [batch][rows]
+  uint32_t* D; // digit planes, [batch][7][rows, or 2 rows for op(B)][ldk]
+  __host__ __device__ unsigned expo_blocks(int K) const {
+    return trans ? (unsigned)((rows + 31) / 32) * ((K + 63) / 64) : (unsigned)((rows + 7) / 8);
+  }
+  __host__ __device__ unsigned pack_blocks(int K) const { return (unsigned)((rows + 31) / 32) * ((K + 31) / 32); }
+};
 
-// the same of every column (E zeroed before; rows in pieces of 64 along blockIdx.y)
-__global__ void __launch_bounds__(256) k_dig_expo_cols(const double2* __restrict__ S, long ld, long ss, int rows,
-                                                       int cols, int* __restrict__ E) {
+// The largest exponents of both operands' rows: of rows as stored by a warp each, of stored columns by 32 columns x 64 of K
+// per block.  Also clears the marks.
+__global__ void __launch_bounds__(256) k_dig_expo(const DigOp A, const DigOp B, int K, const Marks<double2> marks) {
   __shared__ int red[8][32];
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, b = blockIdx.z;
-  const int c = blockIdx.x * 32 + tx, r0 = blockIdx.y * 64;
+  const bool first = blockIdx.x < A.expo_blocks(K);
+  const DigOp& o = first ? A : B;
+  const int blk = first ? blockIdx.x : blockIdx.x - A.expo_blocks(K), b = blockIdx.z;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  marks.clear(((long)b * gridDim.x + blockIdx.x) * 256 + threadIdx.x, (long)gridDim.z * gridDim.x * 256);
+  const double2* S = o.S + (long)b * o.ss;
   int e = 1;
-  if (c < cols) {
+  if (!o.trans) {
+    const int r = blk * 8 + ty;
+    if (r >= o.rows) return;
+    const double2* p = S + (long)r * o.ld;
+#pragma unroll 4
+    for (int k = tx; k < K; k += 32) e = max(e, expo(p[k]));
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (tx == 0) o.E[(long)b * o.rows + r] = e;
+    return;
+  }
+  const int kb = (K + 63) / 64, r = blk / kb * 32 + tx, k0 = blk % kb * 64;
+  if (r < o.rows) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const int r = r0 + ty + 8 * i;
-      if (r < rows) e = max(e, expo(S[(long)b * ss + (long)r * ld + c]));
+      const int k = k0 + ty + 8 * i;
+      if (k < K) e = max(e, expo(S[(long)k * o.ld + r]));
     }
   }
   red[ty][tx] = e;
   __syncthreads();
-  if (ty == 0 && c < cols) {
+  if (ty == 0 && r < o.rows) {
 #pragma unroll
     for (int i = 1; i < 8; ++i) e = max(e, red[i][tx]);
-    atomicMax(E + (long)b * cols + c, e);
+    atomicMax(o.E + (long)b * o.rows + r, e);
   }
 }
 
@@ -118,44 +136,42 @@ __device__ __forceinline__ uint32_t digit_bf16(unsigned long long y, int s) {
   return __float_as_uint(__uint_as_float(0x4B000000u | byte) - (8388608.0f + 128.0f)) >> 16;
 }
 
-// One stored complex matrix to digit planes D[(b * 7 + s)][row][2K] (row length ldk elements).
-//   TRANS: stored K x rows (read through 32 x 32 tiles), else rows x K;
-//   EXPAND: op(B), two rows 2r and 2r + 1 per column r: (yr, -yi) and (yi, yr); else op(A): (ar, ai);
-//   conj: the stored matrix enters conjugated.
-// Blocks of 32 rows x 32 of K, all along blockIdx.x: rows / 32 passes the 65535 of the other two.
-template <bool TRANS, bool EXPAND>
-__global__ void __launch_bounds__(256) k_dig_pack(const double2* __restrict__ S, long ld, long ss, int rows, int K,
-                                                  bool conj, const int* __restrict__ E, uint32_t* __restrict__ D,
-                                                  long ldk) {
-  __shared__ double2 t[TRANS ? 32 : 1][33];
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, b = blockIdx.z;
-  const int kblocks = (K + 31) / 32, k0 = blockIdx.x % kblocks * 32, r0 = blockIdx.x / kblocks * 32;
-  S += (long)b * ss;
-  if (TRANS) {
+// Both operands to digit planes, 32 rows x 32 of K per block (all along blockIdx.x: rows / 32 passes the 65535 of
+// the other dimensions); stored columns are read through a 32 x 32 tile.  op(A): rows (ar, ai); op(B):
+// two rows 2r and 2r + 1 per column r, (yr, -yi) and (yi, yr).
+__global__ void __launch_bounds__(256) k_dig_pack(const DigOp A, const DigOp B, int K, long ldk) {
+  __shared__ double2 t[32][33];
+  const bool first = blockIdx.x < A.pack_blocks(K);
+  const DigOp& o = first ? A : B;
+  const int blk = first ? blockIdx.x : blockIdx.x - A.pack_blocks(K), b = blockIdx.z;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int kblocks = (K + 31) / 32, k0 = blk % kblocks * 32, r0 = blk / kblocks * 32, rows = o.rows;
+  const double2* S = o.S + (long)b * o.ss;
+  if (o.trans) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int k = k0 + ty + 8 * i, r = r0 + tx;
-      t[ty + 8 * i][tx] = (k < K && r < rows) ? S[(long)k * ld + r] : make_double2(0.0, 0.0);
+      t[ty + 8 * i][tx] = (k < K && r < rows) ? S[(long)k * o.ld + r] : make_double2(0.0, 0.0);
     }
     __syncthreads();
   }
   const int k = k0 + tx;
   if (k >= K) return;
-  const long plane = (long)rows * (EXPAND ? 2 : 1) * (ldk / 2);  // 32-bit words of a digit plane
+  const long plane = (long)rows * (first ? 1 : 2) * (ldk / 2);  // 32-bit words of a digit plane
+  const uint32_t sign = (o.conj == first) ? 0x8000u : 0u;  // of the imaginary part in the first row
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int r = r0 + ty + 8 * i;
     if (r >= rows) continue;
-    const double2 v = TRANS ? t[tx][ty + 8 * i] : S[(long)r * ld + k];
-    const int e = E[(long)b * rows + r];
+    const double2 v = o.trans ? t[tx][ty + 8 * i] : S[(long)r * o.ld + k];
+    const int e = o.E[(long)b * rows + r];
     const unsigned long long x = biased_digits(v.x, e), y = biased_digits(v.y, e);
-    uint32_t* dst = D + (long)b * DG_D * plane + (long)(EXPAND ? 2 * r : r) * (ldk / 2) + k;
-    const uint32_t sign = (conj != EXPAND) ? 0x8000u : 0u;  // of the imaginary part in the first row
+    uint32_t* dst = o.D + (long)b * DG_D * plane + (long)(first ? r : 2 * r) * (ldk / 2) + k;
 #pragma unroll
     for (int s = 0; s < DG_D; ++s) {
       const uint32_t re = digit_bf16(x, s), im = digit_bf16(y, s);
       dst[s * plane] = re | ((im ^ sign) << 16);
-      if (EXPAND) dst[s * plane + ldk / 2] = (im ^ (sign ^ 0x8000u)) | (re << 16);
+      if (!first) dst[s * plane + ldk / 2] = (im ^ (sign ^ 0x8000u)) | (re << 16);
     }
   }
 }
@@ -186,8 +202,8 @@ __device__ __forceinline__ double fixed_to_double(long long hi, long long lo, in
 
 __global__ void __launch_bounds__(DG_THREADS, 1) k_dgemm_tc(const __grid_constant__ CUtensorMap tmA,
                                                             const __grid_constant__ CUtensorMap tmB,
-                                                            const __grid_constant__ DotSrc<double2> src,
                                                             const int* __restrict__ EA, const int* __restrict__ EB,
+                                                            const __grid_constant__ Marks<double2> marks,
                                                             double2* __restrict__ C, long ldc, long sC, int M, int N,
                                                             int nk, int batch, double alpha, int beta, int upper) {
   extern __shared__ unsigned char dg_raw[];
@@ -347,29 +363,25 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dgemm_tc(const __grid_constan
         mbar_arrive(tempty);
       }
       const Tile w = tile(t);
-      const int row = w.m0 + (warp & 3) * 32 + lane;
-      if (row < M) {
-        const int ea = EA[(long)w.bz * M + row];
-        double2* crow = C + (long)w.bz * sC + (long)row * ldc;
+      const int row0 = w.m0 + (warp & 3) * 32, row = row0 + lane;
+      if (row0 >= M) continue;
+      const int ea = row < M ? EA[(long)w.bz * M + row] : 0;
+      double2* crow = C + (long)w.bz * sC + (long)row * ldc;
 #pragma unroll
-        for (int q = 0; q < DG_OUT; q += 2) {
-          const int col = (w.n0 + col0 + q) >> 1;
-          if (col < N) {
-            const int eb = EB[(long)w.bz * N + col];
-            double2 v;
-            if (ok && ea < 0x7ff && eb < 0x7ff) {
-              const int e = ea + eb + 40 - 2 * 1077;  // the levels carry 256^5 = 2^40
-              v = make_double2(fixed_to_double(hi[q], lo[q], e), fixed_to_double(hi[q + 1], lo[q + 1], e));
-            } else if (ok && src.A) {  // a row or column holding an infinity or NaN
-              v = direct_dot(src, w.bz, row, col);
-            } else {  // (or its operand overwritten in place, or a pipeline that gave up)
-              v = make_double2(__longlong_as_double(0x7ff8000000000000ll), __longlong_as_double(0x7ff8000000000000ll));
-            }
-            if (alpha != 1.0) v = cscale(v, alpha);
-            if (beta) v = cadd(v, crow[col]);
-            crow[col] = v;
-          }
-        }
+      for (int q = 0; q < DG_OUT; q += 2) {
+        const int col = (w.n0 + col0 + q) >> 1;
+        if (col >= N) continue;  // the same for the whole warp
+        const int eb = EB[(long)w.bz * N + col];
+        // a row or column holding an infinity or NaN: its digits say nothing, left to k_redo
+        const bool mark = ok && row < M && (ea >= 0x7ff || eb >= 0x7ff);
+        marks.put(M, N, w.bz, row0, col, mark, row, col, lane);
+        if (mark || row >= M) continue;
+        const int e = ea + eb + 40 - 2 * 1077;  // the levels carry 256^5 = 2^40
+        double2 v = make_double2(fixed_to_double(hi[q], lo[q], e), fixed_to_double(hi[q + 1], lo[q + 1], e));
+        if (!ok) v = make_double2(__longlong_as_double(0x7ff8000000000000ll), __longlong_as_double(0x7ff8000000000000ll));
+        if (alpha != 1.0) v = cscale(v, alpha);
+        if (beta) v = cadd(v, crow[col]);
+        crow[col] = v;
       }
     }
   }
@@ -400,7 +412,7 @@ static int digit_map(CUtensorMap* tm, const void* ptr, int rows, int K2, long ld
 
 static long dg_ldk(int K) { return (2L * K + 7) / 8 * 8; }
 static size_t dg_slice_bytes(int M, int N, int K) {
-  return (size_t)DG_D * dg_ldk(K) * 2 * (M + 2 * (size_t)N) + 4 * ((size_t)M + N);
+  return (size_t)DG_D * dg_ldk(K) * 2 * (M + 2 * (size_t)N) + 4 * ((size_t)M + N) + Marks<double2>::bytes(M, N, 1);
 }
 size_t dgemm_tc_bytes(int M, int N, int K, int batch) {
   return std::min<size_t>(dg_slice_bytes(M, N, K) * batch, (size_t)3 << 30) + dg_slice_bytes(M, N, K) + 2048;
@@ -426,14 +438,16 @@ int dgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s, bool upp
   const int N2 = 2 * g.N;
   // slices per pass: the digits of both operands in the scratch
   uintptr_t p0 = ((uintptr_t)ws + 255) & ~(uintptr_t)255;
-  const size_t avail = bytes - (p0 - (uintptr_t)ws) - 1024;
-  const int nb = (int)std::min<size_t>(g.batch, avail / dg_slice_bytes(g.M, g.N, g.K));
+  const size_t off = p0 - (uintptr_t)ws + 1024;  // alignments
+  const int nb = bytes < off ? 0 : (int)std::min<size_t>(g.batch, (bytes - off) / dg_slice_bytes(g.M, g.N, g.K));
   if (nb < 1) return TSVD_ERR_WORKSPACE;
+  if (g.C == g.A || g.C == g.B) return TSVD_ERR_INVALID_ARG;  // k_redo reads the operands once more
   auto up = [](uintptr_t p) { return (p + 255) & ~(uintptr_t)255; };
   uint32_t* DA = (uint32_t*)p0;
   uint32_t* DB = (uint32_t*)up(p0 + (size_t)nb * DG_D * g.M * ldk * 2);
   int* EA = (int*)up((uintptr_t)DB + (size_t)nb * DG_D * N2 * ldk * 2);
   int* EB = EA + (size_t)nb * g.M;
+  const Marks<double2> marks = Marks<double2>::at(up((uintptr_t)(EB + (size_t)nb * g.N)), g.M, g.N, nb);
   if (cudaFuncSetAttribute(k_dgemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, DG_SMEM) != cudaSuccess) {
     cudaGetLastError();
     return TSVD_ERR_CUDA;
@@ -443,30 +457,24 @@ int dgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s, bool upp
     const bool ta = g.opA == 'H', tb = g.opB == 'N';
     const double2* A = (const double2*)g.A + (long)b0 * g.sA;
     const double2* B = (const double2*)g.B + (long)b0 * g.sB;
+    const DigOp oa{A, g.lda, g.sA, g.M, ta, ta, EA, DA}, ob{B, g.ldb, g.sB, g.N, tb, !tb, EB, DB};
     if ((ta || tb) && cudaMemsetAsync(EA, 0, sizeof(int) * (size_t)nb * (g.M + g.N), s) != cudaSuccess)
       return TSVD_ERR_CUDA;
-    if (ta) k_dig_expo_cols<<<dim3(cdiv(g.M, 32), cdiv(g.K, 64), n), 256, 0, s>>>(A, g.lda, g.sA, g.K, g.M, EA);
-    else k_dig_expo_rows<<<dim3(cdiv(g.M, 8), n), 256, 0, s>>>(A, g.lda, g.sA, g.M, g.K, EA);
+    k_dig_expo<<<dim3(oa.expo_blocks(g.K) + ob.expo_blocks(g.K), 1, n), 256, 0, s>>>(oa, ob, g.K, marks);
     TSVD_LAUNCHED();
-    if (tb) k_dig_expo_cols<<<dim3(cdiv(g.N, 32), cdiv(g.K, 64), n), 256, 0, s>>>(B, g.ldb, g.sB, g.K, g.N, EB);
-    else k_dig_expo_rows<<<dim3(cdiv(g.N, 8), n), 256, 0, s>>>(B, g.ldb, g.sB, g.N, g.K, EB);
-    TSVD_LAUNCHED();
-    const dim3 ga(cdiv(g.K, 32) * cdiv(g.M, 32), 1, n), gb(cdiv(g.K, 32) * cdiv(g.N, 32), 1, n);
-    if (ta) k_dig_pack<true, false><<<ga, 256, 0, s>>>(A, g.lda, g.sA, g.M, g.K, true, EA, DA, ldk);
-    else k_dig_pack<false, false><<<ga, 256, 0, s>>>(A, g.lda, g.sA, g.M, g.K, false, EA, DA, ldk);
-    TSVD_LAUNCHED();
-    if (tb) k_dig_pack<true, true><<<gb, 256, 0, s>>>(B, g.ldb, g.sB, g.N, g.K, false, EB, DB, ldk);
-    else k_dig_pack<false, true><<<gb, 256, 0, s>>>(B, g.ldb, g.sB, g.N, g.K, true, EB, DB, ldk);
+    k_dig_pack<<<dim3(oa.pack_blocks(g.K) + ob.pack_blocks(g.K), 1, n), 256, 0, s>>>(oa, ob, g.K, ldk);
     TSVD_LAUNCHED();
     CUtensorMap ma, mb;
     TSVD_TRY(digit_map(&ma, DA, g.M, 2 * g.K, ldk, n * DG_D, DG_BM));
     TSVD_TRY(digit_map(&mb, DB, N2, 2 * g.K, ldk, n * DG_D, DG_BN));
     const long tiles = (long)cdiv(N2, DG_BN) * cdiv(g.M, DG_BM) * n;  // one per CTA where some are skipped
     const unsigned grid = (unsigned)(upper ? tiles : std::min<long>(tiles, 152));
-    const DotSrc<double2> src{g.C == g.A || g.C == g.B ? nullptr : A, B, g.lda, g.sA, g.ldb, g.sB, g.K, ta, !tb};
-    k_dgemm_tc<<<grid, DG_THREADS, DG_SMEM, s>>>(ma, mb, src, EA, EB, (double2*)g.C + (long)b0 * g.sC, g.ldc, g.sC, g.M,
-                                                 g.N, cdiv(2L * g.K, DG_KB), n, g.alpha, g.beta != 0.0, upper ? 1 : 0);
+    double2* Cb = (double2*)g.C + (long)b0 * g.sC;
+    k_dgemm_tc<<<grid, DG_THREADS, DG_SMEM, s>>>(ma, mb, EA, EB, marks, Cb, g.ldc, g.sC, g.M, g.N,
+                                                 cdiv(2L * g.K, DG_KB), n, g.alpha, g.beta != 0.0, upper ? 1 : 0);
     TSVD_LAUNCHED();
+    TSVD_TRY(redo_marked<double2>(marks, {A, B, g.lda, g.sA, g.ldb, g.sB, g.K, ta, !tb}, Cb, g.ldc, g.sC, g.M, g.N, n,
+                                  g.alpha, g.beta != 0.0, upper, s));
   }
   return TSVD_OK;
 }

@@ -85,7 +85,8 @@ int cgemm_herm(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStre
 // dgemm_tc.cu -- the FP64 product as exact digit products on the BF16 tensor cores (cgemm and
 // cgemm_herm take it where dgemm_tc_better says so and the scratch holds one slice's digits):
 // bytes of scratch for the whole product (bounded; more slices than fit are done in passes), and
-// the product itself (alpha +-1, beta 0 or 1; upper: only the tiles not wholly below the diagonal)
+// the product itself (alpha +-1, beta 0 or 1, C neither operand; upper: only the tiles not wholly below the
+// diagonal)
 size_t dgemm_tc_bytes(int M, int N, int K, int batch);
 bool dgemm_tc_better(const GemmArgs& g, size_t bytes);
 int dgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s, bool upper);
@@ -116,8 +117,7 @@ int copy_cx(const C* src, long lds, long ss, C* dst, long ldd, long sd, int rows
 template <typename GC>
 int chol_inv(const GC* G, long ldg, long sG, GC* M, long ldm, long sM, int nb, int batch, double shift_rel,
              double dead_rel, uint32_t* dead, cudaStream_t s);
-// O <- W M for the n1 x nb blocks of every slice (M nb x nb dense); O may be W itself (each CTA
-// stages its rows of W before writing).
+// O <- W M for the n1 x nb blocks of every slice (M nb x nb dense)
 template <typename C>
 int rmul_block(const C* W, long ldw, long sW, const C* M, long ldm, long sM, int n1, int nb, int batch, C* O, long ldo,
                long sO, cudaStream_t s);

@@ -25,6 +25,7 @@
 #include "common.cuh"
 #include "kernels.cuh"
 #include "tc_common.cuh"
+#include "tc_redo.cuh"
 
 namespace tsvd {
 
@@ -46,43 +47,56 @@ __device__ __forceinline__ float rna_tf32(float x) {
   return __uint_as_float(r);
 }
 
-// One stored complex matrix to hi / lo rows of 2K floats (row length ldk): TRANS, EXPAND and conj
-// and the blocks as in k_dig_pack.
-template <bool TRANS, bool EXPAND>
-__global__ void __launch_bounds__(256) k_split_pack(const float2* __restrict__ S, long ld, long ss, int rows, int K,
-                                                    bool conj, float* __restrict__ Hi, float* __restrict__ Lo,
-                                                    long ldk) {
-  __shared__ float2 t[TRANS ? 32 : 1][33];
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, b = blockIdx.z;
-  const int kblocks = (K + 31) / 32, k0 = blockIdx.x % kblocks * 32, r0 = blockIdx.x / kblocks * 32;
-  S += (long)b * ss;
-  if (TRANS) {
+// one operand as k_split_pack sees it: rows (columns of op(B)) of K elements
+struct SplitOp {
+  const float2* S;
+  long ld, ss;
+  int rows;
+  bool trans;  // stored K x rows, else rows x K
+  bool conj;   // enters conjugated
+  float *Hi, *Lo;
+  __host__ __device__ unsigned blocks(int K) const { return (unsigned)((rows + 31) / 32) * ((K + 31) / 32); }
+};
+
+// Both operands to hi / lo rows of 2K floats (row length ldk): blocks and rows as in k_dig_pack.  Also clears
+// the marks.
+__global__ void __launch_bounds__(256) k_split_pack(const SplitOp A, const SplitOp B, int K, long ldk,
+                                                    const Marks<float2> marks) {
+  __shared__ float2 t[32][33];
+  const bool first = blockIdx.x < A.blocks(K);
+  const SplitOp& o = first ? A : B;
+  const int blk = first ? blockIdx.x : blockIdx.x - A.blocks(K), b = blockIdx.z;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int kblocks = (K + 31) / 32, k0 = blk % kblocks * 32, r0 = blk / kblocks * 32, rows = o.rows;
+  marks.clear(((long)b * gridDim.x + blockIdx.x) * 256 + threadIdx.x, (long)gridDim.z * gridDim.x * 256);
+  const float2* S = o.S + (long)b * o.ss;
+  if (o.trans) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int k = k0 + ty + 8 * i, r = r0 + tx;
-      t[ty + 8 * i][tx] = (k < K && r < rows) ? S[(long)k * ld + r] : make_float2(0.f, 0.f);
+      t[ty + 8 * i][tx] = (k < K && r < rows) ? S[(long)k * o.ld + r] : make_float2(0.f, 0.f);
     }
     __syncthreads();
   }
   const int k = k0 + tx;
   if (k >= K) return;
-  const long so = (long)b * rows * (EXPAND ? 2 : 1) * ldk;
+  const long so = (long)b * rows * (first ? 1 : 2) * ldk;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int r = r0 + ty + 8 * i;
     if (r >= rows) continue;
-    float2 v = TRANS ? t[tx][ty + 8 * i] : S[(long)r * ld + k];
-    if (conj) v.y = -v.y;
+    float2 v = o.trans ? t[tx][ty + 8 * i] : S[(long)r * o.ld + k];
+    if (o.conj) v.y = -v.y;
     const float hx = rna_tf32(v.x), hy = rna_tf32(v.y), lx = rna_tf32(v.x - hx), ly = rna_tf32(v.y - hy);
-    const long o = so + (long)(EXPAND ? 2 * r : r) * ldk + 2 * k;
-    if (EXPAND) {
-      *(float2*)(Hi + o) = make_float2(hx, -hy);
-      *(float2*)(Lo + o) = make_float2(lx, -ly);
-      *(float2*)(Hi + o + ldk) = make_float2(hy, hx);
-      *(float2*)(Lo + o + ldk) = make_float2(ly, lx);
+    const long at = so + (long)(first ? r : 2 * r) * ldk + 2 * k;
+    if (first) {
+      *(float2*)(o.Hi + at) = make_float2(hx, hy);
+      *(float2*)(o.Lo + at) = make_float2(lx, ly);
     } else {
-      *(float2*)(Hi + o) = make_float2(hx, hy);
-      *(float2*)(Lo + o) = make_float2(lx, ly);
+      *(float2*)(o.Hi + at) = make_float2(hx, -hy);
+      *(float2*)(o.Lo + at) = make_float2(lx, -ly);
+      *(float2*)(o.Hi + at + ldk) = make_float2(hy, hx);
+      *(float2*)(o.Lo + at + ldk) = make_float2(ly, lx);
     }
   }
 }
@@ -91,7 +105,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constan
                                                             const __grid_constant__ CUtensorMap tmAl,
                                                             const __grid_constant__ CUtensorMap tmBh,
                                                             const __grid_constant__ CUtensorMap tmBl,
-                                                            const __grid_constant__ DotSrc<float2> src,
+                                                            const __grid_constant__ Marks<float2> marks,
                                                             float2* __restrict__ C, long ldc, long sC, int M, int N,
                                                             int nk, int batch, float alpha, int beta) {
   extern __shared__ unsigned char sg_raw[];
@@ -216,6 +230,11 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constan
           }
         }
       }
+      // operands that are not finite, or whose hi part overflowed: the warp looks which of its elements (rare)
+      float zero = 0.f;
+#pragma unroll
+      for (int q = 0; q < SG_OUT; ++q) zero = fmaf(tot[q], 0.f, zero);
+      const bool spoiled = __any_sync(0xffffffffu, ok && zero != zero);
       // 32 columns at a time through shared memory, so that eight lanes write 128 bytes of a row
 #pragma unroll
       for (int c0 = 0; c0 < SG_OUT; c0 += 32) {
@@ -225,28 +244,34 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constan
           stg[lane * 8 + (q ^ (lane & 7))] =
               make_float4(tot[c0 + 4 * q], tot[c0 + 4 * q + 1], tot[c0 + 4 * q + 2], tot[c0 + 4 * q + 3]);
         __syncwarp();
-        const int col = ((w.n0 + col0 + c0) >> 1) + 2 * (lane & 7);
-        if (col >= N) continue;
+        const int cb = (w.n0 + col0 + c0) >> 1, col = cb + 2 * (lane & 7);
+        if (cb >= N) continue;
 #pragma unroll 2
         for (int i = 0; i < 8; ++i) {
           const int r = 4 * i + (lane >> 3), row = w.m0 + row0 + r;
-          if (row >= M) break;
+          if (w.m0 + row0 + 4 * i >= M) break;  // the same for the whole warp
           const float4 x = stg[r * 8 + ((lane & 7) ^ (r & 7))];
           float2* dst = C + (long)w.bz * sC + (long)row * ldc + col;
           float2 v[2] = {make_float2(alpha * x.x, alpha * x.y), make_float2(alpha * x.z, alpha * x.w)};
+          bool out[2] = {row < M && col < N, row < M && col + 1 < N};
+          if (spoiled) {
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              const bool mark = out[u] && !(fabsf(v[u].x) <= FLT_MAX && fabsf(v[u].y) <= FLT_MAX);
+              marks.put(M, N, w.bz, w.m0 + row0 + 4 * i, cb + u, mark, row, col + u, lane);
+              out[u] = out[u] && !mark;
+            }
+          }
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
-            if (col + u >= N) continue;
             if (!ok) v[u] = make_float2(__int_as_float(0x7fc00000), __int_as_float(0x7fc00000));
-            else if (src.A && !(fabsf(v[u].x) <= FLT_MAX && fabsf(v[u].y) <= FLT_MAX))  // operands that are not finite
-              v[u] = cscale(direct_dot(src, w.bz, row, col + u), alpha);
-            if (beta) v[u] = cadd(v[u], dst[u]);
+            if (beta && out[u]) v[u] = cadd(v[u], dst[u]);
           }
-          if (col + 1 < N && ((uintptr_t)dst & 15) == 0) {
+          if (out[0] && out[1] && ((uintptr_t)dst & 15) == 0) {
             *(float4*)dst = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
           } else {
-            dst[0] = v[0];
-            if (col + 1 < N) dst[1] = v[1];
+            if (out[0]) dst[0] = v[0];
+            if (out[1]) dst[1] = v[1];
           }
         }
       }
@@ -278,7 +303,9 @@ static int split_map(CUtensorMap* tm, const float* ptr, int rows, int K2, long l
 }
 
 static long sg_ldk(int K) { return (2L * K + 3) / 4 * 4; }
-static size_t sg_slice_bytes(int M, int N, int K) { return 8 * (size_t)sg_ldk(K) * (M + 2 * (size_t)N); }
+static size_t sg_slice_bytes(int M, int N, int K) {
+  return 8 * (size_t)sg_ldk(K) * (M + 2 * (size_t)N) + Marks<float2>::bytes(M, N, 1);
+}
 size_t sgemm_tc_bytes(int M, int N, int K, int batch) {
   return std::min<size_t>(sg_slice_bytes(M, N, K) * batch, (size_t)3 << 30) + sg_slice_bytes(M, N, K) + 2048;
 }
@@ -309,15 +336,17 @@ int sgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s) {
   const long ldk = sg_ldk(g.K);
   const int N2 = 2 * g.N;
   const uintptr_t p0 = ((uintptr_t)ws + 255) & ~(uintptr_t)255;
-  const size_t avail = bytes - (p0 - (uintptr_t)ws) - 1024;
-  const int nb = (int)std::min<size_t>(g.batch, avail / sg_slice_bytes(g.M, g.N, g.K));
+  const size_t off = p0 - (uintptr_t)ws + 1280;  // alignments
+  const int nb = bytes < off ? 0 : (int)std::min<size_t>(g.batch, (bytes - off) / sg_slice_bytes(g.M, g.N, g.K));
   if (nb < 1) return TSVD_ERR_WORKSPACE;
+  if (g.C == g.A || g.C == g.B) return TSVD_ERR_INVALID_ARG;  // k_redo reads the operands once more
   auto up = [](uintptr_t p) { return (p + 255) & ~(uintptr_t)255; };
   const size_t an = (size_t)nb * g.M * ldk * 4, bn = (size_t)nb * N2 * ldk * 4;
   float* Ah = (float*)p0;
   float* Al = (float*)up(p0 + an);
   float* Bh = (float*)up((uintptr_t)Al + an);
   float* Bl = (float*)up((uintptr_t)Bh + bn);
+  const Marks<float2> marks = Marks<float2>::at(up((uintptr_t)Bl + bn), g.M, g.N, nb);
   if (cudaFuncSetAttribute(k_sgemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, SG_SMEM) != cudaSuccess) {
     cudaGetLastError();
     return TSVD_ERR_CUDA;
@@ -326,24 +355,23 @@ int sgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s) {
     const int n = std::min(nb, g.batch - b0);
     const float2* A = (const float2*)g.A + (long)b0 * g.sA;
     const float2* B = (const float2*)g.B + (long)b0 * g.sB;
-    const dim3 ga(cdiv(g.K, 32) * cdiv(g.M, 32), 1, n), gb(cdiv(g.K, 32) * cdiv(g.N, 32), 1, n);
-    if (g.opA == 'H') k_split_pack<true, false><<<ga, 256, 0, s>>>(A, g.lda, g.sA, g.M, g.K, true, Ah, Al, ldk);
-    else k_split_pack<false, false><<<ga, 256, 0, s>>>(A, g.lda, g.sA, g.M, g.K, false, Ah, Al, ldk);
-    TSVD_LAUNCHED();
-    if (g.opB == 'N') k_split_pack<true, true><<<gb, 256, 0, s>>>(B, g.ldb, g.sB, g.N, g.K, false, Bh, Bl, ldk);
-    else k_split_pack<false, true><<<gb, 256, 0, s>>>(B, g.ldb, g.sB, g.N, g.K, true, Bh, Bl, ldk);
+    const SplitOp oa{A, g.lda, g.sA, g.M, g.opA == 'H', g.opA == 'H', Ah, Al};
+    const SplitOp ob{B, g.ldb, g.sB, g.N, g.opB == 'N', g.opB == 'H', Bh, Bl};
+    k_split_pack<<<dim3(oa.blocks(g.K) + ob.blocks(g.K), 1, n), 256, 0, s>>>(oa, ob, g.K, ldk, marks);
     TSVD_LAUNCHED();
     CUtensorMap mah, mal, mbh, mbl;
     TSVD_TRY(split_map(&mah, Ah, g.M, 2 * g.K, ldk, n));
     TSVD_TRY(split_map(&mal, Al, g.M, 2 * g.K, ldk, n));
     TSVD_TRY(split_map(&mbh, Bh, N2, 2 * g.K, ldk, n));
     TSVD_TRY(split_map(&mbl, Bl, N2, 2 * g.K, ldk, n));
-    const DotSrc<float2> src{g.C == g.A || g.C == g.B ? nullptr : A, B, g.lda, g.sA, g.ldb, g.sB, g.K, g.opA == 'H', g.opB == 'H'};
     const long tiles = (long)cdiv(N2, SG_BN) * cdiv(g.M, SG_BM) * n;
+    float2* Cb = (float2*)g.C + (long)b0 * g.sC;
     k_sgemm_tc<<<(unsigned)std::min<long>(tiles, 152), SG_THREADS, SG_SMEM, s>>>(
-        mah, mal, mbh, mbl, src, (float2*)g.C + (long)b0 * g.sC, g.ldc, g.sC, g.M, g.N, cdiv(2L * g.K, SG_KB), n,
-        (float)g.alpha, g.beta != 0.0);
+        mah, mal, mbh, mbl, marks, Cb, g.ldc, g.sC, g.M, g.N, cdiv(2L * g.K, SG_KB), n, (float)g.alpha,
+        g.beta != 0.0);
     TSVD_LAUNCHED();
+    TSVD_TRY(redo_marked<float2>(marks, {A, B, g.lda, g.sA, g.ldb, g.sB, g.K, g.opA == 'H', g.opB == 'H'}, Cb,
+                                 g.ldc, g.sC, g.M, g.N, n, g.alpha, g.beta != 0.0, false, s));
   }
   return TSVD_OK;
 }

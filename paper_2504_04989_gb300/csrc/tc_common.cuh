@@ -117,30 +117,6 @@ __device__ __forceinline__ void ring_drain(Ring<N> r, long filled, uint32_t bar)
   }
 }
 
-// The operands of a complex product as stored, for the elements whose tensor-core sum is not a
-// number because an operand is not finite (its digits or its lo part say nothing): those are summed
-// again directly.
-template <typename C>
-struct DotSrc {
-  const C *A, *B;
-  long lda, sA, ldb, sB;
-  int K;
-  bool ah, bh;
-};
-template <typename C>
-__device__ __noinline__ C direct_dot(const DotSrc<C>& s, int b, int i, int j) {
-  const C* A = s.A + (long)b * s.sA;
-  const C* B = s.B + (long)b * s.sB;
-  C acc;
-  acc.x = acc.y = 0;
-  for (int k = 0; k < s.K; ++k) {
-    const C x = s.ah ? cconj(A[(long)k * s.lda + i]) : A[(long)i * s.lda + k];
-    const C y = s.bh ? cconj(B[(long)j * s.ldb + k]) : B[(long)k * s.ldb + j];
-    cfma(acc, x, y);
-  }
-  return acc;
-}
-
 // the tensor-map encoder of the driver (looked up once)
 inline PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
