@@ -102,12 +102,13 @@ struct Marks {
 };
 
 constexpr int REDO_THREADS = 64;
+constexpr int REDO_RUN = 16;  // terms added one after another, then the runs: the same sum from the list and by tiles
 template <typename C>
 constexpr int redo_tile() { return sizeof(C) == 16 ? 16 : 32; }
 
 // upper: a Hermitian product, whose tiles of 128 rows x 32 columns wholly below the diagonal were left out (no marks there)
 template <typename C>
-__global__ void __launch_bounds__(REDO_THREADS) k_redo(const Marks<C> mk, const __grid_constant__ DotSrc<C> src,
+__global__ void __launch_bounds__(REDO_THREADS, 8) k_redo(const Marks<C> mk, const __grid_constant__ DotSrc<C> src,
                                                        C* __restrict__ Cm, long ldc, long sC, int M, int N, int batch,
                                                        double alpha, int beta, int upper) {
   using R = decltype(C().x);
@@ -123,25 +124,35 @@ __global__ void __launch_bounds__(REDO_THREADS) k_redo(const Marks<C> mk, const 
   if (count <= mk.cap) {
     for (long e = (long)blockIdx.x * 2 + (tid >> 5); e < count; e += (long)gridDim.x * 2) {
       const long at = mk.list[e];
-      const int j = (int)(at % N), i = (int)(at / N % M), b = (int)(at / N / M);
-      C acc = mkc(R(0), R(0));
-      for (int k0 = 0; k0 < src.K; k0 += 128) {
+      const long r = at / N;
+      const int j = (int)(at - r * N), b = (int)(r / M), i = (int)(r - (long)b * M);
+      C tot = mkc(R(0), R(0));
+      for (int k0 = 0; k0 < src.K; k0 += 32 * REDO_RUN) {  // a run per lane, added in their order
+        C acc = mkc(R(0), R(0));
+        const int kb = k0 + REDO_RUN * lane;
+        const int ke = min(kb + REDO_RUN, src.K);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int k = k0 + 32 * u + lane;
-          if (k < src.K) cfma(acc, src.a(b, i, k), src.b(b, k, j));
+        for (int u = 0; u < REDO_RUN; u += 8) {  // eight terms' loads in flight
+          C x[8], y[8];
+#pragma unroll
+          for (int v = 0; v < 8; ++v) {
+            const int k = min(kb + u + v, src.K - 1);
+            x[v] = src.a(b, i, k);
+            y[v] = src.b(b, k, j);
+          }
+#pragma unroll
+          for (int v = 0; v < 8; ++v)
+            if (kb + u + v < ke) cfma(acc, x[v], y[v]);
         }
+        const int runs = min(32, (src.K - k0 + REDO_RUN - 1) / REDO_RUN);
+        for (int q = 0; q < runs; ++q)
+          tot = cadd(tot, mkc(__shfl_sync(0xffffffffu, acc.x, q), __shfl_sync(0xffffffffu, acc.y, q)));
       }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
-      }
-      if (lane == 0) put(b, i, j, acc);
+      if (lane == 0) put(b, i, j, tot);
     }
     return;
   }
-  constexpr int BT = redo_tile<C>(), BK = 16, RT = BT / 8, NS = BT * BK / REDO_THREADS;
+  constexpr int BT = redo_tile<C>(), BK = REDO_RUN, RT = BT / 8, NS = BT * BK / REDO_THREADS;
   __shared__ __align__(16) C As[BK][BT + 1], Bs[BK][BT + 1];
   const int tx = tid & 7, ty = tid >> 3;
   const long tm = (M + BT - 1) / BT, tn = (N + BT - 1) / BT, tiles = tm * tn * batch;
@@ -158,7 +169,7 @@ __global__ void __launch_bounds__(REDO_THREADS) k_redo(const Marks<C> mk, const 
         some |= mark[x][y];
       }
     if (!__syncthreads_or(some)) continue;
-    C acc[RT][RT], tot[RT][RT];  // sums of 64 terms, then their sum
+    C acc[RT][RT], tot[RT][RT];
 #pragma unroll
     for (int x = 0; x < RT; ++x)
 #pragma unroll
@@ -185,15 +196,13 @@ __global__ void __launch_bounds__(REDO_THREADS) k_redo(const Marks<C> mk, const 
 #pragma unroll
           for (int y = 0; y < RT; ++y) cfma(acc[x][y], a[x], c[y]);
       }
-      if ((k0 & 63) == 64 - BK || k0 + BK >= src.K) {
 #pragma unroll
-        for (int x = 0; x < RT; ++x)
+      for (int x = 0; x < RT; ++x)
 #pragma unroll
-          for (int y = 0; y < RT; ++y) {
-            tot[x][y] = cadd(tot[x][y], acc[x][y]);
-            acc[x][y] = mkc(R(0), R(0));
-          }
-      }
+        for (int y = 0; y < RT; ++y) {
+          tot[x][y] = cadd(tot[x][y], acc[x][y]);
+          acc[x][y] = mkc(R(0), R(0));
+        }
       __syncthreads();
     }
 #pragma unroll
