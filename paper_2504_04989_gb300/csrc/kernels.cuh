@@ -91,7 +91,7 @@ size_t dgemm_tc_bytes(int M, int N, int K, int batch);
 bool dgemm_tc_better(const GemmArgs& g, size_t bytes);
 int dgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s, bool upper);
 
-// sgemm_tc.cu -- the FP32 product on the TF32 tensor cores at FP32 accuracy (cgemm takes it where
+// sgemm_tc.cu -- the FP32 product on the BF16 tensor cores, operands in three exact parts (cgemm takes it where
 // sgemm_tc_better says so), as above
 size_t sgemm_tc_bytes(int M, int N, int K, int batch);
 bool sgemm_tc_better(const GemmArgs& g, size_t bytes);

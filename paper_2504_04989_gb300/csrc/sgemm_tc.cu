@@ -1,25 +1,29 @@
-// sgemm_tc.cu -- FP32 complex GEMM on the TF32 tensor cores with FP32 accuracy.
+// sgemm_tc.cu -- FP32 complex GEMM on the BF16 tensor cores, exact operands.
 //
-// Each operand is split x = hi + lo, hi the nearest TF32 and lo the nearest TF32 of
-// the rest (2^-23 relative), and hi hi + hi lo + lo hi is accumulated on tcgen05.  The
-// tensor cores truncate when they add to an accumulator (measured: a sum kept in TMEM
-// shrinks by about 2e-8 per instruction, 1.4e-5 after 1024 complex terms), so an
-// accumulator holds 32 terms of K only -- hi hi and the two small products apart, as B's hi
-// and lo rows lie one after another and one instruction multiplies A hi with both -- and
-// is then read and added to sums in registers, rounded to nearest, in runs of eight
-// readings; two pairs of accumulators alternate so that the reading runs under the next
-// products, and a CTA walks over several tiles so that the next tile's loads and products
-// run under the writing of this one.  Against exact dot products of normal data the result
-// is closer than FP32 multiply-adds' (the figures stand at sgemm_tc_better).
+// Each operand is the sum of three BF16 numbers, x = b0 + b1 + b2, each the nearest to what is left:
+// 8 + 8 + 8 bits, so the split is exact.  The six products b_i b_j with i + j <= 2 are accumulated on
+// tcgen05 (those left out lie below 2^-26 of the product, under half its FP32 rounding), at the price of
+// three of the TF32 rate.  The tensor cores truncate when they add to an accumulator (measured: a sum
+// kept in TMEM shrinks by about 2e-8 per instruction, 1.4e-5 after 1024 complex terms), so an accumulator
+// holds 32 terms of K of b0 b0 only, two instructions on products of 16 bits that rarely lose any,
+// and is then read and added to sums in registers, rounded to nearest, in runs of eight
+// readings; the five small products, 2^-9 of those and less, have accumulators of their own that are read once a run.  Two
+// pairs of accumulators alternate so that the reading runs under the next products, and a CTA walks over several tiles so that the next tile's loads and products
+// run under the writing of this one.  Against exact dot products the result is closer than FP32
+// multiply-adds' at every K (the figures stand at sgemm_tc_better).
+//
+// Near the ends of FP32's range the parts or their products leave it: an entry below 2^-100 (its b2), a sum below 2^-98 per
+// term with products below 2^-100 in it, results that are not finite.  The pass over the operands notes how small the
+// entries of each row get, and the elements concerned are left to k_redo.
 //
 // A complex product is the real product of the interleaved rows of op(A) with the
 // expanded real form of op(B) (rows 2n and 2n + 1 per column n, as in tc_gemm.cu),
-// both written as hi / lo rows by one pass over each operand.
+// both written as three planes by one pass over the operands.
 //
-// Bound: shared memory, 144 KB read and filled per 128 x 128 x 32 block (1125 clocks at 128
-// bytes per clock; the products alone take 768).  K = 100 (2048 x 2048 on 65 slices, most of it
-// writing): 2.13 -> 1.70 ms by walking over tiles; K = 1024: 1.82 -> 1.81 ms by reading A hi
-// once for both, 1.92 with 16 reading warps instead of 8.
+// Bound: shared memory, 136 KB read and filled per 128 x 128 x 32 block (1063 clocks at 128
+// bytes per clock; the products alone take 768).
+#include <cuda_bf16.h>
+
 #include <cmath>
 
 #include "common.cuh"
@@ -29,11 +33,13 @@
 
 namespace tsvd {
 
+constexpr int SG_D = 3;                  // BF16 parts
 constexpr int SG_BM = 128, SG_BN = 128;  // complex rows x real columns
-constexpr int SG_KB = 32;                // K per stage: rows of 128 bytes, 128-byte swizzle
-constexpr int SG_STAGES = 3;
-constexpr int SG_TILE = SG_BM * SG_KB * 4;
-constexpr int SG_STAGE_BYTES = 4 * SG_TILE;  // A hi, A lo, B hi, B lo
+constexpr int SG_KB = 64;                // K per stage: rows of 128 bytes, 128-byte swizzle
+constexpr int SG_STAGES = 2;
+constexpr int SG_KA = 32;                // K per reading of the accumulators
+constexpr int SG_TILE = SG_BM * SG_KB * 2;        // one part of either operand
+constexpr int SG_STAGE_BYTES = 2 * SG_D * SG_TILE;  // A, B
 constexpr int SG_RUN = 8;                // readings summed before they join the total
 constexpr int SG_DRAIN = 256;            // threads reading the accumulators, then one TMA and one MMA warp
 constexpr int SG_THREADS = SG_DRAIN + 64;
@@ -41,25 +47,30 @@ constexpr int SG_OUT = SG_BN / 2;        // columns per reading thread
 constexpr int SG_SMEM = SG_STAGES * SG_STAGE_BYTES + 1024 + 256 + SG_DRAIN / 32 * 4096;  // 4 KB per reading warp
 static_assert(SG_SMEM <= 227 * 1024, "the stages must fit a CTA's shared memory");
 
-__device__ __forceinline__ float rna_tf32(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return __uint_as_float(r);
-}
-
-// one operand as k_split_pack sees it: rows (columns of op(B)) of K elements
+// one operand as its pass sees it: rows (columns of op(B)) of K elements
 struct SplitOp {
   const float2* S;
   long ld, ss;
   int rows;
   bool trans;  // stored K x rows, else rows x K
   bool conj;   // enters conjugated
-  float *Hi, *Lo;
+  uint8_t* low;  // [batch][rows][lowk]: per 32 of K, bits 0 to 3: an entry below 2^-25, 2^-50, 2^-75, 2^-100
+  uint32_t* D;   // planes of the parts, [batch][3][rows, or 2 rows for op(B)][ldk]
   __host__ __device__ unsigned blocks(int K) const { return (unsigned)((rows + 31) / 32) * ((K + 31) / 32); }
 };
+__host__ __device__ __forceinline__ int sg_lowk(int K) { return ((K + 31) / 32 + 7) / 8 * 8; }  // read 8 bytes at a time
 
-// Both operands to hi / lo rows of 2K floats (row length ldk): blocks and rows as in k_dig_pack.  Also clears
-// the marks.
+// the three parts' bits
+__device__ __forceinline__ void bf16_parts(float x, uint32_t (&b)[SG_D]) {
+#pragma unroll
+  for (int s = 0; s < SG_D; ++s) {
+    const __nv_bfloat16 h = __float2bfloat16_rn(x);
+    b[s] = __bfloat16_as_ushort(h);
+    x -= __bfloat162float(h);
+  }
+}
+
+// Both operands to planes of parts: blocks, tiles and rows as in k_dig_pack.  Also clears the marks.
 __global__ void __launch_bounds__(256) k_split_pack(const SplitOp A, const SplitOp B, int K, long ldk,
                                                     const Marks<float2> marks) {
   __shared__ float2 t[32][33];
@@ -67,7 +78,7 @@ __global__ void __launch_bounds__(256) k_split_pack(const SplitOp A, const Split
   const SplitOp& o = first ? A : B;
   const int blk = first ? blockIdx.x : blockIdx.x - A.blocks(K), b = blockIdx.z;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int kblocks = (K + 31) / 32, k0 = blk % kblocks * 32, r0 = blk / kblocks * 32, rows = o.rows;
+  const int kblocks = (K + 31) / 32, kb = blk % kblocks, k0 = kb * 32, r0 = blk / kblocks * 32, rows = o.rows;
   marks.clear(((long)b * gridDim.x + blockIdx.x) * 256 + threadIdx.x, (long)gridDim.z * gridDim.x * 256);
   const float2* S = o.S + (long)b * o.ss;
   if (o.trans) {
@@ -79,36 +90,42 @@ __global__ void __launch_bounds__(256) k_split_pack(const SplitOp A, const Split
     __syncthreads();
   }
   const int k = k0 + tx;
-  if (k >= K) return;
-  const long so = (long)b * rows * (first ? 1 : 2) * ldk;
+  const long plane = (long)rows * (first ? 1 : 2) * (ldk / 2);  // 32-bit words of a plane
+  const uint32_t sign = (o.conj == first) ? 0x8000u : 0u;  // of the imaginary part in the first row
+  const int lowk = sg_lowk(K);
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const int r = r0 + ty + 8 * i;
-    if (r >= rows) continue;
-    float2 v = o.trans ? t[tx][ty + 8 * i] : S[(long)r * o.ld + k];
-    if (o.conj) v.y = -v.y;
-    const float hx = rna_tf32(v.x), hy = rna_tf32(v.y), lx = rna_tf32(v.x - hx), ly = rna_tf32(v.y - hy);
-    const long at = so + (long)(first ? r : 2 * r) * ldk + 2 * k;
-    if (first) {
-      *(float2*)(o.Hi + at) = make_float2(hx, hy);
-      *(float2*)(o.Lo + at) = make_float2(lx, ly);
-    } else {
-      *(float2*)(o.Hi + at) = make_float2(hx, -hy);
-      *(float2*)(o.Lo + at) = make_float2(lx, -ly);
-      *(float2*)(o.Hi + at + ldk) = make_float2(hy, hx);
-      *(float2*)(o.Lo + at + ldk) = make_float2(ly, lx);
+    const int r = r0 + ty + 8 * i;  // the same for the whole warp
+    if (r >= rows) break;
+    float2 v = make_float2(0.f, 0.f);
+    if (k < K) v = o.trans ? t[tx][ty + 8 * i] : S[(long)r * o.ld + k];
+    const float x = v.x != 0.f ? fabsf(v.x) : 1.f, y = v.y != 0.f ? fabsf(v.y) : 1.f;
+    const unsigned least = __reduce_min_sync(0xffffffffu, __float_as_uint(fminf(x, y))) >> 23;  // its exponent
+    if (tx < (kb == kblocks - 1 ? lowk - kb : 1))  // the last block fills up the row
+      o.low[((long)b * rows + r) * lowk + kb + tx] =
+          tx ? 0 : (least < 102) + 2 * (least < 77) + 4 * (least < 52) + 8 * (least < 27);
+    if (k >= K) continue;
+    uint32_t re[SG_D], im[SG_D];
+    bf16_parts(v.x, re);
+    bf16_parts(v.y, im);
+    uint32_t* dst = o.D + (long)b * SG_D * plane + (long)(first ? r : 2 * r) * (ldk / 2) + k;
+#pragma unroll
+    for (int s = 0; s < SG_D; ++s) {
+      dst[s * plane] = re[s] | ((im[s] ^ sign) << 16);
+      if (!first) dst[s * plane + ldk / 2] = (im[s] ^ (sign ^ 0x8000u)) | (re[s] << 16);
     }
   }
 }
 
-__global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constant__ CUtensorMap tmAh,
-                                                            const __grid_constant__ CUtensorMap tmAl,
-                                                            const __grid_constant__ CUtensorMap tmBh,
-                                                            const __grid_constant__ CUtensorMap tmBl,
+__global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constant__ CUtensorMap tmA,
+                                                            const __grid_constant__ CUtensorMap tmB,
+                                                            const uint8_t* __restrict__ lowA,
+                                                            const uint8_t* __restrict__ lowB,
                                                             const __grid_constant__ Marks<float2> marks,
                                                             float2* __restrict__ C, long ldc, long sC, int M, int N,
-                                                            int nk, int batch, float alpha, int beta) {
+                                                            int K, int batch, float alpha, int beta) {
   extern __shared__ unsigned char sg_raw[];
+  const int nk = (2 * K + SG_KB - 1) / SG_KB, na = (2 * K + SG_KA - 1) / SG_KA;  // stages and readings of a tile
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int tn = (2 * N + SG_BN - 1) / SG_BN, tm = (M + SG_BM - 1) / SG_BM;
   const int tiles = tn * tm * batch;  // at least one element each: within an int
@@ -161,34 +178,60 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constan
         }
         const uint32_t dst = smem_u32(base + s * SG_STAGE_BYTES), bar = full0 + 8 * s;
         mbar_expect_tx(bar, SG_STAGE_BYTES);
-        tma_load_3d(dst, &tmAh, kb * SG_KB, w.m0, w.bz, bar);
-        tma_load_3d(dst + 2 * SG_TILE, &tmBh, kb * SG_KB, w.n0, w.bz, bar);
-        tma_load_3d(dst + SG_TILE, &tmAl, kb * SG_KB, w.m0, w.bz, bar);
-        tma_load_3d(dst + 3 * SG_TILE, &tmBl, kb * SG_KB, w.n0, w.bz, bar);
+        tma_load_3d(dst, &tmA, kb * SG_KB, w.m0, w.bz * SG_D, bar);
+        tma_load_3d(dst + SG_D * SG_TILE, &tmB, kb * SG_KB, w.n0, w.bz * SG_D, bar);
       }
     }
     ring_drain(r, filled, full0);
   } else if (tid == SG_DRAIN + 32) {  // MMA issuer
-    const uint32_t idesc0 = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(SG_BM >> 4) << 24);  // FP32 += TF32 TF32^T
+    const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(SG_BM >> 4) << 24);  // FP32 += BF16 BF16^T
     const uint32_t idesc1 = idesc0 | ((uint32_t)(SG_BN >> 3) << 17), idesc2 = idesc0 | ((uint32_t)(2 * SG_BN >> 3) << 17);
-    const long last = (long)((tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1) * nk;
     Ring<SG_STAGES> r;
     Ring<2> ra;
-    for (long g = 0; g < last; ++g, r.next(), ra.next()) {
-      const int s = r.s, a = ra.s;
-      if (!mbar_wait(tempty + 8 * a, ra.ph ^ 1)) break;
-      if (!mbar_wait(full0 + 8 * s, r.ph)) break;
-      asm volatile("tcgen05.fence::after_thread_sync;");
-      const uint32_t sm = smem_u32(base + s * SG_STAGE_BYTES);
-      const uint64_t ah = smem_desc_sw128(sm), al = smem_desc_sw128(sm + SG_TILE);
-      const uint64_t bb = smem_desc_sw128(sm + 2 * SG_TILE);  // B hi, B lo: 256 rows
-      const uint32_t d = tmem + (uint32_t)(a * 2 * SG_BN);
+    bool ok = true;
+    for (int t = blockIdx.x; ok && t < tiles; t += gridDim.x) {
+      for (int kb = 0; ok && kb < nk; ++kb, r.next()) {
+        const int s = r.s;
+        if (!mbar_wait(full0 + 8 * s, r.ph)) {
+          ok = false;
+          break;
+        }
+        const uint32_t sm = smem_u32(base + s * SG_STAGE_BYTES);
+        uint64_t pa[SG_D], pb[SG_D];
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk) mma_issue<false>(d, ah + 2 * kk, bb + 2 * kk, idesc2, kk > 0);  // 32 bytes of K
+        for (int i = 0; i < SG_D; ++i) {
+          pa[i] = smem_desc_sw128(sm + i * SG_TILE);
+          pb[i] = smem_desc_sw128(sm + (SG_D + i) * SG_TILE);
+        }
+        const int parts = min(SG_KB / SG_KA, na - kb * (SG_KB / SG_KA));
+        for (int p = 0; p < parts; ++p, ra.next()) {
+          const int a = ra.s;
+          if (!mbar_wait(tempty + 8 * a, ra.ph ^ 1)) {
+            ok = false;
+            break;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;");
+          const uint32_t d = tmem + (uint32_t)(a * 2 * SG_BN);
+          const int j = kb * (SG_KB / SG_KA) + p;
+          const bool fresh = (j & (SG_RUN - 1)) < 2;  // the run's first use of this pair
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk) mma_issue<false>(d + SG_BN, al + 2 * kk, bb + 2 * kk, idesc1, 1);
-      mma_commit(empty0 + 8 * s);
-      mma_commit(tfull + 8 * a);
+          for (int kk = 0; kk < SG_KA / 16; ++kk) {
+            const int at = 2 * (p * (SG_KA / 16) + kk);  // 32 bytes of K
+            if (kk == 0) {
+              mma_issue<true>(d, pa[0] + at, pb[0] + at, idesc1, 0);
+              mma_issue<true>(d + SG_BN, pa[0] + at, pb[1] + at, idesc1, fresh ? 0 : 1);
+            } else {
+              mma_issue<true>(d, pa[0] + at, pb[0] + at, idesc2, 1);  // b0 b0 | b0 b1
+            }
+            mma_issue<true>(d + SG_BN, pa[0] + at, pb[2] + at, idesc1, 1);
+            mma_issue<true>(d + SG_BN, pa[1] + at, pb[0] + at, idesc1, 1);
+            mma_issue<true>(d + SG_BN, pa[1] + at, pb[1] + at, idesc1, 1);
+            mma_issue<true>(d + SG_BN, pa[2] + at, pb[0] + at, idesc1, 1);
+          }
+          mma_commit(tfull + 8 * a);
+        }
+        if (ok) mma_commit(empty0 + 8 * s);
+      }
     }
   } else if (warp < SG_DRAIN / 32) {
     const int row0 = (warp & 3) * 32, col0 = (warp >> 2) * SG_OUT;
@@ -198,31 +241,40 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constan
     bool ok = true;
     for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
       const Tile w = tile(t);
+      // notes of small entries in this lane's row and column: the first 256 of K ahead of the sums
+      const int lr = min(w.m0 + row0 + lane, M - 1), lc = min((w.n0 + col0) / 2 + lane, N - 1), lowk = sg_lowk(K);
+      const uint2* pr = (const uint2*)(lowA + ((long)w.bz * M + lr) * lowk);
+      const uint2* pc = (const uint2*)(lowB + ((long)w.bz * N + lc) * lowk);
+      const uint2 rl = pr[0], cl = pc[0];
       float run[SG_OUT], tot[SG_OUT];
 #pragma unroll
       for (int q = 0; q < SG_OUT; ++q) run[q] = tot[q] = 0.f;
-      for (int kb = 0; kb < nk && ok; ++kb, ra.next()) {
+      for (int kb = 0; kb < na && ok; ++kb, ra.next()) {
         const int a = ra.s;
         ok = mbar_wait(tfull + 8 * a, ra.ph);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;");
+        // the sums of b0 b0; those of the small products at the run's last use of the pair
+        const int halves = kb + 2 >= min(na, (kb & ~(SG_RUN - 1)) + SG_RUN) ? 2 : 1;
+        for (int h = 0; h < halves; ++h) {
 #pragma unroll
-        for (int q0 = 0; q0 < SG_OUT; q0 += 8) {
-          uint32_t r[2][8];  // hi hi, the small products
+          for (int q0 = 0; q0 < SG_OUT; q0 += 16) {
+            uint32_t r[16];
+            asm volatile(
+                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+                "%14, %15}, [%16];"
+                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                  "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                : "r"(tw + (uint32_t)((2 * a + h) * SG_BN + q0)));
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-          for (int h = 0; h < 2; ++h)
-            asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                         : "=r"(r[h][0]), "=r"(r[h][1]), "=r"(r[h][2]), "=r"(r[h][3]), "=r"(r[h][4]), "=r"(r[h][5]),
-                           "=r"(r[h][6]), "=r"(r[h][7])
-                         : "r"(tw + (uint32_t)((2 * a + h) * SG_BN + q0)));
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-          for (int u = 0; u < 8; ++u) run[q0 + u] += __uint_as_float(r[0][u]) + __uint_as_float(r[1][u]);
+            for (int u = 0; u < 16; ++u) run[q0 + u] += __uint_as_float(r[u]);
+          }
         }
         asm volatile("tcgen05.fence::before_thread_sync;");
         mbar_arrive(tempty + 8 * a);
-        if ((kb & (SG_RUN - 1)) == SG_RUN - 1 || kb == nk - 1) {
+        if ((kb & (SG_RUN - 1)) == SG_RUN - 1 || kb == na - 1) {
 #pragma unroll
           for (int q = 0; q < SG_OUT; ++q) {
             tot[q] += run[q];
@@ -230,11 +282,26 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constan
           }
         }
       }
-      // operands that are not finite, or whose hi part overflowed: the warp looks which of its elements (rare)
+      // results that are not finite, or entries near the lower end of the range: the warp looks which of its elements (rare)
       float zero = 0.f;
 #pragma unroll
       for (int q = 0; q < SG_OUT; ++q) zero = fmaf(tot[q], 0.f, zero);
-      const bool spoiled = __any_sync(0xffffffffu, ok && zero != zero);
+      uint32_t rlow = rl.x | rl.y, clow = cl.x | cl.y;
+#pragma unroll 4
+      for (int q = 1; q < lowk / 8; ++q) {
+        const uint2 x = pr[q], y = pc[q];
+        rlow |= x.x | x.y;
+        clow |= y.x | y.y;
+      }
+      auto level = [](uint32_t x) {  // entries of at least 2^(-25 (level + 1)); 4: smaller ones
+        x |= x >> 16;
+        return __popc((x | x >> 8) & 15u);
+      };
+      const int rlev = level(rlow), clev = level(clow);
+      const int rtop = __reduce_max_sync(0xffffffffu, rlev), ctop = __reduce_max_sync(0xffffffffu, clev);
+      // products below 2^-100 among them, or parts below 2^-124
+      const bool spoiled = ok && (__any_sync(0xffffffffu, zero != zero) || rtop + ctop > 2);
+      const float least = 0x1p-98f * (2.f * (float)K);
       // 32 columns at a time through shared memory, so that eight lanes write 128 bytes of a row
 #pragma unroll
       for (int c0 = 0; c0 < SG_OUT; c0 += 32) {
@@ -257,7 +324,11 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constan
           if (spoiled) {
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
-              const bool mark = out[u] && !(fabsf(v[u].x) <= FLT_MAX && fabsf(v[u].y) <= FLT_MAX);
+              const int rl4 = __shfl_sync(0xffffffffu, rlev, r);
+              const int cl4 = __shfl_sync(0xffffffffu, clev, c0 / 2 + 2 * (lane & 7) + u);
+              const float big = fmaxf(fabsf(v[u].x), fabsf(v[u].y));
+              const bool mark = out[u] && (!(fabsf(v[u].x) <= FLT_MAX && fabsf(v[u].y) <= FLT_MAX) ||
+                                           max(rl4, cl4) > 3 || (rl4 + cl4 > 2 && big < least));
               marks.put(M, N, w.bz, w.m0 + row0 + 4 * i, cb + u, mark, row, col + u, lane);
               out[u] = out[u] && !mark;
             }
@@ -289,32 +360,34 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constan
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-static int split_map(CUtensorMap* tm, const float* ptr, int rows, int K2, long ldk, int batch) {
+static int split_map(CUtensorMap* tm, const void* ptr, int rows, int K2, long ldk, int planes) {
   auto enc = get_encode();
   if (!enc) return TSVD_ERR_CUDA;
-  cuuint64_t dims[3] = {(cuuint64_t)K2, (cuuint64_t)rows, (cuuint64_t)batch};
-  cuuint64_t strides[2] = {(cuuint64_t)(ldk * 4), (cuuint64_t)(ldk * 4 * rows)};
-  cuuint32_t box[3] = {(cuuint32_t)SG_KB, 128, 1};
+  cuuint64_t dims[3] = {(cuuint64_t)K2, (cuuint64_t)rows, (cuuint64_t)planes};
+  cuuint64_t strides[2] = {(cuuint64_t)(ldk * 2), (cuuint64_t)(ldk * 2 * rows)};
+  cuuint32_t box[3] = {(cuuint32_t)SG_KB, 128, (cuuint32_t)SG_D};
   cuuint32_t estr[3] = {1, 1, 1};
-  const CUresult r = enc(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, (void*)ptr, dims, strides, box, estr,
+  const CUresult r = enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, (void*)ptr, dims, strides, box, estr,
                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? TSVD_OK : TSVD_ERR_UNSUPPORTED;
 }
 
-static long sg_ldk(int K) { return (2L * K + 3) / 4 * 4; }
+static long sg_ldk(int K) { return (2L * K + 7) / 8 * 8; }
 static size_t sg_slice_bytes(int M, int N, int K) {
-  return 8 * (size_t)sg_ldk(K) * (M + 2 * (size_t)N) + Marks<float2>::bytes(M, N, 1);
+  return SG_D * 2 * (size_t)sg_ldk(K) * (M + 2 * (size_t)N) + (size_t)sg_lowk(K) * ((size_t)M + N) +
+         Marks<float2>::bytes(M, N, 1);
 }
 size_t sgemm_tc_bytes(int M, int N, int K, int batch) {
   return std::min<size_t>(sg_slice_bytes(M, N, K) * batch, (size_t)3 << 30) + sg_slice_bytes(M, N, K) + 2048;
 }
 
 // Estimated times in microseconds of the two forms: a SIMT tile takes 0.104 (64 x 64) or 0.25 us (128 x
-// 64) per term of K and SM, K split as cgemm splits it.  Measured, product with its operand passes: 1024 x
-// 1024 x 1024 on 33 slices 5.08 -> 1.56 ms (the product alone 1.23: 230 TFLOP/s), 2048 x 100 x 2048 on
-// 17 1230 -> 561 us, 512 x 60 x 512 on 33 109 -> 70.  Error, 2-norm, normal data, K = 97, 512, 1024,
-// 2048, 4096: 1.4, 1.4, 1.4, 1.6, 1.8e-7, the SIMT kernels 1.8, 4.0, 2.6, 4.2, 4.5e-7.
+// 64) per term of K and SM, K split as cgemm splits it.  Measured, product with its operand pass: 1024 x
+// 1024 x 1024 on 33 slices 5.08 -> 1.61 ms (the product alone 1.28: 220 TFLOP/s).  Error, 2-norm, in 2^-24, normal data,
+// K = 32, 60, 128, 512, 2048: 0.8, 0.9, 1.1, 1.4, 1.7, the SIMT kernels 1.7, 2.3, 3.4, 6.8, 13.6; positive data 0.8, 0.9, 1.1, 1.0,
+// 1.2, SIMT 1.4, 2.0, 2.9, 5.9, 11.7 (two TF32 parts and three products, as this was: 2.1 .. 2.6 and 1.7 .. 1.9, from K = 56 on
+// below SIMT only).
 bool sgemm_tc_better(const GemmArgs& g, size_t bytes) {
   if (g.K < 1 || g.M < 1 || g.N < 1 || g.K > (1 << 24)) return false;
   const size_t slice = sg_slice_bytes(g.M, g.N, g.K) + 2048;
@@ -341,12 +414,11 @@ int sgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s) {
   if (nb < 1) return TSVD_ERR_WORKSPACE;
   if (g.C == g.A || g.C == g.B) return TSVD_ERR_INVALID_ARG;  // k_redo reads the operands once more
   auto up = [](uintptr_t p) { return (p + 255) & ~(uintptr_t)255; };
-  const size_t an = (size_t)nb * g.M * ldk * 4, bn = (size_t)nb * N2 * ldk * 4;
-  float* Ah = (float*)p0;
-  float* Al = (float*)up(p0 + an);
-  float* Bh = (float*)up((uintptr_t)Al + an);
-  float* Bl = (float*)up((uintptr_t)Bh + bn);
-  const Marks<float2> marks = Marks<float2>::at(up((uintptr_t)Bl + bn), g.M, g.N, nb);
+  uint32_t* DA = (uint32_t*)p0;
+  uint32_t* DB = (uint32_t*)up(p0 + (size_t)nb * SG_D * g.M * ldk * 2);
+  uint8_t* lowA = (uint8_t*)up((uintptr_t)DB + (size_t)nb * SG_D * N2 * ldk * 2);
+  uint8_t* lowB = lowA + (size_t)nb * g.M * sg_lowk(g.K);
+  const Marks<float2> marks = Marks<float2>::at(up((uintptr_t)(lowB + (size_t)nb * g.N * sg_lowk(g.K))), g.M, g.N, nb);
   if (cudaFuncSetAttribute(k_sgemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, SG_SMEM) != cudaSuccess) {
     cudaGetLastError();
     return TSVD_ERR_CUDA;
@@ -355,20 +427,17 @@ int sgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s) {
     const int n = std::min(nb, g.batch - b0);
     const float2* A = (const float2*)g.A + (long)b0 * g.sA;
     const float2* B = (const float2*)g.B + (long)b0 * g.sB;
-    const SplitOp oa{A, g.lda, g.sA, g.M, g.opA == 'H', g.opA == 'H', Ah, Al};
-    const SplitOp ob{B, g.ldb, g.sB, g.N, g.opB == 'N', g.opB == 'H', Bh, Bl};
+    const SplitOp oa{A, g.lda, g.sA, g.M, g.opA == 'H', g.opA == 'H', lowA, DA};
+    const SplitOp ob{B, g.ldb, g.sB, g.N, g.opB == 'N', g.opB == 'H', lowB, DB};
     k_split_pack<<<dim3(oa.blocks(g.K) + ob.blocks(g.K), 1, n), 256, 0, s>>>(oa, ob, g.K, ldk, marks);
     TSVD_LAUNCHED();
-    CUtensorMap mah, mal, mbh, mbl;
-    TSVD_TRY(split_map(&mah, Ah, g.M, 2 * g.K, ldk, n));
-    TSVD_TRY(split_map(&mal, Al, g.M, 2 * g.K, ldk, n));
-    TSVD_TRY(split_map(&mbh, Bh, N2, 2 * g.K, ldk, n));
-    TSVD_TRY(split_map(&mbl, Bl, N2, 2 * g.K, ldk, n));
+    CUtensorMap ma, mb;
+    TSVD_TRY(split_map(&ma, DA, g.M, 2 * g.K, ldk, n * SG_D));
+    TSVD_TRY(split_map(&mb, DB, N2, 2 * g.K, ldk, n * SG_D));
     const long tiles = (long)cdiv(N2, SG_BN) * cdiv(g.M, SG_BM) * n;
     float2* Cb = (float2*)g.C + (long)b0 * g.sC;
     k_sgemm_tc<<<(unsigned)std::min<long>(tiles, 152), SG_THREADS, SG_SMEM, s>>>(
-        mah, mal, mbh, mbl, marks, Cb, g.ldc, g.sC, g.M, g.N, cdiv(2L * g.K, SG_KB), n, (float)g.alpha,
-        g.beta != 0.0);
+        ma, mb, lowA, lowB, marks, Cb, g.ldc, g.sC, g.M, g.N, g.K, n, (float)g.alpha, g.beta != 0.0);
     TSVD_LAUNCHED();
     TSVD_TRY(redo_marked<float2>(marks, {A, B, g.lda, g.sA, g.ldb, g.sB, g.K, g.opA == 'H', g.opB == 'H'}, Cb,
                                  g.ldc, g.sC, g.M, g.N, n, g.alpha, g.beta != 0.0, false, s));
