@@ -96,10 +96,14 @@ typedef struct {
    64-bit integer multiply-adds on the SIMT units instead of its base-256 digit form on the BF16
    tensor cores.  Both give the same G to the bit; the flag exists to compare them. */
 #define TSVD_FLAG_GRAM_INT 32
+/* bit 6 (TSVD_FLAG_EXPIRE): for tests: every wait in the pipelines of the FP64 and FP32 tensor-core
+   products gives up at once, as after their limit of about a second.  The call ends as usual;
+   info->status is TSVD_ERR_CUDA where such a product was taken, and the outputs mean nothing then. */
+#define TSVD_FLAG_EXPIRE 64
 
 /* ---- device-side outcome, read back only when requested ---- */
 typedef struct {
-  int status;          /* TSVD_OK or TSVD_ERR_NOT_CONVERGED */
+  int status;          /* TSVD_OK, TSVD_ERR_NOT_CONVERGED, or TSVD_ERR_CUDA: a tensor-core product gave up */
   int m_eff;           /* basis columns per slice: min((q+1)(R+P), n1, n2) */
   int dead_columns;    /* Krylov columns found numerically dependent and replaced (all slices) */
   int reserved;

@@ -385,13 +385,13 @@ static int cgemm_tiles(const GemmArgs& g, C* ws, size_t splitk_elems, cudaStream
 }
 
 template <typename C>
-static int cgemm_impl(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t s, int herm) {
+static int cgemm_impl(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t s, int herm, TcOpts st) {
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return TSVD_OK;
   if (g.batch > 65535) return TSVD_ERR_UNSUPPORTED;
   if (g.beta != 0.0 && g.beta != 1.0) return TSVD_ERR_INVALID_ARG;
   if constexpr (std::is_same<C, float2>::value) {
     const size_t bytes = splitk_ws ? splitk_elems * sizeof(C) : 0;
-    if (!g.simt && !herm && sgemm_tc_better(g, bytes)) return sgemm_tc(g, splitk_ws, bytes, s);
+    if (!g.simt && !herm && sgemm_tc_better(g, bytes)) return sgemm_tc(g, splitk_ws, bytes, s, st);
     // the wide tiles where they fill the GPU (two CTAs per SM), directly or by splitting a long K;
     // smaller products keep the 64 x 64 tiles (measured faster there)
     const long wtiles = (long)cdiv(g.M, WBM) * cdiv(g.N, WBN) * g.batch;
@@ -401,7 +401,7 @@ static int cgemm_impl(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, c
   if constexpr (std::is_same<C, double2>::value) {
     const size_t bytes = splitk_ws ? splitk_elems * sizeof(C) : 0;
     if (!g.simt && dgemm_tc_better(g, bytes)) {
-      TSVD_TRY(dgemm_tc(g, splitk_ws, bytes, s, herm != 0));
+      TSVD_TRY(dgemm_tc(g, splitk_ws, bytes, s, herm != 0, st));
       return herm ? mirror_lower<C>(g, s) : TSVD_OK;
     }
   }
@@ -415,8 +415,8 @@ static int cgemm_impl(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, c
 }
 
 template <typename C>
-int cgemm(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t s) {
-  return cgemm_impl<C>(g, splitk_ws, splitk_elems, s, 0);
+int cgemm(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t s, TcOpts st) {
+  return cgemm_impl<C>(g, splitk_ws, splitk_elems, s, 0, st);
 }
 
 template <typename C>
@@ -434,14 +434,14 @@ template size_t cgemm_scratch<double2>(int, int, int, int);
 template size_t cgemm_scratch<float2>(int, int, int, int);
 
 template <typename C>
-int cgemm_herm(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t s) {
+int cgemm_herm(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t s, TcOpts st) {
   if (g.M != g.N || g.beta != 0.0) return TSVD_ERR_INVALID_ARG;
-  return cgemm_impl<C>(g, splitk_ws, splitk_elems, s, 1);
+  return cgemm_impl<C>(g, splitk_ws, splitk_elems, s, 1, st);
 }
-template int cgemm_herm<double2>(const GemmArgs&, void*, size_t, cudaStream_t);
-template int cgemm_herm<float2>(const GemmArgs&, void*, size_t, cudaStream_t);
-template int cgemm<double2>(const GemmArgs&, void*, size_t, cudaStream_t);
-template int cgemm<float2>(const GemmArgs&, void*, size_t, cudaStream_t);
+template int cgemm_herm<double2>(const GemmArgs&, void*, size_t, cudaStream_t, TcOpts);
+template int cgemm_herm<float2>(const GemmArgs&, void*, size_t, cudaStream_t, TcOpts);
+template int cgemm<double2>(const GemmArgs&, void*, size_t, cudaStream_t, TcOpts);
+template int cgemm<float2>(const GemmArgs&, void*, size_t, cudaStream_t, TcOpts);
 
 // ---------------------------------------------------------------------------
 template <typename S, typename D>

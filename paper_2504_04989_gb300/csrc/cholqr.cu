@@ -697,12 +697,12 @@ int orth_block_cols(int n1, int b, int m, int h, const OrthWs& w, int c, int nb,
     // FP32, the fast-decaying spectra of Sec. 5 Ex. 1 in FP64) lose accuracy
     if (c > 0) {
       TSVD_STAGE("orth_cgs", s);
-      TSVD_TRY(cgemm<CL>(gemm('H', 'N', c, nb, n1, 1.0, Q, m, sQ, X, ldx, sX, 0.0, P, nb, sP, h), w.splitk, sk, s));
-      TSVD_TRY(cgemm<CL>(gemm('N', 'N', n1, nb, c, -1.0, Q, m, sQ, P, nb, sP, 1.0, X, ldx, sX, h), w.splitk, sk, s));
+      TSVD_TRY(cgemm<CL>(gemm('H', 'N', c, nb, n1, 1.0, Q, m, sQ, X, ldx, sX, 0.0, P, nb, sP, h), w.splitk, sk, s, w.st));
+      TSVD_TRY(cgemm<CL>(gemm('N', 'N', n1, nb, c, -1.0, Q, m, sQ, P, nb, sP, 1.0, X, ldx, sX, h), w.splitk, sk, s, w.st));
     }
     {
       TSVD_STAGE("orth_gram", s);
-      TSVD_TRY(cgemm<CL>(gemm('H', 'N', nb, nb, n1, 1.0, X, ldx, sX, X, ldx, sX, 0.0, Gs, b, sG, h), w.splitk, sk, s));
+      TSVD_TRY(cgemm<CL>(gemm('H', 'N', nb, nb, n1, 1.0, X, ldx, sX, X, ldx, sX, 0.0, Gs, b, sG, h), w.splitk, sk, s, w.st));
     }
     CL* Mi = (CL*)w.Minv;  // R-tilde^{-1}, nb x nb per slice (leading dimension b)
     {
@@ -713,9 +713,9 @@ int orth_block_cols(int n1, int b, int m, int h, const OrthWs& w, int c, int nb,
       TSVD_STAGE("orth_trsm", s);
       const GemmArgs g = gemm('N', 'N', n1, nb, nb, 1.0, X, ldx, sX, Mi, b, sG, 0.0, Y, ldy, sY, h);
       if (std::is_same<L, double>::value && dgemm_tc_better(g, sk * sizeof(CL)))
-        TSVD_TRY(dgemm_tc(g, w.splitk, sk * sizeof(CL), s, false));
+        TSVD_TRY(dgemm_tc(g, w.splitk, sk * sizeof(CL), s, false, w.st));
       else if (std::is_same<L, float>::value && sgemm_tc_better(g, sk * sizeof(CL)))
-        TSVD_TRY(sgemm_tc(g, w.splitk, sk * sizeof(CL), s));
+        TSVD_TRY(sgemm_tc(g, w.splitk, sk * sizeof(CL), s, w.st));
       else
         TSVD_TRY(rmul_block<CL>(X, ldx, sX, Mi, b, sG, n1, nb, h, Y, ldy, sY, s));
     }

@@ -321,7 +321,8 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dgemm_tc(const __grid_constan
                                                             const uint32_t* __restrict__ nearB,
                                                             const __grid_constant__ Marks<double2> marks,
                                                             double2* __restrict__ C, long ldc, long sC, int M, int N,
-                                                            int K, int batch, double alpha, int beta, int upper) {
+                                                            int K, int batch, double alpha, int beta, int upper,
+                                                            TcOpts st) {
   extern __shared__ unsigned char dg_raw[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int tn = (2 * N + DG_BN - 1) / DG_BN, tm = (M + DG_BM - 1) / DG_BM;
@@ -359,6 +360,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dgemm_tc(const __grid_constan
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = *tslot;
+  auto wait = [&](uint32_t bar, uint32_t parity) { return !st.expire && mbar_wait(bar, parity); };
   const int nk = (2 * K + DG_KB - 1) / DG_KB, chunks = (nk + DG_CHUNK - 1) / DG_CHUNK;
 
   // stages and readings are counted through all tiles of the CTA, so loads and products of the next
@@ -372,7 +374,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dgemm_tc(const __grid_constan
       if (w.skip) continue;
       for (int kb = 0; kb < nk; ++kb, ++filled, r.next()) {
         const int s = r.s;
-        if (!mbar_wait(empty0 + 8 * s, r.ph ^ 1)) {
+        if (!wait(empty0 + 8 * s, r.ph ^ 1)) {
           ok = false;
           break;
         }
@@ -391,7 +393,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dgemm_tc(const __grid_constan
     for (int t = blockIdx.x; ok && t < tiles; t += gridDim.x) {
       if (tile(t).skip) continue;
       for (int c = 0; ok && c < chunks; ++c, ra.next()) {
-        if (!mbar_wait(tempty, ra.ph ^ 1)) {
+        if (!wait(tempty, ra.ph ^ 1)) {
           ok = false;
           break;
         }
@@ -399,7 +401,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dgemm_tc(const __grid_constan
         const int k1 = min(nk, (c + 1) * DG_CHUNK);
         for (int kb = c * DG_CHUNK; kb < k1; ++kb, r.next()) {
           const int s = r.s;
-          if (!mbar_wait(full0 + 8 * s, r.ph)) {
+          if (!wait(full0 + 8 * s, r.ph)) {
             ok = false;
             break;
           }
@@ -444,7 +446,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dgemm_tc(const __grid_constan
 #pragma unroll
       for (int q = 0; q < DG_OUT; ++q) hi[q] = lo[q] = 0;
       for (int c = 0; ok && c < chunks; ++c, ra.next()) {
-        ok = mbar_wait(tfull, ra.ph);
+        ok = wait(tfull, ra.ph);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;");
@@ -478,6 +480,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dgemm_tc(const __grid_constan
         asm volatile("tcgen05.fence::before_thread_sync;");
         mbar_arrive(tempty);
       }
+      if (!ok && lane == 0 && st.err) atomicExch(st.err, 1);
       const Tile w = tile(t);
       const int row0 = w.m0 + (warp & 3) * 32, row = row0 + lane;
       if (row0 >= M) continue;
@@ -563,7 +566,7 @@ bool dgemm_tc_better(const GemmArgs& g, size_t bytes) {
   return simt > 25.0 * calls + pack_us + std::ceil(tiles / 152.0) * tile_us;
 }
 
-int dgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s, bool upper) {
+int dgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s, bool upper, TcOpts st) {
   const long ldk = dg_ldk(g.K);
   const int N2 = 2 * g.N;
   // slices per pass: the digits of both operands in the scratch
@@ -605,7 +608,7 @@ int dgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s, bool upp
     const unsigned grid = (unsigned)(upper ? tiles : std::min<long>(tiles, 152));
     double2* Cb = (double2*)g.C + (long)b0 * g.sC;
     k_dgemm_tc<<<grid, DG_THREADS, DG_SMEM, s>>>(ma, mb, topA, topB, nearA, nearB, marks, Cb, g.ldc, g.sC, g.M, g.N,
-                                                 g.K, n, g.alpha, g.beta != 0.0, upper ? 1 : 0);
+                                                 g.K, n, g.alpha, g.beta != 0.0, upper ? 1 : 0, st);
     TSVD_LAUNCHED();
     TSVD_TRY(redo_marked<double2>(marks, {A, B, g.lda, g.sA, g.ldb, g.sB, g.K, ta, !tb}, Cb, g.ldc, g.sC, g.M, g.N, n,
                                   g.alpha, g.beta != 0.0, upper, s));

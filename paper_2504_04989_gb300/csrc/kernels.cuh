@@ -71,8 +71,14 @@ inline GemmArgs gemm(char opA, char opB, int M, int N, int K, double alpha, cons
   g.batch = batch;
   return g;
 }
+// Where a tensor-core product says that a wait of its pipeline ran out (its elements are NaN then): *err = 1, unless null.
+// expire (tests): the waits give up at once.
+struct TcOpts {
+  int* err = nullptr;
+  bool expire = false;
+};
 template <typename C>
-int cgemm(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t s);
+int cgemm(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t s, TcOpts st = TcOpts());
 // scratch elements with which cgemm can take its tensor-core form for an M x N x K product (0 where
 // it would keep to the SIMT units); a smaller splitk_elems only makes it slower
 template <typename C>
@@ -80,7 +86,7 @@ size_t cgemm_scratch(int M, int N, int K, int batch);
 // C = op(A) op(B) known to be Hermitian (square, beta = 0, e.g. A^H A): only
 // the upper tiles are computed, the lower triangle is mirrored from them
 template <typename C>
-int cgemm_herm(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t s);
+int cgemm_herm(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t s, TcOpts st = TcOpts());
 
 // dgemm_tc.cu -- the FP64 product as exact digit products on the BF16 tensor cores (cgemm and
 // cgemm_herm take it where dgemm_tc_better says so and the scratch holds one slice's digits):
@@ -89,13 +95,13 @@ int cgemm_herm(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStre
 // diagonal)
 size_t dgemm_tc_bytes(int M, int N, int K, int batch);
 bool dgemm_tc_better(const GemmArgs& g, size_t bytes);
-int dgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s, bool upper);
+int dgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s, bool upper, TcOpts st);
 
 // sgemm_tc.cu -- the FP32 product on the BF16 tensor cores, operands in three exact parts (cgemm takes it where
 // sgemm_tc_better says so), as above
 size_t sgemm_tc_bytes(int M, int N, int K, int batch);
 bool sgemm_tc_better(const GemmArgs& g, size_t bytes);
-int sgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s);
+int sgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s, TcOpts st);
 
 // element-wise conversions of batched complex matrices (rows x cols, leading dims)
 int convert_c64_to_c32(const double2* src, long lds, long ss, float2* dst, long ldd, long sd, int rows, int cols,
@@ -160,7 +166,8 @@ struct OrthWs {
   size_t splitk_elems;  // in double2 elements
   int k0;               // Fourier slice index of problem 0
   int nyq;              // index of the (real) Nyquist slice, n3/2 for an even n3, else -1
-  const OrthTc* tc;     // FP32: products on tcgen05 (split TF32), or nullptr for the SIMT GEMMs
+  const OrthTc* tc;     // FP32: products on tcgen05 (split TF32), or nullptr for cgemm's
+  TcOpts st;
 };
 template <typename L>
 int orth_block_cols(int n1, int b, int m, int h, const OrthWs& w, int c, int nb, int block_id, uint64_t seed,

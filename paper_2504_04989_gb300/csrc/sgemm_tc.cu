@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constan
                                                             const uint8_t* __restrict__ lowB,
                                                             const __grid_constant__ Marks<float2> marks,
                                                             float2* __restrict__ C, long ldc, long sC, int M, int N,
-                                                            int K, int batch, float alpha, int beta) {
+                                                            int K, int batch, float alpha, int beta, TcOpts st) {
   extern __shared__ unsigned char sg_raw[];
   const int nk = (2 * K + SG_KB - 1) / SG_KB, na = (2 * K + SG_KA - 1) / SG_KA;  // stages and readings of a tile
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -161,6 +161,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constan
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = *tslot;
+  auto wait = [&](uint32_t bar, uint32_t parity) { return !st.expire && mbar_wait(bar, parity); };
 
   // stages and accumulators are counted through all tiles of the CTA, so loads and products of the
   // next tile run under the writing of this one
@@ -172,7 +173,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constan
       const Tile w = tile(t);
       for (int kb = 0; kb < nk; ++kb, ++filled, r.next()) {
         const int s = r.s;
-        if (!mbar_wait(empty0 + 8 * s, r.ph ^ 1)) {
+        if (!wait(empty0 + 8 * s, r.ph ^ 1)) {
           ok = false;
           break;
         }
@@ -192,7 +193,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constan
     for (int t = blockIdx.x; ok && t < tiles; t += gridDim.x) {
       for (int kb = 0; ok && kb < nk; ++kb, r.next()) {
         const int s = r.s;
-        if (!mbar_wait(full0 + 8 * s, r.ph)) {
+        if (!wait(full0 + 8 * s, r.ph)) {
           ok = false;
           break;
         }
@@ -206,7 +207,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constan
         const int parts = min(SG_KB / SG_KA, na - kb * (SG_KB / SG_KA));
         for (int p = 0; p < parts; ++p, ra.next()) {
           const int a = ra.s;
-          if (!mbar_wait(tempty + 8 * a, ra.ph ^ 1)) {
+          if (!wait(tempty + 8 * a, ra.ph ^ 1)) {
             ok = false;
             break;
           }
@@ -251,7 +252,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constan
       for (int q = 0; q < SG_OUT; ++q) run[q] = tot[q] = 0.f;
       for (int kb = 0; kb < na && ok; ++kb, ra.next()) {
         const int a = ra.s;
-        ok = mbar_wait(tfull + 8 * a, ra.ph);
+        ok = wait(tfull + 8 * a, ra.ph);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;");
@@ -282,6 +283,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constan
           }
         }
       }
+      if (!ok && lane == 0 && st.err) atomicExch(st.err, 1);
       // results that are not finite, or entries near the lower end of the range: the warp looks which of its elements (rare)
       float zero = 0.f;
 #pragma unroll
@@ -405,7 +407,7 @@ bool sgemm_tc_better(const GemmArgs& g, size_t bytes) {
   return simt > 10.0 * calls + pack_us + std::ceil(tiles / 152.0) * tile_us;
 }
 
-int sgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s) {
+int sgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s, TcOpts st) {
   const long ldk = sg_ldk(g.K);
   const int N2 = 2 * g.N;
   const uintptr_t p0 = ((uintptr_t)ws + 255) & ~(uintptr_t)255;
@@ -437,7 +439,7 @@ int sgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s) {
     const long tiles = (long)cdiv(N2, SG_BN) * cdiv(g.M, SG_BM) * n;
     float2* Cb = (float2*)g.C + (long)b0 * g.sC;
     k_sgemm_tc<<<(unsigned)std::min<long>(tiles, 152), SG_THREADS, SG_SMEM, s>>>(
-        ma, mb, lowA, lowB, marks, Cb, g.ldc, g.sC, g.M, g.N, g.K, n, (float)g.alpha, g.beta != 0.0);
+        ma, mb, lowA, lowB, marks, Cb, g.ldc, g.sC, g.M, g.N, g.K, n, (float)g.alpha, g.beta != 0.0, st);
     TSVD_LAUNCHED();
     TSVD_TRY(redo_marked<float2>(marks, {A, B, g.lda, g.sA, g.ldb, g.sB, g.K, g.opA == 'H', g.opB == 'H'}, Cb,
                                  g.ldc, g.sC, g.M, g.N, n, g.alpha, g.beta != 0.0, false, s));

@@ -111,7 +111,8 @@ struct TqrWs {
   C* Tm;     // h x TRI_B x p (pinv)
   C* Xp;     // h x n2 x n1 (pinv)
   uint32_t* dead;
-  int* counters;
+  int* counters;  // [1] dead columns, [2] a product gave up
+  TcOpts st() const { return TcOpts{counters + 2}; }
   double2* splitk;
   size_t splitk_elems;  // double2 elements
   size_t bytes;
@@ -190,6 +191,7 @@ static int tqr_factor(const TqrDims& d, TqrWs<T>& w, const cx_t<T>* M, cudaStrea
   o.k0 = 0;
   o.nyq = (d.n3 % 2 == 0) ? d.n3 / 2 : -1;
   o.tc = nullptr;
+  o.st = w.st();
   for (int c = 0; c < p; c += b) {
     const int nb = std::min(b, p - c);
     TSVD_TRY(copy_cx<C>(M + c, Nc, (long)Mr * Nc, w.W, b, (long)Mr * b, Mr, nb, h, s));
@@ -198,14 +200,14 @@ static int tqr_factor(const TqrDims& d, TqrWs<T>& w, const cx_t<T>* M, cudaStrea
   // R = Q^H M, upper trapezoidal with a real diagonal
   TSVD_TRY(cgemm<C>(gemm('H', 'N', p, Nc, Mr, 1.0, w.Q, p, (long)Mr * p, M, Nc, (long)Mr * Nc, 0.0, w.Rh, Nc,
                          (long)p * Nc, h),
-                    w.splitk, sk, s));
+                    w.splitk, sk, s, w.st()));
   const long total = (long)h * p * Nc;
   k_triu_realdiag<T><<<std::min<long>(cdiv(total, 256), 8192), 256, 0, s>>>(w.Rh, p, Nc, h);
   TSVD_LAUNCHED();
   return TSVD_OK;
 }
 
-// status of the call into *info (synchronises): dead columns found at the
+// status of the call into *info (synchronises): a product that gave up; dead columns found at the
 // CholeskyQR pivots; for the pseudoinverse they mean a rank-deficient slice
 static int read_status(int* counters, cudaStream_t s, tsvd_info* info, int p, bool need_full_rank) {
   if (!info) return TSVD_OK;
@@ -213,7 +215,7 @@ static int read_status(int* counters, cudaStream_t s, tsvd_info* info, int p, bo
   if (cudaMemcpyAsync(host, counters, sizeof(host), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return TSVD_ERR_CUDA;
-  info->status = (need_full_rank && host[1] > 0) ? TSVD_ERR_RANK_DEFICIENT : TSVD_OK;
+  info->status = host[2] ? TSVD_ERR_CUDA : (need_full_rank && host[1] > 0) ? TSVD_ERR_RANK_DEFICIENT : TSVD_OK;
   info->dead_columns = host[1];
   info->m_eff = p;
   info->reserved = 0;
@@ -255,19 +257,19 @@ static int tpinv_run(const T* A, const TqrDims& d, T* Xout, void* ws, cudaStream
     const int r0 = I * TRI_B, e = r0 + TRI_B, rest = p - e;
     TSVD_TRY(cgemm<C>(gemm('N', 'N', TRI_B, rest, rest, 1.0, w.Rh + (long)r0 * p + e, p, sP, w.Rinv + (long)e * p + e,
                            p, sP, 0.0, w.Tm, p, (long)TRI_B * p, h),
-                      w.splitk, sk, s));
+                      w.splitk, sk, s, w.st()));
     TSVD_TRY(cgemm<C>(gemm('N', 'N', TRI_B, rest, TRI_B, -1.0, w.Rinv + (long)r0 * p + r0, p, sP, w.Tm, p,
                            (long)TRI_B * p, 0.0, w.Rinv + (long)r0 * p + e, p, sP, h),
-                      w.splitk, sk, s));
+                      w.splitk, sk, s, w.st()));
   }
   // X^+ = R^{-1} Q^H (p x Mr = n2 x n1) or Q R^{-H} (Mr x p = n2 x n1)
   const long sX = (long)d.n2 * d.n1;
   if (!d.wide)
     TSVD_TRY(cgemm<C>(gemm('N', 'H', p, Mr, p, 1.0, w.Rinv, p, sP, w.Q, p, (long)Mr * p, 0.0, w.Xp, d.n1, sX, h),
-                      w.splitk, sk, s));
+                      w.splitk, sk, s, w.st()));
   else
     TSVD_TRY(cgemm<C>(gemm('N', 'H', Mr, p, p, 1.0, w.Q, p, (long)Mr * p, w.Rinv, p, sP, 0.0, w.Xp, d.n1, sX, h),
-                      w.splitk, sk, s));
+                      w.splitk, sk, s, w.st()));
   TSVD_TRY(launch_irfft3<T>(w.Xp, Xout, sX, d.n3, s));
   return read_status(w.counters, s, info, p, true);
 }

@@ -44,6 +44,7 @@ struct RbkDims {
   int gsl;   // FP32 paths: the exact Gram in its digit form on the BF16 tensor cores
   int mp;    // basis columns used by the projection: m, or R+P with TSVD_FLAG_QTRUNC
   int deflate;  // deflated Rayleigh-Ritz passes for the small SVD (FP64 path)
+  int expire;   // the waits of cgemm's tensor-core products give up at once (tests)
 };
 
 static int rbk_dims(int n1, int n2, int n3, const tsvd_params* p, RbkDims* d) {
@@ -74,6 +75,7 @@ static int rbk_dims(int n1, int n2, int n3, const tsvd_params* p, RbkDims* d) {
   d->gsl = (d->tc3 && !(p->flags & TSVD_FLAG_GRAM_INT) && gram_sliced_ok(n2, d->m)) ? 1 : 0;
   d->mp = (p->flags & TSVD_FLAG_QTRUNC) ? std::min(d->b, d->m) : d->m;
   d->deflate = (p->flags & TSVD_FLAG_DEFLATE) ? 1 : 0;
+  d->expire = (p->flags & TSVD_FLAG_EXPIRE) ? 1 : 0;
   if (d->deflate && p->precision != TSVD_FP64) return TSVD_ERR_UNSUPPORTED;
   if (d->b > 128 || d->m > 512) return TSVD_ERR_UNSUPPORTED;
   if ((long)d->h * n1 * n2 > (1L << 40)) return TSVD_ERR_UNSUPPORTED;
@@ -99,7 +101,7 @@ struct RbkWs {
   int* colexp;    // their per-column exponents
   double2* Rs;
   uint32_t* dead;
-  int* counters;  // [0] status, [1] dead columns
+  int* counters;  // [0] status, [1] dead columns, [2] a tcgen05 pipeline wait ran out (tc_err)
   double2* G;
   double* lam;
   C* Uct;      // U_c (m x R per slice) in the GEMM precision
@@ -117,7 +119,8 @@ struct RbkWs {
   float* Eh;      // expanded real forms of the thin factor (2b rows per slice, leading dim lde)
   float* El;
   long lde;
-  int* tc_err;    // set by a tcgen05 pipeline wait that timed out
+  int* tc_err;
+  TcOpts st;
   double2* splitk;
   size_t splitk_elems;
   // deflated passes (FP64 path with TSVD_FLAG_DEFLATE)
@@ -167,7 +170,8 @@ static RbkWs<T> carve_rbk(void* base, const RbkDims& d) {
   w.eig = cv.take<char>(eig_scratch_bytes(d.m, d.R, d.h));
   w.Aop = nullptr;
   w.Ahi = w.Alo = w.AThi = w.ATlo = w.Eh = w.El = nullptr;
-  w.tc_err = nullptr;
+  w.tc_err = w.counters + 2;
+  w.st = TcOpts{w.tc_err, d.expire != 0};
   w.lda = (2L * d.n2 + 7) / 8 * 8;
   w.ldt = (2L * d.n1 + 7) / 8 * 8;
   w.lde = std::max(w.lda, w.ldt);
@@ -179,7 +183,6 @@ static RbkWs<T> carve_rbk(void* base, const RbkDims& d) {
     w.ATlo = cv.take<float>(h * d.n2 * w.ldt);
     w.Eh = cv.take<float>(h * 2 * (size_t)d.b * w.lde);
     w.El = cv.take<float>(h * 2 * (size_t)d.b * w.lde);
-    w.tc_err = cv.take<int>(4);
     if (d.tc == 2) w.Aop = cv.take<uint16_t>(h * d.n1 * w.lda);
   }
   w.otc = OrthTc{};
@@ -244,6 +247,7 @@ static int orth_block(const RbkDims& d, RbkWs<T>& w, int c, int nb, int block_id
   o.k0 = d.k0;
   o.nyq = (d.n3 % 2 == 0) ? d.n3 / 2 : -1;
   o.tc = d.tco ? &w.otc : nullptr;
+  o.st = w.st;
   return orth_block_cols<L>(d.n1, d.b, d.m, d.h, o, c, nb, block_id, seed, s);
 }
 
@@ -284,7 +288,7 @@ static int basis_product(const RbkDims& d, RbkWs<T>& w, const cx_t<T>* Y, long l
     }
   }
   return cgemm<cx_t<T>>(gemm('N', 'N', n1, nb, n2, 1.0, w.Ah, n2, sA, Y, ldy, sy, 0.0, w.Wt, b, sW, h), w.splitk,
-                        w.splitk_elems * (sizeof(double2) / sizeof(cx_t<T>)), s);
+                        w.splitk_elems * (sizeof(double2) / sizeof(cx_t<T>)), s, w.st);
 }
 
 // columns [col0, col0 + nb) of C^H (n2 x m) = X-hat^H Q(:, col0 : col0 + nb): the
@@ -302,7 +306,7 @@ static int conj_product(const RbkDims& d, RbkWs<T>& w, int col0, int nb, cudaStr
   }
   return cgemm<cx_t<T>>(gemm('H', 'N', n2, nb, n1, 1.0, w.Ah, n2, sA, w.Qt + col0, m, sQ, 0.0, w.CHt + col0, m, sCH,
                              h),
-                        w.splitk, w.splitk_elems * (sizeof(double2) / sizeof(cx_t<T>)), s);
+                        w.splitk, w.splitk_elems * (sizeof(double2) / sizeof(cx_t<T>)), s, w.st);
 }
 
 // Deflated Rayleigh-Ritz passes of the small SVD (FP64 path, deflate.cu):
@@ -319,13 +323,13 @@ static int deflated_passes(const RbkDims& d, RbkWs<double>& w, cudaStream_t s) {
     TSVD_TRY(copy_cx<double2>(w.CH64, m, sCH, w.CpH, mp, sP, n2, mp, h, s));
     for (int sweep = 0; sweep < 2; ++sweep) {  // C_p^H <- C_p^H - (C_p^H U_m) U_m^H, twice
       TSVD_TRY(cgemm<double2>(gemm('N', 'N', n2, R, mp, 1.0, w.CpH, mp, sP, w.Um, R, sU, 0.0, w.T1, R, sT, h), w.splitk,
-                              w.splitk_elems, s));
+                              w.splitk_elems, s, w.st));
       TSVD_TRY(cgemm<double2>(gemm('N', 'H', n2, mp, R, -1.0, w.T1, R, sT, w.Um, R, sU, 1.0, w.CpH, mp, sP, h),
-                              w.splitk, w.splitk_elems, s));
+                              w.splitk, w.splitk_elems, s, w.st));
     }
     TSVD_TRY(cgemm_herm<double2>(gemm('H', 'N', mp, mp, n2, 1.0, w.CpH, mp, sP, w.CpH, mp, sP, 0.0, w.G, mp,
                                       (long)mp * mp, h),
-                                 w.splitk, w.splitk_elems, s));
+                                 w.splitk, w.splitk_elems, s, w.st));
     TSVD_TRY(herm_eig_topR<double2>(w.G, mp, (long)mp * mp, mp, R, h, w.lam, w.Uct, R, sU, w.eig, w.counters, s));
     TSVD_TRY(deflate_merge(w.lam, w.Uct, mp, R, h, w.lamF, w.UF, w.Um, w.acc, false, pass == kPasses - 1, s));
   }
@@ -366,7 +370,6 @@ static int rbk_run(const T* A, const RbkDims& d, const tsvd_params& p, const T* 
 
   if (d.tc3) {  // tensor-core operands of X-hat and X-hat^T (split TF32; BF16 copy for the BF16 path)
     TSVD_STAGE("krylov_split", s);
-    if (cudaMemsetAsync(w.tc_err, 0, sizeof(int), s) != cudaSuccess) return TSVD_ERR_CUDA;
     if constexpr (std::is_same<T, float>::value) {
       // the one TF32 pass of the basis products reads X-hat's FP32 rows as they are (the tensor
       // cores drop the low 13 mantissa bits) when their layout suits TMA, else a padded copy
@@ -434,7 +437,7 @@ static int rbk_run(const T* A, const RbkDims& d, const tsvd_params& p, const T* 
   if constexpr (std::is_same<T, double>::value) {
     TSVD_TRY(cgemm_herm<double2>(gemm('H', 'N', mp, mp, n2, 1.0, w.CH64, m, sCH, w.CH64, m, sCH, 0.0, w.G, mp,
                                       (long)mp * mp, h),
-                                 w.splitk, w.splitk_elems, s));
+                                 w.splitk, w.splitk_elems, s, w.st));
   } else {
     if (w.gsl)
       TSVD_TRY(gram_sliced_fp32((const float2*)w.CHt, m, sCH, n2, mp, h, w.colexp, w.gsl, w.G, mp, (long)mp * mp,
@@ -470,7 +473,7 @@ static int rbk_run(const T* A, const RbkDims& d, const tsvd_params& p, const T* 
       } else {
         TSVD_TRY(cgemm<C>(gemm('N', 'N', n2, R, mp, 1.0, w.CHt, m, sCH, w.Uct, R, (long)mp * R, 0.0, w.Vh, R,
                                (long)n2 * R, h),
-                          w.splitk, w.splitk_elems * (sizeof(double2) / sizeof(cx_t<T>)), s));
+                          w.splitk, w.splitk_elems * (sizeof(double2) / sizeof(cx_t<T>)), s, w.st));
         done = true;
       }
     }
@@ -478,10 +481,10 @@ static int rbk_run(const T* A, const RbkDims& d, const tsvd_params& p, const T* 
   if (!done) {
     TSVD_TRY(cgemm<C>(gemm('N', 'N', n1, R, mp, 1.0, w.Qt, m, sQ, w.Uct, R, (long)mp * R, 0.0, w.Uh, R,
                            (long)n1 * R, h),
-                      w.splitk, w.splitk_elems * (sizeof(double2) / sizeof(cx_t<T>)), s));
+                      w.splitk, w.splitk_elems * (sizeof(double2) / sizeof(cx_t<T>)), s, w.st));
     TSVD_TRY(cgemm<C>(gemm('N', 'N', n2, R, mp, 1.0, w.CHt, m, sCH, w.Uct, R, (long)mp * R, 0.0, w.Vh, R,
                            (long)n2 * R, h),
-                      w.splitk, w.splitk_elems * (sizeof(double2) / sizeof(cx_t<T>)), s));
+                      w.splitk, w.splitk_elems * (sizeof(double2) / sizeof(cx_t<T>)), s, w.st));
   }
   TSVD_TRY(scale_columns_inv<T>(w.Vh, R, (long)n2 * R, n2, R, w.lam, h, s));
   }
@@ -494,12 +497,10 @@ static int rbk_run(const T* A, const RbkDims& d, const tsvd_params& p, const T* 
   }
 
   if (info) {
-    int host[8], tcerr = 0;
+    int host[8];
     if (cudaMemcpyAsync(host, w.counters, sizeof(host), cudaMemcpyDeviceToHost, s) != cudaSuccess) return TSVD_ERR_CUDA;
-    if (w.tc_err && cudaMemcpyAsync(&tcerr, w.tc_err, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess)
-      return TSVD_ERR_CUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return TSVD_ERR_CUDA;
-    info->status = tcerr ? TSVD_ERR_CUDA : host[0];
+    info->status = host[2] ? TSVD_ERR_CUDA : host[0];
     info->dead_columns = host[1];
     info->m_eff = mp;
     info->reserved = 0;
