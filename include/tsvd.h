@@ -76,10 +76,11 @@ typedef struct {
    Q = orth((A A^H)^q A B), orthonormalised after every step (same span), basis of
    min(R+P, n1, n2) columns; the rest of the pipeline as for Alg. 2 */
 #define TSVD_FLAG_ALG1 2
-/* bit 2 (TSVD_FLAG_SIMT): FP32 / mixed paths: run the Krylov products on the FP32 SIMT units
-   instead of the tensor cores (by default the FP32 path runs them on tcgen05 as split TF32,
-   x = hi + lo with hi the nearest TF32, products hi*hi + hi*lo + lo*hi in FP32, about 22
-   significant bits) */
+/* bit 2 (TSVD_FLAG_SIMT): run the complex products on the FP64 and FP32 SIMT units instead of the
+   tensor cores (by default FP32 and mixed Krylov products run on tcgen05 as split TF32, x = hi + lo with
+   hi the nearest TF32, products hi*hi + hi*lo + lo*hi in FP32, about 22 significant bits; the other
+   products on tcgen05 too where that is faster, FP32 from exact BF16 parts, FP64 from integer digits,
+   both with errors below the SIMT units').  The exact Gram has its own flag, TSVD_FLAG_GRAM_INT. */
 #define TSVD_FLAG_SIMT 4
 /* bit 3 (TSVD_FLAG_QTRUNC): Alg. 2 with the basis Q truncated to its leading R+P columns
    before the projection C = Q^T * X (the variant Sec. 5, Ex. 1 reports timings for); the

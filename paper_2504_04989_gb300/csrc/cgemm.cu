@@ -391,7 +391,7 @@ static int cgemm_impl(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, c
   if (g.beta != 0.0 && g.beta != 1.0) return TSVD_ERR_INVALID_ARG;
   if constexpr (std::is_same<C, float2>::value) {
     const size_t bytes = splitk_ws ? splitk_elems * sizeof(C) : 0;
-    if (!g.simt && !herm && sgemm_tc_better(g, bytes)) return sgemm_tc(g, splitk_ws, bytes, s, st);
+    if (!st.simt && !herm && sgemm_tc_better(g, bytes)) return sgemm_tc(g, splitk_ws, bytes, s, st);
     // the wide tiles where they fill the GPU (two CTAs per SM), directly or by splitting a long K;
     // smaller products keep the 64 x 64 tiles (measured faster there)
     const long wtiles = (long)cdiv(g.M, WBM) * cdiv(g.N, WBN) * g.batch;
@@ -400,7 +400,7 @@ static int cgemm_impl(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, c
   }
   if constexpr (std::is_same<C, double2>::value) {
     const size_t bytes = splitk_ws ? splitk_elems * sizeof(C) : 0;
-    if (!g.simt && dgemm_tc_better(g, bytes)) {
+    if (!st.simt && dgemm_tc_better(g, bytes)) {
       TSVD_TRY(dgemm_tc(g, splitk_ws, bytes, s, herm != 0, st));
       return herm ? mirror_lower<C>(g, s) : TSVD_OK;
     }

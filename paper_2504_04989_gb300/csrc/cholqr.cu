@@ -712,9 +712,9 @@ int orth_block_cols(int n1, int b, int m, int h, const OrthWs& w, int c, int nb,
     {
       TSVD_STAGE("orth_trsm", s);
       const GemmArgs g = gemm('N', 'N', n1, nb, nb, 1.0, X, ldx, sX, Mi, b, sG, 0.0, Y, ldy, sY, h);
-      if (std::is_same<L, double>::value && dgemm_tc_better(g, sk * sizeof(CL)))
+      if (std::is_same<L, double>::value && !w.st.simt && dgemm_tc_better(g, sk * sizeof(CL)))
         TSVD_TRY(dgemm_tc(g, w.splitk, sk * sizeof(CL), s, false, w.st));
-      else if (std::is_same<L, float>::value && sgemm_tc_better(g, sk * sizeof(CL)))
+      else if (std::is_same<L, float>::value && !w.st.simt && sgemm_tc_better(g, sk * sizeof(CL)))
         TSVD_TRY(sgemm_tc(g, w.splitk, sk * sizeof(CL), s, w.st));
       else
         TSVD_TRY(rmul_block<CL>(X, ldx, sX, Mi, b, sG, n1, nb, h, Y, ldy, sY, s));

@@ -46,7 +46,6 @@ struct GemmArgs {
   void* C;
   long ldc, sC;
   int batch;
-  bool simt = false;  // keep to the SIMT kernels
 };
 // GemmArgs from its fields (strided batch)
 inline GemmArgs gemm(char opA, char opB, int M, int N, int K, double alpha, const void* A, long lda, long sA,
@@ -72,10 +71,11 @@ inline GemmArgs gemm(char opA, char opB, int M, int N, int K, double alpha, cons
   return g;
 }
 // Where a tensor-core product says that a wait of its pipeline ran out (its elements are NaN then): *err = 1, unless null.
-// expire (tests): the waits give up at once.
+// expire (tests): the waits give up at once.  simt: no tensor-core products.
 struct TcOpts {
   int* err = nullptr;
   bool expire = false;
+  bool simt = false;
 };
 template <typename C>
 int cgemm(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t s, TcOpts st = TcOpts());

@@ -114,8 +114,9 @@ static int tprod_noalloc_run(const T* A, const T* B, T* Cout, int n1, int n2, in
   g.ldc = n4;
   g.sC = (long)n1 * n4;
   g.batch = (int)h;
-  g.simt = true;  // no kernel beyond those the first call loads
-  TSVD_TRY(cgemm<C>(g, sk_elems > 0 ? sk : nullptr, sk_elems, s));
+  TcOpts simt;  // the tensor-core kernels would have to be loaded too
+  simt.simt = true;
+  TSVD_TRY(cgemm<C>(g, sk_elems > 0 ? sk : nullptr, sk_elems, s, simt));
   TSVD_TRY(launch_irfft3<T>(Ch, Cout, (long)n1 * n4, n3, s));
   return TSVD_OK;
 }

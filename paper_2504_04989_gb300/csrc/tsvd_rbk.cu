@@ -44,6 +44,7 @@ struct RbkDims {
   int gsl;   // FP32 paths: the exact Gram in its digit form on the BF16 tensor cores
   int mp;    // basis columns used by the projection: m, or R+P with TSVD_FLAG_QTRUNC
   int deflate;  // deflated Rayleigh-Ritz passes for the small SVD (FP64 path)
+  int simt;     // TSVD_FLAG_SIMT
   int expire;   // the waits of cgemm's tensor-core products give up at once (tests)
 };
 
@@ -75,6 +76,7 @@ static int rbk_dims(int n1, int n2, int n3, const tsvd_params* p, RbkDims* d) {
   d->gsl = (d->tc3 && !(p->flags & TSVD_FLAG_GRAM_INT) && gram_sliced_ok(n2, d->m)) ? 1 : 0;
   d->mp = (p->flags & TSVD_FLAG_QTRUNC) ? std::min(d->b, d->m) : d->m;
   d->deflate = (p->flags & TSVD_FLAG_DEFLATE) ? 1 : 0;
+  d->simt = (p->flags & TSVD_FLAG_SIMT) ? 1 : 0;
   d->expire = (p->flags & TSVD_FLAG_EXPIRE) ? 1 : 0;
   if (d->deflate && p->precision != TSVD_FP64) return TSVD_ERR_UNSUPPORTED;
   if (d->b > 128 || d->m > 512) return TSVD_ERR_UNSUPPORTED;
@@ -171,7 +173,7 @@ static RbkWs<T> carve_rbk(void* base, const RbkDims& d) {
   w.Aop = nullptr;
   w.Ahi = w.Alo = w.AThi = w.ATlo = w.Eh = w.El = nullptr;
   w.tc_err = w.counters + 2;
-  w.st = TcOpts{w.tc_err, d.expire != 0};
+  w.st = TcOpts{w.tc_err, d.expire != 0, d.simt != 0};
   w.lda = (2L * d.n2 + 7) / 8 * 8;
   w.ldt = (2L * d.n1 + 7) / 8 * 8;
   w.lde = std::max(w.lda, w.ldt);

@@ -8,7 +8,7 @@ pytestmark = pytest.mark.gpu
 
 torch = pytest.importorskip("torch")
 
-EXPIRE = 64  # TSVD_FLAG_EXPIRE
+SIMT, EXPIRE = 4, 64  # TSVD_FLAG_SIMT, TSVD_FLAG_EXPIRE
 
 
 @pytest.fixture(scope="module")
@@ -46,3 +46,9 @@ def test_products_that_give_up(lib, precision, n, n3):
     assert _status(lib, precision, 0, n, n3) == 0
     assert _status(lib, precision, EXPIRE, n, n3) == -3  # TSVD_ERR_CUDA
     assert _status(lib, precision, 0, n, n3) == 0
+
+
+@pytest.mark.parametrize("precision,n,n3", [("fp64", 384, 16), ("fp32", 512, 64)])
+def test_simt_takes_no_such_product(lib, precision, n, n3):
+    """TSVD_FLAG_SIMT: no tensor-core product that could give up."""
+    assert _status(lib, precision, SIMT | EXPIRE, n, n3) == 0
