@@ -375,7 +375,8 @@ TSVD_API int tpinv(const void* A, int n1, int n2, int n3, int precision, void* X
  * All calls share the array: calls whose kernels overlap on the GPU race.
  * The array sits in a module of the library that holds no kernel; with CUDA's
  * lazy module loading (the default) that module, and its 16 MiB, is loaded on
- * a device by the first call there, so make that first call before sealing a
+ * a device by the first call there, and with it every kernel that a later call of
+ * any size and precision can take, so make one call before sealing a
  * pool that must not grow and before capturing a CUDA graph.  Every call
  * outside a capture looks the array's address up again (nothing is allocated
  * by that once the module is loaded), so a device reset is followed; inside a

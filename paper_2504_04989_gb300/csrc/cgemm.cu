@@ -420,6 +420,16 @@ int cgemm(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t 
 }
 
 template <typename C>
+int load_simt_products() {
+  TSVD_TRY(load_kernel(k_cgemm<C, false, false, false>));
+  TSVD_TRY(load_kernel(k_cgemm<C, false, false, true>));
+  if constexpr (std::is_same<C, float2>::value) TSVD_TRY(load_kernel(k_cgemm_w<false, false>));
+  return load_kernel(k_splitk_reduce<C>);
+}
+template int load_simt_products<double2>();
+template int load_simt_products<float2>();
+
+template <typename C>
 size_t cgemm_scratch(int M, int N, int K, int batch) {
   GemmArgs g = gemm('N', 'N', M, N, K, 1.0, nullptr, K, 0, nullptr, N, 0, 0.0, nullptr, N, 0, batch);
   if constexpr (std::is_same<C, double2>::value) {

@@ -109,6 +109,15 @@ __device__ __forceinline__ double inv_sqrt(double d) {
   return __hiloint2double(__double2hiint(y) - (e2 << 19), __double2loint(y));  // y 2^(-e2/2)
 }
 
+// f's code on the current device, without a launch
+template <typename F>
+inline int load_kernel(F* f) {
+  cudaFuncAttributes a;
+  if (cudaFuncGetAttributes(&a, f) == cudaSuccess) return TSVD_OK;
+  cudaGetLastError();
+  return TSVD_ERR_CUDA;
+}
+
 // warp reductions
 __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

@@ -1278,6 +1278,29 @@ int launch_irfft3(const cx_t<T>* Xh, T* X, long plane, int n3, cudaStream_t s) {
   return TSVD_OK;
 }
 
+template <typename T>
+int load_transforms() {
+  int rc = TSVD_OK;
+  auto load = [&](auto forward, auto inverse) {
+    if (rc == TSVD_OK) rc = load_kernel(forward);
+    if (rc == TSVD_OK) rc = load_kernel(inverse);
+  };
+  load(k_rfft3_reg<T, 2>, k_irfft3_reg<T, 2>);
+  load(k_rfft3_reg<T, 4>, k_irfft3_reg<T, 4>);
+  load(k_rfft3_reg<T, 8>, k_irfft3_reg<T, 8>);
+  load(k_rfft3_reg<T, 16>, k_irfft3_reg<T, 16>);
+  load(k_rfft3_reg<T, 32>, k_irfft3_reg<T, 32>);
+  load(k_rfft3_reg<T, 64>, k_irfft3_reg<T, 64>);
+  if constexpr (sizeof(T) == 4) load(k_rfft3_reg<T, 128>, k_irfft3_reg<T, 128>);
+  else load(k_rfft3_reg2<T, 128>, k_irfft3_reg2<T, 128>);
+  load(k_rdft3<T>, k_irdft3<T>);
+  load(k_rfft3_fft<T>, k_irfft3_fft<T>);
+  load(k_rfft3<T>, k_irfft3<T>);
+  return rc;
+}
+template int load_transforms<double>();
+template int load_transforms<float>();
+
 template int launch_rfft3<double>(const double*, double2*, long, int, cudaStream_t);
 template int launch_rfft3<float>(const float*, float2*, long, int, cudaStream_t);
 template int launch_irfft3<double>(const double2*, double*, long, int, cudaStream_t);

@@ -26,6 +26,10 @@ template <typename T>
 int launch_rfft3(const T* X, cx_t<T>* Xh, long plane, int n3, cudaStream_t s);
 template <typename T>
 int launch_irfft3(const cx_t<T>* Xh, T* X, long plane, int n3, cudaStream_t s);
+// load every kernel of the two transforms on the current device (under lazy loading a kernel's first launch does,
+// and may take device memory)
+template <typename T>
+int load_transforms();
 template <typename T>
 int launch_gaussian(uint64_t seed, uint32_t stream_id, uint32_t tensor_id, long n, T* out, cudaStream_t s);
 
@@ -79,6 +83,9 @@ struct TcOpts {
 };
 template <typename C>
 int cgemm(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t s, TcOpts st = TcOpts());
+// load the kernels of the SIMT form of op 'N' x 'N', as load_transforms
+template <typename C>
+int load_simt_products();
 // scratch elements with which cgemm can take its tensor-core form for an M x N x K product (0 where
 // it would keep to the SIMT units); a smaller splitk_elems only makes it slower
 template <typename C>

@@ -22,6 +22,9 @@
 //    16 MiB, is loaded on a device at the first call there (the address
 //    lookup below), so make that first call before sealing a pool or arena
 //    that must not grow afterwards, and before any CUDA graph capture;
+//  * that first call also loads every kernel that a later one can take, whatever
+//    its sizes and precision (transforms by length, products by tile), so one
+//    call of any size is enough;
 //  * every call outside stream capture looks the address up again
 //    (cudaGetSymbolAddress allocates nothing once the module is loaded), so a
 //    device reset that reloads the module at another address is followed;
@@ -60,6 +63,12 @@ static int scratch_address(cudaStream_t s, void** out) {
     if (cudaGetSymbolAddress(&p, g_tprod_scratch) != cudaSuccess || !p) {
       cudaGetLastError();
       return TSVD_ERR_CUDA;
+    }
+    if (__atomic_load_n(&g_scratch_ptr[dev], __ATOMIC_ACQUIRE) != p) {  // the first call (two at once do no harm)
+      TSVD_TRY(load_transforms<double>());
+      TSVD_TRY(load_transforms<float>());
+      TSVD_TRY(load_simt_products<double2>());
+      TSVD_TRY(load_simt_products<float2>());
     }
     __atomic_store_n(&g_scratch_ptr[dev], p, __ATOMIC_RELEASE);
   } else {
@@ -114,7 +123,7 @@ static int tprod_noalloc_run(const T* A, const T* B, T* Cout, int n1, int n2, in
   g.ldc = n4;
   g.sC = (long)n1 * n4;
   g.batch = (int)h;
-  TcOpts simt;  // the tensor-core kernels would have to be loaded too
+  TcOpts simt;  // no kernel beyond those that the first call loads
   simt.simt = true;
   TSVD_TRY(cgemm<C>(g, sk_elems > 0 ? sk : nullptr, sk_elems, s, simt));
   TSVD_TRY(launch_irfft3<T>(Ch, Cout, (long)n1 * n4, n3, s));
