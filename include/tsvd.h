@@ -102,6 +102,12 @@ typedef struct {
    info->status is TSVD_ERR_CUDA where such a product was taken, and the outputs mean nothing then. */
 #define TSVD_FLAG_EXPIRE 64
 
+/* The *_workspace_size calls report the workspace that a call gains by: most of it beyond the operands holds
+   the parts of a tensor-core product's operands.  With this bit in their precision argument, or in
+   params->flags, they report the least with which the call runs: its products are done in passes then, or on
+   the SIMT units, to the same accuracy but slower.  Every size from there on is accepted. */
+#define TSVD_WS_LEAST 256
+
 /* ---- device-side outcome, read back only when requested ---- */
 typedef struct {
   int status;          /* TSVD_OK, TSVD_ERR_NOT_CONVERGED, or TSVD_ERR_CUDA: a tensor-core product gave up */

@@ -18,6 +18,7 @@ TSVD_FLAG_QTRUNC = 8
 TSVD_FLAG_DEFLATE = 16
 TSVD_FLAG_GRAM_INT = 32
 TSVD_FLAG_EXPIRE = 64
+TSVD_WS_LEAST = 256
 PRECISIONS = {"fp64": TSVD_FP64, "fp32": TSVD_FP32, "tf32": TSVD_MIXED_TF32, "bf16": TSVD_MIXED_BF16,
               "tf32x3": TSVD_SPLIT_TF32}
 

@@ -44,6 +44,35 @@ def _workspace(nbytes, device):
     return torch.empty(max(int(nbytes), 256), dtype=torch.uint8, device=device)
 
 
+def _workspace_for(size, device):
+    """The workspace that size(0) asks for or, where that is more than the device has left, the least
+    with which the call runs, size(TSVD_WS_LEAST)."""
+    try:
+        return _workspace(size(0), device)
+    except torch.OutOfMemoryError:
+        return _workspace(size(_lib.TSVD_WS_LEAST), device)
+
+
+def _sized(call, *args, precision, what):
+    """size function for _workspace_for of a *_workspace_size call that takes its precision last"""
+    def size(flag):
+        nbytes = C.c_size_t()
+        _lib.check(call(*args, precision | flag, C.byref(nbytes)), what)
+        return nbytes.value
+    return size
+
+
+def _sized_params(call, *args, params, what):
+    """the same of a call that takes params"""
+    def size(flag):
+        p = _lib.TsvdParams.from_buffer_copy(params)
+        p.flags |= flag
+        nbytes = C.c_size_t()
+        _lib.check(call(*args, C.byref(p), C.byref(nbytes)), what)
+        return nbytes.value
+    return size
+
+
 def _flags(fp64_qr, alg1, q_trunc, deflate=False, gram_int=False):
     return ((_lib.TSVD_FLAG_FP64_QR if fp64_qr else 0) | (_lib.TSVD_FLAG_ALG1 if alg1 else 0) |
             (_lib.TSVD_FLAG_QTRUNC if q_trunc else 0) | (_lib.TSVD_FLAG_DEFLATE if deflate else 0) |
@@ -74,10 +103,9 @@ def rbk(A, R, P=10, q=2, seed=0, precision="fp32", omega=None, return_info=False
     n3, n1, n2 = A.shape
     flags = _flags(fp64_qr, alg1, q_trunc, deflate, gram_int)
     p = _lib.TsvdParams(R=int(R), P=int(P), q=int(q), precision=pr, seed=int(seed), flags=flags)
-    nbytes = C.c_size_t()
-    _lib.check(lib.tsvd_rbk_workspace_size(n1, n2, n3, C.byref(p), C.byref(nbytes)), "tsvd_rbk_workspace_size")
     dev = A.device
-    ws = _workspace(nbytes.value, dev)
+    ws = _workspace_for(_sized_params(lib.tsvd_rbk_workspace_size, n1, n2, n3, params=p,
+                                      what="tsvd_rbk_workspace_size"), dev)
     h = n3 // 2 + 1
     U = torch.empty((n3, n1, R), dtype=dt, device=dev)
     S = torch.empty((n3, R), dtype=dt, device=dev)
@@ -90,7 +118,7 @@ def rbk(A, R, P=10, q=2, seed=0, precision="fp32", omega=None, return_info=False
     info = _lib.TsvdInfo()
     with torch.cuda.device(dev):
         rc = lib.tsvd_rbk(_ptr(A), n1, n2, n3, C.byref(p), _ptr(omega), _ptr(U), _ptr(S), _ptr(V), _ptr(sig),
-                          _ptr(ws), nbytes.value, _stream(dev), C.byref(info) if return_info else None)
+                          _ptr(ws), ws.numel(), _stream(dev), C.byref(info) if return_info else None)
     _lib.check(rc, "tsvd_rbk")
     if return_info:
         return U, S, V, sig, {"status": info.status, "m_eff": info.m_eff, "dead_columns": info.dead_columns}
@@ -109,11 +137,10 @@ class RbkPlan:
         self.p = _lib.TsvdParams(R=int(R), P=int(P), q=int(q), precision=_prec(precision), seed=int(seed),
                                  flags=flags)
         self.shape = (n1, n2, n3)
-        nbytes = C.c_size_t()
-        _lib.check(self.lib.tsvd_rbk_workspace_size(n1, n2, n3, C.byref(self.p), C.byref(nbytes)), "workspace")
-        self.nbytes = nbytes.value
         self.device = torch.device(device)
-        self.ws = _workspace(self.nbytes, self.device)
+        self.ws = _workspace_for(_sized_params(self.lib.tsvd_rbk_workspace_size, n1, n2, n3, params=self.p,
+                                               what="workspace"), self.device)
+        self.nbytes = self.ws.numel()
         self.U = torch.empty((n3, n1, R), dtype=self.dt, device=self.device)
         self.S = torch.empty((n3, R), dtype=self.dt, device=self.device)
         self.V = torch.empty((n3, n2, R), dtype=self.dt, device=self.device)
@@ -161,11 +188,21 @@ class RbkBatchPlan:
             d.U, d.S, d.V = self.U[-1].data_ptr(), self.S[-1].data_ptr(), self.V[-1].data_ptr()
             d.sigma_hat = self.sig[-1].data_ptr()
         self.count = n
-        nbytes = C.c_size_t()
-        _lib.check(self.lib.tsvd_rbk_batched_workspace_size(self.descs, n, self.lanes, C.byref(nbytes)),
-                   "tsvd_rbk_batched_workspace_size")
-        self.nbytes = nbytes.value
-        self.ws = _workspace(max(self.nbytes, 256), self.device)
+
+        def size(flag):
+            nbytes = C.c_size_t()
+            for d in self.descs[:n]:
+                d.params.flags |= flag
+            try:
+                _lib.check(self.lib.tsvd_rbk_batched_workspace_size(self.descs, n, self.lanes, C.byref(nbytes)),
+                           "tsvd_rbk_batched_workspace_size")
+            finally:
+                for d in self.descs[:n]:
+                    d.params.flags &= ~flag
+            return nbytes.value
+
+        self.ws = _workspace_for(size, self.device)
+        self.nbytes = self.ws.numel()
         self.graph = None
         if graph:
             self._launch()                      # first call creates the lane streams outside the capture
@@ -212,12 +249,10 @@ def _tprod_raw(A, B, precision):
     n3b, n2b, n4 = B.shape
     if n3b != n3 or n2b != n2:
         raise ValueError("tprod: shapes (n3,n1,n2) and (n3,n2,n4) required")
-    nbytes = C.c_size_t()
-    _lib.check(lib.tprod_workspace_size(n1, n2, n4, n3, pr, C.byref(nbytes)), "tprod_workspace_size")
-    ws = _workspace(nbytes.value, A.device)
+    ws = _workspace_for(_sized(lib.tprod_workspace_size, n1, n2, n4, n3, precision=pr, what="tprod_workspace_size"), A.device)
     out = torch.empty((n3, n1, n4), dtype=A.dtype, device=A.device)
     with torch.cuda.device(A.device):
-        _lib.check(lib.tprod(_ptr(A), _ptr(B), _ptr(out), n1, n2, n4, n3, pr, _ptr(ws), nbytes.value,
+        _lib.check(lib.tprod(_ptr(A), _ptr(B), _ptr(out), n1, n2, n4, n3, pr, _ptr(ws), ws.numel(),
                              _stream(A.device)), "tprod")
     return out
 
@@ -230,14 +265,12 @@ def tprod_backward(A, B, dC, precision="fp32", need_dA=True, need_dB=True):
     _need_cuda(A, B, dC, dtype=_DT[precision])
     n3, n1, n2 = A.shape
     n4 = B.shape[2]
-    nbytes = C.c_size_t()
-    _lib.check(lib.tprod_backward_workspace_size(n1, n2, n4, n3, pr, C.byref(nbytes)), "workspace")
-    ws = _workspace(nbytes.value, A.device)
+    ws = _workspace_for(_sized(lib.tprod_backward_workspace_size, n1, n2, n4, n3, precision=pr, what="workspace"), A.device)
     dA = torch.empty_like(A) if need_dA else None
     dB = torch.empty_like(B) if need_dB else None
     with torch.cuda.device(A.device):
         _lib.check(lib.tprod_backward(_ptr(A), _ptr(B), _ptr(dC), _ptr(dA), _ptr(dB), n1, n2, n4, n3, pr, _ptr(ws),
-                                      nbytes.value, _stream(A.device)), "tprod_backward")
+                                      ws.numel(), _stream(A.device)), "tprod_backward")
     return dA, dB
 
 
@@ -248,12 +281,10 @@ def _tproj_raw(Q, A, precision):
     _need_cuda(Q, A, dtype=_DT[precision])
     n3, n1, m = Q.shape
     n2 = A.shape[2]
-    nbytes = C.c_size_t()
-    _lib.check(lib.tproj_workspace_size(n1, m, n2, n3, pr, C.byref(nbytes)), "workspace")
-    ws = _workspace(nbytes.value, Q.device)
+    ws = _workspace_for(_sized(lib.tproj_workspace_size, n1, m, n2, n3, precision=pr, what="workspace"), Q.device)
     Y = torch.empty_like(A)
     with torch.cuda.device(Q.device):
-        _lib.check(lib.tproj(_ptr(Q), _ptr(A), _ptr(Y), n1, m, n2, n3, pr, _ptr(ws), nbytes.value,
+        _lib.check(lib.tproj(_ptr(Q), _ptr(A), _ptr(Y), n1, m, n2, n3, pr, _ptr(ws), ws.numel(),
                              _stream(Q.device)), "tproj")
     return Y
 
@@ -266,14 +297,12 @@ def tproj_backward(Q, A, dY, precision="fp32", need_dQ=True, need_dA=True):
     _need_cuda(Q, A, dY, dtype=_DT[precision])
     n3, n1, m = Q.shape
     n2 = A.shape[2]
-    nbytes = C.c_size_t()
-    _lib.check(lib.tproj_backward_workspace_size(n1, m, n2, n3, pr, C.byref(nbytes)), "workspace")
-    ws = _workspace(nbytes.value, Q.device)
+    ws = _workspace_for(_sized(lib.tproj_backward_workspace_size, n1, m, n2, n3, precision=pr, what="workspace"), Q.device)
     dQ = torch.empty_like(Q) if need_dQ else None
     dA = torch.empty_like(A) if need_dA else None
     with torch.cuda.device(Q.device):
         _lib.check(lib.tproj_backward(_ptr(Q), _ptr(A), _ptr(dY), _ptr(dQ), _ptr(dA), n1, m, n2, n3, pr, _ptr(ws),
-                                      nbytes.value, _stream(Q.device)), "tproj_backward")
+                                      ws.numel(), _stream(Q.device)), "tproj_backward")
     return dQ, dA
 
 
@@ -430,14 +459,12 @@ def tqr(A, precision=None, return_info=False):
     _need_cuda(A, dtype=_DT[precision])
     n3, n1, n2 = A.shape
     p = min(n1, n2)
-    nbytes = C.c_size_t()
-    _lib.check(lib.tqr_workspace_size(n1, n2, n3, pr, C.byref(nbytes)), "tqr_workspace_size")
-    ws = _workspace(nbytes.value, A.device)
+    ws = _workspace_for(_sized(lib.tqr_workspace_size, n1, n2, n3, precision=pr, what="tqr_workspace_size"), A.device)
     Q = torch.empty((n3, n1, p), dtype=A.dtype, device=A.device)
     R = torch.empty((n3, p, n2), dtype=A.dtype, device=A.device)
     info = _lib.TsvdInfo()
     with torch.cuda.device(A.device):
-        _lib.check(lib.tqr(_ptr(A), n1, n2, n3, pr, _ptr(Q), _ptr(R), _ptr(ws), nbytes.value, _stream(A.device),
+        _lib.check(lib.tqr(_ptr(A), n1, n2, n3, pr, _ptr(Q), _ptr(R), _ptr(ws), ws.numel(), _stream(A.device),
                            C.byref(info) if return_info else None), "tqr")
     if return_info:
         return Q, R, {"status": info.status, "dead_columns": info.dead_columns}
@@ -454,13 +481,12 @@ def tpinv(A, precision=None, return_info=False):
     A = A.contiguous()
     _need_cuda(A, dtype=_DT[precision])
     n3, n1, n2 = A.shape
-    nbytes = C.c_size_t()
-    _lib.check(lib.tpinv_workspace_size(n1, n2, n3, pr, C.byref(nbytes)), "tpinv_workspace_size")
-    ws = _workspace(nbytes.value, A.device)
+    ws = _workspace_for(_sized(lib.tpinv_workspace_size, n1, n2, n3, precision=pr, what="tpinv_workspace_size"),
+                        A.device)
     X = torch.empty((n3, n2, n1), dtype=A.dtype, device=A.device)
     info = _lib.TsvdInfo()
     with torch.cuda.device(A.device):
-        _lib.check(lib.tpinv(_ptr(A), n1, n2, n3, pr, _ptr(X), _ptr(ws), nbytes.value, _stream(A.device),
+        _lib.check(lib.tpinv(_ptr(A), n1, n2, n3, pr, _ptr(X), _ptr(ws), ws.numel(), _stream(A.device),
                              C.byref(info) if return_info else None), "tpinv")
     if return_info:
         return X, {"status": info.status, "dead_columns": info.dead_columns}
@@ -515,11 +541,8 @@ def rbk_fourier(Ahat, n3, k0, R, P=10, q=2, seed=0, precision="fp32", omega=None
     p = _lib.TsvdParams(R=int(R), P=int(P), q=int(q), precision=pr, seed=int(seed), flags=_flags(**{
         "fp64_qr": flags.get("fp64_qr", False), "alg1": flags.get("alg1", False),
         "q_trunc": flags.get("q_trunc", False), "deflate": flags.get("deflate", False)}))
-    nbytes = C.c_size_t()
-    _lib.check(lib.tsvd_rbk_fourier_workspace_size(n1, n2, n3, k0, ns, C.byref(p), C.byref(nbytes)),
-               "tsvd_rbk_fourier_workspace_size")
-    dev = Ahat.device
-    ws = _workspace(nbytes.value, dev)
+    ws = _workspace_for(_sized_params(lib.tsvd_rbk_fourier_workspace_size, n1, n2, n3, k0, ns, params=p,
+                                      what="tsvd_rbk_fourier_workspace_size"), dev)
     Uh = torch.empty((ns, n1, R), dtype=cdt, device=dev)
     Vh = torch.empty((ns, n2, R), dtype=cdt, device=dev)
     sig = torch.empty((ns, R), dtype=torch.float64, device=dev)
@@ -529,11 +552,18 @@ def rbk_fourier(Ahat, n3, k0, R, P=10, q=2, seed=0, precision="fp32", omega=None
     info = _lib.TsvdInfo()
     with torch.cuda.device(dev):
         _lib.check(lib.tsvd_rbk_fourier(_ptr(Ahat), n1, n2, n3, k0, ns, C.byref(p), _ptr(omega), _ptr(Uh), _ptr(Vh),
-                                        _ptr(sig), _ptr(ws), nbytes.value, _stream(dev),
+                                        _ptr(sig), _ptr(ws), ws.numel(), _stream(dev),
                                         C.byref(info) if return_info else None), "tsvd_rbk_fourier")
     if return_info:
         return Uh, Vh, sig, {"status": info.status, "m_eff": info.m_eff, "dead_columns": info.dead_columns}
     return Uh, Vh, sig
+
+
+def lowrank_workspace(U, V):
+    """The workspace of lowrank for factors of these shapes."""
+    n3, n1, R = U.shape
+    return _workspace_for(_sized(_lib.load().tsvd_lowrank_workspace_size, n1, V.shape[1], n3, R,
+                                 precision=_prec(_precision_of(U, None)), what="lowrank ws"), U.device)
 
 
 def lowrank(U, S, V, out=None, ws=None):
@@ -545,13 +575,12 @@ def lowrank(U, S, V, out=None, ws=None):
     _need_cuda(U, S, V, dtype=U.dtype)
     n3, n1, R = U.shape
     n2 = V.shape[1]
-    nbytes = C.c_size_t()
-    _lib.check(lib.tsvd_lowrank_workspace_size(n1, n2, n3, R, _prec(precision), C.byref(nbytes)), "lowrank ws")
-    ws = _workspace(nbytes.value, U.device) if ws is None else ws
+    if ws is None:
+        ws = lowrank_workspace(U, V)
     X = torch.empty((n3, n1, n2), dtype=U.dtype, device=U.device) if out is None else out
     with torch.cuda.device(U.device):
         _lib.check(lib.tsvd_lowrank(_ptr(U), _ptr(S), _ptr(V), n1, n2, n3, R, _prec(precision), _ptr(X), _ptr(ws),
-                                    nbytes.value, _stream(U.device)), "tsvd_lowrank")
+                                    ws.numel(), _stream(U.device)), "tsvd_lowrank")
     return X
 
 

@@ -115,13 +115,7 @@ class FillInPlan:
     def _iterate(self):
         U, S, V, _ = self.plan(self.C)
         if self.lr_ws is None:
-            import ctypes as C
-            from . import _lib
-            nbytes = C.c_size_t()
-            n3, n1, R = U.shape
-            _lib.check(_lib.load().tsvd_lowrank_workspace_size(n1, V.shape[1], n3, R, _lib.PRECISIONS[
-                "fp64" if U.dtype == torch.float64 else "fp32"], C.byref(nbytes)), "lowrank ws")
-            self.lr_ws = torch.empty(nbytes.value, dtype=torch.uint8, device=U.device)
+            self.lr_ws = api.lowrank_workspace(U, V)
         api.lowrank(U, S, V, out=self.X, ws=self.lr_ws)
         api.fill_in(self.C, self.M, self.mask, self.X, self.change2, self.partial)
 

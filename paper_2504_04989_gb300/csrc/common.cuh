@@ -188,6 +188,16 @@ struct Carver {
   size_t bytes() const { return (off + 255) & ~(size_t)255; }
 };
 
+// The product scratch at the end of a workspace, in elements of C: `least` with which the call runs, `best` beyond which no
+// product gains; between them what `have` bytes leave.
+constexpr size_t WS_ALL = (size_t)-1;
+template <typename C>
+size_t fit_scratch(const Carver& cv, size_t have, size_t least, size_t best) {
+  if (have == WS_ALL) return std::max(least, best);
+  const size_t used = cv.bytes(), room = have > used ? (have - used) / sizeof(C) : 0;
+  return std::max(least, std::min(best, room));
+}
+
 inline int launch_status() { return cudaGetLastError() == cudaSuccess ? TSVD_OK : TSVD_ERR_CUDA; }
 
 #define TSVD_TRY(expr)          \

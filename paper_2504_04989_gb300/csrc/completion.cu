@@ -83,7 +83,7 @@ struct LrWs {
 };
 
 template <typename T>
-static LrWs<T> carve_lr(void* base, int n1, int n2, int n3, int R) {
+static LrWs<T> carve_lr(void* base, int n1, int n2, int n3, int R, size_t have) {
   using C = cx_t<T>;
   const size_t h = n3 / 2 + 1;
   Carver cv(base);
@@ -92,8 +92,8 @@ static LrWs<T> carve_lr(void* base, int n1, int n2, int n3, int R) {
   w.Vh = cv.take<C>(h * n2 * R);
   w.Sh = cv.take<C>(h * R);
   w.Xh = cv.take<C>(h * n1 * n2);
-  w.sk_elems = std::max(std::min<size_t>((size_t)1 << 20, 4 * h * (size_t)n1 * n2),
-                        cgemm_scratch<C>(n1, n2, R, (int)h));
+  w.sk_elems = fit_scratch<C>(cv, have, std::min<size_t>((size_t)1 << 20, 4 * h * (size_t)n1 * n2),
+                              cgemm_scratch<C>(n1, n2, R, (int)h));
   w.sk = cv.take<C>(w.sk_elems);
   w.bytes = cv.bytes();
   return w;
@@ -101,9 +101,9 @@ static LrWs<T> carve_lr(void* base, int n1, int n2, int n3, int R) {
 
 template <typename T>
 static int lowrank_run(const T* U, const T* S, const T* V, int n1, int n2, int n3, int R, T* X, void* ws,
-                       cudaStream_t s) {
+                       size_t have, cudaStream_t s) {
   using C = cx_t<T>;
-  LrWs<T> w = carve_lr<T>(ws, n1, n2, n3, R);
+  LrWs<T> w = carve_lr<T>(ws, n1, n2, n3, R, have);
   const int h = n3 / 2 + 1;
   TSVD_TRY(launch_rfft3<T>(U, w.Uh, (long)n1 * R, n3, s));
   TSVD_TRY(launch_rfft3<T>(V, w.Vh, (long)n2 * R, n3, s));
@@ -123,8 +123,10 @@ using namespace tsvd;
 
 extern "C" int tsvd_lowrank_workspace_size(int n1, int n2, int n3, int R, int precision, size_t* bytes) {
   if (!bytes || n1 < 1 || n2 < 1 || n3 < 1 || R < 1) return TSVD_ERR_INVALID_ARG;
-  if (precision == TSVD_FP64) *bytes = carve_lr<double>(nullptr, n1, n2, n3, R).bytes;
-  else if (precision == TSVD_FP32) *bytes = carve_lr<float>(nullptr, n1, n2, n3, R).bytes;
+  const size_t have = (precision & TSVD_WS_LEAST) ? 0 : WS_ALL;
+  precision &= ~TSVD_WS_LEAST;
+  if (precision == TSVD_FP64) *bytes = carve_lr<double>(nullptr, n1, n2, n3, R, have).bytes;
+  else if (precision == TSVD_FP32) *bytes = carve_lr<float>(nullptr, n1, n2, n3, R, have).bytes;
   else return TSVD_ERR_INVALID_ARG;
   return TSVD_OK;
 }
@@ -132,14 +134,15 @@ extern "C" int tsvd_lowrank_workspace_size(int n1, int n2, int n3, int R, int pr
 extern "C" int tsvd_lowrank(const void* U, const void* S, const void* V, int n1, int n2, int n3, int R, int precision,
                             void* X, void* ws, size_t ws_bytes, void* stream) {
   size_t need = 0;
-  TSVD_TRY(tsvd_lowrank_workspace_size(n1, n2, n3, R, precision, &need));
+  if (precision != TSVD_FP64 && precision != TSVD_FP32) return TSVD_ERR_INVALID_ARG;
+  TSVD_TRY(tsvd_lowrank_workspace_size(n1, n2, n3, R, precision | TSVD_WS_LEAST, &need));
   if (!U || !S || !V || !X || !ws || ((uintptr_t)ws & 255) != 0) return TSVD_ERR_INVALID_ARG;
   if (ws_bytes < need) return TSVD_ERR_WORKSPACE;
   cudaStream_t s = (cudaStream_t)stream;
   if (precision == TSVD_FP64)
     return lowrank_run<double>((const double*)U, (const double*)S, (const double*)V, n1, n2, n3, R, (double*)X, ws,
-                               s);
-  return lowrank_run<float>((const float*)U, (const float*)S, (const float*)V, n1, n2, n3, R, (float*)X, ws, s);
+                               ws_bytes, s);
+  return lowrank_run<float>((const float*)U, (const float*)S, (const float*)V, n1, n2, n3, R, (float*)X, ws, ws_bytes, s);
 }
 
 extern "C" int tsvd_sigma_tubes(const double* sigma_hat, int R, int n3, double power, int precision, void* tubes,

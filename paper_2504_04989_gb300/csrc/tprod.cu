@@ -51,11 +51,12 @@ static GemmArgs gm(char opA, char opB, int M, int N, int K, double alpha, const 
   return g;
 }
 
-// complex elements of product scratch: split-K partials, or the operands of the tensor-core form of
-// the products M x N x K given
+constexpr size_t SPLITK_ELEMS = (size_t)1 << 22;  // complex elements of split-K scratch, the least that a call takes
+
+// complex elements of scratch for the operands of the tensor-core form of the products M x N x K given
 template <typename C>
 static size_t scratch_elems(int batch, std::initializer_list<std::array<int, 3>> shapes) {
-  size_t n = (size_t)1 << 22;
+  size_t n = 0;
   for (const auto& t : shapes) n = std::max(n, cgemm_scratch<C>(t[0], t[1], t[2], batch));
   return n;
 }
@@ -69,22 +70,23 @@ struct TprodWs {
   size_t bytes;
 };
 template <typename T>
-static TprodWs<T> carve_tprod(void* base, int n1, int n2, int n4, int n3) {
+static TprodWs<T> carve_tprod(void* base, int n1, int n2, int n4, int n3, size_t have) {
   Carver cv(base);
   const size_t h = n3 / 2 + 1;
   TprodWs<T> w;
   w.Ah = cv.take<cx_t<T>>(h * n1 * n2);
   w.Bh = cv.take<cx_t<T>>(h * n2 * n4);
   w.Ch = cv.take<cx_t<T>>(h * n1 * n4);
-  w.sk_elems = scratch_elems<cx_t<T>>((int)h, {std::array<int, 3>{n1, n4, n2}});
+  w.sk_elems = fit_scratch<cx_t<T>>(cv, have, SPLITK_ELEMS, scratch_elems<cx_t<T>>((int)h, {std::array<int, 3>{n1, n4, n2}}));
   w.sk = cv.take<cx_t<T>>(w.sk_elems);
   w.bytes = cv.bytes();
   return w;
 }
 
 template <typename T>
-static int tprod_run(const T* A, const T* B, T* Cout, int n1, int n2, int n4, int n3, void* ws, cudaStream_t s) {
-  TprodWs<T> w = carve_tprod<T>(ws, n1, n2, n4, n3);
+static int tprod_run(const T* A, const T* B, T* Cout, int n1, int n2, int n4, int n3, void* ws, size_t have,
+                     cudaStream_t s) {
+  TprodWs<T> w = carve_tprod<T>(ws, n1, n2, n4, n3, have);
   const int h = n3 / 2 + 1;
   {
     TSVD_STAGE("tprod_rfft", s);
@@ -189,7 +191,7 @@ struct TbwdWs {
   size_t bytes;
 };
 template <typename T>
-static TbwdWs<T> carve_tbwd(void* base, int n1, int n2, int n4, int n3) {
+static TbwdWs<T> carve_tbwd(void* base, int n1, int n2, int n4, int n3, size_t have) {
   Carver cv(base);
   const size_t h = n3 / 2 + 1;
   TbwdWs<T> w;
@@ -198,16 +200,18 @@ static TbwdWs<T> carve_tbwd(void* base, int n1, int n2, int n4, int n3) {
   w.dCh = cv.take<cx_t<T>>(h * n1 * n4);
   w.dAh = cv.take<cx_t<T>>(h * n1 * n2);
   w.dBh = cv.take<cx_t<T>>(h * n2 * n4);
-  w.sk_elems = scratch_elems<cx_t<T>>((int)h, {std::array<int, 3>{n1, n2, n4}, std::array<int, 3>{n2, n4, n1}});
+  w.sk_elems = fit_scratch<cx_t<T>>(
+      cv, have, SPLITK_ELEMS,
+      scratch_elems<cx_t<T>>((int)h, {std::array<int, 3>{n1, n2, n4}, std::array<int, 3>{n2, n4, n1}}));
   w.sk = cv.take<cx_t<T>>(w.sk_elems);
   w.bytes = cv.bytes();
   return w;
 }
 
 template <typename T>
-static int tbwd_run(const T* A, const T* B, const T* dC, T* dA, T* dB, int n1, int n2, int n4, int n3, void* ws,
+static int tbwd_run(const T* A, const T* B, const T* dC, T* dA, T* dB, int n1, int n2, int n4, int n3, void* ws, size_t have,
                     cudaStream_t s) {
-  TbwdWs<T> w = carve_tbwd<T>(ws, n1, n2, n4, n3);
+  TbwdWs<T> w = carve_tbwd<T>(ws, n1, n2, n4, n3, have);
   const int h = n3 / 2 + 1;
   TSVD_TRY(launch_rfft3<T>(dC, w.dCh, (long)n1 * n4, n3, s));
   if (dA) {
@@ -234,7 +238,7 @@ struct TprojWs {
   size_t bytes;
 };
 template <typename T>
-static TprojWs<T> carve_tproj(void* base, int n1, int m, int n2, int n3) {
+static TprojWs<T> carve_tproj(void* base, int n1, int m, int n2, int n3, size_t have) {
   Carver cv(base);
   const size_t h = n3 / 2 + 1;
   TprojWs<T> w;
@@ -245,16 +249,19 @@ static TprojWs<T> carve_tproj(void* base, int n1, int m, int n2, int n3) {
   w.T2 = cv.take<cx_t<T>>(h * (size_t)n2 * m);
   w.dAh = cv.take<cx_t<T>>(h * n1 * n2);
   w.dQh = cv.take<cx_t<T>>(h * n1 * m);
-  w.sk_elems = scratch_elems<cx_t<T>>((int)h, {std::array<int, 3>{m, n2, n1}, std::array<int, 3>{n1, n2, m}, std::array<int, 3>{n2, m, n1}, std::array<int, 3>{n1, m, n2}});
+  w.sk_elems = fit_scratch<cx_t<T>>(
+      cv, have, SPLITK_ELEMS,
+      scratch_elems<cx_t<T>>((int)h, {std::array<int, 3>{m, n2, n1}, std::array<int, 3>{n1, n2, m},
+                                      std::array<int, 3>{n2, m, n1}, std::array<int, 3>{n1, m, n2}}));
   w.sk = cv.take<cx_t<T>>(w.sk_elems);
   w.bytes = cv.bytes();
   return w;
 }
 
 template <typename T>
-static int tproj_run(const T* Q, const T* A, const T* dY, T* dQ, T* dA, int n1, int m, int n2, int n3, void* ws,
+static int tproj_run(const T* Q, const T* A, const T* dY, T* dQ, T* dA, int n1, int m, int n2, int n3, void* ws, size_t have,
                      cudaStream_t s) {
-  TprojWs<T> w = carve_tproj<T>(ws, n1, m, n2, n3);
+  TprojWs<T> w = carve_tproj<T>(ws, n1, m, n2, n3, have);
   const int h = n3 / 2 + 1;
   using C = cx_t<T>;
   TSVD_TRY(launch_rfft3<T>(Q, w.Qh, (long)n1 * m, n3, s));
@@ -279,8 +286,8 @@ static int tproj_run(const T* Q, const T* A, const T* dY, T* dQ, T* dA, int n1, 
 }
 
 template <typename T>
-static int tproj_fwd_run(const T* Q, const T* A, T* Y, int n1, int m, int n2, int n3, void* ws, cudaStream_t s) {
-  TprojWs<T> w = carve_tproj<T>(ws, n1, m, n2, n3);
+static int tproj_fwd_run(const T* Q, const T* A, T* Y, int n1, int m, int n2, int n3, void* ws, size_t have, cudaStream_t s) {
+  TprojWs<T> w = carve_tproj<T>(ws, n1, m, n2, n3, have);
   const int h = n3 / 2 + 1;
   using C = cx_t<T>;
   TSVD_TRY(launch_rfft3<T>(Q, w.Qh, (long)n1 * m, n3, s));
@@ -300,9 +307,11 @@ using namespace tsvd;
 
 extern "C" int tprod_workspace_size(int n1, int n2, int n4, int n3, int precision, size_t* bytes) {
   if (!bytes || !dims_ok(n1, n2, n4, n3)) return TSVD_ERR_INVALID_ARG;
+  const size_t have = (precision & TSVD_WS_LEAST) ? 0 : WS_ALL;
+  precision &= ~TSVD_WS_LEAST;
   TSVD_TRY(check_prec_fwd(precision));
-  if (precision == TSVD_FP64) *bytes = carve_tprod<double>(nullptr, n1, n2, n4, n3).bytes;
-  else if (precision == TSVD_FP32) *bytes = carve_tprod<float>(nullptr, n1, n2, n4, n3).bytes;
+  if (precision == TSVD_FP64) *bytes = carve_tprod<double>(nullptr, n1, n2, n4, n3, have).bytes;
+  else if (precision == TSVD_FP32) *bytes = carve_tprod<float>(nullptr, n1, n2, n4, n3, have).bytes;
   else *bytes = carve_tprod_tc(nullptr, n1, n2, n4, n3, precision - TSVD_MIXED_TF32).bytes;
   return TSVD_OK;
 }
@@ -311,13 +320,14 @@ extern "C" int tprod(const void* A, const void* B, void* C, int n1, int n2, int 
                      size_t ws_bytes, void* stream) {
   if (!A || !B || !C || !ws || !dims_ok(n1, n2, n4, n3) || !aligned(ws)) return TSVD_ERR_INVALID_ARG;
   size_t need;
-  TSVD_TRY(tprod_workspace_size(n1, n2, n4, n3, precision, &need));
+  TSVD_TRY(check_prec_fwd(precision));
+  TSVD_TRY(tprod_workspace_size(n1, n2, n4, n3, precision | TSVD_WS_LEAST, &need));
   if (ws_bytes < need) return TSVD_ERR_WORKSPACE;
   cudaStream_t s = (cudaStream_t)stream;
   if (precision == TSVD_FP64)
-    return tprod_run<double>((const double*)A, (const double*)B, (double*)C, n1, n2, n4, n3, ws, s);
+    return tprod_run<double>((const double*)A, (const double*)B, (double*)C, n1, n2, n4, n3, ws, ws_bytes, s);
   if (precision == TSVD_FP32)
-    return tprod_run<float>((const float*)A, (const float*)B, (float*)C, n1, n2, n4, n3, ws, s);
+    return tprod_run<float>((const float*)A, (const float*)B, (float*)C, n1, n2, n4, n3, ws, ws_bytes, s);
   // TF32 (mode 0), BF16 (1), split TF32 (2) on tcgen05
   return tprod_tc_run((const float*)A, (const float*)B, (float*)C, n1, n2, n4, n3, precision - TSVD_MIXED_TF32, ws,
                       s);
@@ -325,9 +335,11 @@ extern "C" int tprod(const void* A, const void* B, void* C, int n1, int n2, int 
 
 extern "C" int tprod_backward_workspace_size(int n1, int n2, int n4, int n3, int precision, size_t* bytes) {
   if (!bytes || !dims_ok(n1, n2, n4, n3)) return TSVD_ERR_INVALID_ARG;
+  const size_t have = (precision & TSVD_WS_LEAST) ? 0 : WS_ALL;
+  precision &= ~TSVD_WS_LEAST;
   TSVD_TRY(check_prec(precision));
-  *bytes = precision == TSVD_FP64 ? carve_tbwd<double>(nullptr, n1, n2, n4, n3).bytes
-                                  : carve_tbwd<float>(nullptr, n1, n2, n4, n3).bytes;
+  *bytes = precision == TSVD_FP64 ? carve_tbwd<double>(nullptr, n1, n2, n4, n3, have).bytes
+                                  : carve_tbwd<float>(nullptr, n1, n2, n4, n3, have).bytes;
   return TSVD_OK;
 }
 
@@ -336,21 +348,24 @@ extern "C" int tprod_backward(const void* A, const void* B, const void* dC, void
   if (!dC || !ws || !dims_ok(n1, n2, n4, n3) || !aligned(ws)) return TSVD_ERR_INVALID_ARG;
   if ((dA && !B) || (dB && !A)) return TSVD_ERR_INVALID_ARG;
   size_t need;
-  TSVD_TRY(tprod_backward_workspace_size(n1, n2, n4, n3, precision, &need));
+  TSVD_TRY(check_prec(precision));
+  TSVD_TRY(tprod_backward_workspace_size(n1, n2, n4, n3, precision | TSVD_WS_LEAST, &need));
   if (ws_bytes < need) return TSVD_ERR_WORKSPACE;
   cudaStream_t s = (cudaStream_t)stream;
   if (precision == TSVD_FP64)
     return tbwd_run<double>((const double*)A, (const double*)B, (const double*)dC, (double*)dA, (double*)dB, n1, n2,
-                            n4, n3, ws, s);
+                            n4, n3, ws, ws_bytes, s);
   return tbwd_run<float>((const float*)A, (const float*)B, (const float*)dC, (float*)dA, (float*)dB, n1, n2, n4, n3,
-                         ws, s);
+                         ws, ws_bytes, s);
 }
 
 extern "C" int tproj_backward_workspace_size(int n1, int m, int n2, int n3, int precision, size_t* bytes) {
   if (!bytes || !dims_ok(n1, m, n2, n3)) return TSVD_ERR_INVALID_ARG;
+  const size_t have = (precision & TSVD_WS_LEAST) ? 0 : WS_ALL;
+  precision &= ~TSVD_WS_LEAST;
   TSVD_TRY(check_prec(precision));
-  *bytes = precision == TSVD_FP64 ? carve_tproj<double>(nullptr, n1, m, n2, n3).bytes
-                                  : carve_tproj<float>(nullptr, n1, m, n2, n3).bytes;
+  *bytes = precision == TSVD_FP64 ? carve_tproj<double>(nullptr, n1, m, n2, n3, have).bytes
+                                  : carve_tproj<float>(nullptr, n1, m, n2, n3, have).bytes;
   return TSVD_OK;
 }
 
@@ -359,14 +374,15 @@ extern "C" int tproj_backward(const void* Q, const void* A, const void* dY, void
   if (!Q || !dY || !ws || !dims_ok(n1, m, n2, n3) || !aligned(ws)) return TSVD_ERR_INVALID_ARG;
   if (dQ && !A) return TSVD_ERR_INVALID_ARG;
   size_t need;
-  TSVD_TRY(tproj_backward_workspace_size(n1, m, n2, n3, precision, &need));
+  TSVD_TRY(check_prec(precision));
+  TSVD_TRY(tproj_backward_workspace_size(n1, m, n2, n3, precision | TSVD_WS_LEAST, &need));
   if (ws_bytes < need) return TSVD_ERR_WORKSPACE;
   cudaStream_t s = (cudaStream_t)stream;
   if (precision == TSVD_FP64)
     return tproj_run<double>((const double*)Q, (const double*)A, (const double*)dY, (double*)dQ, (double*)dA, n1, m,
-                             n2, n3, ws, s);
+                             n2, n3, ws, ws_bytes, s);
   return tproj_run<float>((const float*)Q, (const float*)A, (const float*)dY, (float*)dQ, (float*)dA, n1, m, n2, n3,
-                          ws, s);
+                          ws, ws_bytes, s);
 }
 
 extern "C" int tproj_workspace_size(int n1, int m, int n2, int n3, int precision, size_t* bytes) {
@@ -377,10 +393,11 @@ extern "C" int tproj(const void* Q, const void* A, void* Y, int n1, int m, int n
                      size_t ws_bytes, void* stream) {
   if (!Q || !A || !Y || !ws || !dims_ok(n1, m, n2, n3) || !aligned(ws)) return TSVD_ERR_INVALID_ARG;
   size_t need;
-  TSVD_TRY(tproj_workspace_size(n1, m, n2, n3, precision, &need));
+  TSVD_TRY(check_prec(precision));
+  TSVD_TRY(tproj_workspace_size(n1, m, n2, n3, precision | TSVD_WS_LEAST, &need));
   if (ws_bytes < need) return TSVD_ERR_WORKSPACE;
   cudaStream_t s = (cudaStream_t)stream;
   if (precision == TSVD_FP64)
-    return tproj_fwd_run<double>((const double*)Q, (const double*)A, (double*)Y, n1, m, n2, n3, ws, s);
-  return tproj_fwd_run<float>((const float*)Q, (const float*)A, (float*)Y, n1, m, n2, n3, ws, s);
+    return tproj_fwd_run<double>((const double*)Q, (const double*)A, (double*)Y, n1, m, n2, n3, ws, ws_bytes, s);
+  return tproj_fwd_run<float>((const float*)Q, (const float*)A, (float*)Y, n1, m, n2, n3, ws, ws_bytes, s);
 }

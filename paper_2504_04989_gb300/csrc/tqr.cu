@@ -142,7 +142,7 @@ static int tqr_dims(int n1, int n2, int n3, int precision, bool pinv, TqrDims* d
 }
 
 template <typename T>
-static TqrWs<T> carve_tqr(void* base, const TqrDims& d, bool pinv) {
+static TqrWs<T> carve_tqr(void* base, const TqrDims& d, bool pinv, size_t have) {
   using C = cx_t<T>;
   Carver cv(base);
   TqrWs<T> w;
@@ -160,11 +160,13 @@ static TqrWs<T> carve_tqr(void* base, const TqrDims& d, bool pinv) {
   w.Xp = pinv ? cv.take<C>(h * d.n2 * d.n1) : nullptr;
   w.dead = cv.take<uint32_t>(h * 4);
   w.counters = cv.take<int>(8);
-  w.splitk_elems = std::min<size_t>((size_t)1 << 22, 8 * h * (size_t)d.p * std::max(d.b, 64));
   const int hb = (int)h, shapes[][3] = {{d.p, d.Nc, d.Mr}, {d.b, d.b, d.Mr}, {d.p, d.b, d.Mr}, {d.Mr, d.b, d.p},
                                         {d.Mr, d.b, d.b}, {d.p, d.Mr, d.p}, {d.Mr, d.p, d.p}};
+  size_t best = 0;
   for (const auto& t : shapes)
-    w.splitk_elems = std::max(w.splitk_elems, cgemm_scratch<C>(t[0], t[1], t[2], hb) * sizeof(C) / sizeof(double2) + 1);
+    best = std::max(best, cgemm_scratch<C>(t[0], t[1], t[2], hb) * sizeof(C) / sizeof(double2) + 1);
+  w.splitk_elems = fit_scratch<double2>(cv, have, std::min<size_t>((size_t)1 << 22, 8 * h * (size_t)d.p * std::max(d.b, 64)),
+                                        best);
   w.splitk = cv.take<double2>(w.splitk_elems);
   w.bytes = cv.bytes();
   return w;
@@ -223,8 +225,8 @@ static int read_status(int* counters, cudaStream_t s, tsvd_info* info, int p, bo
 }
 
 template <typename T>
-static int tqr_run(const T* A, const TqrDims& d, T* Qout, T* Rout, void* ws, cudaStream_t s, tsvd_info* info) {
-  TqrWs<T> w = carve_tqr<T>(ws, d, false);
+static int tqr_run(const T* A, const TqrDims& d, T* Qout, T* Rout, void* ws, size_t have, cudaStream_t s, tsvd_info* info) {
+  TqrWs<T> w = carve_tqr<T>(ws, d, false, have);
   TSVD_TRY(launch_rfft3<T>(A, w.Ah, (long)d.n1 * d.n2, d.n3, s));
   TSVD_TRY(tqr_factor<T>(d, w, w.Ah, s));
   TSVD_TRY(launch_irfft3<T>(w.Q, Qout, (long)d.n1 * d.p, d.n3, s));
@@ -233,9 +235,9 @@ static int tqr_run(const T* A, const TqrDims& d, T* Qout, T* Rout, void* ws, cud
 }
 
 template <typename T>
-static int tpinv_run(const T* A, const TqrDims& d, T* Xout, void* ws, cudaStream_t s, tsvd_info* info) {
+static int tpinv_run(const T* A, const TqrDims& d, T* Xout, void* ws, size_t have, cudaStream_t s, tsvd_info* info) {
   using C = cx_t<T>;
-  TqrWs<T> w = carve_tqr<T>(ws, d, true);
+  TqrWs<T> w = carve_tqr<T>(ws, d, true, have);
   const int p = d.p, Mr = d.Mr, h = d.h;
   const long sP = (long)p * p;
   const size_t sk = std::is_same<T, double>::value ? w.splitk_elems : 2 * w.splitk_elems;
@@ -281,8 +283,11 @@ using namespace tsvd;
 extern "C" int tqr_workspace_size(int n1, int n2, int n3, int precision, size_t* bytes) {
   if (!bytes) return TSVD_ERR_INVALID_ARG;
   TqrDims d;
+  const size_t have = (precision & TSVD_WS_LEAST) ? 0 : WS_ALL;
+  precision &= ~TSVD_WS_LEAST;
   TSVD_TRY(tqr_dims(n1, n2, n3, precision, false, &d));
-  *bytes = precision == TSVD_FP64 ? carve_tqr<double>(nullptr, d, false).bytes : carve_tqr<float>(nullptr, d, false).bytes;
+  *bytes = precision == TSVD_FP64 ? carve_tqr<double>(nullptr, d, false, have).bytes
+                                  : carve_tqr<float>(nullptr, d, false, have).bytes;
   return TSVD_OK;
 }
 
@@ -292,18 +297,21 @@ extern "C" int tqr(const void* A, int n1, int n2, int n3, int precision, void* Q
   TSVD_TRY(tqr_dims(n1, n2, n3, precision, false, &d));
   if (!A || !Q || !R || !ws || ((uintptr_t)ws & 255) != 0) return TSVD_ERR_INVALID_ARG;
   size_t need = 0;
-  TSVD_TRY(tqr_workspace_size(n1, n2, n3, precision, &need));
+  TSVD_TRY(tqr_workspace_size(n1, n2, n3, precision | TSVD_WS_LEAST, &need));
   if (ws_bytes < need) return TSVD_ERR_WORKSPACE;
   cudaStream_t s = (cudaStream_t)stream;
-  if (precision == TSVD_FP64) return tqr_run<double>((const double*)A, d, (double*)Q, (double*)R, ws, s, info);
-  return tqr_run<float>((const float*)A, d, (float*)Q, (float*)R, ws, s, info);
+  if (precision == TSVD_FP64) return tqr_run<double>((const double*)A, d, (double*)Q, (double*)R, ws, ws_bytes, s, info);
+  return tqr_run<float>((const float*)A, d, (float*)Q, (float*)R, ws, ws_bytes, s, info);
 }
 
 extern "C" int tpinv_workspace_size(int n1, int n2, int n3, int precision, size_t* bytes) {
   if (!bytes) return TSVD_ERR_INVALID_ARG;
   TqrDims d;
+  const size_t have = (precision & TSVD_WS_LEAST) ? 0 : WS_ALL;
+  precision &= ~TSVD_WS_LEAST;
   TSVD_TRY(tqr_dims(n1, n2, n3, precision, true, &d));
-  *bytes = precision == TSVD_FP64 ? carve_tqr<double>(nullptr, d, true).bytes : carve_tqr<float>(nullptr, d, true).bytes;
+  *bytes = precision == TSVD_FP64 ? carve_tqr<double>(nullptr, d, true, have).bytes
+                                  : carve_tqr<float>(nullptr, d, true, have).bytes;
   return TSVD_OK;
 }
 
@@ -313,9 +321,9 @@ extern "C" int tpinv(const void* A, int n1, int n2, int n3, int precision, void*
   TSVD_TRY(tqr_dims(n1, n2, n3, precision, true, &d));
   if (!A || !X || !ws || ((uintptr_t)ws & 255) != 0) return TSVD_ERR_INVALID_ARG;
   size_t need = 0;
-  TSVD_TRY(tpinv_workspace_size(n1, n2, n3, precision, &need));
+  TSVD_TRY(tpinv_workspace_size(n1, n2, n3, precision | TSVD_WS_LEAST, &need));
   if (ws_bytes < need) return TSVD_ERR_WORKSPACE;
   cudaStream_t s = (cudaStream_t)stream;
-  if (precision == TSVD_FP64) return tpinv_run<double>((const double*)A, d, (double*)X, ws, s, info);
-  return tpinv_run<float>((const float*)A, d, (float*)X, ws, s, info);
+  if (precision == TSVD_FP64) return tpinv_run<double>((const double*)A, d, (double*)X, ws, ws_bytes, s, info);
+  return tpinv_run<float>((const float*)A, d, (float*)X, ws, ws_bytes, s, info);
 }

@@ -137,7 +137,7 @@ struct RbkWs {
 };
 
 template <typename T, typename L>
-static RbkWs<T> carve_rbk(void* base, const RbkDims& d) {
+static RbkWs<T> carve_rbk(void* base, const RbkDims& d, size_t have) {
   using C = cx_t<T>;
   using CL = cx_t<L>;
   constexpr bool dbl = std::is_same<T, double>::value;
@@ -205,15 +205,6 @@ static RbkWs<T> carve_rbk(void* base, const RbkDims& d) {
     t.Qdlo = cv.take<float>(h * 2 * (size_t)d.m * (t.ldq2 / 2));
     t.err = w.tc_err;
   }
-  w.splitk_elems = 8 * h * (size_t)d.m * std::max(d.b, 64);
-  const int hb = d.h, shapes[][3] = {{d.n1, d.b, d.n2}, {d.n2, d.b, d.n1}, {d.m, d.b, d.n1}, {d.n1, d.b, d.m},
-                                     {d.b, d.b, d.n1},  {d.n1, d.b, d.b}, {d.mp, d.mp, d.n2}, {d.n1, d.R, d.mp},
-                                     {d.n2, d.R, d.mp}};
-  for (const auto& t : shapes) {  // the orthonormalisation's products run in L, the others in T
-    w.splitk_elems = std::max(w.splitk_elems, cgemm_scratch<CL>(t[0], t[1], t[2], hb) * sizeof(CL) / sizeof(double2) + 1);
-    w.splitk_elems = std::max(w.splitk_elems, cgemm_scratch<C>(t[0], t[1], t[2], hb) * sizeof(C) / sizeof(double2) + 1);
-  }
-  w.splitk = cv.take<double2>(w.splitk_elems);
   w.lamF = nullptr;
   w.UF = w.Um = w.T1 = w.CpH = nullptr;
   w.acc = nullptr;
@@ -225,10 +216,19 @@ static RbkWs<T> carve_rbk(void* base, const RbkDims& d) {
     w.CpH = cv.take<double2>(h * d.n2 * d.mp);
     w.acc = cv.take<int>(h);
   }
+  const int hb = d.h, shapes[][3] = {{d.n1, d.b, d.n2}, {d.n2, d.b, d.n1}, {d.m, d.b, d.n1}, {d.n1, d.b, d.m},
+                                     {d.b, d.b, d.n1},  {d.n1, d.b, d.b}, {d.mp, d.mp, d.n2}, {d.n1, d.R, d.mp},
+                                     {d.n2, d.R, d.mp}};
+  size_t best = 0;
+  for (const auto& t : shapes) {  // the orthonormalisation's products run in L, the others in T
+    best = std::max(best, cgemm_scratch<CL>(t[0], t[1], t[2], hb) * sizeof(CL) / sizeof(double2) + 1);
+    best = std::max(best, cgemm_scratch<C>(t[0], t[1], t[2], hb) * sizeof(C) / sizeof(double2) + 1);
+  }
+  w.splitk_elems = fit_scratch<double2>(cv, have, 8 * h * (size_t)d.m * std::max(d.b, 64), best);
+  w.splitk = cv.take<double2>(w.splitk_elems);
   w.bytes = cv.bytes();
   return w;
 }
-
 
 // Orthonormalise the nb leading columns of the Krylov block W against the c
 // finished columns of Q (orth_block_cols in cholqr.cu: shifted CholeskyQR3
@@ -343,10 +343,10 @@ static int deflated_passes(const RbkDims& d, RbkWs<double>& w, cudaStream_t s) {
 
 template <typename T, typename L>
 static int rbk_run(const T* A, const RbkDims& d, const tsvd_params& p, const T* Omega, T* U, T* S, T* V,
-                   double* sig, void* ws, cudaStream_t s, tsvd_info* info, const cx_t<T>* Ahat = nullptr,
+                   double* sig, void* ws, size_t have, cudaStream_t s, tsvd_info* info, const cx_t<T>* Ahat = nullptr,
                    cx_t<T>* Uhat = nullptr, cx_t<T>* Vhat = nullptr) {
   using C = cx_t<T>;
-  RbkWs<T> w = carve_rbk<T, L>(ws, d);
+  RbkWs<T> w = carve_rbk<T, L>(ws, d, have);
   if (d.fourier) {  // Fourier slices k0 .. k0+h-1 given and returned by the caller
     w.Ah = const_cast<C*>(Ahat);
     w.Uh = Uhat;
@@ -514,17 +514,19 @@ static int rbk_run(const T* A, const RbkDims& d, const tsvd_params& p, const T* 
 
 using namespace tsvd;
 
-static size_t rbk_bytes(const RbkDims& d, const tsvd_params* p) {
-  if (p->precision == TSVD_FP64) return carve_rbk<double, double>(nullptr, d).bytes;
-  if (p->flags & TSVD_FLAG_FP64_QR) return carve_rbk<float, double>(nullptr, d).bytes;
-  return carve_rbk<float, float>(nullptr, d).bytes;
+// the workspace with which the call runs (least) or that its products gain by
+static size_t rbk_bytes(const RbkDims& d, const tsvd_params* p, bool least) {
+  const size_t have = least ? 0 : WS_ALL;
+  if (p->precision == TSVD_FP64) return carve_rbk<double, double>(nullptr, d, have).bytes;
+  if (p->flags & TSVD_FLAG_FP64_QR) return carve_rbk<float, double>(nullptr, d, have).bytes;
+  return carve_rbk<float, float>(nullptr, d, have).bytes;
 }
 
 extern "C" int tsvd_rbk_workspace_size(int n1, int n2, int n3, const tsvd_params* params, size_t* bytes) {
   if (!bytes) return TSVD_ERR_INVALID_ARG;
   RbkDims d;
   TSVD_TRY(rbk_dims(n1, n2, n3, params, &d));
-  *bytes = rbk_bytes(d, params);
+  *bytes = rbk_bytes(d, params, (params->flags & TSVD_WS_LEAST) != 0);
   return TSVD_OK;
 }
 
@@ -535,16 +537,16 @@ extern "C" int tsvd_rbk(const void* A, int n1, int n2, int n3, const tsvd_params
   TSVD_TRY(rbk_dims(n1, n2, n3, params, &d));
   if (!A || !U || !S || !V || !ws) return TSVD_ERR_INVALID_ARG;
   if (((uintptr_t)ws & 255) != 0) return TSVD_ERR_INVALID_ARG;
-  if (ws_bytes < rbk_bytes(d, params)) return TSVD_ERR_WORKSPACE;
+  if (ws_bytes < rbk_bytes(d, params, true)) return TSVD_ERR_WORKSPACE;
   cudaStream_t s = (cudaStream_t)stream;
   if (params->precision == TSVD_FP64)
     return rbk_run<double, double>((const double*)A, d, *params, (const double*)Omega, (double*)U, (double*)S,
-                                   (double*)V, sigma_hat, ws, s, info);
+                                   (double*)V, sigma_hat, ws, ws_bytes, s, info);
   if (params->flags & TSVD_FLAG_FP64_QR)
     return rbk_run<float, double>((const float*)A, d, *params, (const float*)Omega, (float*)U, (float*)S, (float*)V,
-                                  sigma_hat, ws, s, info);
+                                  sigma_hat, ws, ws_bytes, s, info);
   return rbk_run<float, float>((const float*)A, d, *params, (const float*)Omega, (float*)U, (float*)S, (float*)V,
-                               sigma_hat, ws, s, info);
+                               sigma_hat, ws, ws_bytes, s, info);
 }
 
 // Alg. 2 on a block of Fourier slices [k0, k0 + ns) of an n1 x n2 x n3 tensor
@@ -567,7 +569,7 @@ extern "C" int tsvd_rbk_fourier_workspace_size(int n1, int n2, int n3, int k0, i
   if (!bytes) return TSVD_ERR_INVALID_ARG;
   RbkDims d;
   TSVD_TRY(rbk_fourier_dims(n1, n2, n3, k0, ns, params, &d));
-  *bytes = rbk_bytes(d, params);
+  *bytes = rbk_bytes(d, params, (params->flags & TSVD_WS_LEAST) != 0);
   return TSVD_OK;
 }
 
@@ -578,15 +580,15 @@ extern "C" int tsvd_rbk_fourier(const void* Ahat, int n1, int n2, int n3, int k0
   TSVD_TRY(rbk_fourier_dims(n1, n2, n3, k0, ns, params, &d));
   if (!Ahat || !Uhat || !Vhat || !sigma_hat || !ws) return TSVD_ERR_INVALID_ARG;
   if (((uintptr_t)ws & 255) != 0) return TSVD_ERR_INVALID_ARG;
-  if (ws_bytes < rbk_bytes(d, params)) return TSVD_ERR_WORKSPACE;
+  if (ws_bytes < rbk_bytes(d, params, true)) return TSVD_ERR_WORKSPACE;
   cudaStream_t s = (cudaStream_t)stream;
   if (params->precision == TSVD_FP64)
     return rbk_run<double, double>(nullptr, d, *params, (const double*)Omega, nullptr, nullptr, nullptr, sigma_hat,
-                                   ws, s, info, (const double2*)Ahat, (double2*)Uhat, (double2*)Vhat);
+                                   ws, ws_bytes, s, info, (const double2*)Ahat, (double2*)Uhat, (double2*)Vhat);
   if (params->flags & TSVD_FLAG_FP64_QR)
     return rbk_run<float, double>(nullptr, d, *params, (const float*)Omega, nullptr, nullptr, nullptr, sigma_hat, ws,
-                                  s, info, (const float2*)Ahat, (float2*)Uhat, (float2*)Vhat);
-  return rbk_run<float, float>(nullptr, d, *params, (const float*)Omega, nullptr, nullptr, nullptr, sigma_hat, ws, s,
+                                  ws_bytes, s, info, (const float2*)Ahat, (float2*)Uhat, (float2*)Vhat);
+  return rbk_run<float, float>(nullptr, d, *params, (const float*)Omega, nullptr, nullptr, nullptr, sigma_hat, ws, ws_bytes, s,
                                info, (const float2*)Ahat, (float2*)Uhat, (float2*)Vhat);
 }
 
@@ -655,7 +657,7 @@ struct BatchPlan {
 
 static size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
-static int plan_batch(const tsvd_rbk_desc* descs, int count, int lanes, BatchPlan* bp) {
+static int plan_batch(const tsvd_rbk_desc* descs, int count, int lanes, bool least, BatchPlan* bp) {
   if (!descs || count < 0 || lanes < 1) return TSVD_ERR_INVALID_ARG;
   bp->lanes = std::max(1, std::min({lanes, kMaxLanes, std::max(count, 1)}));
   std::vector<double> cost(count);
@@ -664,7 +666,7 @@ static int plan_batch(const tsvd_rbk_desc* descs, int count, int lanes, BatchPla
     RbkDims d;
     TSVD_TRY(rbk_dims(descs[i].n1, descs[i].n2, descs[i].n3, &descs[i].params, &d));
     cost[i] = rbk_cost(d);
-    bytes[i] = align256(rbk_bytes(d, &descs[i].params));
+    bytes[i] = align256(rbk_bytes(d, &descs[i].params, least || (descs[i].params.flags & TSVD_WS_LEAST)));
   }
   bp->order.resize(count);
   for (int i = 0; i < count; ++i) bp->order[i] = i;
@@ -685,19 +687,19 @@ static int plan_batch(const tsvd_rbk_desc* descs, int count, int lanes, BatchPla
   return TSVD_OK;
 }
 
-static int rbk_one(const tsvd_rbk_desc& t, void* ws, cudaStream_t s) {
+static int rbk_one(const tsvd_rbk_desc& t, void* ws, size_t have, cudaStream_t s) {
   RbkDims d;
   TSVD_TRY(rbk_dims(t.n1, t.n2, t.n3, &t.params, &d));
   if (!t.A || !t.U || !t.S || !t.V) return TSVD_ERR_INVALID_ARG;
   const tsvd_params& p = t.params;
   if (p.precision == TSVD_FP64)
     return rbk_run<double, double>((const double*)t.A, d, p, (const double*)t.Omega, (double*)t.U, (double*)t.S,
-                                   (double*)t.V, t.sigma_hat, ws, s, nullptr);
+                                   (double*)t.V, t.sigma_hat, ws, have, s, nullptr);
   if (p.flags & TSVD_FLAG_FP64_QR)
     return rbk_run<float, double>((const float*)t.A, d, p, (const float*)t.Omega, (float*)t.U, (float*)t.S,
-                                  (float*)t.V, t.sigma_hat, ws, s, nullptr);
+                                  (float*)t.V, t.sigma_hat, ws, have, s, nullptr);
   return rbk_run<float, float>((const float*)t.A, d, p, (const float*)t.Omega, (float*)t.U, (float*)t.S, (float*)t.V,
-                               t.sigma_hat, ws, s, nullptr);
+                               t.sigma_hat, ws, have, s, nullptr);
 }
 
 }  // namespace tsvd
@@ -705,7 +707,7 @@ static int rbk_one(const tsvd_rbk_desc& t, void* ws, cudaStream_t s) {
 extern "C" int tsvd_rbk_batched_workspace_size(const tsvd_rbk_desc* descs, int count, int lanes, size_t* bytes) {
   if (!bytes) return TSVD_ERR_INVALID_ARG;
   BatchPlan bp;
-  TSVD_TRY(plan_batch(descs, count, lanes, &bp));
+  TSVD_TRY(plan_batch(descs, count, lanes, false, &bp));
   *bytes = bp.lane_off[bp.lanes];
   return TSVD_OK;
 }
@@ -713,14 +715,15 @@ extern "C" int tsvd_rbk_batched_workspace_size(const tsvd_rbk_desc* descs, int c
 extern "C" int tsvd_rbk_batched(const tsvd_rbk_desc* descs, int count, int lanes, void* ws, size_t ws_bytes,
                                 void* stream) {
   BatchPlan bp;
-  TSVD_TRY(plan_batch(descs, count, lanes, &bp));
+  TSVD_TRY(plan_batch(descs, count, lanes, false, &bp));
+  if (ws_bytes < bp.lane_off[bp.lanes]) TSVD_TRY(plan_batch(descs, count, lanes, true, &bp));
   if (count == 0) return TSVD_OK;
   if (!ws || ((uintptr_t)ws & 255) != 0) return TSVD_ERR_INVALID_ARG;
   if (ws_bytes < bp.lane_off[bp.lanes]) return TSVD_ERR_WORKSPACE;
   cudaStream_t s = (cudaStream_t)stream;
   char* base = (char*)ws;
   if (bp.lanes == 1) {
-    for (int i : bp.order) TSVD_TRY(rbk_one(descs[i], base, s));
+    for (int i : bp.order) TSVD_TRY(rbk_one(descs[i], base, bp.lane_off[1], s));
     return TSVD_OK;
   }
   LanePool* lp = nullptr;
@@ -731,7 +734,7 @@ extern "C" int tsvd_rbk_batched(const tsvd_rbk_desc* descs, int count, int lanes
   int rc = TSVD_OK;
   for (int i : bp.order) {
     const int l = bp.lane_of[i];
-    rc = rbk_one(descs[i], base + bp.lane_off[l], lp->s[l]);
+    rc = rbk_one(descs[i], base + bp.lane_off[l], bp.lane_off[l + 1] - bp.lane_off[l], lp->s[l]);
     if (rc != TSVD_OK) break;
   }
   // join every lane back into the caller's stream, also after an error
