@@ -15,6 +15,7 @@
 //                           sum for tubes too long for those.
 #include "common.cuh"
 #include "kernels.cuh"
+#include "unit_circle.cuh"
 
 namespace tsvd {
 
@@ -431,35 +432,6 @@ __global__ void __launch_bounds__(FFT_WARPS * 32) k_irfft3_fft(const cx_t<T>* __
 // in FP64 (64: 539 -> 341 us).
 // ---------------------------------------------------------------------------
 namespace ct {
-constexpr double kTau = 6.283185307179586476925286766559;
-constexpr double csin(double x) {
-  double t = x, s = x;
-  for (int k = 1; k < 12; ++k) {
-    t *= -x * x / (2.0 * k * (2.0 * k + 1.0));
-    s += t;
-  }
-  return s;
-}
-constexpr double ccos(double x) {
-  double t = 1.0, s = 1.0;
-  for (int k = 1; k < 12; ++k) {
-    t *= -x * x / ((2.0 * k - 1.0) * 2.0 * k);
-    s += t;
-  }
-  return s;
-}
-// cos and sin of 2 pi p / n (Taylor series on the first octant; exact on the axes)
-constexpr double cos2pi(long p, long n) {
-  p %= n;
-  if (2 * p > n) p = n - p;
-  if (4 * p == n) return 0.0;
-  if (4 * p > n) return -cos2pi(n - 2 * p, 2 * n);
-  if (8 * p > n) return csin(kTau * (double)(n - 4 * p) / (4.0 * (double)n));
-  return ccos(kTau * (double)p / (double)n);
-}
-constexpr double sin2pi(long p, long n) {  // cos(theta - pi/2)
-  return cos2pi(((4 * p - n) % (4 * n) + 4 * n) % (4 * n), 4 * n);
-}
 // position of frequency k in the output of dif_fft<., M, .>
 constexpr int pos(int k, int len) { return len <= 2 ? k : (k % 4) * (len / 4) + pos(k / 4, len / 4); }
 }  // namespace ct
