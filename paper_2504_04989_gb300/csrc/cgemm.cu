@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(GemmCfg<C, SMALL>::TD* GemmCfg<C, SMALL>::TD) 
   }
 }
 
-// FP32 (float2) products other than the Hermitian form: 128 x 64 tiles, each
+// FP32 (float2) products: 128 x 64 tiles, each
 // of the 256 threads holding an 8 x 4 complex register tile (rows 8 ty .. +7,
 // columns 4 tx .. +3), read from shared memory in 16-byte pieces: 6 loads per
 // 128 FMAs instead of 8 per 64.  Rows of the staged tiles are padded by 16
@@ -385,17 +385,17 @@ static int cgemm_tiles(const GemmArgs& g, C* ws, size_t splitk_elems, cudaStream
 }
 
 template <typename C>
-static int cgemm_impl(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t s, int herm, TcOpts st) {
+static int cgemm_impl(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t s, int herm, TcOpts st) {  // herm: FP64
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return TSVD_OK;
   if (g.batch > 65535) return TSVD_ERR_UNSUPPORTED;
   if (g.beta != 0.0 && g.beta != 1.0) return TSVD_ERR_INVALID_ARG;
   if constexpr (std::is_same<C, float2>::value) {
     const size_t bytes = splitk_ws ? splitk_elems * sizeof(C) : 0;
-    if (!st.simt && !herm && sgemm_tc_better(g, bytes)) return sgemm_tc(g, splitk_ws, bytes, s, st);
+    if (!st.simt && sgemm_tc_better(g, bytes)) return sgemm_tc(g, splitk_ws, bytes, s, st);
     // the wide tiles where they fill the GPU (two CTAs per SM), directly or by splitting a long K;
     // smaller products keep the 64 x 64 tiles (measured faster there)
     const long wtiles = (long)cdiv(g.M, WBM) * cdiv(g.N, WBN) * g.batch;
-    if (!herm && g.K > 0 && (wtiles >= 2L * 152 || (g.K >= 1024 && splitk_ws)))
+    if (g.K > 0 && (wtiles >= 2L * 152 || (g.K >= 1024 && splitk_ws)))
       return cgemm_wide(g, (float2*)splitk_ws, splitk_ws ? splitk_elems : 0, s);
   }
   if constexpr (std::is_same<C, double2>::value) {
@@ -443,13 +443,10 @@ size_t cgemm_scratch(int M, int N, int K, int batch) {
 template size_t cgemm_scratch<double2>(int, int, int, int);
 template size_t cgemm_scratch<float2>(int, int, int, int);
 
-template <typename C>
 int cgemm_herm(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t s, TcOpts st) {
   if (g.M != g.N || g.beta != 0.0) return TSVD_ERR_INVALID_ARG;
-  return cgemm_impl<C>(g, splitk_ws, splitk_elems, s, 1, st);
+  return cgemm_impl<double2>(g, splitk_ws, splitk_elems, s, 1, st);
 }
-template int cgemm_herm<double2>(const GemmArgs&, void*, size_t, cudaStream_t, TcOpts);
-template int cgemm_herm<float2>(const GemmArgs&, void*, size_t, cudaStream_t, TcOpts);
 template int cgemm<double2>(const GemmArgs&, void*, size_t, cudaStream_t, TcOpts);
 template int cgemm<float2>(const GemmArgs&, void*, size_t, cudaStream_t, TcOpts);
 

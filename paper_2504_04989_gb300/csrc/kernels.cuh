@@ -90,9 +90,8 @@ int load_simt_products();
 // it would keep to the SIMT units); a smaller splitk_elems only makes it slower
 template <typename C>
 size_t cgemm_scratch(int M, int N, int K, int batch);
-// C = op(A) op(B) known to be Hermitian (square, beta = 0, e.g. A^H A): only
+// FP64 C = op(A) op(B) known to be Hermitian (square, beta = 0, e.g. A^H A): only
 // the upper tiles are computed, the lower triangle is mirrored from them
-template <typename C>
 int cgemm_herm(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t s, TcOpts st = TcOpts());
 
 // dgemm_tc.cu -- the FP64 product as exact digit products on the BF16 tensor cores (cgemm and
@@ -209,10 +208,6 @@ int split_rows(const float* x, long ldx, float* hi, float* lo, long ldy, int col
 int split_block(const float* x, long ldx, float* hi, float* lo, long ldy, int cols, long rows, cudaStream_t s);
 // per slice complex X (rows x cols) -> X^T as real rows of 2 rows floats (leading dim ldt), hi / lo
 int split_transpose(const float2* X, int rows, int cols, int batch, float* hi, float* lo, long ldt, cudaStream_t s);
-// the same for a strided block (leading dim ldx, batch stride sx) into rows of leading dim ldt, batch stride st
-// (padding columns are not touched)
-int split_transpose_ld(const float2* X, int rows, int cols, long ldx, long sx, int batch, float* hi, float* lo,
-                       long ldt, long st, cudaStream_t s);
 // per slice the columns c of a complex X (rows x cols, leading dim ldx, batch stride sx) as real
 // rows 2c (real parts) and 2c+1 (imaginary parts) of length rows, split into hi / lo (leading dim
 // ldt, batch stride st; padding not touched)

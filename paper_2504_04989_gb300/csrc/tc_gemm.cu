@@ -562,16 +562,6 @@ int split_transpose(const float2* X, int rows, int cols, int batch, float* hi, f
   return TSVD_OK;
 }
 
-int split_transpose_ld(const float2* X, int rows, int cols, long ldx, long sx, int batch, float* hi, float* lo,
-                       long ldt, long st, cudaStream_t s) {
-  if (rows <= 0 || cols <= 0 || batch <= 0) return TSVD_OK;
-  if (batch > 65535) return TSVD_ERR_UNSUPPORTED;
-  dim3 grid(cdiv(cols, 32), cdiv(rows, 32), batch), block(32, 8);
-  k_split_transpose<<<grid, block, 0, s>>>(X, rows, cols, ldx, sx, hi, lo, ldt, st);
-  TSVD_LAUNCHED();
-  return TSVD_OK;
-}
-
 // per slice: the columns of a complex X (rows x cols, leading dim ldx) as real rows of
 // length `rows`: row 2c the real parts of column c, row 2c+1 the imaginary parts, split
 // into hi / lo (leading dim ldt, batch stride st); 32 x 32 complex tiles through shared memory

@@ -329,7 +329,7 @@ static int deflated_passes(const RbkDims& d, RbkWs<double>& w, cudaStream_t s) {
       TSVD_TRY(cgemm<double2>(gemm('N', 'H', n2, mp, R, -1.0, w.T1, R, sT, w.Um, R, sU, 1.0, w.CpH, mp, sP, h),
                               w.splitk, w.splitk_elems, s, w.st));
     }
-    TSVD_TRY(cgemm_herm<double2>(gemm('H', 'N', mp, mp, n2, 1.0, w.CpH, mp, sP, w.CpH, mp, sP, 0.0, w.G, mp,
+    TSVD_TRY(cgemm_herm(gemm('H', 'N', mp, mp, n2, 1.0, w.CpH, mp, sP, w.CpH, mp, sP, 0.0, w.G, mp,
                                       (long)mp * mp, h),
                                  w.splitk, w.splitk_elems, s, w.st));
     TSVD_TRY(herm_eig_topR<double2>(w.G, mp, (long)mp * mp, mp, R, h, w.lam, w.Uct, R, sU, w.eig, w.counters, s));
@@ -437,7 +437,7 @@ static int rbk_run(const T* A, const RbkDims& d, const tsvd_params& p, const T* 
   {
   TSVD_STAGE("gram_c", s);
   if constexpr (std::is_same<T, double>::value) {
-    TSVD_TRY(cgemm_herm<double2>(gemm('H', 'N', mp, mp, n2, 1.0, w.CH64, m, sCH, w.CH64, m, sCH, 0.0, w.G, mp,
+    TSVD_TRY(cgemm_herm(gemm('H', 'N', mp, mp, n2, 1.0, w.CH64, m, sCH, w.CH64, m, sCH, 0.0, w.G, mp,
                                       (long)mp * mp, h),
                                  w.splitk, w.splitk_elems, s, w.st));
   } else {
