@@ -28,23 +28,23 @@ template <typename C, bool SMALL>
 struct GemmCfg;
 template <bool SMALL>
 struct GemmCfg<double2, SMALL> {
-  static constexpr int BT = 16, TD = 8, BK = 16, KMIN = 16, TARGET = 2 * 152;
+  static constexpr int BT = 16, TD = 8, BK = 16, KMIN = 16, TARGET = 2 * SMS;
   using R = double;
 };
 template <>
 struct GemmCfg<float2, false> {
-  static constexpr int BT = 64, TD = 16, BK = 16, KMIN = 64, TARGET = 2 * 152;
+  static constexpr int BT = 64, TD = 16, BK = 16, KMIN = 64, TARGET = 2 * SMS;
   using R = float;
 };
 template <>
 struct GemmCfg<float2, true> {
-  static constexpr int BT = 32, TD = 8, BK = 16, KMIN = 32, TARGET = 4 * 152;
+  static constexpr int BT = 32, TD = 8, BK = 16, KMIN = 32, TARGET = 4 * SMS;
   using R = float;
 };
 
 template <typename C, bool AH, bool BH, bool SMALL>
-__global__ void __launch_bounds__(GemmCfg<C, SMALL>::TD* GemmCfg<C, SMALL>::TD) k_cgemm(GemmArgs g, C* __restrict__ ws, int ksplit, int kchunk, int tiles_m,
-                                               int herm_upper) {
+__global__ void __launch_bounds__(GemmCfg<C, SMALL>::TD* GemmCfg<C, SMALL>::TD)
+    k_cgemm(GemmArgs g, C* __restrict__ ws, int ksplit, int kchunk, int tiles_m, int herm_upper) {
   using Cfg = GemmCfg<C, SMALL>;
   constexpr int BK = Cfg::BK, GBM = Cfg::BT, GBN = GBM, TD = Cfg::TD, NT = TD * TD;
   constexpr int RT = GBM / TD;                           // rows and columns of a thread
@@ -333,7 +333,7 @@ static int mirror_lower(const GemmArgs& g, cudaStream_t s) {
 // k_cgemm_w over the FP32 product g: split-K until about two waves of two CTAs per SM
 static int cgemm_wide(const GemmArgs& g, float2* ws, size_t splitk_elems, cudaStream_t s) {
   const long tiles = (long)cdiv(g.M, WBM) * cdiv(g.N, WBN) * g.batch;
-  int ks = (int)std::max(1L, std::min(16L, (4L * 152 + tiles - 1) / tiles));
+  int ks = (int)std::max(1L, std::min(16L, (4L * SMS + tiles - 1) / tiles));
   ks = std::min(ks, std::max(1, g.K / 64));
   if (!ws) ks = 1;
   while (ks > 1 && (size_t)ks * g.batch * g.M * g.N > splitk_elems) --ks;
@@ -384,8 +384,9 @@ static int cgemm_tiles(const GemmArgs& g, C* ws, size_t splitk_elems, cudaStream
   return herm ? mirror_lower<C>(g, s) : TSVD_OK;
 }
 
+// herm: a Hermitian product (FP64 only)
 template <typename C>
-static int cgemm_impl(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t s, int herm, TcOpts st) {  // herm: FP64
+static int cgemm_impl(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, cudaStream_t s, int herm, TcOpts st) {
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return TSVD_OK;
   if (g.batch > 65535) return TSVD_ERR_UNSUPPORTED;
   if (g.beta != 0.0 && g.beta != 1.0) return TSVD_ERR_INVALID_ARG;
@@ -395,7 +396,7 @@ static int cgemm_impl(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, c
     // the wide tiles where they fill the GPU (two CTAs per SM), directly or by splitting a long K;
     // smaller products keep the 64 x 64 tiles (measured faster there)
     const long wtiles = (long)cdiv(g.M, WBM) * cdiv(g.N, WBN) * g.batch;
-    if (g.K > 0 && (wtiles >= 2L * 152 || (g.K >= 1024 && splitk_ws)))
+    if (g.K > 0 && (wtiles >= 2L * SMS || (g.K >= 1024 && splitk_ws)))
       return cgemm_wide(g, (float2*)splitk_ws, splitk_ws ? splitk_elems : 0, s);
   }
   if constexpr (std::is_same<C, double2>::value) {
@@ -409,7 +410,7 @@ static int cgemm_impl(const GemmArgs& g, void* splitk_ws, size_t splitk_elems, c
   // small tiles where the 64 x 64 ones would be mostly padding or, even with K split, leave SMs idle
   const long tiles64 = (long)cdiv(g.M, 64) * cdiv(g.N, 64) * g.batch;
   if (std::is_same<C, float2>::value &&
-      (g.N <= 32 || g.M <= 32 || tiles64 * std::max(1, std::min(16, g.K / 64)) < 152))
+      (g.N <= 32 || g.M <= 32 || tiles64 * std::max(1, std::min(16, g.K / 64)) < SMS))
     return cgemm_tiles<C, true>(g, (C*)splitk_ws, sk, s, herm);
   return cgemm_tiles<C, false>(g, (C*)splitk_ws, sk, s, herm);
 }

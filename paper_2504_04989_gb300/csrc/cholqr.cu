@@ -468,7 +468,8 @@ template int rmul_block<float2>(const float2*, long, long, const float2*, long, 
 // Dependent Krylov columns (exact low rank, zero data): replace column c+j by
 // a Philox Gaussian direction (stream 3) projected twice against every other
 // live column of the basis, then normalised.  Any orthonormal completion of
-// span(K) leaves the Rayleigh-Ritz result of Alg. 2 optimal (Sec. 4: Q (Q^T A)_k is the best rank-k approximation within range(Q)).
+// span(K) leaves the Rayleigh-Ritz result of Alg. 2 optimal (Sec. 4: Q (Q^T A)_k is the best rank-k approximation
+// within range(Q)).
 // ---------------------------------------------------------------------------
 template <typename C>
 __global__ void __launch_bounds__(256) k_repair_dead(C* __restrict__ Q, long ldq, long sQ, int n1, int c, int nb,

@@ -12,6 +12,8 @@
 
 namespace tsvd {
 
+constexpr int SMS = 152;  // SMs of a GB300, which grids and tiles are chosen for
+
 // complex element type for a real type
 template <typename T>
 struct Cx;
@@ -91,11 +93,12 @@ __device__ __forceinline__ float2 from_c64<float2>(double2 a) {
   return make_float2((float)a.x, (float)a.y);
 }
 
-// 1 / sqrt(d) for d > 0.  FP64, to a rounding or two of the last place: the hardware's FP32 estimate y and one step of its
-// series in e = 1 - d y^2 to e^2 (the correctly rounded root and division, and even a second Newton step, weigh
-// on a serial chain).  FP32 keeps the root and the division: the pivots of a last pass lie within a few units of 1, where
-// the estimate with a Newton step, and a correctly rounded 1 / sqrt too, come out below them on average: columns of Q 3
-// to 4e-8 shorter, which the singular values show (24 uneven T-SVDs: error 3.44e-6 so, 3.47e-6 and 3.48e-6 with those).
+// 1 / sqrt(d) for d > 0.  FP64, to a rounding or two of the last place: the hardware's FP32 estimate y and one step
+// of its series in e = 1 - d y^2 to e^2 (the correctly rounded root and division, and even a second Newton step, weigh
+// on a serial chain).  FP32 keeps the root and the division: the pivots of a last pass lie within a few units of 1,
+// where the estimate with a Newton step, and a correctly rounded 1 / sqrt too, come out below them on average:
+// columns of Q 3 to 4e-8 shorter, which the singular values show (24 uneven T-SVDs: error 3.44e-6 so, 3.47e-6 and
+// 3.48e-6 with those).
 __device__ __forceinline__ float inv_sqrt(float d) { return 1.0f / sqrtf(d); }
 __device__ __forceinline__ double inv_sqrt(double d) {
   const int h = (__double2hiint(d) >> 20) - 1023;  // d = m 4^e with m in [1, 4)
@@ -187,8 +190,8 @@ struct Carver {
   size_t bytes() const { return (off + 255) & ~(size_t)255; }
 };
 
-// The product scratch at the end of a workspace, in elements of C: `least` with which the call runs, `best` beyond which no
-// product gains; between them what `have` bytes leave.
+// The product scratch at the end of a workspace, in elements of C: `least` with which the call runs, `best` beyond
+// which no product gains; between them what `have` bytes leave.
 constexpr size_t WS_ALL = (size_t)-1;
 template <typename C>
 size_t fit_scratch(const Carver& cv, size_t have, size_t least, size_t best) {

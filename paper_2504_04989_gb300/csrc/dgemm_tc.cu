@@ -24,9 +24,9 @@
 // small next to its scales, or is left to k_redo, which adds them up in FP64:
 //   |C_ij| is at least 2^-7 of (scale of row i) (scale of column j), or
 //   the entry of row i that meets the largest one of column j is within 2^-5 of its scale, or the other way round.
-// Either says that sum |a||b| is at least 2^-7 of the scales, against an error of at most about 2^-59 of them per term: 2.4 times
-// the worst case of FP64 multiply-adds, 2 K u sum |a||b|, where those are only just met.  Errors as measured stand at
-// dgemm_tc_better.
+// Either says that sum |a||b| is at least 2^-7 of the scales, against an error of at most about 2^-59 of them per
+// term: 2.4 times the worst case of FP64 multiply-adds, 2 K u sum |a||b|, where those are only just met.  Errors as
+// measured stand at dgemm_tc_better.
 //
 // A complex product is the real product of the interleaved rows of op(A) with the
 // expanded real form of op(B) (rows 2n and 2n + 1 per column n, as in tc_gemm.cu).
@@ -84,7 +84,8 @@ struct DigOp {
   bool trans;  // stored K x rows, else rows x K
   bool conj;   // enters conjugated
   int sign;    // its entries of k take sign * shift[k] to their exponents
-  unsigned long long* top;  // [batch][rows] 2^32 (bound of the row's exponents + DG_OFF, 0, DG_INF) + the k of the largest entry
+  // [batch][rows] 2^32 (bound of the row's exponents + DG_OFF, 0, DG_INF) + the k of the largest entry
+  unsigned long long* top;
   uint32_t* near;           // [batch][rows][K / 32] which entries are within 2^-5 of that bound
   uint32_t* D;              // digit planes, [batch][8][rows, or 2 rows for op(B)][ldk]
   __host__ __device__ unsigned expo_blocks(int K) const {
@@ -93,8 +94,8 @@ struct DigOp {
   __host__ __device__ unsigned pack_blocks(int K) const { return (unsigned)((rows + 31) / 32) * ((K + 31) / 32); }
 };
 
-// Of 32 entries of op(A)(:, k) and of op(B)(k, :), spread over it, the mean exponent (0 where all are zero) and how far the
-// largest lies above it, zeros counted as 64 below: 32 k per block, 8 of its threads on each.  Also zeroes what
+// Of 32 entries of op(A)(:, k) and of op(B)(k, :), spread over it, the mean exponent (0 where all are zero) and how
+// far the largest lies above it, zeros counted as 64 below: 32 k per block, 8 of its threads on each.  Also zeroes what
 // the next pass takes maxima into.
 __global__ void __launch_bounds__(256) k_dig_sample(const DigOp A, const DigOp B, int K, float4* __restrict__ stat) {
   __shared__ int red[2][3][8][32];
@@ -144,10 +145,10 @@ __global__ void __launch_bounds__(256) k_dig_sample(const DigOp A, const DigOp B
   out[2] = cnt ? ((float)big - mean) + 64.f * (float)(n - cnt) / (float)n : 64.f;
 }
 
-// The power of two that op(A)(:, k) takes over from op(B)(k, :): what brings the mean exponent of the more even operand's
-// column or row to that of 32 k spread over K, if it is off by more than 1.25 (a sample of evenly scaled data stays below,
-// and an entry more or less does not change it); where that is all zero, what brings the other's there.  A sample that misleads
-// costs time, not accuracy.
+// The power of two that op(A)(:, k) takes over from op(B)(k, :): what brings the mean exponent of the more even
+// operand's column or row to that of 32 k spread over K, if it is off by more than 1.25 (a sample of evenly scaled
+// data stays below, and an entry more or less does not change it); where that is all zero, what brings the other's
+// there.  A sample that misleads costs time, not accuracy.
 struct DigShift {
   const float4* stat;
   float ra, rb;
@@ -172,8 +173,8 @@ struct DigShift {
   }
 };
 
-// The largest shifted exponents of both operands' rows: of rows as stored by a warp each, of stored columns by 32 columns
-// x 64 of K per block.  Also clears the marks.
+// The largest shifted exponents of both operands' rows: of rows as stored by a warp each, of stored columns by 32
+// columns x 64 of K per block.  Also clears the marks.
 __global__ void __launch_bounds__(256) k_dig_expo(const DigOp A, const DigOp B, int K, const float4* __restrict__ stat,
                                                   const Marks<double2> marks) {
   __shared__ unsigned long long red[8][32];
@@ -541,7 +542,8 @@ static int digit_map(CUtensorMap* tm, const void* ptr, int rows, int K2, long ld
 
 static long dg_ldk(int K) { return (2L * K + 7) / 8 * 8; }
 static size_t dg_slice_bytes(int M, int N, int K) {
-  return (size_t)DG_D * dg_ldk(K) * 2 * (M + 2 * (size_t)N) + (8 + 4 * (size_t)((K + 31) / 32)) * ((size_t)M + N) + 16 * (size_t)K + Marks<double2>::bytes(M, N, 1);
+  return (size_t)DG_D * dg_ldk(K) * 2 * (M + 2 * (size_t)N) + (8 + 4 * (size_t)((K + 31) / 32)) * ((size_t)M + N) +
+         16 * (size_t)K + Marks<double2>::bytes(M, N, 1);
 }
 size_t dgemm_tc_bytes(int M, int N, int K, int batch) {
   return std::min<size_t>(dg_slice_bytes(M, N, K) * batch, (size_t)3 << 30) + dg_slice_bytes(M, N, K) + 2048;
@@ -550,10 +552,11 @@ size_t dgemm_tc_bytes(int M, int N, int K, int batch) {
 // Estimated times in microseconds of the two forms; the digit form from about 2e7 multiply-adds on
 // (128 x 64 x 128 on 5 slices: 265 us on the FP64 units, 78 us here; 64 x 15 x 64 on 9 slices: 19 us
 // there, about 25 us of launches here).
-// Error, 2-norm, and the largest of an element in u sum |a||b|, FP64 multiply-adds (GemmCfg<double2>) in brackets: normal data,
-// K = 16: 4.7e-17, 1.5 (1.4e-16, 4.4), 97: 4.7e-17, 0.5 (3.3e-16, 4.5), 2048: 4.7e-17, 0.1 (4.0e-16, 0.6); every entry over
-// twelve decades of its own 1.5e-16, 7.8 (2.6e-16, 12); columns of A over eight decades 5.0e-17, 1.0 (3.6e-16, 8.3); columns of A
-// and rows of B against each other over 3, 6, 12, 17 decades 4.8e-17, 0.4 (2.8e-16, 1.8) each.
+// Error, 2-norm, and the largest of an element in u sum |a||b|, FP64 multiply-adds (GemmCfg<double2>) in brackets:
+// normal data, K = 16: 4.7e-17, 1.5 (1.4e-16, 4.4), 97: 4.7e-17, 0.5 (3.3e-16, 4.5), 2048: 4.7e-17, 0.1 (4.0e-16,
+// 0.6); every entry over twelve decades of its own 1.5e-16, 7.8 (2.6e-16, 12); columns of A over eight decades
+// 5.0e-17, 1.0 (3.6e-16, 8.3); columns of A and rows of B against each other over 3, 6, 12, 17 decades 4.8e-17, 0.4
+// (2.8e-16, 1.8) each.
 bool dgemm_tc_better(const GemmArgs& g, size_t bytes) {
   if (g.K < 1 || g.M < 1 || g.N < 1 || g.K > (1 << 20)) return false;
   const size_t slice = dg_slice_bytes(g.M, g.N, g.K) + 2048;
@@ -563,7 +566,7 @@ bool dgemm_tc_better(const GemmArgs& g, size_t bytes) {
   const double tile_us = 2.0 + (cdiv(2L * g.K, DG_KB) * 1.5 + cdiv(2L * g.K, DG_KB * DG_CHUNK) * 1.5);
   const double pack_us = ((double)slice * 1.3 * g.batch) / 3.0e6;
   const double calls = std::ceil((double)g.batch * slice / (double)bytes);
-  return simt > 25.0 * calls + pack_us + std::ceil(tiles / 152.0) * tile_us;
+  return simt > 25.0 * calls + pack_us + std::ceil(tiles / SMS) * tile_us;
 }
 
 int dgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s, bool upper, TcOpts st) {
@@ -594,7 +597,8 @@ int dgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s, bool upp
     const bool ta = g.opA == 'H', tb = g.opB == 'N';
     const double2* A = (const double2*)g.A + (long)b0 * g.sA;
     const double2* B = (const double2*)g.B + (long)b0 * g.sB;
-    const DigOp oa{A, g.lda, g.sA, g.M, ta, ta, 1, topA, nearA, DA}, ob{B, g.ldb, g.sB, g.N, tb, !tb, -1, topB, nearB, DB};
+    const DigOp oa{A, g.lda, g.sA, g.M, ta, ta, 1, topA, nearA, DA};
+    const DigOp ob{B, g.ldb, g.sB, g.N, tb, !tb, -1, topB, nearB, DB};
     k_dig_sample<<<dim3(cdiv(g.K, 32), 1, n), 256, 0, s>>>(oa, ob, g.K, stat);
     TSVD_LAUNCHED();
     k_dig_expo<<<dim3(oa.expo_blocks(g.K) + ob.expo_blocks(g.K), 1, n), 256, 0, s>>>(oa, ob, g.K, stat, marks);
@@ -605,7 +609,7 @@ int dgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s, bool upp
     TSVD_TRY(digit_map(&ma, DA, g.M, 2 * g.K, ldk, n * DG_D, DG_BM));
     TSVD_TRY(digit_map(&mb, DB, N2, 2 * g.K, ldk, n * DG_D, DG_BN));
     const long tiles = (long)cdiv(N2, DG_BN) * cdiv(g.M, DG_BM) * n;  // one per CTA where some are skipped
-    const unsigned grid = (unsigned)(upper ? tiles : std::min<long>(tiles, 152));
+    const unsigned grid = (unsigned)(upper ? tiles : std::min<long>(tiles, SMS));
     double2* Cb = (double2*)g.C + (long)b0 * g.sC;
     k_dgemm_tc<<<grid, DG_THREADS, DG_SMEM, s>>>(ma, mb, topA, topB, nearA, nearB, marks, Cb, g.ldc, g.sC, g.M, g.N,
                                                  g.K, n, g.alpha, g.beta != 0.0, upper ? 1 : 0, st);

@@ -1526,7 +1526,7 @@ static int launch_backtransform(int m, int R, int batch, const EigScratch& e, C*
   int parts = cdiv(R, BT_VPC);
   long best = -1;
   for (int p = parts; p <= std::max<int>(parts, cdiv(R, 4)); ++p) {
-    const long load = (long)cdiv((long)p * batch, 152) * cdiv(R, p);
+    const long load = (long)cdiv((long)p * batch, SMS) * cdiv(R, p);
     if (best < 0 || load < best) {
       best = load;
       parts = p;
@@ -1603,8 +1603,8 @@ static int hetrd_clusters(int CL) {
 // How a batch of m x m reductions is laid out (k_hetrd): the largest cluster in {8, 4, 2, 1} whose CTAs are
 // all resident at once, with at least 20 rows each while they take a quarter of the SMs (m = 90 on 9
 // slices: 604 us on clusters of 1, 508 on 2, 455 on 4), else 32 (a CTA keeps its SM: in a batch of 24
-// tensors, 32 rows throughout gave 9.4 ms, 20 rows 10.3), and whose packed rows fit in shared memory beside the vectors, with the warps' partials there
-// too or, where only those do not fit, in L2; else rows in L2.
+// tensors, 32 rows throughout gave 9.4 ms, 20 rows 10.3), and whose packed rows fit in shared memory beside the
+// vectors, with the warps' partials there too or, where only those do not fit, in L2; else rows in L2.
 struct HetrdPlan {
   int CL;
   bool global_rows, cp_global;
@@ -1616,7 +1616,7 @@ static HetrdPlan hetrd_plan(int m, int batch) {
   const size_t el = sizeof(double2), vec = 7 * (size_t)m * el, part = (size_t)(HETRD_NT / 32) * m * el;
   int most = 1;
   for (int CL = 8; CL >= 1; CL >>= 1) {
-    if (CL > 1 && (m / CL < (4 * batch * CL <= 152 ? 20 : 32) || batch > hetrd_clusters(CL))) continue;
+    if (CL > 1 && (m / CL < (4 * batch * CL <= SMS ? 20 : 32) || batch > hetrd_clusters(CL))) continue;
     most = std::max(most, CL);
     const size_t rows = hetrd_row_elems(m, CL) * el;
     if (rows + vec + part <= smax) return HetrdPlan{CL, false, false, rows + vec + part};

@@ -123,8 +123,8 @@ static int tile_e(int n3, size_t elem, size_t celem, bool inverse) {
 
 // ---------------------------------------------------------------------------
 // Mixed-radix FFT of the tubes for the lengths above 160 and the smooth FP64 ones
-// (Stockham autosort, radices 4, 2, 3, 5 and any remaining prime).  A CTA owns a tile of FFT_TUBES consecutive tubes; two real
-// tubes are packed into one complex sequence z = x + i y and each warp
+// (Stockham autosort, radices 4, 2, 3, 5 and any remaining prime).  A CTA owns a tile of FFT_TUBES consecutive tubes;
+// two real tubes are packed into one complex sequence z = x + i y and each warp
 // transforms whole sequences in shared memory (lane-parallel butterflies,
 // warp barriers between passes).  The half spectra are separated as
 // X_k = (Z_k + conj Z_{n-k}) / 2, Y_k = (Z_k - conj Z_{n-k}) / (2i); the inverse
@@ -670,8 +670,9 @@ __global__ void __launch_bounds__(128) k_irfft3_reg2(const cx_t<T>* __restrict__
 constexpr int RDFT_MAX = 160;
 template <typename T>
 struct RVec;
+// (64 tubes x 8 frequencies per warp and 256 threads measured slower: 121 -> 140 us at n = 100 with the former loads)
 template <>
-struct RVec<float> {  // (64 tubes x 8 frequencies per warp and 256 threads measured slower: 121 -> 140 us at n = 100 with the former loads)
+struct RVec<float> {
   using type = float4;
   static constexpr int V = 4, KB = 4, THREADS = 128;
 };
@@ -740,183 +741,183 @@ __global__ void __launch_bounds__(RVec<T>::THREADS, 4) k_rdft3(const T* __restri
   }
   // persistent CTAs: the table is made once for all the tiles a CTA takes
   for (long tile = blockIdx.x; (tile << lgE) < plane; tile += gridDim.x) {
-  const long e0 = tile << lgE;
-  __syncthreads();  // the previous tile's samples have been read
-  auto ld = [&](int j, long ge) { return ge < plane ? __ldg(X + (long)j * plane + ge) : T(0); };
-  // 16 bytes per load where the planes are aligned (W tubes), else one sample; 8 or 16 loads in flight
-  auto fold = [&](auto w_) {
-    constexpr int W = decltype(w_)::value;
-    using VW = typename std::conditional<W == 1, T, VT>::type;
-    constexpr int UB = W == 1 ? 8 : 4;  // items of two loads at a time
-    const int lgW = lgE - (W == 4 ? 2 : W == 2 ? 1 : 0), items = J << lgW;
-    auto get = [&](int j, long ge, T* o) {
-      if (ge < plane) {
-        const VW x = __ldg((const VW*)(X + (long)j * plane + ge));
-        if constexpr (W == 1) o[0] = x;
-        else unpack(x, o);
+    const long e0 = tile << lgE;
+    __syncthreads();  // the previous tile's samples have been read
+    auto ld = [&](int j, long ge) { return ge < plane ? __ldg(X + (long)j * plane + ge) : T(0); };
+    // 16 bytes per load where the planes are aligned (W tubes), else one sample; 8 or 16 loads in flight
+    auto fold = [&](auto w_) {
+      constexpr int W = decltype(w_)::value;
+      using VW = typename std::conditional<W == 1, T, VT>::type;
+      constexpr int UB = W == 1 ? 8 : 4;  // items of two loads at a time
+      const int lgW = lgE - (W == 4 ? 2 : W == 2 ? 1 : 0), items = J << lgW;
+      auto get = [&](int j, long ge, T* o) {
+        if (ge < plane) {
+          const VW x = __ldg((const VW*)(X + (long)j * plane + ge));
+          if constexpr (W == 1) o[0] = x;
+          else unpack(x, o);
+        } else {
+#pragma unroll
+          for (int q = 0; q < W; ++q) o[q] = T(0);
+        }
+      };
+      auto put = [&](T* dst, const T* v) {
+        if constexpr (W == 4) *(float4*)dst = make_float4(v[0], v[1], v[2], v[3]);
+        else if constexpr (W == 2) *(double2*)dst = make_double2(v[0], v[1]);
+        else dst[0] = v[0];
+      };
+      if (d.types == 1) {
+        for (int i0 = tid; i0 < items; i0 += UB * THR) {
+          T x[UB][2][W];
+#pragma unroll
+          for (int u = 0; u < UB; ++u) {
+            const int i = min(i0 + u * THR, items - 1), j = (i >> lgW) + 1;
+            const long ge = e0 + (i & ((1 << lgW) - 1)) * W;
+            get(j, ge, x[u][0]);
+            get(n - j, ge, x[u][1]);
+          }
+#pragma unroll
+          for (int u = 0; u < UB; ++u) {
+            const int i = i0 + u * THR;
+            if (i >= items) break;
+            T p[W], q[W];
+#pragma unroll
+            for (int k = 0; k < W; ++k) {
+              p[k] = x[u][0][k] + x[u][1][k];
+              q[k] = x[u][0][k] - x[u][1][k];
+            }
+            put(dat + (long)i * W, p);
+            put(dat + J * E + (long)i * W, q);
+          }
+        }
       } else {
+        T* o = dat + (size_t)rows * E;
+        for (int i0 = tid; i0 < items; i0 += UB / 2 * THR) {
+          T x[UB / 2][4][W];
 #pragma unroll
-        for (int q = 0; q < W; ++q) o[q] = T(0);
+          for (int u = 0; u < UB / 2; ++u) {
+            const int i = min(i0 + u * THR, items - 1), j = (i >> lgW) + 1;
+            const long ge = e0 + (i & ((1 << lgW) - 1)) * W;
+            get(j, ge, x[u][0]);
+            get(m - j, ge, x[u][1]);
+            get(m + j, ge, x[u][2]);
+            get(n - j, ge, x[u][3]);
+          }
+#pragma unroll
+          for (int u = 0; u < UB / 2; ++u) {
+            const int i = i0 + u * THR;
+            if (i >= items) break;
+            T p0[W], q0[W], p1[W], q1[W];
+#pragma unroll
+            for (int k = 0; k < W; ++k) {
+              const T s0 = x[u][0][k] + x[u][2][k], s1 = x[u][1][k] + x[u][3][k];
+              const T d0 = x[u][0][k] - x[u][2][k], d1 = x[u][1][k] - x[u][3][k];
+              p0[k] = s0 + s1;
+              q0[k] = s0 - s1;
+              p1[k] = d0 - d1;
+              q1[k] = d0 + d1;
+            }
+            put(dat + (long)i * W, p0);
+            put(dat + J * E + (long)i * W, q0);
+            put(o + (long)i * W, p1);
+            put(o + J * E + (long)i * W, q1);
+          }
+        }
       }
     };
-    auto put = [&](T* dst, const T* v) {
-      if constexpr (W == 4) *(float4*)dst = make_float4(v[0], v[1], v[2], v[3]);
-      else if constexpr (W == 2) *(double2*)dst = make_double2(v[0], v[1]);
-      else dst[0] = v[0];
-    };
-    if (d.types == 1) {
-      for (int i0 = tid; i0 < items; i0 += UB * THR) {
-        T x[UB][2][W];
-#pragma unroll
-        for (int u = 0; u < UB; ++u) {
-          const int i = min(i0 + u * THR, items - 1), j = (i >> lgW) + 1;
-          const long ge = e0 + (i & ((1 << lgW) - 1)) * W;
-          get(j, ge, x[u][0]);
-          get(n - j, ge, x[u][1]);
+    if (plane % V == 0 && ((uintptr_t)X & 15) == 0) fold(IntC<V>());
+    else fold(IntC<1>());
+    for (int e = tid; e < E; e += THR) {
+      const long ge = e0 + e;
+      T* f0 = dat + 2 * J * E + e;
+      if (d.types == 1) {
+        f0[0] = ld(0, ge);
+      } else {
+        const T a = ld(0, ge), b = ld(m, ge);
+        T* f1 = f0 + (size_t)rows * E;
+        f0[0] = a + b;
+        f1[0] = a - b;
+        if (d.half) {
+          const T c = ld(m / 2, ge), f = ld(m / 2 + m, ge);
+          f0[E] = c + f;
+          f1[E] = c - f;
         }
+      }
+    }
+    __syncthreads();
+    const int L = E / V, items = d.HP / KB * L;
+    for (int it = tid; it < items; it += THR) {
+      const int lane = it % L, c0 = it / L * KB;
+      const int t = c0 >= d.hp[0];
+      const T* P = dat + (size_t)t * rows * E + lane * V;
+      const T* Q = P + J * E;
+      T re[KB][V], im[KB][V];
+      {
+        T f[V], g[V];
+        unpack(*(const VT*)(P + 2 * J * E), f);
 #pragma unroll
-        for (int u = 0; u < UB; ++u) {
-          const int i = i0 + u * THR;
-          if (i >= items) break;
-          T p[W], q[W];
+        for (int u = 0; u < V; ++u) g[u] = T(0);
+        if (d.half) unpack(*(const VT*)(P + (2 * J + 1) * E), g);
 #pragma unroll
-          for (int k = 0; k < W; ++k) {
-            p[k] = x[u][0][k] + x[u][1][k];
-            q[k] = x[u][0][k] - x[u][1][k];
+        for (int q = 0; q < KB; ++q) {
+          // the middle sample: (-1)^k' on the real part (even frequencies) or on -Im (odd ones)
+          const T sg = ((c0 - (t ? d.hp[0] : 0) + q) & 1) ? T(-1) : T(1);
+#pragma unroll
+          for (int u = 0; u < V; ++u) {
+            re[q][u] = t ? f[u] : f[u] + sg * g[u];
+            im[q][u] = t ? sg * g[u] : T(0);
           }
-          put(dat + (long)i * W, p);
-          put(dat + J * E + (long)i * W, q);
         }
       }
-    } else {
-      T* o = dat + (size_t)rows * E;
-      for (int i0 = tid; i0 < items; i0 += UB / 2 * THR) {
-        T x[UB / 2][4][W];
+      const C* w = tab + c0;
+      for (int j0 = 0; j0 < J; j0 += 8) {
+        T sr[KB][V], si[KB][V];
 #pragma unroll
-        for (int u = 0; u < UB / 2; ++u) {
-          const int i = min(i0 + u * THR, items - 1), j = (i >> lgW) + 1;
-          const long ge = e0 + (i & ((1 << lgW) - 1)) * W;
-          get(j, ge, x[u][0]);
-          get(m - j, ge, x[u][1]);
-          get(m + j, ge, x[u][2]);
-          get(n - j, ge, x[u][3]);
-        }
+        for (int q = 0; q < KB; ++q)
 #pragma unroll
-        for (int u = 0; u < UB / 2; ++u) {
-          const int i = i0 + u * THR;
-          if (i >= items) break;
-          T p0[W], q0[W], p1[W], q1[W];
-#pragma unroll
-          for (int k = 0; k < W; ++k) {
-            const T s0 = x[u][0][k] + x[u][2][k], s1 = x[u][1][k] + x[u][3][k];
-            const T d0 = x[u][0][k] - x[u][2][k], d1 = x[u][1][k] - x[u][3][k];
-            p0[k] = s0 + s1;
-            q0[k] = s0 - s1;
-            p1[k] = d0 - d1;
-            q1[k] = d0 + d1;
-          }
-          put(dat + (long)i * W, p0);
-          put(dat + J * E + (long)i * W, q0);
-          put(o + (long)i * W, p1);
-          put(o + J * E + (long)i * W, q1);
-        }
-      }
-    }
-  };
-  if (plane % V == 0 && ((uintptr_t)X & 15) == 0) fold(IntC<V>());
-  else fold(IntC<1>());
-  for (int e = tid; e < E; e += THR) {
-    const long ge = e0 + e;
-    T* f0 = dat + 2 * J * E + e;
-    if (d.types == 1) {
-      f0[0] = ld(0, ge);
-    } else {
-      const T a = ld(0, ge), b = ld(m, ge);
-      T* f1 = f0 + (size_t)rows * E;
-      f0[0] = a + b;
-      f1[0] = a - b;
-      if (d.half) {
-        const T c = ld(m / 2, ge), f = ld(m / 2 + m, ge);
-        f0[E] = c + f;
-        f1[E] = c - f;
-      }
-    }
-  }
-  __syncthreads();
-  const int L = E / V, items = d.HP / KB * L;
-  for (int it = tid; it < items; it += THR) {
-    const int lane = it % L, c0 = it / L * KB;
-    const int t = c0 >= d.hp[0];
-    const T* P = dat + (size_t)t * rows * E + lane * V;
-    const T* Q = P + J * E;
-    T re[KB][V], im[KB][V];
-    {
-      T f[V], g[V];
-      unpack(*(const VT*)(P + 2 * J * E), f);
-#pragma unroll
-      for (int u = 0; u < V; ++u) g[u] = T(0);
-      if (d.half) unpack(*(const VT*)(P + (2 * J + 1) * E), g);
-#pragma unroll
-      for (int q = 0; q < KB; ++q) {
-        // the middle sample: (-1)^k' on the real part (even frequencies) or on -Im (odd ones)
-        const T sg = ((c0 - (t ? d.hp[0] : 0) + q) & 1) ? T(-1) : T(1);
-#pragma unroll
-        for (int u = 0; u < V; ++u) {
-          re[q][u] = t ? f[u] : f[u] + sg * g[u];
-          im[q][u] = t ? sg * g[u] : T(0);
-        }
-      }
-    }
-    const C* w = tab + c0;
-    for (int j0 = 0; j0 < J; j0 += 8) {
-      T sr[KB][V], si[KB][V];
-#pragma unroll
-      for (int q = 0; q < KB; ++q)
-#pragma unroll
-        for (int u = 0; u < V; ++u) sr[q][u] = si[q][u] = T(0);
-      const int j1 = min(J, j0 + 8);
+          for (int u = 0; u < V; ++u) sr[q][u] = si[q][u] = T(0);
+        const int j1 = min(J, j0 + 8);
 #pragma unroll 4
-      for (int j = j0; j < j1; ++j) {
-        T pv[V], qv[V];
-        unpack(*(const VT*)(P + j * E), pv);
-        unpack(*(const VT*)(Q + j * E), qv);
-        C c[KB];
-        load_row<KB>(w + (size_t)j * d.HP, c);
+        for (int j = j0; j < j1; ++j) {
+          T pv[V], qv[V];
+          unpack(*(const VT*)(P + j * E), pv);
+          unpack(*(const VT*)(Q + j * E), qv);
+          C c[KB];
+          load_row<KB>(w + (size_t)j * d.HP, c);
+#pragma unroll
+          for (int q = 0; q < KB; ++q)
+#pragma unroll
+            for (int u = 0; u < V; ++u) {
+              sr[q][u] = fma(pv[u], c[q].x, sr[q][u]);
+              si[q][u] = fma(qv[u], c[q].y, si[q][u]);
+            }
+        }
 #pragma unroll
         for (int q = 0; q < KB; ++q)
 #pragma unroll
           for (int u = 0; u < V; ++u) {
-            sr[q][u] = fma(pv[u], c[q].x, sr[q][u]);
-            si[q][u] = fma(qv[u], c[q].y, si[q][u]);
+            re[q][u] += sr[q][u];
+            im[q][u] += si[q][u];
           }
       }
+      const int q0 = c0 - (t ? d.hp[0] : 0);
 #pragma unroll
-      for (int q = 0; q < KB; ++q)
+      for (int q = 0; q < KB; ++q) {
+        if (q0 + q >= d.hc[t]) continue;
+        const int k = d.types == 2 ? 2 * (q0 + q) + t : q0 + q;
+        const long ge = e0 + lane * V;
+        C* dst = Xh + (long)k * plane + ge;
+        if (sizeof(T) == 4 && ge + V <= plane && ((uintptr_t)dst & 15) == 0) {
 #pragma unroll
-        for (int u = 0; u < V; ++u) {
-          re[q][u] += sr[q][u];
-          im[q][u] += si[q][u];
+          for (int u = 0; u < V; u += 2)
+            *(float4*)(dst + u) = make_float4((float)re[q][u], (float)-im[q][u], (float)re[q][u + 1],
+                                              (float)-im[q][u + 1]);
+        } else {
+#pragma unroll
+          for (int u = 0; u < V; ++u)
+            if (ge + u < plane) dst[u] = mkc(re[q][u], -im[q][u]);
         }
-    }
-    const int q0 = c0 - (t ? d.hp[0] : 0);
-#pragma unroll
-    for (int q = 0; q < KB; ++q) {
-      if (q0 + q >= d.hc[t]) continue;
-      const int k = d.types == 2 ? 2 * (q0 + q) + t : q0 + q;
-      const long ge = e0 + lane * V;
-      C* dst = Xh + (long)k * plane + ge;
-      if (sizeof(T) == 4 && ge + V <= plane && ((uintptr_t)dst & 15) == 0) {
-#pragma unroll
-        for (int u = 0; u < V; u += 2)
-          *(float4*)(dst + u) = make_float4((float)re[q][u], (float)-im[q][u], (float)re[q][u + 1],
-                                            (float)-im[q][u + 1]);
-      } else {
-#pragma unroll
-        for (int u = 0; u < V; ++u)
-          if (ge + u < plane) dst[u] = mkc(re[q][u], -im[q][u]);
       }
     }
-  }
   }
 }
 
@@ -944,149 +945,149 @@ __global__ void __launch_bounds__(RVec<T>::THREADS, 3) k_irdft3(const cx_t<T>* _
     tab[i] = tw[(freq(r) * t) % n];
   }
   for (long tile = blockIdx.x; (tile << lgE) < plane; tile += gridDim.x) {
-  const long e0 = tile << lgE;
-  __syncthreads();  // the previous tile's samples have been read
-  // FP32: two tubes per load where the planes are aligned; 8 loads in flight
-  auto stage = [&](auto w_) {
-    constexpr int W = decltype(w_)::value, UB = 8;
-    const int lgW = lgE - (W == 2 ? 1 : 0), cnt = K << lgW;
-    for (int i0 = tid; i0 < cnt; i0 += UB * THR) {
-      C x[UB][W];
+    const long e0 = tile << lgE;
+    __syncthreads();  // the previous tile's samples have been read
+    // FP32: two tubes per load where the planes are aligned; 8 loads in flight
+    auto stage = [&](auto w_) {
+      constexpr int W = decltype(w_)::value, UB = 8;
+      const int lgW = lgE - (W == 2 ? 1 : 0), cnt = K << lgW;
+      for (int i0 = tid; i0 < cnt; i0 += UB * THR) {
+        C x[UB][W];
 #pragma unroll
-      for (int u = 0; u < UB; ++u) {
-        const int i = min(i0 + u * THR, cnt - 1);
-        const long ge = e0 + (i & ((1 << lgW) - 1)) * W;
-        const C* src = Xh + (long)freq(i >> lgW) * plane + ge;
-        if constexpr (W == 2) {
-          const float4 y = ge < plane ? *(const float4*)src : make_float4(0.f, 0.f, 0.f, 0.f);
-          x[u][0] = mkc(T(y.x), T(y.y));
-          x[u][1] = mkc(T(y.z), T(y.w));
-        } else {
-          x[u][0] = ge < plane ? *src : mkc(T(0), T(0));
+        for (int u = 0; u < UB; ++u) {
+          const int i = min(i0 + u * THR, cnt - 1);
+          const long ge = e0 + (i & ((1 << lgW) - 1)) * W;
+          const C* src = Xh + (long)freq(i >> lgW) * plane + ge;
+          if constexpr (W == 2) {
+            const float4 y = ge < plane ? *(const float4*)src : make_float4(0.f, 0.f, 0.f, 0.f);
+            x[u][0] = mkc(T(y.x), T(y.y));
+            x[u][1] = mkc(T(y.z), T(y.w));
+          } else {
+            x[u][0] = ge < plane ? *src : mkc(T(0), T(0));
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < UB; ++u) {
+          const int i = i0 + u * THR;
+          if (i >= cnt) break;
+#pragma unroll
+          for (int k = 0; k < W; ++k) {
+            dr[i * W + k] = T(2) * x[u][k].x;
+            di[i * W + k] = T(2) * x[u][k].y;
+          }
         }
       }
-#pragma unroll
-      for (int u = 0; u < UB; ++u) {
-        const int i = i0 + u * THR;
-        if (i >= cnt) break;
-#pragma unroll
-        for (int k = 0; k < W; ++k) {
-          dr[i * W + k] = T(2) * x[u][k].x;
-          di[i * W + k] = T(2) * x[u][k].y;
-        }
-      }
+    };
+    if (sizeof(T) == 4 && plane % 2 == 0 && ((uintptr_t)Xh & 15) == 0) stage(IntC<sizeof(T) == 4 ? 2 : 1>());
+    else stage(IntC<1>());
+    for (int e = tid; e < E; e += THR) {
+      const long ge = e0 + e;
+      dr[K * E + e] = ge < plane ? Xh[ge].x : T(0);
+      dr[(K + 1) * E + e] = (types == 2 && ge < plane) ? Xh[(long)m * plane + ge].x : T(0);
     }
-  };
-  if (sizeof(T) == 4 && plane % 2 == 0 && ((uintptr_t)Xh & 15) == 0) stage(IntC<sizeof(T) == 4 ? 2 : 1>());
-  else stage(IntC<1>());
-  for (int e = tid; e < E; e += THR) {
-    const long ge = e0 + e;
-    dr[K * E + e] = ge < plane ? Xh[ge].x : T(0);
-    dr[(K + 1) * E + e] = (types == 2 && ge < plane) ? Xh[(long)m * plane + ge].x : T(0);
-  }
-  __syncthreads();
-  const T inv = T(1) / T(n);
-  const int L = E / V, items = HP / KB * L;
-  for (int it = tid; it < items; it += THR) {
-    const int lane = it % L, t0 = it / L * KB;
-    T a[2][KB][V], b[2][KB][V];  // sums over the even and the odd frequencies
-    {
-      T f[V], g[V];
-      unpack(*(const VT*)(dr + (size_t)K * E + lane * V), f);
-      unpack(*(const VT*)(dr + (size_t)(K + 1) * E + lane * V), g);
+    __syncthreads();
+    const T inv = T(1) / T(n);
+    const int L = E / V, items = HP / KB * L;
+    for (int it = tid; it < items; it += THR) {
+      const int lane = it % L, t0 = it / L * KB;
+      T a[2][KB][V], b[2][KB][V];  // sums over the even and the odd frequencies
+      {
+        T f[V], g[V];
+        unpack(*(const VT*)(dr + (size_t)K * E + lane * V), f);
+        unpack(*(const VT*)(dr + (size_t)(K + 1) * E + lane * V), g);
 #pragma unroll
-      for (int q = 0; q < KB; ++q) {
-        const T sg = ((t0 + q) & 1) ? T(-1) : T(1);  // Nyquist: (-1)^t, with the frequencies of m's parity
+        for (int q = 0; q < KB; ++q) {
+          const T sg = ((t0 + q) & 1) ? T(-1) : T(1);  // Nyquist: (-1)^t, with the frequencies of m's parity
 #pragma unroll
-        for (int u = 0; u < V; ++u) {
-          a[0][q][u] = (m & 1) ? f[u] : f[u] + sg * g[u];
-          a[1][q][u] = (m & 1) ? sg * g[u] : T(0);
-          b[0][q][u] = b[1][q][u] = T(0);
+          for (int u = 0; u < V; ++u) {
+            a[0][q][u] = (m & 1) ? f[u] : f[u] + sg * g[u];
+            a[1][q][u] = (m & 1) ? sg * g[u] : T(0);
+            b[0][q][u] = b[1][q][u] = T(0);
+          }
         }
       }
-    }
 #pragma unroll
-    for (int ty = 0; ty < 2; ++ty) {
-      const int rb = ty ? K0 : 0, re = ty ? K : K0;
-      for (int r0 = rb; r0 < re; r0 += 8) {
-        T sr[KB][V], si[KB][V];
+      for (int ty = 0; ty < 2; ++ty) {
+        const int rb = ty ? K0 : 0, re = ty ? K : K0;
+        for (int r0 = rb; r0 < re; r0 += 8) {
+          T sr[KB][V], si[KB][V];
 #pragma unroll
-        for (int q = 0; q < KB; ++q)
+          for (int q = 0; q < KB; ++q)
 #pragma unroll
-          for (int u = 0; u < V; ++u) sr[q][u] = si[q][u] = T(0);
-        const int r1 = min(re, r0 + 8);
+            for (int u = 0; u < V; ++u) sr[q][u] = si[q][u] = T(0);
+          const int r1 = min(re, r0 + 8);
 #pragma unroll 4
-        for (int r = r0; r < r1; ++r) {
-          T pv[V], qv[V];
-          unpack(*(const VT*)(dr + (size_t)r * E + lane * V), pv);
-          unpack(*(const VT*)(di + (size_t)r * E + lane * V), qv);
-          C c[KB];
-          load_row<KB>(tab + (size_t)r * HP + t0, c);
+          for (int r = r0; r < r1; ++r) {
+            T pv[V], qv[V];
+            unpack(*(const VT*)(dr + (size_t)r * E + lane * V), pv);
+            unpack(*(const VT*)(di + (size_t)r * E + lane * V), qv);
+            C c[KB];
+            load_row<KB>(tab + (size_t)r * HP + t0, c);
+#pragma unroll
+            for (int q = 0; q < KB; ++q)
+#pragma unroll
+              for (int u = 0; u < V; ++u) {
+                sr[q][u] = fma(pv[u], c[q].x, sr[q][u]);
+                si[q][u] = fma(qv[u], c[q].y, si[q][u]);
+              }
+          }
 #pragma unroll
           for (int q = 0; q < KB; ++q)
 #pragma unroll
             for (int u = 0; u < V; ++u) {
-              sr[q][u] = fma(pv[u], c[q].x, sr[q][u]);
-              si[q][u] = fma(qv[u], c[q].y, si[q][u]);
+              a[ty][q][u] += sr[q][u];
+              b[ty][q][u] += si[q][u];
             }
         }
-#pragma unroll
-        for (int q = 0; q < KB; ++q)
-#pragma unroll
-          for (int u = 0; u < V; ++u) {
-            a[ty][q][u] += sr[q][u];
-            b[ty][q][u] += si[q][u];
-          }
       }
-    }
-    const long ge = e0 + lane * V;
-    auto put = [&](int t, const T* v) {
-      T* dst = X + (long)t * plane + ge;
-      if (ge + V <= plane && ((uintptr_t)dst & (sizeof(VT) - 1)) == 0) {
-        if constexpr (V == 4) *(float4*)dst = make_float4(v[0], v[1], v[2], v[3]);
-        else *(double2*)dst = make_double2(v[0], v[1]);
-      } else {
+      const long ge = e0 + lane * V;
+      auto put = [&](int t, const T* v) {
+        T* dst = X + (long)t * plane + ge;
+        if (ge + V <= plane && ((uintptr_t)dst & (sizeof(VT) - 1)) == 0) {
+          if constexpr (V == 4) *(float4*)dst = make_float4(v[0], v[1], v[2], v[3]);
+          else *(double2*)dst = make_double2(v[0], v[1]);
+        } else {
 #pragma unroll
-        for (int u = 0; u < V; ++u)
-          if (ge + u < plane) dst[u] = v[u];
-      }
-    };
-#pragma unroll
-    for (int q = 0; q < KB; ++q) {
-      const int t = t0 + q;
-      if (t >= tc) continue;
-      T v[V];
-      if (types == 1) {
-#pragma unroll
-        for (int u = 0; u < V; ++u) v[u] = (a[0][q][u] - b[0][q][u]) * inv;
-        put(t, v);
-        if (t > 0) {
-#pragma unroll
-          for (int u = 0; u < V; ++u) v[u] = (a[0][q][u] + b[0][q][u]) * inv;
-          put(n - t, v);
+          for (int u = 0; u < V; ++u)
+            if (ge + u < plane) dst[u] = v[u];
         }
-        continue;
-      }
+      };
 #pragma unroll
-      for (int u = 0; u < V; ++u) v[u] = ((a[0][q][u] + a[1][q][u]) - (b[0][q][u] + b[1][q][u])) * inv;
-      put(t, v);
-      if (2 * t < m) {
+      for (int q = 0; q < KB; ++q) {
+        const int t = t0 + q;
+        if (t >= tc) continue;
+        T v[V];
+        if (types == 1) {
 #pragma unroll
-        for (int u = 0; u < V; ++u) v[u] = ((a[0][q][u] - a[1][q][u]) + (b[0][q][u] - b[1][q][u])) * inv;
-        put(m - t, v);
-      }
-      if (t > 0) {
+          for (int u = 0; u < V; ++u) v[u] = (a[0][q][u] - b[0][q][u]) * inv;
+          put(t, v);
+          if (t > 0) {
 #pragma unroll
-        for (int u = 0; u < V; ++u) v[u] = ((a[0][q][u] + a[1][q][u]) + (b[0][q][u] + b[1][q][u])) * inv;
-        put(n - t, v);
+            for (int u = 0; u < V; ++u) v[u] = (a[0][q][u] + b[0][q][u]) * inv;
+            put(n - t, v);
+          }
+          continue;
+        }
+#pragma unroll
+        for (int u = 0; u < V; ++u) v[u] = ((a[0][q][u] + a[1][q][u]) - (b[0][q][u] + b[1][q][u])) * inv;
+        put(t, v);
         if (2 * t < m) {
 #pragma unroll
-          for (int u = 0; u < V; ++u) v[u] = ((a[0][q][u] - a[1][q][u]) - (b[0][q][u] - b[1][q][u])) * inv;
-          put(m + t, v);
+          for (int u = 0; u < V; ++u) v[u] = ((a[0][q][u] - a[1][q][u]) + (b[0][q][u] - b[1][q][u])) * inv;
+          put(m - t, v);
+        }
+        if (t > 0) {
+#pragma unroll
+          for (int u = 0; u < V; ++u) v[u] = ((a[0][q][u] + a[1][q][u]) + (b[0][q][u] + b[1][q][u])) * inv;
+          put(n - t, v);
+          if (2 * t < m) {
+#pragma unroll
+            for (int u = 0; u < V; ++u) v[u] = ((a[0][q][u] - a[1][q][u]) - (b[0][q][u] - b[1][q][u])) * inv;
+            put(m + t, v);
+          }
         }
       }
     }
-  }
   }
 }
 
@@ -1095,13 +1096,13 @@ template <typename T>
 static int rdft_tile(int n, long plane) {
   int lg = 9;
   while (lg > 6 && ((size_t)n * sizeof(T) << lg) > 34 * 1024) --lg;
-  while (lg > 5 && cdiv(plane, 1 << lg) < 2 * 152) --lg;
+  while (lg > 5 && cdiv(plane, 1 << lg) < 2 * SMS) --lg;
   return lg;
 }
 // persistent CTAs: as many per SM as registers (the launch bounds) and shared memory allow
 static unsigned rdft_grid(long plane, int lgE, size_t smem, bool inverse) {
   const unsigned fit = std::max<unsigned>(1, 227 * 1024 / (unsigned)(smem + 1024));
-  return std::min<unsigned>(cdiv(plane, 1L << lgE), 152 * std::min(fit, inverse ? 3u : 4u));
+  return std::min<unsigned>(cdiv(plane, 1L << lgE), SMS * std::min(fit, inverse ? 3u : 4u));
 }
 // FP64 arithmetic runs at 1/64 of FP32's rate, so there the operation count decides: picoseconds per
 // sample of the two forms as measured on a 512 x 512 plane (the mixed-radix passes by radix; the
@@ -1150,7 +1151,7 @@ static bool fft_setup(int n, FftPlan* P, size_t* smem) {
 }
 
 // threads per CTA of the register kernels: fewer where the plane would leave SMs idle
-static int reg_fft_threads(long plane) { return cdiv(plane, 128) >= 152 ? 128 : cdiv(plane, 64) >= 152 ? 64 : 32; }
+static int reg_fft_threads(long plane) { return cdiv(plane, 128) >= SMS ? 128 : cdiv(plane, 64) >= SMS ? 64 : 32; }
 
 template <typename T>
 int launch_rfft3(const T* X, cx_t<T>* Xh, long plane, int n3, cudaStream_t s) {

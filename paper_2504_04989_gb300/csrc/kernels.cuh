@@ -74,8 +74,8 @@ inline GemmArgs gemm(char opA, char opB, int M, int N, int K, double alpha, cons
   g.batch = batch;
   return g;
 }
-// Where a tensor-core product says that a wait of its pipeline ran out (its elements are NaN then): *err = 1, unless null.
-// expire (tests): the waits give up at once.  simt: no tensor-core products.
+// Where a tensor-core product says that a wait of its pipeline ran out (its elements are NaN then): *err = 1, unless
+// null. expire (tests): the waits give up at once.  simt: no tensor-core products.
 struct TcOpts {
   int* err = nullptr;
   bool expire = false;

@@ -7,14 +7,14 @@
 // kept in TMEM shrinks by about 2e-8 per instruction, 1.4e-5 after 1024 complex terms), so an accumulator
 // holds 32 terms of K of b0 b0 only, two instructions on products of 16 bits that rarely lose any,
 // and is then read and added to sums in registers, rounded to nearest, in runs of eight
-// readings; the five small products, 2^-9 of those and less, have accumulators of their own that are read once a run.  Two
-// pairs of accumulators alternate so that the reading runs under the next products, and a CTA walks over several tiles so that the next tile's loads and products
-// run under the writing of this one.  Against exact dot products the result is closer than FP32
-// multiply-adds' at every K (the figures stand at sgemm_tc_better).
+// readings; the five small products, 2^-9 of those and less, have accumulators of their own that are read once a run.
+// Two pairs of accumulators alternate so that the reading runs under the next products, and a CTA walks over several
+// tiles so that the next tile's loads and products run under the writing of this one.  Against exact dot products the
+// result is closer than FP32 multiply-adds' at every K (the figures stand at sgemm_tc_better).
 //
-// Near the ends of FP32's range the parts or their products leave it: an entry below 2^-100 (its b2), a sum below 2^-98 per
-// term with products below 2^-100 in it, results that are not finite.  The pass over the operands notes how small the
-// entries of each row get, and the elements concerned are left to k_redo.
+// Near the ends of FP32's range the parts or their products leave it: an entry below 2^-100 (its b2), a sum below
+// 2^-98 per term with products below 2^-100 in it, results that are not finite.  The pass over the operands notes how
+// small the entries of each row get, and the elements concerned are left to k_redo.
 //
 // A complex product is the real product of the interleaved rows of op(A) with the
 // expanded real form of op(B) (rows 2n and 2n + 1 per column n, as in tc_gemm.cu),
@@ -284,7 +284,8 @@ __global__ void __launch_bounds__(SG_THREADS, 1) k_sgemm_tc(const __grid_constan
         }
       }
       if (!ok && lane == 0 && st.err) atomicExch(st.err, 1);
-      // results that are not finite, or entries near the lower end of the range: the warp looks which of its elements (rare)
+      // results that are not finite, or entries near the lower end of the range: the warp looks which of its elements
+      // (rare)
       float zero = 0.f;
 #pragma unroll
       for (int q = 0; q < SG_OUT; ++q) zero = fmaf(tot[q], 0.f, zero);
@@ -386,25 +387,25 @@ size_t sgemm_tc_bytes(int M, int N, int K, int batch) {
 
 // Estimated times in microseconds of the two forms: a SIMT tile takes 0.104 (64 x 64) or 0.25 us (128 x
 // 64) per term of K and SM, K split as cgemm splits it.  Measured, product with its operand pass: 1024 x
-// 1024 x 1024 on 33 slices 5.08 -> 1.61 ms (the product alone 1.28: 220 TFLOP/s).  Error, 2-norm, in 2^-24, normal data,
-// K = 32, 60, 128, 512, 2048: 0.8, 0.9, 1.1, 1.4, 1.7, the SIMT kernels 1.7, 2.3, 3.4, 6.8, 13.6; positive data 0.8, 0.9, 1.1, 1.0,
-// 1.2, SIMT 1.4, 2.0, 2.9, 5.9, 11.7 (two TF32 parts and three products, as this was: 2.1 .. 2.6 and 1.7 .. 1.9, from K = 56 on
-// below SIMT only).
+// 1024 x 1024 on 33 slices 5.08 -> 1.61 ms (the product alone 1.28: 220 TFLOP/s).  Error, 2-norm, in 2^-24, normal
+// data, K = 32, 60, 128, 512, 2048: 0.8, 0.9, 1.1, 1.4, 1.7, the SIMT kernels 1.7, 2.3, 3.4, 6.8, 13.6; positive data
+// 0.8, 0.9, 1.1, 1.0, 1.2, SIMT 1.4, 2.0, 2.9, 5.9, 11.7 (two TF32 parts and three products, as this was: 2.1 .. 2.6
+// and 1.7 .. 1.9, from K = 56 on below SIMT only).
 bool sgemm_tc_better(const GemmArgs& g, size_t bytes) {
   if (g.K < 1 || g.M < 1 || g.N < 1 || g.K > (1 << 24)) return false;
   const size_t slice = sg_slice_bytes(g.M, g.N, g.K) + 2048;
   if (bytes < slice) return false;
   const double wtiles = (double)cdiv(g.M, 128) * cdiv(g.N, 64) * g.batch;
-  const bool wide = g.K >= 1024 || wtiles >= 2 * 152;
+  const bool wide = g.K >= 1024 || wtiles >= 2 * SMS;
   const double stiles = wide ? wtiles : (double)cdiv(g.M, 64) * cdiv(g.N, 64) * g.batch;
-  double ks = std::min(16.0, std::max(1.0, std::floor(wide ? (4 * 152 + stiles - 1) / stiles : 2 * 152 / stiles)));
+  double ks = std::min(16.0, std::max(1.0, std::floor(wide ? (4 * SMS + stiles - 1) / stiles : 2 * SMS / stiles)));
   ks = std::min(ks, std::max(1.0, g.K / 64.0));
-  const double simt = 4.0 + (ks > 1.0 ? 3.0 : 0.0) + std::ceil(stiles * ks / 152) * (g.K / ks) * (wide ? 0.25 : 0.104);
+  const double simt = 4.0 + (ks > 1.0 ? 3.0 : 0.0) + std::ceil(stiles * ks / SMS) * (g.K / ks) * (wide ? 0.25 : 0.104);
   const double tiles = (double)cdiv(g.M, SG_BM) * cdiv(2L * g.N, SG_BN) * g.batch;
   const double tile_us = 3.0 + cdiv(2L * g.K, SG_KB) * 0.55;
   const double pack_us = ((double)slice * 1.4 * g.batch) / 4.0e6;
   const double calls = std::ceil((double)g.batch * slice / (double)bytes);
-  return simt > 10.0 * calls + pack_us + std::ceil(tiles / 152.0) * tile_us;
+  return simt > 10.0 * calls + pack_us + std::ceil(tiles / SMS) * tile_us;
 }
 
 int sgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s, TcOpts st) {
@@ -438,7 +439,7 @@ int sgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s, TcOpts s
     TSVD_TRY(split_map(&mb, DB, N2, 2 * g.K, ldk, n * SG_D));
     const long tiles = (long)cdiv(N2, SG_BN) * cdiv(g.M, SG_BM) * n;
     float2* Cb = (float2*)g.C + (long)b0 * g.sC;
-    k_sgemm_tc<<<(unsigned)std::min<long>(tiles, 152), SG_THREADS, SG_SMEM, s>>>(
+    k_sgemm_tc<<<(unsigned)std::min<long>(tiles, SMS), SG_THREADS, SG_SMEM, s>>>(
         ma, mb, lowA, lowB, marks, Cb, g.ldc, g.sC, g.M, g.N, g.K, n, (float)g.alpha, g.beta != 0.0, st);
     TSVD_LAUNCHED();
     TSVD_TRY(redo_marked<float2>(marks, {A, B, g.lda, g.sA, g.ldb, g.sB, g.K, g.opA == 'H', g.opB == 'H'}, Cb,

@@ -14,8 +14,8 @@
 // lanes (C = alpha A B^T + beta C, the old values loaded before any store).  A
 // CTA walks over several tiles with two accumulators, so the next tile's loads
 // and products run under the storing of this one (2048 x 120 x 360 on 65 slices,
-// added to C with split copies: 357 -> 258 us; TF32, 2048 x 120 x 2048: 470 -> 440).  Every wait is bounded: on a timeout the kernel records
-// an error flag instead of hanging.  The split-TF32 epilogue can also write
+// added to C with split copies: 357 -> 258 us; TF32, 2048 x 120 x 2048: 470 -> 440).  Every wait is bounded: on a
+// timeout the kernel records an error flag instead of hanging.  The split-TF32 epilogue can also write
 // hi / lo copies of C for a following product.
 //
 // A third mode keeps FP32 accuracy on the TF32 units ("split TF32"): each
@@ -323,7 +323,7 @@ static int tc_launch(const CUtensorMap& ta, const CUtensorMap& tb, const CUtenso
     cudaGetLastError();
     return TSVD_ERR_CUDA;
   }
-  k_tc_gemm<MODE, BN><<<(unsigned)std::min<long>(tiles, 152), TC_THREADS, tc_smem<MODE, BN>(), s>>>(
+  k_tc_gemm<MODE, BN><<<(unsigned)std::min<long>(tiles, SMS), TC_THREADS, tc_smem<MODE, BN>(), s>>>(
       ta, tb, ta2, tb2, C, ldc, sC, M, N, nk, batch, err, alpha, beta, o2);
   TSVD_LAUNCHED();
   return TSVD_OK;
@@ -360,7 +360,7 @@ int tc_gemm_split(const float* Ahi, const float* Alo, long lda, long sA, int M, 
   // clock), so a term of K costs a tile of 256 about 1.5 times one of 128.  The 48 products of a T-SVD
   // of 2048 x 2048 x 128 took 12.2 ms with 128 columns throughout, 11.1 so (one tile per CTA).
   const long rows = (long)cdiv(M, TC_BM) * batch;
-  const bool wide = 3 * cdiv(rows * cdiv(N, 256), 152) <= 2 * cdiv(rows * cdiv(N, 128), 152);
+  const bool wide = 3 * cdiv(rows * cdiv(N, 256), SMS) <= 2 * cdiv(rows * cdiv(N, 128), SMS);
   const int bn = wide ? 256 : 128, row = wide ? 64 : 128;
   CUtensorMap ta, tb, ta2, tb2;
   TSVD_TRY(make_map(&ta, Ahi, M, K, lda, sA, batch, false, TC_BM, row));
@@ -500,7 +500,7 @@ static int split_fill(const float* x, long ldx, float* hi, float* lo, long ldy, 
                    cols % 4 == 0 && fill % 4 == 0;
   int lg = 0;
   while (lg < 5 && (vec ? 4 : 1) << lg < fill) ++lg;
-  const unsigned grid = (unsigned)std::min<long>(cdiv(rows, 8L << (5 - lg)), 152 * 16);
+  const unsigned grid = (unsigned)std::min<long>(cdiv(rows, 8L << (5 - lg)), SMS * 16);
   if (vec) k_split_rows<4><<<grid, 256, 0, s>>>(x, ldx, hi, lo, ldy, cols, fill, rows, lg);
   else k_split_rows<1><<<grid, 256, 0, s>>>(x, ldx, hi, lo, ldy, cols, fill, rows, lg);
   TSVD_LAUNCHED();

@@ -6,8 +6,8 @@
 // readers took 0.4 ms for 1024 terms, and the waits give up after a second).  Few elements are taken from the
 // list, a warp each with its lanes along K, spread over the GPU; where there are more than the list
 // holds, the tiles with marks are computed as k_cgemm does.  Without marks it reads one word.
-// t-product of 512 x 512 x 512, n3 = 16, against sums by the product's own readers: FP32 (finite data: 106 us) one row not
-// finite 695 -> 153 us, every row 6212 -> 748; FP64 (finite: 490) 3412 -> 522 and 14120 -> 8720.
+// t-product of 512 x 512 x 512, n3 = 16, against sums by the product's own readers: FP32 (finite data: 106 us) one
+// row not finite 695 -> 153 us, every row 6212 -> 748; FP64 (finite: 490) 3412 -> 522 and 14120 -> 8720.
 #pragma once
 
 #include <algorithm>
@@ -106,7 +106,8 @@ constexpr int REDO_RUN = 16;  // terms added one after another, then the runs: t
 template <typename C>
 constexpr int redo_tile() { return sizeof(C) == 16 ? 16 : 32; }
 
-// upper: a Hermitian product, whose tiles of 128 rows x 32 columns wholly below the diagonal were left out (no marks there)
+// upper: a Hermitian product, whose tiles of 128 rows x 32 columns wholly below the diagonal were left out (no marks
+// there)
 template <typename C>
 __global__ void __launch_bounds__(REDO_THREADS, 8) k_redo(const Marks<C> mk, const __grid_constant__ DotSrc<C> src,
                                                        C* __restrict__ Cm, long ldc, long sC, int M, int N, int batch,
@@ -218,7 +219,7 @@ int redo_marked(const Marks<C>& mk, const DotSrc<C>& src, C* Cm, long ldc, long 
                 double alpha, bool beta, bool upper, cudaStream_t s) {
   constexpr int BT = redo_tile<C>();
   const long tiles = (long)cdiv(M, BT) * cdiv(N, BT) * batch;
-  k_redo<C><<<(unsigned)std::min<long>(tiles, 152 * 8), REDO_THREADS, 0, s>>>(mk, src, Cm, ldc, sC, M, N, batch, alpha,
+  k_redo<C><<<(unsigned)std::min<long>(tiles, SMS * 8), REDO_THREADS, 0, s>>>(mk, src, Cm, ldc, sC, M, N, batch, alpha,
                                                                                beta ? 1 : 0, upper ? 1 : 0);
   TSVD_LAUNCHED();
   return TSVD_OK;
