@@ -541,6 +541,7 @@ def rbk_fourier(Ahat, n3, k0, R, P=10, q=2, seed=0, precision="fp32", omega=None
     p = _lib.TsvdParams(R=int(R), P=int(P), q=int(q), precision=pr, seed=int(seed), flags=_flags(**{
         "fp64_qr": flags.get("fp64_qr", False), "alg1": flags.get("alg1", False),
         "q_trunc": flags.get("q_trunc", False), "deflate": flags.get("deflate", False)}))
+    dev = Ahat.device
     ws = _workspace_for(_sized_params(lib.tsvd_rbk_fourier_workspace_size, n1, n2, n3, k0, ns, params=p,
                                       what="tsvd_rbk_fourier_workspace_size"), dev)
     Uh = torch.empty((ns, n1, R), dtype=cdt, device=dev)
