@@ -44,33 +44,23 @@ def _workspace(nbytes, device):
     return torch.empty(max(int(nbytes), 256), dtype=torch.uint8, device=device)
 
 
-def _workspace_for(size, device):
-    """The workspace that size(0) asks for or, where that is more than the device has left, the least
-    with which the call runs, size(TSVD_WS_LEAST)."""
+def _workspace_for(device, what, call, args, last):
+    """The workspace that a *_workspace_size call asks for (last: its precision or params) or, where that is more
+    than the device has left, the least with which the call it belongs to runs (TSVD_WS_LEAST)."""
+    nbytes = C.c_size_t()
+    whole = isinstance(last, int)
+    _lib.check(call(*args, last if whole else C.byref(last), C.byref(nbytes)), what)
     try:
-        return _workspace(size(0), device)
+        return torch.empty(max(nbytes.value, 256), dtype=torch.uint8, device=device)
     except torch.OutOfMemoryError:
-        return _workspace(size(_lib.TSVD_WS_LEAST), device)
-
-
-def _sized(call, *args, precision, what):
-    """size function for _workspace_for of a *_workspace_size call that takes its precision last"""
-    def size(flag):
-        nbytes = C.c_size_t()
-        _lib.check(call(*args, precision | flag, C.byref(nbytes)), what)
-        return nbytes.value
-    return size
-
-
-def _sized_params(call, *args, params, what):
-    """the same of a call that takes params"""
-    def size(flag):
-        p = _lib.TsvdParams.from_buffer_copy(params)
-        p.flags |= flag
-        nbytes = C.c_size_t()
-        _lib.check(call(*args, C.byref(p), C.byref(nbytes)), what)
-        return nbytes.value
-    return size
+        pass
+    if whole:
+        last |= _lib.TSVD_WS_LEAST
+    else:
+        last = _lib.TsvdParams.from_buffer_copy(last)
+        last.flags |= _lib.TSVD_WS_LEAST
+    _lib.check(call(*args, last if whole else C.byref(last), C.byref(nbytes)), what)
+    return _workspace(nbytes.value, device)
 
 
 def _flags(fp64_qr, alg1, q_trunc, deflate=False, gram_int=False):
@@ -104,8 +94,7 @@ def rbk(A, R, P=10, q=2, seed=0, precision="fp32", omega=None, return_info=False
     flags = _flags(fp64_qr, alg1, q_trunc, deflate, gram_int)
     p = _lib.TsvdParams(R=int(R), P=int(P), q=int(q), precision=pr, seed=int(seed), flags=flags)
     dev = A.device
-    ws = _workspace_for(_sized_params(lib.tsvd_rbk_workspace_size, n1, n2, n3, params=p,
-                                      what="tsvd_rbk_workspace_size"), dev)
+    ws = _workspace_for(dev, "tsvd_rbk_workspace_size", lib.tsvd_rbk_workspace_size, (n1, n2, n3), p)
     h = n3 // 2 + 1
     U = torch.empty((n3, n1, R), dtype=dt, device=dev)
     S = torch.empty((n3, R), dtype=dt, device=dev)
@@ -138,8 +127,7 @@ class RbkPlan:
                                  flags=flags)
         self.shape = (n1, n2, n3)
         self.device = torch.device(device)
-        self.ws = _workspace_for(_sized_params(self.lib.tsvd_rbk_workspace_size, n1, n2, n3, params=self.p,
-                                               what="workspace"), self.device)
+        self.ws = _workspace_for(self.device, "workspace", self.lib.tsvd_rbk_workspace_size, (n1, n2, n3), self.p)
         self.nbytes = self.ws.numel()
         self.U = torch.empty((n3, n1, R), dtype=self.dt, device=self.device)
         self.S = torch.empty((n3, R), dtype=self.dt, device=self.device)
@@ -189,19 +177,18 @@ class RbkBatchPlan:
             d.sigma_hat = self.sig[-1].data_ptr()
         self.count = n
 
-        def size(flag):
+        def size():
             nbytes = C.c_size_t()
-            for d in self.descs[:n]:
-                d.params.flags |= flag
-            try:
-                _lib.check(self.lib.tsvd_rbk_batched_workspace_size(self.descs, n, self.lanes, C.byref(nbytes)),
-                           "tsvd_rbk_batched_workspace_size")
-            finally:
-                for d in self.descs[:n]:
-                    d.params.flags &= ~flag
+            _lib.check(self.lib.tsvd_rbk_batched_workspace_size(self.descs, n, self.lanes, C.byref(nbytes)),
+                       "tsvd_rbk_batched_workspace_size")
             return nbytes.value
 
-        self.ws = _workspace_for(size, self.device)
+        try:
+            self.ws = _workspace(size(), self.device)
+        except torch.OutOfMemoryError:  # the least instead, as _workspace_for
+            for d in self.descs[:n]:
+                d.params.flags |= _lib.TSVD_WS_LEAST
+            self.ws = _workspace(size(), self.device)
         self.nbytes = self.ws.numel()
         self.graph = None
         if graph:
@@ -249,7 +236,7 @@ def _tprod_raw(A, B, precision):
     n3b, n2b, n4 = B.shape
     if n3b != n3 or n2b != n2:
         raise ValueError("tprod: shapes (n3,n1,n2) and (n3,n2,n4) required")
-    ws = _workspace_for(_sized(lib.tprod_workspace_size, n1, n2, n4, n3, precision=pr, what="tprod_workspace_size"), A.device)
+    ws = _workspace_for(A.device, "tprod_workspace_size", lib.tprod_workspace_size, (n1, n2, n4, n3), pr)
     out = torch.empty((n3, n1, n4), dtype=A.dtype, device=A.device)
     with torch.cuda.device(A.device):
         _lib.check(lib.tprod(_ptr(A), _ptr(B), _ptr(out), n1, n2, n4, n3, pr, _ptr(ws), ws.numel(),
@@ -265,7 +252,7 @@ def tprod_backward(A, B, dC, precision="fp32", need_dA=True, need_dB=True):
     _need_cuda(A, B, dC, dtype=_DT[precision])
     n3, n1, n2 = A.shape
     n4 = B.shape[2]
-    ws = _workspace_for(_sized(lib.tprod_backward_workspace_size, n1, n2, n4, n3, precision=pr, what="workspace"), A.device)
+    ws = _workspace_for(A.device, "workspace", lib.tprod_backward_workspace_size, (n1, n2, n4, n3), pr)
     dA = torch.empty_like(A) if need_dA else None
     dB = torch.empty_like(B) if need_dB else None
     with torch.cuda.device(A.device):
@@ -281,7 +268,7 @@ def _tproj_raw(Q, A, precision):
     _need_cuda(Q, A, dtype=_DT[precision])
     n3, n1, m = Q.shape
     n2 = A.shape[2]
-    ws = _workspace_for(_sized(lib.tproj_workspace_size, n1, m, n2, n3, precision=pr, what="workspace"), Q.device)
+    ws = _workspace_for(Q.device, "workspace", lib.tproj_workspace_size, (n1, m, n2, n3), pr)
     Y = torch.empty_like(A)
     with torch.cuda.device(Q.device):
         _lib.check(lib.tproj(_ptr(Q), _ptr(A), _ptr(Y), n1, m, n2, n3, pr, _ptr(ws), ws.numel(),
@@ -297,7 +284,7 @@ def tproj_backward(Q, A, dY, precision="fp32", need_dQ=True, need_dA=True):
     _need_cuda(Q, A, dY, dtype=_DT[precision])
     n3, n1, m = Q.shape
     n2 = A.shape[2]
-    ws = _workspace_for(_sized(lib.tproj_backward_workspace_size, n1, m, n2, n3, precision=pr, what="workspace"), Q.device)
+    ws = _workspace_for(Q.device, "workspace", lib.tproj_backward_workspace_size, (n1, m, n2, n3), pr)
     dQ = torch.empty_like(Q) if need_dQ else None
     dA = torch.empty_like(A) if need_dA else None
     with torch.cuda.device(Q.device):
@@ -459,7 +446,7 @@ def tqr(A, precision=None, return_info=False):
     _need_cuda(A, dtype=_DT[precision])
     n3, n1, n2 = A.shape
     p = min(n1, n2)
-    ws = _workspace_for(_sized(lib.tqr_workspace_size, n1, n2, n3, precision=pr, what="tqr_workspace_size"), A.device)
+    ws = _workspace_for(A.device, "tqr_workspace_size", lib.tqr_workspace_size, (n1, n2, n3), pr)
     Q = torch.empty((n3, n1, p), dtype=A.dtype, device=A.device)
     R = torch.empty((n3, p, n2), dtype=A.dtype, device=A.device)
     info = _lib.TsvdInfo()
@@ -481,8 +468,7 @@ def tpinv(A, precision=None, return_info=False):
     A = A.contiguous()
     _need_cuda(A, dtype=_DT[precision])
     n3, n1, n2 = A.shape
-    ws = _workspace_for(_sized(lib.tpinv_workspace_size, n1, n2, n3, precision=pr, what="tpinv_workspace_size"),
-                        A.device)
+    ws = _workspace_for(A.device, "tpinv_workspace_size", lib.tpinv_workspace_size, (n1, n2, n3), pr)
     X = torch.empty((n3, n2, n1), dtype=A.dtype, device=A.device)
     info = _lib.TsvdInfo()
     with torch.cuda.device(A.device):
@@ -542,8 +528,8 @@ def rbk_fourier(Ahat, n3, k0, R, P=10, q=2, seed=0, precision="fp32", omega=None
         "fp64_qr": flags.get("fp64_qr", False), "alg1": flags.get("alg1", False),
         "q_trunc": flags.get("q_trunc", False), "deflate": flags.get("deflate", False)}))
     dev = Ahat.device
-    ws = _workspace_for(_sized_params(lib.tsvd_rbk_fourier_workspace_size, n1, n2, n3, k0, ns, params=p,
-                                      what="tsvd_rbk_fourier_workspace_size"), dev)
+    ws = _workspace_for(dev, "tsvd_rbk_fourier_workspace_size", lib.tsvd_rbk_fourier_workspace_size,
+                        (n1, n2, n3, k0, ns), p)
     Uh = torch.empty((ns, n1, R), dtype=cdt, device=dev)
     Vh = torch.empty((ns, n2, R), dtype=cdt, device=dev)
     sig = torch.empty((ns, R), dtype=torch.float64, device=dev)
@@ -563,8 +549,8 @@ def rbk_fourier(Ahat, n3, k0, R, P=10, q=2, seed=0, precision="fp32", omega=None
 def lowrank_workspace(U, V):
     """The workspace of lowrank for factors of these shapes."""
     n3, n1, R = U.shape
-    return _workspace_for(_sized(_lib.load().tsvd_lowrank_workspace_size, n1, V.shape[1], n3, R,
-                                 precision=_prec(_precision_of(U, None)), what="lowrank ws"), U.device)
+    return _workspace_for(U.device, "lowrank ws", _lib.load().tsvd_lowrank_workspace_size, (n1, V.shape[1], n3, R),
+                          _prec(_precision_of(U, None)))
 
 
 def lowrank(U, S, V, out=None, ws=None):
