@@ -403,9 +403,9 @@ def main():
         t = stages[stage] * 1e-3
         if "flops" in work:
             if args.precision == "fp64" and stage != "eig_hetrd":
-                # exact digit products on the BF16 tensor cores, 34 digit pairs
+                # exact digit products on the BF16 tensor cores, 36 digit pairs
                 peak = pk.get("bf16_tflops")
-                peak, src = peak and peak / 34, "MEASURED_PEAKS.json bf16_tflops / 34 (digit-pair products)"
+                peak, src = peak and peak / 36, "MEASURED_PEAKS.json bf16_tflops / 36 (digit-pair products)"
             elif args.precision == "fp64":
                 peak, src = alu["fp64"], "measured here: cuBLAS FP64 GEMM"
             elif stage == "eig_hetrd":
