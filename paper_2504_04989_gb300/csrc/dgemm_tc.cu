@@ -23,8 +23,12 @@
 // times R^-1, C^H times U_c and U S times V^H become even; (2) every element shows that its terms are not
 // small next to its scales, or is left to k_redo, which adds them up in FP64:
 //   |C_ij| is at least 2^-7 of (scale of row i) (scale of column j), or
-//   the entry of row i that meets the largest one of column j is within 2^-5 of its scale, or the other way round.
-// Either says that sum |a||b| is at least 2^-7 of the scales, against an error of at most about 2^-59 of them per
+//   the entry of row i that meets the largest one of column j is within 2^-5 of its scale, or the other way round, or
+//   the entries within 2^-5 and within 2^-8 of their scales that meet one another add up to 2^-7: bits of the two
+//   levels, counted word by word until they do.  This shows it for the products of orthonormal columns, which cancel
+//   to zeros, where the columns are concentrated and have their largest entries in different rows (of a
+//   2048 x 2048 x 128 T-SVD's Q^H Q and Q^H W the two tests above leave 7 to 25 % of the elements, this one 1 %).
+// Each says that sum |a||b| is at least 2^-7 of the scales, against an error of at most about 2^-59 of them per
 // term: 2.4 times the worst case of FP64 multiply-adds, 2 K u sum |a||b|, where those are only just met.  Errors as
 // measured stand at dgemm_tc_better.
 //
@@ -86,7 +90,7 @@ struct DigOp {
   int sign;    // its entries of k take sign * shift[k] to their exponents
   // [batch][rows] 2^32 (bound of the row's exponents + DG_OFF, 0, DG_INF) + the k of the largest entry
   unsigned long long* top;
-  uint32_t* near;           // [batch][rows][K / 32] which entries are within 2^-5 of that bound
+  uint2* near;              // [batch][rows][K / 32] which entries are within 2^-5 and within 2^-8 of that bound
   uint32_t* D;              // digit planes, [batch][8][rows, or 2 rows for op(B)][ldk]
   __host__ __device__ unsigned expo_blocks(int K) const {
     return trans ? (unsigned)((rows + 31) / 32) * ((K + 63) / 64) : (unsigned)((rows + 7) / 8);
@@ -276,7 +280,9 @@ __global__ void __launch_bounds__(256) k_dig_pack(const DigOp A, const DigOp B, 
     double2 v = make_double2(0.0, 0.0);
     if (in) v = o.trans ? t[tx][ty + 8 * i] : S[(long)r * o.ld + k];
     const long long X = digit_int(v.x, e), Y = digit_int(v.y, e);
-    const unsigned near = __ballot_sync(0xffffffffu, max(llabs(X), llabs(Y)) >= 1ll << 57);
+    const long long big = max(llabs(X), llabs(Y));
+    const uint2 near =
+        make_uint2(__ballot_sync(0xffffffffu, big >= 1ll << 57), __ballot_sync(0xffffffffu, big >= 1ll << 54));
     if (tx == 0) o.near[br * kblocks + blk % kblocks] = near;
     if (!in) continue;
     const unsigned long long x = 0x8080808080808080ull + X, y = 0x8080808080808080ull + Y;
@@ -318,8 +324,8 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dgemm_tc(const __grid_constan
                                                             const __grid_constant__ CUtensorMap tmB,
                                                             const unsigned long long* __restrict__ topA,
                                                             const unsigned long long* __restrict__ topB,
-                                                            const uint32_t* __restrict__ nearA,
-                                                            const uint32_t* __restrict__ nearB,
+                                                            const uint2* __restrict__ nearA,
+                                                            const uint2* __restrict__ nearB,
                                                             const __grid_constant__ Marks<double2> marks,
                                                             double2* __restrict__ C, long ldc, long sC, int M, int N,
                                                             int K, int batch, double alpha, int beta, int upper,
@@ -501,7 +507,18 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dgemm_tc(const __grid_constan
         bool mark = ok && row < M && min(ea, eb) > 0 && !large(hi[q], lo[q]) && !large(hi[q + 1], lo[q + 1]);
         if (mark) {
           const int ka = (int)(uint32_t)ta, kb = (int)(uint32_t)tb, kw = (K + 31) / 32;
-          mark = !((nearA[ra * kw + kb / 32] >> (kb & 31) | nearB[rb * kw + ka / 32] >> (ka & 31)) & 1u);
+          const uint2 *na = nearA + ra * kw, *nb = nearB + rb * kw;
+          mark = !((na[kb / 32].x >> (kb & 31) | nb[ka / 32].x >> (ka & 31)) & 1u);
+          if (mark) {
+            // each pair is worth the product of its levels, 2^-5 = 2^-8 (1 + 7): in units of 2^-16
+            int sum = 0;
+#pragma unroll 4
+            for (int w = 0; w < kw && sum < 512; ++w) {
+              const uint2 x = na[w], y = nb[w];
+              sum += __popc(x.y & y.y) + 7 * (__popc(x.x & y.y) + __popc(x.y & y.x)) + 49 * __popc(x.x & y.x);
+            }
+            mark = sum < 512;
+          }
         }
         mark |= ok && row < M && max(ea, eb) >= DG_INF;
         marks.put(M, N, w.bz, row0, col, mark, row, col, lane);
@@ -542,7 +559,7 @@ static int digit_map(CUtensorMap* tm, const void* ptr, int rows, int K2, long ld
 
 static long dg_ldk(int K) { return (2L * K + 7) / 8 * 8; }
 static size_t dg_slice_bytes(int M, int N, int K) {
-  return (size_t)DG_D * dg_ldk(K) * 2 * (M + 2 * (size_t)N) + (8 + 4 * (size_t)((K + 31) / 32)) * ((size_t)M + N) +
+  return (size_t)DG_D * dg_ldk(K) * 2 * (M + 2 * (size_t)N) + 8 * (1 + (size_t)((K + 31) / 32)) * ((size_t)M + N) +
          16 * (size_t)K + Marks<double2>::bytes(M, N, 1);
 }
 size_t dgemm_tc_bytes(int M, int N, int K, int batch) {
@@ -585,8 +602,8 @@ int dgemm_tc(const GemmArgs& g, void* ws, size_t bytes, cudaStream_t s, bool upp
   unsigned long long* topA = (unsigned long long*)(stat + (size_t)nb * g.K);
   unsigned long long* topB = topA + (size_t)nb * g.M;
   const size_t kw = cdiv(g.K, 32);
-  uint32_t* nearA = (uint32_t*)(topB + (size_t)nb * g.N);
-  uint32_t* nearB = nearA + (size_t)nb * g.M * kw;
+  uint2* nearA = (uint2*)(topB + (size_t)nb * g.N);
+  uint2* nearB = nearA + (size_t)nb * g.M * kw;
   const Marks<double2> marks = Marks<double2>::at(up((uintptr_t)(nearB + (size_t)nb * g.N * kw)), g.M, g.N, nb);
   if (cudaFuncSetAttribute(k_dgemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, DG_SMEM) != cudaSuccess) {
     cudaGetLastError();
