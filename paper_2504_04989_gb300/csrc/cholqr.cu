@@ -40,6 +40,8 @@ namespace tsvd {
 // smallest tiles that fit (an instruction costs the same whatever the lanes).
 // Against one step and barrier per row, 33 slices: FP32 nb = 25: 23 -> 16 us, 60:
 // 59 -> 29, 120: 272 -> 61; FP64 15: 35 -> 28, 60: 271 -> 202, 120: 1910 -> 1240.
+// Roots of FP32 pivots by root and division instead of the estimate: + 11 % (60 on 33 slices 24.6 -> 27.4 us, 120 on
+// 65 slices 56.5 -> 62.2, as they run in a T-SVD).
 // ---------------------------------------------------------------------------
 
 __device__ __forceinline__ float2 shfl_c(float2 v, int l) {
